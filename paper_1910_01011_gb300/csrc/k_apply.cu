@@ -20,6 +20,7 @@
 //   s = delta.(2D + delta) = r^2 - R_c^2,   r - R_c = s / (r + R_c),
 //   phase = (Re k R_c mod 2 pi, FP64) + Re k (r - R_c).
 #include <cstdio>
+#include <type_traits>
 
 #include "internal.h"
 #include "pair_math.h"
@@ -89,51 +90,67 @@ __device__ __forceinline__ float reduce_phase(double t) {
 
 // ----------------------------------------------------------------- gather (trial densities)
 
-__global__ void gather_kernel(GatherArgs a) {
-    const int64_t s = a.s_begin + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= a.s_end) return;
-    int4 v = a.slot_v[s];
+// One thread per (triangle, rule point): each point takes ~16 FP64
+// operations, which GB300 issues at 1/64 of its FP32 rate, so the kernel is
+// bound by how many SMs share them (one thread per triangle: 10 us at any
+// size up to a few thousand triangles; now 6-7 us, cold caches).  Thread q of a triangle
+// also forms one of the six real curl components.
+constexpr int GATHER_THREADS = 96;  // 16 triangles
+static_assert(GATHER_THREADS % QP == 0 && QP == 6, "six threads per triangle, one curl component each");
+
+__global__ void __launch_bounds__(GATHER_THREADS) gather_kernel(GatherArgs a) {
+    const int64_t i = a.s_begin * QP + (int64_t)blockIdx.x * GATHER_THREADS + threadIdx.x;
+    const int64_t s = i / QP;
+    const int q = (int)(i - s * QP);
+    const bool live = s < a.s_end;
+    const int4 v = live ? a.slot_v[s] : make_int4(-1, -1, -1, 0);
+    const bool real = v.x >= 0;
     double2 xs[3], xf[3];
-    bool real = v.x >= 0;
+#pragma unroll
     for (int k = 0; k < 3; k++) {
-        int vid = k == 0 ? v.x : k == 1 ? v.y : v.z;
-        if (real) {
-            xs[k] = a.x[a.v_dof1[vid]];
-            xf[k] = a.x[a.v_dof2[vid]];
-        } else {
-            xs[k] = make_double2(0, 0);
-            xf[k] = make_double2(0, 0);
-        }
+        const int vid = k == 0 ? v.x : k == 1 ? v.y : v.z;
+        xs[k] = real ? a.x[a.v_dof1[vid]] : make_double2(0, 0);
+        xf[k] = real ? a.x[a.v_dof2[vid]] : make_double2(0, 0);
     }
-    float4 p32[QP];
-    for (int q = 0; q < QP; q++) {
-        double w = real ? a.pt_w[s * QP + q] : 0.0;
-        double sr = 0, si = 0, dr = 0, di = 0;
-        for (int k = 0; k < 3; k++) {
-            sr += a.lam[q][k] * xs[k].x;
-            si += a.lam[q][k] * xs[k].y;
-            dr += a.lam[q][k] * xf[k].x;
-            di += a.lam[q][k] * xf[k].y;
-        }
-        p32[q] = make_float4((float)(w * sr), (float)(w * si), (float)(w * dr), (float)(w * di));
-        if (a.pd64) a.pd64[s * QP + q] = make_double4(w * sr, w * si, w * dr, w * di);
+    const double w = real ? a.pt_w[i] : 0.0;
+    double sr = 0, si = 0, dr = 0, di = 0;
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const double l = a.lam[q][k];
+        sr += l * xs[k].x;
+        si += l * xs[k].y;
+        dr += l * xf[k].x;
+        di += l * xf[k].y;
     }
-    if (a.pd32) pair_interleave(p32, a.pd32 + s * QP);
-    double cr[3] = {0, 0, 0}, ci[3] = {0, 0, 0};
+    sr *= w;
+    si *= w;
+    dr *= w;
+    di *= w;
+    // curl component c, real (q < 3) or imaginary part
+    const int c = q < 3 ? q : q - 3;
+    double cu = 0;
     if (real)
-        for (int k = 0; k < 3; k++)
-            for (int c = 0; c < 3; c++) {
-                double cu = a.slot_curl[s * 9 + 3 * k + c];
-                cr[c] += xf[k].x * cu;
-                ci[c] += xf[k].y * cu;
-            }
+#pragma unroll
+        for (int k = 0; k < 3; k++) cu += (q < 3 ? xf[k].x : xf[k].y) * a.slot_curl[s * 9 + 3 * k + c];
+    if (a.pd32) {
+        // pair-interleaved: the even point of a pair writes (x_a, x_b, y_a, y_b), the odd one (z_a, z_b, w_a, w_b)
+        const float4 p = make_float4((float)sr, (float)si, (float)dr, (float)di);
+        const bool odd = q & 1;
+        const float ox = __shfl_xor_sync(0xffffffffu, odd ? p.x : p.z, 1);
+        const float oy = __shfl_xor_sync(0xffffffffu, odd ? p.y : p.w, 1);
+        if (live) a.pd32[i] = odd ? make_float4(ox, p.z, oy, p.w) : make_float4(p.x, ox, p.y, oy);
+    }
+    if (!live) return;
+    if (a.pd64) a.pd64[i] = make_double4(sr, si, dr, di);
     if (a.tcurl32) {
-        a.tcurl32[2 * s] = make_float4((float)cr[0], (float)cr[1], (float)cr[2], 0.f);
-        a.tcurl32[2 * s + 1] = make_float4((float)ci[0], (float)ci[1], (float)ci[2], 0.f);
+        float* t = reinterpret_cast<float*>(a.tcurl32 + 2 * s + (q >= 3));
+        t[c] = (float)cu;
+        if (c == 0) t[3] = 0.f;
     }
     if (a.tcurl64) {
-        a.tcurl64[2 * s] = make_double4(cr[0], cr[1], cr[2], 0.0);
-        a.tcurl64[2 * s + 1] = make_double4(ci[0], ci[1], ci[2], 0.0);
+        double* t = reinterpret_cast<double*>(a.tcurl64 + 2 * s + (q >= 3));
+        t[c] = cu;
+        if (c == 0) t[3] = 0.0;
     }
 }
 
@@ -842,188 +859,225 @@ cudaError_t launch_far64_multi(const FarArgs64M& a, int n_tgt_tiles, int n_chunk
 
 // ----------------------------------------------------------------- projection onto P1 test functions
 
-// One CTA per target tile.  Its TP threads first sum, each for its own
-// point, the chunk partials of both slots (reads coalesced across the CTA);
-// then one thread per triangle projects onto the P1 test functions from
-// shared memory.  FP32 partials are summed with a compensated (TwoSum)
-// FP32 sum in chunk order, converted to FP64 once: the GPU's FP64 rate is
-// a small fraction of its FP32 rate, and the compensation carries the
-// rounding error of every addition, so the result matches an FP64 sum of
-// the same FP32 values to about 1e-15 of the sum of their magnitudes.
-__global__ void __launch_bounds__(TP) project_kernel(ProjectArgs a) {
-    __shared__ double Ps[2][NCOMP][TP];
-    const int tile = a.tgt_begin + blockIdx.x;
-    const int tid = threadIdx.x;
-    const int tdom = a.tdom[tile];
-    {
-        const int64_t p = (int64_t)tile * TP + tid;
-        for (int sl = 0; sl < 2; sl++) {
-            const SlotCoef cf = a.coef[tdom * 2 + sl];
-            if (cf.cV == 0 && cf.cK == 0 && cf.cKp == 0 && cf.cW == 0) continue;
-            const int64_t step = 2 * NCOMP * a.n_pts;  // one chunk
-            if (a.partial32) {
-                // all components at once: NCOMP independent loads per chunk
-                const float* src = a.partial32 + (int64_t)sl * NCOMP * a.n_pts + (p - a.p_off);
-                float hi[NCOMP], lo[NCOMP];
-#pragma unroll
-                for (int c = 0; c < NCOMP; c++) hi[c] = lo[c] = 0.f;
-                for (int ch = 0; ch < a.n_chunks; ch++, src += step) {
-                    float x[NCOMP];
-#pragma unroll
-                    for (int c = 0; c < NCOMP; c++) x[c] = src[(int64_t)c * a.n_pts];
-#pragma unroll
-                    for (int c = 0; c < NCOMP; c++) {
-                        const float u = hi[c] + x[c];  // TwoSum: hi + x = u + (rounding error)
-                        const float xb = u - hi[c];
-                        lo[c] += (hi[c] - (u - xb)) + (x[c] - xb);
-                        hi[c] = u;
-                    }
-                }
-#pragma unroll
-                for (int c = 0; c < NCOMP; c++) Ps[sl][c][tid] = (double)hi[c] + (double)lo[c];
-            } else {
-                for (int c = 0; c < NCOMP; c++) {
-                    const double* src = a.partial64 + ((int64_t)sl * NCOMP + c) * a.n_pts + (p - a.p_off);
-                    double sum = 0.0;
-                    for (int ch = 0; ch < a.n_chunks; ch++) sum += src[ch * step];
-                    Ps[sl][c][tid] = sum;
-                }
-            }
-        }
-    }
-    __syncthreads();
-    // far part: thread tid < TT owns slot tile * TT + tid
-    const int64_t s = (int64_t)tile * TT + tid;
-    const bool own = tid < TT && a.slot_v[s].x >= 0;
-    double r1[3][2] = {{0, 0}, {0, 0}, {0, 0}}, r2[3][2] = {{0, 0}, {0, 0}, {0, 0}};
-    if (own) {
-        const int dom = tdom;  // a tile holds triangles of one domain
-        const double inv4pi = 0.07957747154594767;
-        for (int sl = 0; sl < 2; sl++) {
-            const SlotCoef cf = a.coef[dom * 2 + sl];
-            if (cf.cV == 0 && cf.cK == 0 && cf.cKp == 0 && cf.cW == 0) continue;
-            double wc[6] = {0, 0, 0, 0, 0, 0};
-            for (int q = 0; q < QP; q++) {
-                const int64_t p = s * QP + q;
-                double P[NCOMP];
-                for (int c = 0; c < NCOMP; c++) P[c] = Ps[sl][c][tid * QP + q];
-                const double w = a.pt_w[p] * inv4pi;
-                // row1 potential: cV PV - cK PK ; row2 (pointwise part): cKp PKp - cW k^2 PWm
-                const double t1r = cf.cV * P[0] - cf.cK * P[2], t1i = cf.cV * P[1] - cf.cK * P[3];
-                const double kwr = cf.k2re * P[6] - cf.k2im * P[7], kwi = cf.k2re * P[7] + cf.k2im * P[6];
-                const double t2r = cf.cKp * P[4] - cf.cW * kwr, t2i = cf.cKp * P[5] - cf.cW * kwi;
-                for (int k = 0; k < 3; k++) {
-                    const double wl = w * a.lam[q][k];
-                    r1[k][0] += wl * t1r;
-                    r1[k][1] += wl * t1i;
-                    r2[k][0] += wl * t2r;
-                    r2[k][1] += wl * t2i;
-                }
-                for (int c = 0; c < 6; c++) wc[c] += w * P[8 + c];
-            }
-            for (int k = 0; k < 3; k++) {
-                const double* cu = &a.slot_curl[s * 9 + 3 * k];
-                r2[k][0] += cf.cW * (cu[0] * wc[0] + cu[1] * wc[1] + cu[2] * wc[2]);
-                r2[k][1] += cf.cW * (cu[0] * wc[3] + cu[1] * wc[4] + cu[2] * wc[5]);
-            }
-        }
-    }
-    // near pairs (touching and near band): combined 3x3 sub-blocks (row1<-psi,
-    // row1<-phi, row2<-psi, row2<-phi).  Every thread takes part: thread
-    // (j, sub) = (tid / NSUB, tid % NSUB) sums every NSUB-th pair of slot
-    // tile * TT + j; the NSUB partial sums meet in shared memory (Ps is free
-    // again) and are added in a fixed order, so results are deterministic.
-    // FP32 blocks (the FP32 operator) take FP32 products and sums.
+// One CTA per PS = 8 slots (a quarter of a target tile), three phases:
+//  1. near pairs (touching and near band), one warp per slot, one pair per
+//     lane and pass: the combined 3x3 sub-blocks (row1<-psi, row1<-phi,
+//     row2<-psi, row2<-phi) times the pair's source values.  The FP32
+//     operator takes FP32 products; a lane sums its two or three pairs.
+//  2. chunk partials: the CTA's 2 x NCOMP x 48 sums over the chunks, one
+//     (component, point) per thread and pass, points coalesced.  FP32
+//     partials are summed with a compensated (TwoSum) FP32 sum in chunk
+//     order, converted to FP64 once: the GPU's FP64 rate is a small fraction
+//     of its FP32 rate, and the compensation carries the rounding error of
+//     every addition, so the result matches an FP64 sum of the same FP32
+//     values to about 1e-15 of the sum of their magnitudes.
+//  3. the projection onto the P1 test functions in FP64, spread over the
+//     (slot, point) and (slot, vertex) pairs, and the lanes' near sums
+//     (compensated again) in lane order.
+// The kernel is a chain of dependent loads and of FP64 operations at 1/64 of
+// the FP32 rate, so its time at small sizes is the length of that chain on
+// one SM.  One CTA per tile with six threads per slot walked ten pairs one
+// after another and ran a tile's FP64 on one SM; a quarter of a tile per CTA
+// and 32 lanes per slot shorten both: 76 -> 24 us on 300 triangles, 234 -> 98 us
+// on 8,172 (FP32), 319 -> 159 us on 1,452 (FP64), cold caches.
+constexpr int PS = 8;                  // slots per CTA
+constexpr int PP = PS * QP;            // points per CTA
+constexpr int PROJ_THREADS = PS * 32;
+constexpr int PROJ_PAD = 32 * 12 + 4;  // near partial sums of one slot, padded against bank conflicts
+static_assert(TT % PS == 0, "a CTA's slots lie in one tile");
+static_assert(2 * PP + 12 * PS <= PROJ_THREADS && 3 * PS <= 32 && 32 + 6 * PS <= PROJ_THREADS, "phase 3 work fits the CTA");
+
+__device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float x) {
+    const float u = hi + x;  // TwoSum: hi + x = u + (rounding error)
+    const float xb = u - hi;
+    lo += (hi - (u - xb)) + (x - xb);
+    hi = u;
+}
+
+template <bool F64>
+__global__ void __launch_bounds__(PROJ_THREADS) project_kernel(ProjectArgs a) {
+    typedef typename std::conditional<F64, double, float>::type real_t;
+    __shared__ double Ps[2][NCOMP][PP];
+    __shared__ real_t red[PS * PROJ_PAD];
+    __shared__ double nsum[PS][12], csum[PS][6];
+    const int64_t s0 = (int64_t)a.tgt_begin * TT + (int64_t)blockIdx.x * PS;  // first slot
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tdom = a.tdom[s0 / TT];  // a tile holds triangles of one domain
+    // 1. near pairs
     if (a.np_ptr) {
-        constexpr int NSUB = TP / TT;
-        double* red = &Ps[0][0][0];  // [TT][NSUB][12]
-        static_assert(TT * NSUB * 12 <= 2 * NCOMP * TP, "near partial sums fit in the potential buffer");
-        __syncthreads();
-        const int j = tid / NSUB, sub = tid % NSUB;
-        const int64_t sj = (int64_t)tile * TT + j;
-        double acc[12];
+        const int64_t s = s0 + warp;
+        real_t f[12];
 #pragma unroll
-        for (int c = 0; c < 12; c++) acc[c] = 0;
-        if (a.slot_v[sj].x >= 0) {
-            const int64_t pe = a.np_ptr[sj + 1];
-            if (a.nb32) {
-                float f[12];
+        for (int c = 0; c < 12; c++) f[c] = 0;
+        if (a.slot_v[s].x >= 0) {
+            const int64_t pe = a.np_ptr[s + 1];
+            // two pairs per pass: the dependent loads pair -> slot -> unknowns -> values overlap
+            for (int64_t pi = a.np_ptr[s] + lane; pi < pe; pi += 64) {
+                const int64_t pj[2] = {pi, min(pi + 32, pe - 1)};
+                int4 vt[2];
 #pragma unroll
-                for (int c = 0; c < 12; c++) f[c] = 0.f;
-                for (int64_t pi = a.np_ptr[sj] + sub; pi < pe; pi += NSUB) {
-                    const int4 vt = a.slot_v[a.np_src[pi]];
-                    const int vid[3] = {vt.x, vt.y, vt.z};
-                    float2 xv[2][3];
+                for (int u = 0; u < 2; u++) vt[u] = a.slot_v[a.np_src[pj[u]]];
+                real_t xv[2][2][3][2];
+#pragma unroll
+                for (int u = 0; u < 2; u++)
 #pragma unroll
                     for (int b = 0; b < 3; b++) {
-                        const double2 x1 = a.x[a.v_dof1[vid[b]]], x2 = a.x[a.v_dof2[vid[b]]];
-                        xv[0][b] = make_float2((float)x1.x, (float)x1.y);
-                        xv[1][b] = make_float2((float)x2.x, (float)x2.y);
+                        const int vid = b == 0 ? vt[u].x : b == 1 ? vt[u].y : vt[u].z;
+                        const double2 x1 = a.x[a.v_dof1[vid]], x2 = a.x[a.v_dof2[vid]];
+                        xv[u][0][b][0] = (real_t)x1.x;
+                        xv[u][0][b][1] = (real_t)x1.y;
+                        xv[u][1][b][0] = (real_t)x2.x;
+                        xv[u][1][b][1] = (real_t)x2.y;
                     }
-                    // 36 complex entries as 18 aligned float4 (pair stride 288 bytes)
-                    const float4* B4 = reinterpret_cast<const float4*>(a.nb32 + pi * 36);
 #pragma unroll
-                    for (int e2 = 0; e2 < 18; e2++) {
-                        const float4 B = B4[e2];
-#pragma unroll
-                        for (int h = 0; h < 2; h++) {
-                            const int e = 2 * e2 + h, blk = e / 9, k = (e % 9) / 3, b = e % 3;
-                            const float br = h ? B.z : B.x, bi = h ? B.w : B.y;
-                            const float2 x = xv[blk & 1][b];
-                            const int o = (blk < 2 ? 0 : 6) + 2 * k;
-                            f[o] = fmaf(br, x.x, fmaf(-bi, x.y, f[o]));
-                            f[o + 1] = fmaf(br, x.y, fmaf(bi, x.x, f[o + 1]));
-                        }
-                    }
-                }
-#pragma unroll
-                for (int c = 0; c < 12; c++) acc[c] = f[c];
-            } else {
-                for (int64_t pi = a.np_ptr[sj] + sub; pi < pe; pi += NSUB) {
-                    const int4 vt = a.slot_v[a.np_src[pi]];
-                    const int vid[3] = {vt.x, vt.y, vt.z};
-                    double2 xv[2][3];
-                    for (int b = 0; b < 3; b++) {
-                        xv[0][b] = a.x[a.v_dof1[vid[b]]];
-                        xv[1][b] = a.x[a.v_dof2[vid[b]]];
-                    }
+                for (int u = 0; u < 2; u++) {
+                    if (u && pi + 32 >= pe) break;
+                    // 36 complex entries as 18 loads of two (FP32, 16-byte aligned: pair stride 288 bytes) or 36 of one
 #pragma unroll
                     for (int e = 0; e < 36; e++) {
-                        const int blk = e / 9, k = (e % 9) / 3, b = e % 3;
-                        const double2 B = a.nb64[pi * 36 + e];
-                        const double2 x = xv[blk & 1][b];
-                        const int o = (blk < 2 ? 0 : 6) + 2 * k;
-                        acc[o] += B.x * x.x - B.y * x.y;
-                        acc[o + 1] += B.x * x.y + B.y * x.x;
+                        real_t br, bi;
+                        if constexpr (F64) {
+                            const double2 B = a.nb64[pj[u] * 36 + e];
+                            br = B.x;
+                            bi = B.y;
+                        } else {
+                            const float4 B = reinterpret_cast<const float4*>(a.nb32 + pj[u] * 36)[e >> 1];
+                            br = (e & 1) ? B.z : B.x;
+                            bi = (e & 1) ? B.w : B.y;
+                        }
+                        const int blk = e / 9, k = (e % 9) / 3, b = e % 3, o = (blk < 2 ? 0 : 6) + 2 * k;
+                        const real_t xr = xv[u][blk & 1][b][0], xi = xv[u][blk & 1][b][1];
+                        f[o] += br * xr - bi * xi;
+                        f[o + 1] += br * xi + bi * xr;
                     }
                 }
             }
         }
 #pragma unroll
-        for (int c = 0; c < 12; c++) red[(j * NSUB + sub) * 12 + c] = acc[c];
-        __syncthreads();
-        if (own)
-            for (int u = 0; u < NSUB; u++) {
-                const double* q = red + (tid * NSUB + u) * 12;
-                for (int k = 0; k < 3; k++) {
-                    r1[k][0] += q[2 * k];
-                    r1[k][1] += q[2 * k + 1];
-                    r2[k][0] += q[6 + 2 * k];
-                    r2[k][1] += q[6 + 2 * k + 1];
-                }
-            }
+        for (int c = 0; c < 12; c++) red[warp * PROJ_PAD + lane * 12 + c] = f[c];
     }
+    // 2. chunk partials
+    const int64_t p0 = s0 * QP - a.p_off;
+    const int64_t step = 2 * NCOMP * a.n_pts;  // one chunk
+    // a thread's sums side by side: their loads of one chunk are independent
+    constexpr int NS = (2 * NCOMP * PP + PROJ_THREADS - 1) / PROJ_THREADS;
+    const SlotCoef &cf0 = a.coef[tdom * 2], &cf1 = a.coef[tdom * 2 + 1];
+    const bool on[2] = {cf0.cV != 0 || cf0.cK != 0 || cf0.cKp != 0 || cf0.cW != 0,
+                        cf1.cV != 0 || cf1.cK != 0 || cf1.cKp != 0 || cf1.cW != 0};
+    int64_t at[NS];
+    bool use[NS];
+#pragma unroll
+    for (int u = 0; u < NS; u++) {
+        const int i = tid + u * PROJ_THREADS, row = i / PP;
+        use[u] = i < 2 * NCOMP * PP && on[row >= NCOMP];
+        at[u] = (int64_t)row * a.n_pts + p0 + (i - row * PP);
+    }
+    if constexpr (F64) {
+        double sum[NS];
+#pragma unroll
+        for (int u = 0; u < NS; u++) sum[u] = 0.0;
+#pragma unroll 2
+        for (int ch = 0; ch < a.n_chunks; ch++)
+#pragma unroll
+            for (int u = 0; u < NS; u++)
+                if (use[u]) sum[u] += a.partial64[ch * step + at[u]];
+#pragma unroll
+        for (int u = 0; u < NS; u++)
+            if (use[u]) (&Ps[0][0][0])[tid + u * PROJ_THREADS] = sum[u];
+    } else {
+        float hi[NS], lo[NS];
+#pragma unroll
+        for (int u = 0; u < NS; u++) hi[u] = lo[u] = 0.f;
+#pragma unroll 4
+        for (int ch = 0; ch < a.n_chunks; ch++) {
+            float x[NS];
+#pragma unroll
+            for (int u = 0; u < NS; u++) x[u] = use[u] ? a.partial32[ch * step + at[u]] : 0.f;
+#pragma unroll
+            for (int u = 0; u < NS; u++) two_sum_acc(hi[u], lo[u], x[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < NS; u++)
+            if (use[u]) (&Ps[0][0][0])[tid + u * PROJ_THREADS] = (double)hi[u] + (double)lo[u];
+    }
+    __syncthreads();
+    // 3a. one thread per (slot, wavenumber slot, point): the point's weighted
+    // row potentials and curl terms, in place; beside them one thread per
+    // (slot, component) adds the lanes' near sums
+    if (tid < 2 * PP) {
+        const int sl = tid / PP, pt = tid - sl * PP;
+        if (on[sl] && a.slot_v[s0 + pt / QP].x >= 0) {
+            const SlotCoef& cf = sl ? cf1 : cf0;
+            const double w = a.pt_w[s0 * QP + pt] * 0.07957747154594767;  // 1 / (4 pi)
+            const double P6 = Ps[sl][6][pt], P7 = Ps[sl][7][pt];
+            // row1 potential: cV PV - cK PK ; row2 (pointwise part): cKp PKp - cW k^2 PWm
+            const double t1r = cf.cV * Ps[sl][0][pt] - cf.cK * Ps[sl][2][pt];
+            const double t1i = cf.cV * Ps[sl][1][pt] - cf.cK * Ps[sl][3][pt];
+            const double t2r = cf.cKp * Ps[sl][4][pt] - cf.cW * (cf.k2re * P6 - cf.k2im * P7);
+            const double t2i = cf.cKp * Ps[sl][5][pt] - cf.cW * (cf.k2re * P7 + cf.k2im * P6);
+            Ps[sl][0][pt] = w * t1r;
+            Ps[sl][1][pt] = w * t1i;
+            Ps[sl][2][pt] = w * t2r;
+            Ps[sl][3][pt] = w * t2i;
+            const double wc = w * cf.cW;
+#pragma unroll
+            for (int c = 8; c < NCOMP; c++) Ps[sl][c][pt] *= wc;
+        }
+    } else if (a.np_ptr && tid < 2 * PP + PS * 12) {
+        const int u = tid - 2 * PP, j = u / 12, c = u - 12 * j;
+        real_t n = 0, lo = 0;
+        for (int l = 0; l < 32; l++) {
+            const real_t x = red[j * PROJ_PAD + l * 12 + c];
+            if constexpr (F64) n += x;
+            else two_sum_acc(n, lo, x);
+        }
+        nsum[j][c] = (double)n + (double)lo;
+    }
+    __syncthreads();
+    // 3b. thread (j, k): rows of vertex k of slot s0 + j; beside them the slots' curl sums, one component per thread
+    const int j = tid / 3, k = tid - 3 * j;
+    const bool own = tid < 3 * PS && a.slot_v[s0 + j].x >= 0;
+    double r[4] = {0, 0, 0, 0};
+    if (own) {
+#pragma unroll
+        for (int sl = 0; sl < 2; sl++)
+            if (on[sl])
+#pragma unroll
+                for (int q = 0; q < QP; q++)
+#pragma unroll
+                    for (int c = 0; c < 4; c++) r[c] += a.lam[q][k] * Ps[sl][c][j * QP + q];
+    } else if (tid >= 32 && tid < 32 + 6 * PS) {
+        const int jj = (tid - 32) / 6, c = tid - 32 - 6 * jj;
+        double t = 0;
+#pragma unroll
+        for (int sl = 0; sl < 2; sl++)
+            if (on[sl])
+#pragma unroll
+                for (int q = 0; q < QP; q++) t += Ps[sl][8 + c][jj * QP + q];
+        csum[jj][c] = t;
+    }
+    __syncthreads();
     if (!own) return;
-    for (int k = 0; k < 3; k++) {
-        a.tri_out[(s * 3 + k) * 2] = make_double2(r1[k][0], r1[k][1]);
-        a.tri_out[(s * 3 + k) * 2 + 1] = make_double2(r2[k][0], r2[k][1]);
+    const int64_t s = s0 + j;
+    const double* cu = &a.slot_curl[s * 9 + 3 * k];
+    r[2] += cu[0] * csum[j][0] + cu[1] * csum[j][1] + cu[2] * csum[j][2];
+    r[3] += cu[0] * csum[j][3] + cu[1] * csum[j][4] + cu[2] * csum[j][5];
+    if (a.np_ptr) {
+        r[0] += nsum[j][2 * k];
+        r[1] += nsum[j][2 * k + 1];
+        r[2] += nsum[j][6 + 2 * k];
+        r[3] += nsum[j][6 + 2 * k + 1];
     }
+    a.tri_out[(s * 3 + k) * 2] = make_double2(r[0], r[1]);
+    a.tri_out[(s * 3 + k) * 2 + 1] = make_double2(r[2], r[3]);
 }
 
 cudaError_t launch_project(const ProjectArgs& a, cudaStream_t s) {
     const int n_tiles = a.tgt_end - a.tgt_begin;
     if (n_tiles <= 0) return cudaSuccess;
-    project_kernel<<<(unsigned)n_tiles, TP, 0, s>>>(a);
+    const unsigned grid = (unsigned)n_tiles * (TT / PS);
+    if (a.partial32) project_kernel<false><<<grid, PROJ_THREADS, 0, s>>>(a);
+    else project_kernel<true><<<grid, PROJ_THREADS, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -1033,7 +1087,9 @@ __global__ void reduce_kernel(ReduceArgs a) {
     const int64_t v = a.v_begin + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (v >= a.v_end) return;
     double s1r = 0, s1i = 0, s2r = 0, s2i = 0;
-    for (int64_t i = a.vc_ptr[v]; i < a.vc_ptr[v + 1]; i++) {
+    const int64_t e = a.vc_ptr[v + 1];
+#pragma unroll 4
+    for (int64_t i = a.vc_ptr[v]; i < e; i++) {
         const int64_t c = a.vc_idx[i];
         const double2 u = a.tri_out[c * 2], w = a.tri_out[c * 2 + 1];
         s1r += u.x;
@@ -1048,14 +1104,14 @@ __global__ void reduce_kernel(ReduceArgs a) {
 cudaError_t launch_reduce(const ReduceArgs& a, cudaStream_t s) {
     int64_t n = a.v_end - a.v_begin;
     if (n <= 0) return cudaSuccess;
-    reduce_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(a);
+    reduce_kernel<<<(unsigned)((n + 63) / 64), 64, 0, s>>>(a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_gather(const GatherArgs& a, cudaStream_t s) {
     int64_t n = a.s_end - a.s_begin;
     if (n <= 0) return cudaSuccess;
-    gather_kernel<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(a);
+    gather_kernel<<<(unsigned)((n * QP + GATHER_THREADS - 1) / GATHER_THREADS), GATHER_THREADS, 0, s>>>(a);
     return cudaGetLastError();
 }
 
