@@ -206,10 +206,11 @@ int64_t estimate_solve_bytes(const bem_ctx* ctx, int64_t n_exc, const bem_solve_
     b += pts * 152 + slots * 460 + pairs * 12 + N * 64 + tiles * 64;
     // near-field blocks (c128 + c64) and their build scratch
     b += pairs * 36 * 24 + std::min<int64_t>(pairs, 1 << 20) * 2 * 27 * 16;
-    // far-field partial potentials (FP64 residual is the larger)
-    int nc = 1, ct = 1;
-    ctx->chunking((int)tiles, (int)tiles, &nc, &ct);
-    b += (int64_t)nc * 2 * NCOMP * pts * 8;
+    // far-field partial potentials (one buffer for the FP32 operator and the FP64 residual)
+    int nc = 1, nc64 = 1, ct = 1;
+    ctx->chunking((int)tiles, (int)tiles, &nc, &ct, false);
+    ctx->chunking((int)tiles, (int)tiles, &nc64, &ct, true);
+    b += std::max((int64_t)nc * 4, (int64_t)nc64 * 8) * 2 * NCOMP * pts;
     // right-hand sides, solutions, piston data
     b += n_exc * (2 * N * 16 + slots * 6 * 16 + ne * 16) + ne * 32 * 32 + 3 * N * 16;
     // GMRES basis and work (per lockstep column)
@@ -491,9 +492,19 @@ int bem_ctx::ensure_far_work(int tgt_b, int tgt_e, int src_b, int src_e, int chu
     return BEM_OK;
 }
 
-void bem_ctx::chunking(int n_tgt, int n_src, int* n_chunks, int* chunk_tiles) const {
+// FP32 chunks are at most FAR32_CHUNK tiles long: the six warps of a CTA drift
+// apart inside its four-stage ring, and in a long chunk the leading warps end
+// up waiting for the slowest one at every tile (long-scoreboard stalls, FMA
+// pipe 63 % busy at 128 tiles against 74 % at 16).  Measured far-field time on
+// the 20,988-triangle rib scene: 31.7-31.9 ms at 6-16 tiles, 33.4 at 24, 36.8
+// at 64, 39.1 at the up to 219 tiles taken before; on 41,292 triangles 123 ms
+// against 147.5.  The double-float far field has no ring and keeps its own rule.
+constexpr int FAR32_CHUNK = 12;
+
+void bem_ctx::chunking(int n_tgt, int n_src, int* n_chunks, int* chunk_tiles, bool fp64) const {
     int want = std::max(1, (152 * 2 * 8 + n_tgt - 1) / std::max(1, n_tgt));
     int nc = std::max(want, (n_src + CHUNK_MAX - 1) / CHUNK_MAX);
+    if (!fp64) nc = std::max(nc, (n_src + FAR32_CHUNK - 1) / FAR32_CHUNK);
     if (opts.chunk_tiles > 0) nc = (n_src + opts.chunk_tiles - 1) / opts.chunk_tiles;
     // the partial potentials grow as chunks x points: at most 8 GiB of them at
     // FP64 (4 GiB at FP32), unless CHUNK_MAX forces more chunks
@@ -519,8 +530,12 @@ int bem_ctx::plan_apply(const double2* x, double2* y, int precision, const Apply
     const int tgt_b = g.dom_tile_begin[m.tgt_dom_lo], tgt_e = g.dom_tile_end[m.tgt_dom_hi - 1];
     const int src_b = g.dom_tile_begin[m.src_dom_lo], src_e = g.dom_tile_end[m.src_dom_hi - 1];
     int n_chunks, chunk_tiles;
-    chunking(fill_tiles > 0 ? fill_tiles : tgt_e - tgt_b, src_e - src_b, &n_chunks, &chunk_tiles);
+    chunking(fill_tiles > 0 ? fill_tiles : tgt_e - tgt_b, src_e - src_b, &n_chunks, &chunk_tiles, fp64);
     int rc = ensure_partial(n_chunks, fp64);
+    if (rc == BEM_ERR_OUT_OF_BUDGET && !fp64) {  // longer chunks where the budget does not hold the partials of short ones
+        chunking(fill_tiles > 0 ? fill_tiles : tgt_e - tgt_b, src_e - src_b, &n_chunks, &chunk_tiles, true);
+        rc = ensure_partial(n_chunks, fp64);
+    }
     if (rc) return rc;
     P.n_tgt = tgt_e - tgt_b;
     P.n_chunks = n_chunks;

@@ -179,7 +179,7 @@ struct bem_ctx {
     int ensure_near();
     int ensure_partial(int n_chunks, bool fp64);
     int ensure_far_work(int tgt_b, int tgt_e, int src_b, int src_e, int chunk_tiles, int n_chunks, int slot1);
-    void chunking(int n_tgt, int n_src, int* n_chunks, int* chunk_tiles) const;
+    void chunking(int n_tgt, int n_src, int* n_chunks, int* chunk_tiles, bool fp64) const;
     int plan_apply(const double2* x, double2* y, int precision, const gbem::ApplyMode& m, gbem::ApplyPlan& P,
                    int fill_tiles = 0);
     int run_apply(const double2* x, double2* y, int precision, const gbem::ApplyMode& m);

@@ -63,7 +63,7 @@ extern "C" int bem_apply_noalloc(bem_ctx* ctx, const bem_z* x, bem_z* y) {
     const Geometry& g = ctx->geo;
     const int n_tiles = g.n_tiles;
     int n_chunks, chunk_tiles;
-    ctx->chunking(n_tiles, n_tiles, &n_chunks, &chunk_tiles);
+    ctx->chunking(n_tiles, n_tiles, &n_chunks, &chunk_tiles, false);
     const size_t per_tile = (size_t)n_chunks * 2 * NCOMP * TP;  // floats of scratch per target tile
     if (per_tile > NOALLOC_SCRATCH_FLOATS)
         return ctx->fail(BEM_ERR_OUT_OF_BUDGET, "problem too large for the 64 MiB allocation-free scratch (" +
