@@ -153,6 +153,7 @@ namespace gbem {
 
 void invalidate_basis(bem_ctx* ctx);
 void invalidate_recycle(bem_ctx* ctx);
+size_t gemm_work_bytes(int64_t mpad, int64_t kpad, int64_t n_rhs);  // k_gemm.cu
 
 // Eviction by the request loop: every device allocation of the context goes;
 // the host description (meshes, materials, transducer) stays and the device
@@ -255,10 +256,9 @@ int64_t estimate_solve_bytes(const bem_ctx* ctx, int64_t n_exc, const bem_solve_
     if (o.operator_mode == 1) {
         const int64_t mp = (N + 127) / 128 * 128, kp = (N + 31) / 32 * 32;
         const int64_t planes = 6 * mp * kp * 2;
-        const int64_t nbpad = (R + 63) / 64 * 128;
         const int64_t a64 = 16 * N * N;
         if (o.precision == BEM_PREC_FP32)
-            b += std::max(planes + 8 * N * N, planes + a64) + R * N * 16 + 3 * nbpad * kp * 2;
+            b += std::max(planes + 8 * N * N, planes + a64) + (int64_t)gemm_work_bytes(mp, kp, R);
         else
             b += a64;
     }

@@ -476,21 +476,11 @@ __global__ void add_near_kernel(int64_t n_pairs, const int32_t* pair_tgt, const 
             }
 }
 
-__global__ void c128_to_c64(int64_t n, const double2* x, float2* y) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) y[i] = make_float2((float)x[i].x, (float)x[i].y);
-}
-
-__global__ void c64_to_c128(int64_t n, const float2* x, double2* y) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) y[i] = make_double2(x[i].x, x[i].y);
-}
-
 int gemm_bf16x3(bem_ctx* ctx, const __nv_bfloat16* Aplanes, int64_t m, int64_t k, int64_t mpad, int64_t kpad,
-                const float2* X, int64_t n_rhs, float2* Y, __nv_bfloat16* xplanes, int64_t nbpad);
+                const float2* X, const double2* X64, int64_t n_rhs, float2* Y, double2* Y64, void* work);
+size_t gemm_work_bytes(int64_t mpad, int64_t kpad, int64_t n_rhs);
 int split_a(bem_ctx* ctx, const float2* A, int64_t m, int64_t k, int64_t mpad, int64_t kpad, __nv_bfloat16* P);
 int gemm_a_planes();
-int gemm_b_planes();
 int gemm_k_align();
 
 }  // namespace gbem
@@ -628,26 +618,15 @@ int bem_ctx::apply_assembled64(const double2* x, double2* y, int64_t n_rhs) {
 // Y = A_hat X for n_rhs system-order vectors (complex128, device), through
 // the assembled operator and the tensor-core GEMM.
 int bem_ctx::apply_assembled(const double2* x, double2* y, int64_t n_rhs) {
-    bem_ctx* const ctx = this;
     int rc = ensure_assembled();
     if (rc) return rc;
     const int64_t n = geo.n_dof;
-    const int64_t nbpad = (n_rhs + 63) / 64 * 128;
-    const size_t need = (size_t)n_rhs * n * sizeof(float2) * 2 + (size_t)gemm_b_planes() * nbpad * asm_kpad * 2;
+    const size_t need = gemm_work_bytes(asm_mpad, asm_kpad, n_rhs);
     if (need > asm_work_bytes) {
         if (asm_work) dfree(asm_work);
         asm_work = dalloc(need, &rc);
         if (rc) { asm_work = nullptr; asm_work_bytes = 0; return rc; }
         asm_work_bytes = need;
     }
-    float2* xs = (float2*)asm_work;
-    float2* ys = xs + n_rhs * n;
-    __nv_bfloat16* xp = (__nv_bfloat16*)(ys + n_rhs * n);
-    const int64_t tot = n_rhs * n;
-    c128_to_c64<<<(unsigned)((tot + 255) / 256), 256, 0, stream>>>(tot, x, xs);
-    if ((rc = gemm_bf16x3(this, asm_planes, n, n, asm_mpad, asm_kpad, xs, n_rhs, ys, xp, nbpad))) return rc;
-    c64_to_c128<<<(unsigned)((tot + 255) / 256), 256, 0, stream>>>(tot, ys, y);
-    launches += 2;
-    CK(cudaGetLastError());
-    return BEM_OK;
+    return gemm_bf16x3(this, asm_planes, n, n, asm_mpad, asm_kpad, nullptr, x, n_rhs, nullptr, y, asm_work);
 }

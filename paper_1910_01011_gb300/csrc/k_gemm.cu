@@ -13,17 +13,29 @@
 // The complex product is two real GEMMs sharing the B operand
 // B = [X_re | X_im] (k x 2n):  C1 = A_re B,  C2 = A_im B, then
 //   Y_re = C1[:, :n] - C2[:, n:],   Y_im = C1[:, n:] + C2[:, :n].
-// A CTA owns a 128-row tile of A and a 128-column tile of B (64 right-hand
-// sides, real and imaginary parts), so C1 and C2 are two 128 x 128 FP32
-// accumulators in tensor memory (256 TMEM columns, double-buffered over 512).
-// Operands stream in by TMA (64-byte swizzle, K-major, 32 of K per stage)
-// through a three-stage ring (GSTAGES); one thread issues the MMAs and
-// commits each stage back to the producer.
+// A unit of work is a 128-row tile of A times a GN-column tile of B over 256
+// of K; C1 and C2 are two 128 x GN FP32 accumulators in tensor memory,
+// double-buffered.  GN = 32 (up to 16 right-hand sides, real and imaginary
+// parts) or 128 (64 right-hand sides).  Operands stream in by TMA (64-byte
+// swizzle, K-major, 32 of K per stage) through a ring of 216 KB; one thread
+// issues the MMAs and commits each stage back to the producer.
+//
+// Up to 64 right-hand sides the product is bound by reading the 12 N^2 bytes
+// of A once, so every SM has to stream all the time: each of 152 CTAs takes
+// an equal, contiguous range of units (tile-major), crossing tile borders, and
+// the pieces of a tile that several CTAs share are summed in CTA order by
+// gemm_finish_kernel.  One CTA per tile left SMs idle (165 tiles on 152 SMs
+// are two waves, 65 tiles use 65 SMs): N = 21,016, 16 right-hand sides took
+// 1,364 us against 774 us (12 N^2 bytes at 6.85 TB/s), N = 8,200
+// 258 us against 132 us.  With more right-hand sides the
+// tensor cores bind it, and one CTA per tile over all of K (column tiles
+// fastest) lets the column tiles of a row share A through L2.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <cstring>
 #include <string>
@@ -34,24 +46,33 @@
 namespace gbem {
 
 constexpr int GM = 128;                       // rows of A per CTA
-constexpr int GN = 128;                       // columns of B per CTA (64 rhs x re/im)
 constexpr int GK = 32;                        // k per stage (64 bytes of bf16, 64-byte swizzle)
 constexpr int NSPLIT = 3;                     // BF16 terms per real number
-constexpr int GSTAGES = 3;
-constexpr int TILE_BYTES = GM * GK * 2;       // 8 KB per operand tile
+constexpr int TILE_BYTES = GM * GK * 2;       // 8 KB per A operand tile
 constexpr int A_TILES = 2 * NSPLIT;           // A re (3 terms), A im (3 terms)
-constexpr int G_STAGE_BYTES = (A_TILES + NSPLIT) * TILE_BYTES;
 constexpr int GEMM_THREADS = 192;             // warp 0 TMA, warp 1 MMA, warps 2-5 accumulate / epilogue
-constexpr uint32_t TMEM_COLS = 512;           // two accumulator buffers of 256 columns (C1 | C2)
 constexpr int KCH_STAGES = 8;                 // stages per accumulation chunk (K = 256)
+constexpr int GEMM_CTAS = 152;                // CTAs of a split product: one per SM
 
-struct GemmSmem {
-    alignas(1024) uint8_t stage[GSTAGES][G_STAGE_BYTES];
-    uint64_t full[GSTAGES];
-    uint64_t empty[GSTAGES];
-    uint64_t accf[2];   // chunk accumulated in TMEM buffer b (MMA commit)
-    uint64_t acce[2];   // TMEM buffer b drained (4 epilogue warps)
-    uint32_t tmem_base;
+template <int GN>
+struct GemmCfg {
+    static constexpr int HN = GN / 2;                 // right-hand sides per column tile
+    static constexpr int BT_BYTES = GN * GK * 2;      // bytes per B operand tile
+    static constexpr int STAGE_BYTES = A_TILES * TILE_BYTES + NSPLIT * BT_BYTES;
+    static constexpr int STAGES = 216 * 1024 / STAGE_BYTES;
+    static constexpr uint32_t TMEM_COLS = 4 * GN;     // two buffers of C1 | C2
+    // instruction descriptor, kind::f16: BF16 A and B, FP32 D, both K-major, M = 128, N = GN
+    static constexpr uint32_t IDESC =
+        (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(GN >> 3) << 17) | ((uint32_t)(GM >> 4) << 24);
+    struct Smem {
+        alignas(1024) uint8_t stage[STAGES][STAGE_BYTES];
+        uint64_t full[STAGES];
+        uint64_t empty[STAGES];
+        uint64_t accf[2];   // chunk accumulated in TMEM buffer b (MMA commit)
+        uint64_t acce[2];   // TMEM buffer b drained (4 epilogue warps)
+        uint32_t tmem_base;
+    };
+    static_assert(STAGE_BYTES % 1024 == 0 && sizeof(Smem) + 1024 <= 227 * 1024, "gemm smem");
 };
 
 __device__ __forceinline__ uint32_t s_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -105,15 +126,11 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
     return d;
 }
 
-// Instruction descriptor, kind::f16: BF16 A and B, FP32 D, both K-major,
-// M = 128, N = 128.
-constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(GN >> 3) << 17) | ((uint32_t)(GM >> 4) << 24);
-
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t accumulate) {
+__device__ __forceinline__ void mma_bf16(uint32_t idesc, uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
-        "l"(a), "l"(b), "r"(IDESC), "r"(accumulate)
+        "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 
@@ -122,34 +139,56 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
                  : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-    for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
+    for (int i = 0; i < 8; i++) v[i] = __uint_as_float(r[i]);
 }
 
 // The tensor cores accumulate FP32 with truncation, so a long K sum drifts
 // by ~K x 2^-24 relative.  The MMAs therefore accumulate only KCH_STAGES*GK
 // of K in tensor memory (two buffers, double-buffered); four epilogue warps
 // drain each chunk into round-to-nearest FP32 registers.
-// grid: (n_col_tiles, m_tiles); the column tile runs fastest so that the
-// CTAs sharing an A row tile run together and share it through L2.
+//
+// Unit u = tile * nch + chunk, tile = row tile * n_ct + column tile; CTA b
+// takes units [units b / CTAs, units (b + 1) / CTAs).  part != null: each
+// CTA's sum over its units of a tile goes to part[tile][piece][rhs][128]
+// (piece: the CTA's place among those of the tile); else (whole tiles per CTA)
+// straight to Y or Y64.
+struct GemmArgs {
+    int64_t mpad, nbpad;
+    int kblocks, m, n_rhs, n_ct, nch, pieces, units;
+    float2* Y;
+    double2* Y64;
+    float2* part;
+    int* err;
+};
+
+__host__ __device__ inline int gemm_first_unit(int units, int ctas, int b) { return (int)((int64_t)units * b / ctas); }
+// the first of the CTAs that hold units of `tile`
+__host__ __device__ inline int gemm_first_cta(int units, int ctas, int nch, int tile) {
+    const int u = tile * nch;
+    int b = (int)((int64_t)u * ctas / units);
+    while (b + 1 < ctas && gemm_first_unit(units, ctas, b + 1) <= u) b++;
+    while (b > 0 && gemm_first_unit(units, ctas, b) > u) b--;
+    return b;
+}
+
+template <int GN>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
-    gemm_bf16x3_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                       int64_t mpad, int64_t nbpad, int kblocks, int m, int n_rhs, float2* Y, int* err) {
+    gemm_bf16x3_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmArgs a) {
+    typedef GemmCfg<GN> C;
+    constexpr int GSTAGES = C::STAGES, HN = C::HN;
     extern __shared__ uint8_t smem_raw[];
-    GemmSmem& sm = *reinterpret_cast<GemmSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    typename C::Smem& sm =
+        *reinterpret_cast<typename C::Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int ct = blockIdx.x, mt = blockIdx.y;
-    const int m0 = mt * GM;
-    const int b0 = ct * GN;  // B rows (rhs re block then rhs im block)
-    const int nchunks = (kblocks + KCH_STAGES - 1) / KCH_STAGES;
+    const int u0 = gemm_first_unit(a.units, gridDim.x, blockIdx.x), u1 = gemm_first_unit(a.units, gridDim.x, blockIdx.x + 1);
+    int* const err = a.err;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < GSTAGES; s++) {
@@ -164,7 +203,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     }
     if (warp == 2) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s_u32(&sm.tmem_base)),
-                     "r"(TMEM_COLS)
+                     "r"(C::TMEM_COLS)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -175,104 +214,134 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
 
     if (warp == 0) {
         if (lane == 0) {
-            // producer
-            for (int kb = 0; kb < kblocks; kb++) {
-                const int s = kb % GSTAGES, u = kb / GSTAGES;
-                if (kb >= GSTAGES && !g_mbar_wait(&sm.empty[s], (uint32_t)((u - 1) & 1), err)) break;
-                uint8_t* st = sm.stage[s];
-                g_mbar_expect_tx(&sm.full[s], G_STAGE_BYTES);
-                const int kx = kb * GK;
-                for (int pl = 0; pl < A_TILES; pl++)
-                    tma_2d(st + pl * TILE_BYTES, &tmA, kx, (int)(pl * mpad + m0), &sm.full[s]);
-                for (int pl = 0; pl < NSPLIT; pl++)
-                    tma_2d(st + (A_TILES + pl) * TILE_BYTES, &tmB, kx, (int)(pl * nbpad + b0), &sm.full[s]);
+            // producer: the stages of all units one after another
+            int s = 0;
+            uint32_t ph = 1;  // parity of the ring's previous round (the first wait on a fresh barrier passes)
+            bool ok = true;
+            for (int u = u0; u < u1 && ok; u++) {
+                const int tile = u / a.nch;
+                const int c = u - tile * a.nch;
+                const int m0 = tile / a.n_ct * GM, b0 = tile % a.n_ct * GN;
+                const int ke = min(a.kblocks, (c + 1) * KCH_STAGES);
+                for (int kb = c * KCH_STAGES; kb < ke; kb++) {
+                    if (!(ok = g_mbar_wait(&sm.empty[s], ph, err))) break;
+                    uint8_t* st = sm.stage[s];
+                    g_mbar_expect_tx(&sm.full[s], C::STAGE_BYTES);
+                    const int kx = kb * GK;
+                    for (int pl = 0; pl < A_TILES; pl++)
+                        tma_2d(st + pl * TILE_BYTES, &tmA, kx, (int)(pl * a.mpad + m0), &sm.full[s]);
+                    for (int pl = 0; pl < NSPLIT; pl++)
+                        tma_2d(st + A_TILES * TILE_BYTES + pl * C::BT_BYTES, &tmB, kx, (int)(pl * a.nbpad + b0), &sm.full[s]);
+                    if (++s == GSTAGES) {
+                        s = 0;
+                        ph ^= 1;
+                    }
+                }
             }
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            // MMA issuer: per chunk, buffer b: C1 (cols 256b..256b+127) = A_re B,
-            // C2 (256b+128..256b+255) = A_im B, each as the six products A_i B_j, i + j <= 2
+            // MMA issuer: per unit, buffer b: C1 (cols 2 GN b ...) = A_re B,
+            // C2 (cols 2 GN b + GN ...) = A_im B, each as the six products A_i B_j, i + j <= 2
             bool ok = true;
-            for (int kb = 0; kb < kblocks && ok; kb++) {
-                const int c = kb / KCH_STAGES, first = (kb % KCH_STAGES) == 0;
-                const int buf = c & 1;
-                const uint32_t acc_base = tmem + (uint32_t)(buf * 256);
-                if (first && c >= 2) {
-                    ok = g_mbar_wait(&sm.acce[buf], (uint32_t)(((c >> 1) - 1) & 1), err);
+            int s = 0;
+            uint32_t ph = 0;
+            for (int u = u0; u < u1 && ok; u++) {
+                const int c = u % a.nch, cc = u - u0, buf = cc & 1;
+                const uint32_t acc_base = tmem + (uint32_t)(buf * 2 * GN);
+                if (cc >= 2) {
+                    ok = g_mbar_wait(&sm.acce[buf], (uint32_t)(((cc >> 1) - 1) & 1), err);
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 }
-                const int s = kb % GSTAGES, u = kb / GSTAGES;
-                ok = ok && g_mbar_wait(&sm.full[s], (uint32_t)(u & 1), err);
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t base = s_u32(sm.stage[s]);
+                const int kb0 = c * KCH_STAGES, ke = min(a.kblocks, kb0 + KCH_STAGES);
+                for (int kb = kb0; kb < ke && ok; kb++) {
+                    if (!(ok = g_mbar_wait(&sm.full[s], ph, err))) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint32_t base = s_u32(sm.stage[s]);
 #pragma unroll
-                for (int kk = 0; kk < GK / 16; kk++) {
-                    const uint32_t off = kk * 32;
-                    uint64_t ar[NSPLIT], ai[NSPLIT], bd[NSPLIT];
+                    for (int kk = 0; kk < GK / 16; kk++) {
+                        const uint32_t off = kk * 32;
+                        uint64_t ar[NSPLIT], ai[NSPLIT], bd[NSPLIT];
 #pragma unroll
-                    for (int t = 0; t < NSPLIT; t++) {
-                        ar[t] = smem_desc(base + t * TILE_BYTES + off);
-                        ai[t] = smem_desc(base + (NSPLIT + t) * TILE_BYTES + off);
-                        bd[t] = smem_desc(base + (A_TILES + t) * TILE_BYTES + off);
+                        for (int t = 0; t < NSPLIT; t++) {
+                            ar[t] = smem_desc(base + t * TILE_BYTES + off);
+                            ai[t] = smem_desc(base + (NSPLIT + t) * TILE_BYTES + off);
+                            bd[t] = smem_desc(base + A_TILES * TILE_BYTES + t * C::BT_BYTES + off);
+                        }
+                        const uint32_t acc = (kb > kb0 || kk > 0) ? 1u : 0u;
+#pragma unroll
+                        for (int h = 0; h < 2; h++) {
+                            const uint64_t* A = h ? ai : ar;
+                            const uint32_t d = acc_base + h * GN;
+                            mma_bf16(C::IDESC, d, A[0], bd[0], acc);
+                            mma_bf16(C::IDESC, d, A[0], bd[1], 1u);
+                            mma_bf16(C::IDESC, d, A[1], bd[0], 1u);
+                            mma_bf16(C::IDESC, d, A[0], bd[2], 1u);
+                            mma_bf16(C::IDESC, d, A[1], bd[1], 1u);
+                            mma_bf16(C::IDESC, d, A[2], bd[0], 1u);
+                        }
                     }
-                    const uint32_t acc = (!first || kk > 0) ? 1u : 0u;
-                    mma_bf16(acc_base, ar[0], bd[0], acc);
-                    mma_bf16(acc_base, ar[0], bd[1], 1u);
-                    mma_bf16(acc_base, ar[1], bd[0], 1u);
-                    mma_bf16(acc_base, ar[0], bd[2], 1u);
-                    mma_bf16(acc_base, ar[1], bd[1], 1u);
-                    mma_bf16(acc_base, ar[2], bd[0], 1u);
-                    mma_bf16(acc_base + 128, ai[0], bd[0], acc);
-                    mma_bf16(acc_base + 128, ai[0], bd[1], 1u);
-                    mma_bf16(acc_base + 128, ai[1], bd[0], 1u);
-                    mma_bf16(acc_base + 128, ai[0], bd[2], 1u);
-                    mma_bf16(acc_base + 128, ai[1], bd[1], 1u);
-                    mma_bf16(acc_base + 128, ai[2], bd[0], 1u);
+                    mma_commit(&sm.empty[s]);
+                    if (++s == GSTAGES) {
+                        s = 0;
+                        ph ^= 1;
+                    }
                 }
-                mma_commit(&sm.empty[s]);
-                if ((kb % KCH_STAGES) == KCH_STAGES - 1 || kb == kblocks - 1) mma_commit(&sm.accf[buf]);
+                if (ok) mma_commit(&sm.accf[buf]);
             }
-            // a chunk cut short by a timeout still signals its buffer
+            // a unit cut short by a timeout still signals its buffer
             if (!ok) {
                 mma_commit(&sm.accf[0]);
                 mma_commit(&sm.accf[1]);
             }
         }
     } else {
-        // accumulate each chunk (round-to-nearest FP32) and write Y
+        // accumulate each unit (round-to-nearest FP32); at the end of a tile or of the CTA's range write the sums
         const int q = warp & 3;  // TMEM lane quarter this warp may access
-        const int row = m0 + q * 32 + lane;
-        float yr[64], yi[64];
+        float yr[HN], yi[HN];
 #pragma unroll
-        for (int j = 0; j < 64; j++) yr[j] = yi[j] = 0.f;
-        for (int c = 0; c < nchunks; c++) {
-            const int buf = c & 1;
-            g_mbar_wait(&sm.accf[buf], (uint32_t)((c >> 1) & 1), err);
+        for (int j = 0; j < HN; j++) yr[j] = yi[j] = 0.f;
+        for (int u = u0; u < u1; u++) {
+            const int tile = u / a.nch;
+            const int cc = u - u0, buf = cc & 1;
+            g_mbar_wait(&sm.accf[buf], (uint32_t)((cc >> 1) & 1), err);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t lb = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 256);
+            const uint32_t lb = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 2 * GN);
 #pragma unroll
-            for (int jc = 0; jc < 64; jc += 16) {
-                float ta[16], tb[16];
-                tmem_ld16(lb + jc, ta);         // A_re X_re
-                tmem_ld16(lb + 192 + jc, tb);   // A_im X_im
+            for (int jc = 0; jc < HN; jc += 8) {
+                float ta[8], tb[8];
+                tmem_ld8(lb + jc, ta);                // A_re X_re
+                tmem_ld8(lb + GN + HN + jc, tb);      // A_im X_im
 #pragma unroll
-                for (int j = 0; j < 16; j++) yr[jc + j] += ta[j] - tb[j];
-                tmem_ld16(lb + 64 + jc, ta);    // A_re X_im
-                tmem_ld16(lb + 128 + jc, tb);   // A_im X_re
+                for (int j = 0; j < 8; j++) yr[jc + j] += ta[j] - tb[j];
+                tmem_ld8(lb + HN + jc, ta);           // A_re X_im
+                tmem_ld8(lb + GN + jc, tb);           // A_im X_re
 #pragma unroll
-                for (int j = 0; j < 16; j++) yi[jc + j] += ta[j] + tb[j];
+                for (int j = 0; j < 8; j++) yi[jc + j] += ta[j] + tb[j];
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0)
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s_u32(&sm.acce[buf])) : "memory");
-        }
-        if (row < m) {
+            if (u + 1 < u1 && (u + 1) % a.nch != 0) continue;
+            const int ct = tile % a.n_ct, r = q * 32 + lane, row = tile / a.n_ct * GM + r;
+            if (a.part) {
+                const int piece = blockIdx.x - gemm_first_cta(a.units, gridDim.x, a.nch, tile);
+                float2* out = a.part + (int64_t)(tile * a.pieces + piece) * HN * GM + r;
 #pragma unroll
-            for (int j = 0; j < 64; j++) {
-                const int rhs = ct * 64 + j;
-                if (rhs < n_rhs) Y[(int64_t)rhs * m + row] = make_float2(yr[j], yi[j]);
+                for (int j = 0; j < HN; j++)
+                    if (ct * HN + j < a.n_rhs) out[j * GM] = make_float2(yr[j], yi[j]);
+            } else if (row < a.m) {
+#pragma unroll
+                for (int j = 0; j < HN; j++) {
+                    const int rhs = ct * HN + j;
+                    if (rhs >= a.n_rhs) continue;
+                    if (a.Y64) a.Y64[(int64_t)rhs * a.m + row] = make_double2(yr[j], yi[j]);
+                    else a.Y[(int64_t)rhs * a.m + row] = make_float2(yr[j], yi[j]);
+                }
             }
+#pragma unroll
+            for (int j = 0; j < HN; j++) yr[j] = yi[j] = 0.f;
         }
     }
     __syncwarp();
@@ -280,8 +349,25 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     __syncthreads();
     if (warp == 2) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::TMEM_COLS) : "memory");
     }
+}
+
+// Y = the pieces of every tile summed in CTA order (one column tile: n_rhs <= HN).
+__global__ void gemm_finish_kernel(GemmArgs a, int ctas, int hn) {
+    const int row = blockIdx.x * blockDim.x + threadIdx.x, rhs = blockIdx.y;
+    if (row >= a.m) return;
+    const int tile = row / GM;
+    const int first = gemm_first_cta(a.units, ctas, a.nch, tile);
+    float2 y = make_float2(0.f, 0.f);
+    for (int p = 0; p < a.pieces; p++) {
+        if (first + p >= ctas || gemm_first_unit(a.units, ctas, first + p) >= (tile + 1) * a.nch) break;
+        const float2 v = a.part[((int64_t)(tile * a.pieces + p) * hn + rhs) * GM + row % GM];
+        y.x += v.x;
+        y.y += v.y;
+    }
+    if (a.Y64) a.Y64[(int64_t)rhs * a.m + row] = make_double2(y.x, y.y);
+    else a.Y[(int64_t)rhs * a.m + row] = y;
 }
 
 // x -> three BF16 terms, x ~ t0 + t1 + t2
@@ -304,18 +390,19 @@ __global__ void split_a_kernel(const float2* A, int64_t m, int64_t k, int64_t mp
     split3(v.y, P[3 * plane + idx], P[4 * plane + idx], P[5 * plane + idx]);
 }
 
-// X (n_rhs x k, complex64, rhs-major) -> bf16 planes [t0, t1, t2][nbpad][kpad];
-// B row of rhs j, part p (0 re, 1 im) = (j / 64) * 128 + p * 64 + j % 64.
-__global__ void split_x_kernel(const float2* X, int64_t n_rhs, int64_t k, int64_t nbpad, int64_t kpad,
+// X (n_rhs x k, complex64 or complex128 rounded to it, rhs-major) -> bf16 planes [t0, t1, t2][nbpad][kpad];
+// B row of rhs j, part p (0 re, 1 im) = (j / hn) * 2 hn + p * hn + j % hn.
+template <class T>
+__global__ void split_x_kernel(const T* X, int64_t n_rhs, int64_t k, int64_t nbpad, int64_t kpad, int hn,
                                __nv_bfloat16* P) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= nbpad * kpad) return;
     const int64_t brow = idx / kpad, c = idx % kpad;
-    const int64_t blk = brow / 128, within = brow % 128, part = within / 64, j = blk * 64 + within % 64;
+    const int64_t blk = brow / (2 * hn), within = brow % (2 * hn), part = within / hn, j = blk * hn + within % hn;
     float x = 0.f;
     if (j < n_rhs && c < k) {
-        const float2 v = X[j * k + c];
-        x = part ? v.y : v.x;
+        const T v = X[j * k + c];
+        x = (float)(part ? v.y : v.x);
     }
     split3(x, P[idx], P[nbpad * kpad + idx], P[2 * nbpad * kpad + idx]);
 }
@@ -335,12 +422,12 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     return fn;
 }
 
-static bool make_map(CUtensorMap* map, void* base, int64_t rows, int64_t kpad) {
+static bool make_map(CUtensorMap* map, void* base, int64_t rows, int64_t kpad, int box_rows) {
     auto fn = encode_fn();
     if (!fn) return false;
     cuuint64_t dims[2] = {(cuuint64_t)kpad, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)kpad * 2};
-    cuuint32_t box[2] = {GK, GM};
+    cuuint32_t box[2] = {GK, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -348,31 +435,76 @@ static bool make_map(CUtensorMap* map, void* base, int64_t rows, int64_t kpad) {
     return r == CUDA_SUCCESS;
 }
 
+// Right-hand sides per column tile and bytes of scratch (X planes, then the
+// pieces of a split product) for n_rhs right-hand sides.
+static int gemm_hn(int64_t n_rhs) { return n_rhs <= 16 ? 16 : 64; }
+static int gemm_pieces(int64_t units, int64_t ctas, int nch) {
+    const int q = (int)(units / ctas);  // a CTA holds q or q + 1 units
+    return (nch + q - 1) / q + 1;
+}
+size_t gemm_work_bytes(int64_t mpad, int64_t kpad, int64_t n_rhs) {
+    const int hn = gemm_hn(n_rhs);
+    const int64_t nbpad = (n_rhs + hn - 1) / hn * 2 * hn;
+    size_t b = (size_t)NSPLIT * nbpad * kpad * 2;
+    if (n_rhs <= hn) {
+        const int nch = (int)((kpad / GK + KCH_STAGES - 1) / KCH_STAGES);
+        const int64_t units = mpad / GM * nch, ctas = std::min<int64_t>(GEMM_CTAS, units);
+        b = (b + 15) / 16 * 16 + (size_t)(mpad / GM) * gemm_pieces(units, ctas, nch) * hn * GM * sizeof(float2);
+    }
+    return b;
+}
+
+template <int GN>
+static cudaError_t launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, const GemmArgs& a, unsigned ctas, cudaStream_t s) {
+    constexpr size_t smem = sizeof(typename GemmCfg<GN>::Smem) + 1024;
+    static const cudaError_t attr_e =
+        cudaFuncSetAttribute(gemm_bf16x3_kernel<GN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (attr_e != cudaSuccess) return attr_e;
+    gemm_bf16x3_kernel<GN><<<ctas, GEMM_THREADS, smem, s>>>(ta, tb, a);
+    return cudaGetLastError();
+}
+
 // Planes of A are kept by the caller (they are the assembled operator); X
-// is split per call.  Y (n_rhs x m complex64) = A X.
+// is split per call into work (gemm_work_bytes).  X is complex64 (X) or
+// complex128 (X64), and Y (n_rhs x m) = A X likewise.
 int gemm_bf16x3(bem_ctx* ctx, const __nv_bfloat16* Aplanes, int64_t m, int64_t k, int64_t mpad, int64_t kpad,
-                const float2* X, int64_t n_rhs, float2* Y, __nv_bfloat16* xplanes, int64_t nbpad) {
-    static_assert(sizeof(GemmSmem) <= 227 * 1024 - 1024, "gemm smem");
+                const float2* X, const double2* X64, int64_t n_rhs, float2* Y, double2* Y64, void* work) {
+    const int hn = gemm_hn(n_rhs);
+    const int64_t nbpad = (n_rhs + hn - 1) / hn * 2 * hn;
+    __nv_bfloat16* xplanes = (__nv_bfloat16*)work;
     CUtensorMap ta, tb;
-    if (!make_map(&ta, (void*)Aplanes, A_TILES * mpad, kpad) || !make_map(&tb, (void*)xplanes, NSPLIT * nbpad, kpad))
+    if (!make_map(&ta, (void*)Aplanes, A_TILES * mpad, kpad, GM) || !make_map(&tb, (void*)xplanes, NSPLIT * nbpad, kpad, 2 * hn))
         return ctx->fail(BEM_ERR_CUDA, "cuTensorMapEncodeTiled failed");
     const int64_t nx = nbpad * kpad;
-    split_x_kernel<<<(unsigned)((nx + 255) / 256), 256, 0, ctx->stream>>>(X, n_rhs, k, nbpad, kpad, xplanes);
-    const size_t smem = sizeof(GemmSmem) + 1024;
-    static const cudaError_t attr_e =
-        cudaFuncSetAttribute(gemm_bf16x3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (attr_e != cudaSuccess) return ctx->fail(BEM_ERR_CUDA, std::string("gemm attribute: ") + cudaGetErrorString(attr_e));
-    const dim3 grid((unsigned)(nbpad / GN), (unsigned)(mpad / GM));
-    gemm_bf16x3_kernel<<<grid, GEMM_THREADS, smem, ctx->stream>>>(ta, tb, mpad, nbpad, (int)(kpad / GK), (int)m,
-                                                                  (int)n_rhs, Y, ctx->dev.err);
+    const unsigned nbx = (unsigned)((nx + 255) / 256);
+    if (X64) split_x_kernel<<<nbx, 256, 0, ctx->stream>>>(X64, n_rhs, k, nbpad, kpad, hn, xplanes);
+    else split_x_kernel<<<nbx, 256, 0, ctx->stream>>>(X, n_rhs, k, nbpad, kpad, hn, xplanes);
+    GemmArgs a{};
+    a.mpad = mpad; a.nbpad = nbpad; a.kblocks = (int)(kpad / GK); a.m = (int)m; a.n_rhs = (int)n_rhs;
+    a.n_ct = (int)(nbpad / (2 * hn));
+    a.nch = (a.kblocks + KCH_STAGES - 1) / KCH_STAGES;
+    a.units = (int)(mpad / GM * a.n_ct * a.nch);
+    a.Y = Y; a.Y64 = Y64; a.err = ctx->dev.err;
+    const bool split = a.n_ct == 1;
+    int64_t ctas = mpad / GM * a.n_ct;  // whole tiles
+    if (split) {
+        ctas = std::min<int64_t>(GEMM_CTAS, a.units);
+        a.pieces = gemm_pieces(a.units, ctas, a.nch);
+        a.part = (float2*)((char*)work + ((size_t)NSPLIT * nx * 2 + 15) / 16 * 16);
+    }
+    cudaError_t e = hn == 16 ? launch_gemm<32>(ta, tb, a, (unsigned)ctas, ctx->stream)
+                             : launch_gemm<128>(ta, tb, a, (unsigned)ctas, ctx->stream);
     ctx->launches += 2;
-    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess && split) {
+        gemm_finish_kernel<<<dim3((unsigned)((m + 255) / 256), (unsigned)n_rhs), 256, 0, ctx->stream>>>(a, (int)ctas, hn);
+        ctx->launches++;
+        e = cudaGetLastError();
+    }
     if (e != cudaSuccess) return ctx->fail(BEM_ERR_CUDA, std::string("gemm launch: ") + cudaGetErrorString(e));
     return BEM_OK;
 }
 
 int gemm_a_planes() { return A_TILES; }
-int gemm_b_planes() { return NSPLIT; }
 int gemm_k_align() { return GK; }
 
 int split_a(bem_ctx* ctx, const float2* A, int64_t m, int64_t k, int64_t mpad, int64_t kpad, __nv_bfloat16* P) {
@@ -401,17 +533,16 @@ extern "C" int bem_zgemm_bf16x3(bem_ctx* ctx, int64_t m, int64_t k, int64_t n_rh
         cudaMemsetAsync(ctx->dev.err, 0, sizeof(int), ctx->stream);
     }
     const int64_t mpad = (m + GM - 1) / GM * GM, kpad = (k + GK - 1) / GK * GK;
-    const int64_t nbpad = (n_rhs + 63) / 64 * 128;
     int rc;
     __nv_bfloat16* ap = (__nv_bfloat16*)ctx->dalloc((size_t)A_TILES * mpad * kpad * 2, &rc);
     if (rc) return rc;
-    __nv_bfloat16* xp = (__nv_bfloat16*)ctx->dalloc((size_t)NSPLIT * nbpad * kpad * 2, &rc);
+    void* work = ctx->dalloc(gemm_work_bytes(mpad, kpad, n_rhs), &rc);
     if (rc) { ctx->dfree(ap); return rc; }
     rc = split_a(ctx, (const float2*)A, m, k, mpad, kpad, ap);
-    if (!rc) rc = gemm_bf16x3(ctx, ap, m, k, mpad, kpad, (const float2*)X, n_rhs, (float2*)Y, xp, nbpad);
+    if (!rc) rc = gemm_bf16x3(ctx, ap, m, k, mpad, kpad, (const float2*)X, nullptr, n_rhs, (float2*)Y, nullptr, work);
     cudaStreamSynchronize(ctx->stream);
     ctx->dfree(ap);
-    ctx->dfree(xp);
+    ctx->dfree(work);
     if (!rc) rc = ctx->check_device_error();
     return rc;
 }

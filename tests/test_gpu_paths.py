@@ -35,3 +35,26 @@ def test_short_chunks_fall_back_under_a_budget(api):
     assert np.array_equal(y, ref)
     assert c.memory()[0] < used - (1 << 28)
     c.close()
+
+
+@pytest.mark.parametrize("m,k,n", [(1, 1, 1), (128, 32, 16), (129, 33, 3), (130, 2049, 16), (19500, 40, 2), (257, 8200, 1),
+                                   (640, 300, 17), (384, 513, 64), (150, 290, 65)])
+def test_gemm_split_over_ctas(m, k, n):
+    """The split-BF16 product with its units spread over the CTAs (up to 64
+    right-hand sides) and with whole tiles (more), at ragged sizes; each of the
+    k terms is good to ~2^-23, and rounding of FP32 sums grows like sqrt(k)."""
+    import torch
+    from paper_1910_01011_gb300 import _lib
+    from paper_1910_01011_gb300.api import Context
+    g = torch.Generator().manual_seed(m + k + n)
+    A = torch.randn(m, k, 2, generator=g)
+    X = torch.randn(n, k, 2, generator=g)
+    Ac, Xc = torch.view_as_complex(A), torch.view_as_complex(X)
+    ref = Xc.to(torch.complex128) @ Ac.to(torch.complex128).T
+    c = Context(0, hbm_budget_bytes=0)
+    d, x, y = Ac.cuda(), Xc.cuda(), torch.full((n, m), float("nan"), dtype=torch.complex64, device="cuda")
+    rc = c.lib.bem_zgemm_bf16x3(c.h, m, k, n, d.data_ptr(), x.data_ptr(), y.data_ptr())
+    _lib.check(rc, c.h)
+    err = (y.cpu().to(torch.complex128) - ref).norm() / ref.norm()
+    c.close()
+    assert err < 2e-6
