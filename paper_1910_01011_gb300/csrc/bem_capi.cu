@@ -323,13 +323,21 @@ int bem_ctx::finalize() {
     if ((rc = upload(this, &d.np_tgt, ptgt))) return rc;
     for (int r = 0; r <= 3; r++) {  // 0: the near-pair rule, 1-3: Sauter-Schwab
         if ((rc = upload(this, &d.ss_tab[r], quad.ss[r]))) return rc;
-        const size_t m = quad.ss[r].size();
-        std::vector<float> f(2 * m);  // double-float copy for the near build
-        for (size_t i = 0; i < m; i++) {
-            f[i] = (float)quad.ss[r][i];
-            f[m + i] = (float)(quad.ss[r][i] - (double)f[i]);
+        std::vector<float4> f;  // groups of the double-float near build: hi, then lo of each row
+        for (size_t i = 0; i < quad.grp[r].size(); i += 8) {
+            float h[8], l[8];
+            for (int c = 0; c < 8; c++) {
+                h[c] = (float)quad.grp[r][i + c];
+                l[c] = (float)(quad.grp[r][i + c] - (long double)h[c]);
+            }
+            for (const float* v : {h, h + 4, l, l + 4}) f.push_back(make_float4(v[0], v[1], v[2], v[3]));
         }
-        if ((rc = upload(this, &d.ss_tabf[r], f))) return rc;
+        if ((rc = upload(this, &d.grp[r], f))) return rc;
+    }
+    {
+        std::vector<float2> f;
+        for (const long double v : quad.inner) f.push_back(make_float2((float)v, (float)(v - (long double)(float)v)));
+        if ((rc = upload(this, &d.inner, f))) return rc;
     }
     // working buffers
     d.pd32 = (float4*)dalloc(g.n_pts * sizeof(float4), &rc); if (rc) return rc;
@@ -407,7 +415,12 @@ int bem_ctx::build_near(NearSet& ns, int n_slot_k, double kre, double kim, const
         if (opts.fp64_far == 0) {  // double-float point evaluations (the default), else native FP64
             if ((rc = ensure_fardf()) || (rc = check_df_phase(kre, false))) return rc;
             a.use_df = 1;
-            for (int r = 0; r <= 3; r++) a.ss_tabf[r] = dev.ss_tabf[r];
+            for (int r = 0; r <= 3; r++) {
+                a.grp[r] = dev.grp[r];
+                a.grp_n[r] = (int)(quad.grp[r].size() / 8);
+            }
+            a.inner = dev.inner;
+            a.ng = quad.ng;
             a.sctab = dfg.sctab;
             a.extab = dfg.extab;
             a.c = dfg.c;
@@ -419,7 +432,6 @@ int bem_ctx::build_near(NearSet& ns, int n_slot_k, double kre, double kim, const
             split((long double)kre, a.k0df.x, a.k0df.y);
             split((long double)kim, a.k0df.z, a.k0df.w);
             for (int q = 0; q < 3 * QP; q++) split((long double)a.rule[q], a.rule_h[q], a.rule_l[q]);
-            split(1.0L / (4.0L * 3.141592653589793238462643383279502884L), a.i4h, a.i4l);
         }
         CK(launch_near_build(a, stream));
         NearCombineArgs c{};
@@ -874,7 +886,7 @@ int bem_create(bem_ctx** out, int device, void* cuda_stream, const bem_opts* opt
     c->stream = (cudaStream_t)cuda_stream;
     bem_default_opts(&c->opts);
     if (opts) c->opts = *opts;
-    if (c->opts.n_gauss_singular < 2 || c->opts.n_gauss_singular > 20 || !(c->opts.osrc_tol > 0) ||
+    if (c->opts.n_gauss_singular < 2 || c->opts.n_gauss_singular > NEAR_NG_MAX || !(c->opts.osrc_tol > 0) ||
         !(c->opts.osrc_tol < 1) || c->opts.osrc_solver < 0 || c->opts.osrc_solver > 4 ||
         c->opts.osrc_wavenumber < 0 || c->opts.osrc_wavenumber > 1 || c->opts.fp64_far < 0 || c->opts.fp64_far > 1) {
         delete c;

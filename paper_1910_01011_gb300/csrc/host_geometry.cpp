@@ -113,9 +113,10 @@ bool gauss_legendre01(int n, std::vector<double>& x, std::vector<double>& w) {
 // reference points s (test), t (trial) in {0 <= s2 <= s1 <= 1} and the
 // Jacobian.  Identical: 6 regions; common edge on s2 = t2 = 0: 5 regions;
 // common vertex at the origin: 2 regions.
-static void ss_map(int rel, int reg, double xi, double e1, double e2, double e3, double s[2], double t[2]) {
+template <class R>
+static void ss_map(int rel, int reg, R xi, R e1, R e2, R e3, R s[2], R t[2]) {
     if (rel == 3) {
-        const double a = e1 * e2 * e3, b = e1 * e2;
+        const R a = e1 * e2 * e3, b = e1 * e2;
         switch (reg) {
             case 0: s[0] = xi; s[1] = xi * (1 - e1 + b); t[0] = xi * (1 - a); t[1] = xi * (1 - e1); break;
             case 1: s[0] = xi * (1 - a); s[1] = xi * (1 - e1); t[0] = xi; t[1] = xi * (1 - e1 + b); break;
@@ -138,9 +139,10 @@ static void ss_map(int rel, int reg, double xi, double e1, double e2, double e3,
     }
 }
 
-static double ss_jac(int rel, int reg, double xi, double e1, double e2) {
+template <class R>
+static R ss_jac(int rel, int reg, R xi, R e1, R e2) {
     if (rel == 3) return xi * xi * xi * e1 * e1 * e2;
-    if (rel == 2) return xi * xi * xi * e1 * e1 * (reg == 0 ? 1.0 : e2);
+    if (rel == 2) return xi * xi * xi * e1 * e1 * (reg == 0 ? (R)1 : e2);
     return xi * xi * xi * e2;
 }
 
@@ -182,6 +184,39 @@ bool build_quadrature(Quadrature& q, int n_gauss) {
                             double wt = gw[a] * gw[b] * gw[c] * gw[d] * ss_jac(rel, reg, gx[a], gx[b], gx[c]);
                             tab.insert(tab.end(), {s[0], s[1], t[0], t[1], wt});
                         }
+    }
+    // the tables as groups along the innermost direction, in which every map is linear
+    typedef long double ld;
+    q.inner.clear();
+    for (int d = 0; d < n_gauss; d++) {
+        const ld g = gx[d], w = gw[d];
+        q.inner.insert(q.inner.end(), {g, w, w * g, w * g * g});
+    }
+    for (int rel = 0; rel <= 3; rel++) {
+        const int nreg = rel == 3 ? 6 : rel == 2 ? 5 : rel == 1 ? 2 : 1;
+        auto& tab = q.grp[rel];
+        tab.clear();
+        for (int reg = 0; reg < nreg; reg++)
+            for (int a = 0; a < n_gauss; a++)
+                for (int b = 0; b < n_gauss; b++)
+                    for (int c = 0; c < n_gauss; c++) {
+                        ld s[2][2], t[2][2];  // both points at g = 0 and 1
+                        for (int e = 0; e < 2; e++) {
+                            if (rel) ss_map<ld>(rel, reg, gx[a], gx[b], gx[c], e, s[e], t[e]);
+                            else {
+                                s[e][0] = gx[a];
+                                s[e][1] = (ld)gx[a] * gx[b];
+                                t[e][0] = gx[c];
+                                t[e][1] = (ld)gx[c] * e;
+                            }
+                        }
+                        const bool first = s[0][0] != s[1][0] || s[0][1] != s[1][1];
+                        const ld(*m)[2] = first ? s : t, *f = first ? t[0] : s[0];
+                        const ld w = (ld)gw[a] * gw[b] * gw[c] *
+                                     (rel ? ss_jac<ld>(rel, reg, gx[a], gx[b], gx[c]) : (ld)gx[a] * gx[c]);
+                        tab.insert(tab.end(), {f[0], f[1], m[0][0], m[0][1], m[1][0] - m[0][0], m[1][1] - m[0][1], w,
+                                               first ? (ld)1 : (ld)0});
+                    }
     }
     return true;
 }

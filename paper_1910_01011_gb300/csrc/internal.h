@@ -23,6 +23,7 @@ constexpr int TT = 32;          // triangles per tile
 constexpr int QP = 6;           // regular-rule points per triangle
 constexpr int TP = TT * QP;     // points per tile = threads of a far-field CTA
 constexpr int NCOMP = 14;       // potentials per target point and wavenumber slot
+constexpr int NEAR_NG_MAX = 20; // Gauss points per direction of the near-field rules, at most
 constexpr int CHUNK_MAX = 256;  // source tiles per far-field CTA (shared-memory table bound)
 
 // ------------------------------------------------------------------ host geometry
@@ -35,6 +36,10 @@ struct Quadrature {
     // triangle; 1 vertex, 2 edge, 3 identical: Sauter-Schwab):
     // rows (s1, s2, t1, t2, weight * jacobian)
     std::vector<double> ss[4];
+    // the same tables without their innermost direction g in [0, 1], which moves one of the two points along a
+    // line: rows (fixed point f1, f2; moving point m1, m2 at g = 0 and its change d1, d2 over g = 0..1; weight *
+    // jacobian; 1 if the first point moves, else 0), and that direction's rows (g, w, w g, w g^2)
+    std::vector<long double> grp[4], inner;
 };
 
 struct HostDomain {
@@ -292,17 +297,20 @@ struct NearArgs {
     const int* slot_dom;        // via slot_v.w
     int n_slot_k;               // 1 or 2
     double2* raw;               // [pair][slot][27]: V, K, K' (SS minus regular)
-    // double-float point evaluations (use_df): tables as (hi, lo) floats,
-    // sin / cos / exp tables and constants, wavenumbers, regular rule, 1 / (4 pi)
+    // double-float point evaluations (use_df): sin / cos / exp tables and constants, wavenumbers, regular rule
     int use_df;
-    const float* ss_tabf[4];
+    // the same rules as groups of points along a line (4 float4 each: hi then lo
+    // of f1, f2, m1, m2 | d1, d2, weight, side), and the innermost rule (g, w, w g, w g^2)
+    const float4* grp[4];
+    int grp_n[4];
+    const float2* inner;
+    int ng;
     const float4* sctab;
     const float2* extab;
     DfConsts c;
     const float4* kdf;
     float4 k0df;
     float rule_h[3 * QP], rule_l[3 * QP];
-    float i4h, i4l;
 };
 
 struct NearCombineArgs {

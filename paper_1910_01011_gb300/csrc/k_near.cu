@@ -137,15 +137,33 @@ __global__ void __launch_bounds__(NEAR_THREADS) near_build_kernel(NearArgs A) {
 
 // ---- the same integrals with double-float point evaluations (df_math.cuh):
 // GB300 runs FP64 at ~1/64 of its FP32 rate and every point pair costs a
-// square root, a reciprocal and a sincos; the pair's geometry is split once
-// into shared memory, the table points are read as (hi, lo) floats, and the
-// 27 complex moments of each thread are converted to FP64 once for the
-// block reduction (relative accuracy ~1e-13).
+// square root, a reciprocal and a sincos.
+//
+// Every rule is a tensor product whose innermost direction moves the point of
+// one triangle along a line and leaves the other point where it is, so a
+// table row is a group: the fixed point, the line of the moving one, the
+// weight without the innermost factor.  A thread evaluates the points of one
+// group.  Along the line the moving P1 functions and the one of (y - x).n_y,
+// (x - y).n_x that is not constant are linear in the innermost coordinate, so
+// five complex sums per point carry everything: G, G g, F, F g, F g^2.
+// They are expanded to three sums per moving vertex for each of V, K and K'
+// (relative accuracy ~1e-13, as the evaluations), and the CTA's groups meet
+// in shared memory, where lane (operator, i, j) of each warp multiplies them
+// with the fixed point's P1 values and adds them up; four warps' sums are
+// added in FP64.  One point per thread with all 27 complex moments in
+// registers (255 of them, eight warps per SM), each reduced over the CTA by
+// FP64 shuffles, which ran on the 1/64-rate pipe for longer than the points
+// on theirs, took 198 ms (4,620-triangle rib scene); now 57.6 ms.
+//
+// The regular rule is subtracted by six more groups (one per fixed point)
+// whose points do not lie on a line; they sum the expanded form directly.
+
+constexpr int NEAR_S = 9;                    // complex sums of a group: V, K, K' x moving vertex
+constexpr int NEAR_ROW = 2 * NEAR_S + 3 + 1;  // (h, l) pairs of a group in shared memory: sums, P1 values, side
 
 struct NearGeomDF {
-    dfl X0[3], X1[3], X2[3], Y0[3], Y1[3], Y2[3];  // Sauter-Schwab parametrisations (reordered vertices)
-    dfl O0[3], Ou[3], Ov[3], Q0[3], Qu[3], Qv[3];  // regular-rule parametrisations (original order)
-    dfl nx[3], ny[3], scale, axay;
+    dfl v[14][3];  // X0, X1, X2, Y0, Y1, Y2 (reordered vertices), O0, Ou, Ov, Q0, Qu, Qv (original), nx, ny
+    dfl scale, axay;
 };
 
 __device__ __forceinline__ dfl split_d(double v) {
@@ -153,166 +171,271 @@ __device__ __forceinline__ dfl split_d(double v) {
     return dfl{h, (float)(v - (double)h)};
 }
 
-template <bool ATTEN>
-__device__ __forceinline__ void kernel_eval_df(const dfl (&x)[3], const dfl (&y)[3], const NearGeomDF& G, dfl kr,
-                                               dfl ki, dfl w, const dfl (&lx)[3], const dfl (&ly)[3],
-                                               const NearArgs& A, const float4* __restrict__ tab,
-                                               const float2* __restrict__ etab, dfl (&acc)[NACC][2]) {
-    const dfl d0 = dsub(x[0], y[0]), d1 = dsub(x[1], y[1]), d2 = dsub(x[2], y[2]);
-    dfl r, ri;
-    dsqrt_rinv(dadd(dadd(dsqr(d0), dsqr(d1)), dsqr(d2)), r, ri);
-    dfl sn, cs;
-    dsincos(dmul(kr, r), A.c, tab, sn, cs);
-    dfl a = dmul(dmul(ri, dfl{A.i4h, A.i4l}), w);  // w G magnitude
-    if (ATTEN) a = dmul(a, dexp_neg(dmul(ki, r), A.c, etab));
-    const dfl Gr = dmul(a, cs), Gi = dmul(a, sn);
-    const dfl u = dsub(dneg(ki), ri);  // Re(ik - 1/r)
-    const dfl Fr = dmul(dsub(dmul(Gr, u), dmul(Gi, kr)), ri);
-    const dfl Fi = dmul(dadd(dmul(Gr, kr), dmul(Gi, u)), ri);
-    const dfl dny = dneg(dadd(dadd(dmul(d0, G.ny[0]), dmul(d1, G.ny[1])), dmul(d2, G.ny[2])));  // (y - x).n_y
-    const dfl dnx = dadd(dadd(dmul(d0, G.nx[0]), dmul(d1, G.nx[1])), dmul(d2, G.nx[2]));        // (x - y).n_x
-    const dfl Fyr = dmul(Fr, dny), Fyi = dmul(Fi, dny), Fxr = dmul(Fr, dnx), Fxi = dmul(Fi, dnx);
-#pragma unroll
-    for (int i = 0; i < 3; i++)
-#pragma unroll
-        for (int j = 0; j < 3; j++) {
-            const dfl pp = dmul(lx[i], ly[j]);
-            dmac(acc[3 * i + j][0], Gr, pp, 1.0f);
-            dmac(acc[3 * i + j][1], Gi, pp, 1.0f);
-            dmac(acc[9 + 3 * i + j][0], Fyr, pp, 1.0f);
-            dmac(acc[9 + 3 * i + j][1], Fyi, pp, 1.0f);
-            dmac(acc[18 + 3 * i + j][0], Fxr, pp, 1.0f);
-            dmac(acc[18 + 3 * i + j][1], Fxi, pp, 1.0f);
-        }
+__device__ __forceinline__ dfl ddot3(const dfl (&a)[3], const dfl (&b)[3]) {
+    return dadd(dadd(dmul(a[0], b[0]), dmul(a[1], b[1])), dmul(a[2], b[2]));
 }
 
-// lx[pa[i]] = v[i] for a permutation pa, without run-time register indexing
+// G r^0 = e^{ikr} / r and F = G (ik - 1/r) / r at the difference e (without the 1 / (4 pi))
+template <bool ATTEN>
+__device__ __forceinline__ void near_gf(const dfl (&e)[3], dfl kr, dfl ki, const NearArgs& A,
+                                        const float4* __restrict__ tab, const float2* __restrict__ etab, dfl& Gr, dfl& Gi,
+                                        dfl& Fr, dfl& Fi) {
+    dfl r, ri;
+    dsqrt_rinv(dadd(dadd(dsqr(e[0]), dsqr(e[1])), dsqr(e[2])), r, ri);
+    dfl sn, cs;
+    dsincos(dmul(kr, r), A.c, tab, sn, cs);
+    dfl a = ri;
+    if (ATTEN) a = dmul(a, dexp_neg(dmul(ki, r), A.c, etab));
+    Gr = dmul(a, cs);
+    Gi = dmul(a, sn);
+    const dfl u = ATTEN ? dsub(dneg(ki), ri) : dneg(ri);  // Re(ik - 1/r)
+    Fr = dmul(dsub(dmul(Gr, u), dmul(Gi, kr)), ri);
+    Fi = dmul(dadd(dmul(Gr, kr), dmul(Gi, u)), ri);
+}
+
+// out[j] = v[i] with pa[i] = j, without run-time register indexing
 __device__ __forceinline__ void permute3(const dfl (&v)[3], const int (&pa)[3], dfl (&out)[3]) {
 #pragma unroll
     for (int j = 0; j < 3; j++) out[j] = pa[0] == j ? v[0] : pa[1] == j ? v[1] : v[2];
 }
+// P1 values (1 - s1, s1 - s2, s2), or with c = 0 their change along (s1, s2)
+__device__ __forceinline__ void bary(dfl s1, dfl s2, float c, const int (&pa)[3], dfl (&out)[3]) {
+    const dfl v[3] = {dsub(dfl{c, 0.0f}, s1), dsub(s1, s2), s2};
+    permute3(v, pa, out);
+}
 
 template <bool ATTEN>
-__device__ __forceinline__ void near_df_body(const NearArgs& A, const NearGeomDF& G, int rel, const int (&pa)[3],
-                                             const int (&pb)[3], dfl kr, dfl ki, bool live,
-                                             const float4* __restrict__ tab, const float2* __restrict__ etab,
-                                             dfl (&acc)[NACC][2]) {
-    const int n = live ? A.ss_n[rel] : 0;
-    const float* th = A.ss_tabf[rel];
-    const float* tl = th + 5 * (int64_t)A.ss_n[rel];
-    for (int idx = threadIdx.x; idx < n; idx += NEAR_THREADS) {
-        const dfl s1 = {th[5 * idx], tl[5 * idx]}, s2 = {th[5 * idx + 1], tl[5 * idx + 1]};
-        const dfl t1 = {th[5 * idx + 2], tl[5 * idx + 2]}, t2 = {th[5 * idx + 3], tl[5 * idx + 3]};
-        const dfl w = dmul(dfl{th[5 * idx + 4], tl[5 * idx + 4]}, G.scale);
-        dfl x[3], y[3];
+__device__ __forceinline__ void near_group(const NearArgs& A, const NearGeomDF& G, int rel, int idx, const int (&pa)[3],
+                                           const int (&pb)[3], dfl kr, dfl ki, const float4* __restrict__ tab,
+                                           const float2* __restrict__ etab, const float2 (*__restrict__ inner)[4],
+                                           float2* __restrict__ row) {
+    const float4* T = A.grp[rel] + 4 * (int64_t)idx;
+    const float4 fh = T[0], wh = T[1], fl = T[2], wl = T[3];
+    const dfl f1 = {fh.x, fl.x}, f2 = {fh.y, fl.y}, m1 = {fh.z, fl.z}, m2 = {fh.w, fl.w};
+    const dfl d1 = {wh.x, wl.x}, d2 = {wh.y, wl.y}, w = dmul(dfl{wh.z, wl.z}, G.scale);
+    const bool ymoves = wh.w == 0.0f;  // x fixed
+    // e = x - y = e0 + g dv along the line
+    const dfl(*Fx)[3] = G.v + (ymoves ? 0 : 3);
+    const dfl(*Mv)[3] = G.v + (ymoves ? 3 : 0);
+    dfl e0[3], dv[3];
 #pragma unroll
-        for (int c = 0; c < 3; c++) {
-            x[c] = dadd(dadd(G.X0[c], dmul(s1, G.X1[c])), dmul(s2, G.X2[c]));
-            y[c] = dadd(dadd(G.Y0[c], dmul(t1, G.Y1[c])), dmul(t2, G.Y2[c]));
-        }
-        const dfl lxr[3] = {dsub(dfl{1.0f, 0.0f}, s1), dsub(s1, s2), s2};
-        const dfl lyr[3] = {dsub(dfl{1.0f, 0.0f}, t1), dsub(t1, t2), t2};
-        dfl lx[3], ly[3];
-        permute3(lxr, pa, lx);
-        permute3(lyr, pb, ly);
-        kernel_eval_df<ATTEN>(x, y, G, kr, ki, w, lx, ly, A, tab, etab, acc);
+    for (int c = 0; c < 3; c++) {
+        const dfl fx = dadd(dadd(Fx[0][c], dmul(f1, Fx[1][c])), dmul(f2, Fx[2][c]));
+        const dfl mv = dadd(dadd(Mv[0][c], dmul(m1, Mv[1][c])), dmul(m2, Mv[2][c]));
+        const dfl sl = dadd(dmul(d1, Mv[1][c]), dmul(d2, Mv[2][c]));
+        e0[c] = ymoves ? dsub(fx, mv) : dsub(mv, fx);
+        dv[c] = ymoves ? dneg(sl) : sl;
     }
-    // minus the regular rule the far-field kernel applied (not for identical pairs)
-    if (rel != 3 && live)
-        for (int idx = threadIdx.x; idx < QP * QP; idx += NEAR_THREADS) {
-            const int qa = idx / QP, qb = idx % QP;
-            const dfl l1 = {A.rule_h[3 * qa], A.rule_l[3 * qa]}, l2 = {A.rule_h[3 * qa + 1], A.rule_l[3 * qa + 1]};
-            const dfl wa = {A.rule_h[3 * qa + 2], A.rule_l[3 * qa + 2]};
-            const dfl m1 = {A.rule_h[3 * qb], A.rule_l[3 * qb]}, m2 = {A.rule_h[3 * qb + 1], A.rule_l[3 * qb + 1]};
-            const dfl wb = {A.rule_h[3 * qb + 2], A.rule_l[3 * qb + 2]};
-            dfl x[3], y[3];
+    dfl g0[2], g1[2], h0[2], h1[2], h2[2];
 #pragma unroll
-            for (int c = 0; c < 3; c++) {
-                x[c] = dadd(dadd(G.O0[c], dmul(l1, G.Ou[c])), dmul(l2, G.Ov[c]));
-                y[c] = dadd(dadd(G.Q0[c], dmul(m1, G.Qu[c])), dmul(m2, G.Qv[c]));
-            }
-            const dfl lx[3] = {dsub(dsub(dfl{1.0f, 0.0f}, l1), l2), l1, l2};
-            const dfl ly[3] = {dsub(dsub(dfl{1.0f, 0.0f}, m1), m2), m1, m2};
-            kernel_eval_df<ATTEN>(x, y, G, kr, ki, dneg(dmul(dmul(wa, wb), G.axay)), lx, ly, A, tab, etab, acc);
+    for (int c = 0; c < 2; c++) g0[c] = g1[c] = h0[c] = h1[c] = h2[c] = dfl{0.0f, 0.0f};
+    for (int q = 0; q < A.ng; q++) {
+        const float2 gq = inner[q][0], w0 = inner[q][1], w1 = inner[q][2], w2 = inner[q][3];
+        const dfl g = {gq.x, gq.y}, c0 = {w0.x, w0.y}, c1 = {w1.x, w1.y}, c2 = {w2.x, w2.y};
+        dfl e[3];
+#pragma unroll
+        for (int c = 0; c < 3; c++) e[c] = dadd(e0[c], dmul(g, dv[c]));
+        dfl Gr, Gi, Fr, Fi;
+        near_gf<ATTEN>(e, kr, ki, A, tab, etab, Gr, Gi, Fr, Fi);
+        dmac(g0[0], Gr, c0, 1.0f);
+        dmac(g0[1], Gi, c0, 1.0f);
+        dmac(g1[0], Gr, c1, 1.0f);
+        dmac(g1[1], Gi, c1, 1.0f);
+        dmac(h0[0], Fr, c0, 1.0f);
+        dmac(h0[1], Fi, c0, 1.0f);
+        dmac(h1[0], Fr, c1, 1.0f);
+        dmac(h1[1], Fi, c1, 1.0f);
+        dmac(h2[0], Fr, c2, 1.0f);
+        dmac(h2[1], Fi, c2, 1.0f);
+    }
+    // (y - x).n_y = -e.n_y and (x - y).n_x = e.n_x: the one of the moving triangle is constant along the line
+    const dfl(&nf)[3] = G.v[ymoves ? 12 : 13];
+    const dfl(&nm)[3] = G.v[ymoves ? 13 : 12];
+    dfl cst = ddot3(e0, nm), lr = ddot3(e0, nf), ls = ddot3(dv, nf);
+    if (ymoves) cst = dneg(cst);
+    else {
+        lr = dneg(lr);
+        ls = dneg(ls);
+    }
+    dfl u[3], p[3], s[3];
+    bary(f1, f2, 1.0f, ymoves ? pa : pb, u);
+    bary(m1, m2, 1.0f, ymoves ? pb : pa, p);
+    bary(d1, d2, 0.0f, ymoves ? pb : pa, s);
+    // sums per moving vertex: V from G; the constant factor's operator and the linear one's from F
+    const int oc = ymoves ? 3 : 6, ol = ymoves ? 6 : 3;  // K, K' rows
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+        g0[c] = two_sum(g0[c].h, g0[c].l);
+        g1[c] = two_sum(g1[c].h, g1[c].l);
+        h0[c] = two_sum(h0[c].h, h0[c].l);
+        h1[c] = two_sum(h1[c].h, h1[c].l);
+        h2[c] = two_sum(h2[c].h, h2[c].l);
+        // F times the linear factor: l0 + l1 g, as moments 0 and 1
+        const dfl l0 = dadd(dmul(lr, h0[c]), dmul(ls, h1[c])), l1 = dadd(dmul(lr, h1[c]), dmul(ls, h2[c]));
+        const dfl k0 = dmul(cst, h0[c]), k1 = dmul(cst, h1[c]);
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            const dfl pw = dmul(p[j], w), sw = dmul(s[j], w);
+            const dfl V = dadd(dmul(pw, g0[c]), dmul(sw, g1[c]));
+            const dfl K = dadd(dmul(pw, k0), dmul(sw, k1)), L = dadd(dmul(pw, l0), dmul(sw, l1));
+            row[2 * j + c] = make_float2(V.h, V.l);
+            row[2 * (oc + j) + c] = make_float2(K.h, K.l);
+            row[2 * (ol + j) + c] = make_float2(L.h, L.l);
         }
+    }
+#pragma unroll
+    for (int i = 0; i < 3; i++) row[2 * NEAR_S + i] = make_float2(u[i].h, u[i].l);
+    row[2 * NEAR_S + 3] = make_float2(ymoves ? 0.0f : 1.0f, 0.0f);
+}
+
+// Minus the regular rule the far-field kernel applied: point qa of the target against the source's points.
+template <bool ATTEN>
+__device__ __forceinline__ void near_regular(const NearArgs& A, const NearGeomDF& G, int qa, dfl kr, dfl ki,
+                                             const float4* __restrict__ tab, const float2* __restrict__ etab,
+                                             float2* __restrict__ row) {
+    const dfl l1 = {A.rule_h[3 * qa], A.rule_l[3 * qa]}, l2 = {A.rule_h[3 * qa + 1], A.rule_l[3 * qa + 1]};
+    const dfl wa = {A.rule_h[3 * qa + 2], A.rule_l[3 * qa + 2]};
+    const dfl w = dneg(dmul(wa, G.axay));
+    dfl x[3];
+#pragma unroll
+    for (int c = 0; c < 3; c++) x[c] = dadd(dadd(G.v[6][c], dmul(l1, G.v[7][c])), dmul(l2, G.v[8][c]));
+    dfl acc[NEAR_S][2];
+#pragma unroll
+    for (int k = 0; k < NEAR_S; k++) acc[k][0] = acc[k][1] = dfl{0.0f, 0.0f};
+    for (int qb = 0; qb < QP; qb++) {
+        const dfl m1 = {A.rule_h[3 * qb], A.rule_l[3 * qb]}, m2 = {A.rule_h[3 * qb + 1], A.rule_l[3 * qb + 1]};
+        const dfl wb = {A.rule_h[3 * qb + 2], A.rule_l[3 * qb + 2]};
+        dfl e[3];
+#pragma unroll
+        for (int c = 0; c < 3; c++)
+            e[c] = dsub(x[c], dadd(dadd(G.v[9][c], dmul(m1, G.v[10][c])), dmul(m2, G.v[11][c])));
+        dfl Gr, Gi, Fr, Fi;
+        near_gf<ATTEN>(e, kr, ki, A, tab, etab, Gr, Gi, Fr, Fi);
+        const dfl wt = dmul(w, wb), dy = dneg(ddot3(e, G.v[13])), dx = ddot3(e, G.v[12]);
+        const dfl ly[3] = {dsub(dsub(dfl{1.0f, 0.0f}, m1), m2), m1, m2};
+        const dfl f[3][2] = {{dmul(Gr, wt), dmul(Gi, wt)},
+                             {dmul(dmul(Fr, wt), dy), dmul(dmul(Fi, wt), dy)},
+                             {dmul(dmul(Fr, wt), dx), dmul(dmul(Fi, wt), dx)}};
+#pragma unroll
+        for (int o = 0; o < 3; o++)
+#pragma unroll
+            for (int j = 0; j < 3; j++)
+#pragma unroll
+                for (int c = 0; c < 2; c++) dmac(acc[3 * o + j][c], f[o][c], ly[j], 1.0f);
+    }
+#pragma unroll
+    for (int k = 0; k < NEAR_S; k++)
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            const dfl v = two_sum(acc[k][c].h, acc[k][c].l);
+            row[2 * k + c] = make_float2(v.h, v.l);
+        }
+    const dfl lx[3] = {dsub(dsub(dfl{1.0f, 0.0f}, l1), l2), l1, l2};
+#pragma unroll
+    for (int i = 0; i < 3; i++) row[2 * NEAR_S + i] = make_float2(lx[i].h, lx[i].l);
+    row[2 * NEAR_S + 3] = make_float2(0.0f, 0.0f);
 }
 
 // grid: (pair, wavenumber slot); one CTA integrates one pair at one k.
-__global__ void __launch_bounds__(NEAR_THREADS) near_build_df_kernel(NearArgs A) {
+__global__ void __launch_bounds__(NEAR_THREADS, 4) near_build_df_kernel(NearArgs A) {
     __shared__ float4 tab[128];
     __shared__ float2 etab[64];
+    __shared__ float2 inner[NEAR_NG_MAX][4];  // innermost rule: g, w, w g, w g^2
     __shared__ NearGeomDF G;
+    __shared__ float2 rows[NEAR_THREADS][NEAR_ROW];
+    __shared__ double red[NEAR_THREADS / 32][NACC][2];
     const int64_t pi = blockIdx.x;
-    const int sl = blockIdx.y;
+    const int sl = blockIdx.y, tid = threadIdx.x;
     const int tgt = A.pair_tgt[pi], src = A.pair_src[pi];
     const int code = A.pair_code[pi];
     const int rel = code & 15;
+    double* out = reinterpret_cast<double*>(A.raw + ((int64_t)pi * A.n_slot_k + sl) * NACC);
+    const int dom = A.slot_dom[4 * tgt + 3];
+    // the own-domain wavenumber applies only to pairs within the target's domain
+    if (sl != 0 && A.slot_dom[4 * src + 3] != dom) {
+        if (tid < NACC * 2) out[tid] = 0.0;
+        return;
+    }
     int pa[3], pb[3];
+#pragma unroll
     for (int i = 0; i < 3; i++) {
         pa[i] = (code >> (4 + 2 * i)) & 3;
         pb[i] = (code >> (10 + 2 * i)) & 3;
     }
-    const int dom = A.slot_dom[4 * tgt + 3];
     const float4 kk = sl == 0 ? A.k0df : A.kdf[dom];
     const dfl kr = {kk.x, kk.y}, ki = {kk.z, kk.w};
-    const bool live = sl == 0 || A.slot_dom[4 * src + 3] == dom;
-    for (int i = threadIdx.x; i < 128; i += NEAR_THREADS) tab[i] = A.sctab[i];
-    for (int i = threadIdx.x; i < 64; i += NEAR_THREADS) etab[i] = A.extab[i];
-    if (threadIdx.x == 0) {
-        // the pair's geometry in FP64, differences formed before the split
-        const double* P = A.slot_P;
-        for (int c = 0; c < 3; c++) {
-            const double px[3] = {P[(int64_t)tgt * 9 + 3 * pa[0] + c], P[(int64_t)tgt * 9 + 3 * pa[1] + c],
-                                  P[(int64_t)tgt * 9 + 3 * pa[2] + c]};
-            const double py[3] = {P[(int64_t)src * 9 + 3 * pb[0] + c], P[(int64_t)src * 9 + 3 * pb[1] + c],
-                                  P[(int64_t)src * 9 + 3 * pb[2] + c]};
-            const double ox[3] = {P[(int64_t)tgt * 9 + c], P[(int64_t)tgt * 9 + 3 + c], P[(int64_t)tgt * 9 + 6 + c]};
-            const double oy[3] = {P[(int64_t)src * 9 + c], P[(int64_t)src * 9 + 3 + c], P[(int64_t)src * 9 + 6 + c]};
-            G.X0[c] = split_d(px[0]);
-            G.X1[c] = split_d(px[1] - px[0]);
-            G.X2[c] = split_d(px[2] - px[1]);
-            G.Y0[c] = split_d(py[0]);
-            G.Y1[c] = split_d(py[1] - py[0]);
-            G.Y2[c] = split_d(py[2] - py[1]);
-            G.O0[c] = split_d(ox[0]);
-            G.Ou[c] = split_d(ox[1] - ox[0]);
-            G.Ov[c] = split_d(ox[2] - ox[0]);
-            G.Q0[c] = split_d(oy[0]);
-            G.Qu[c] = split_d(oy[1] - oy[0]);
-            G.Qv[c] = split_d(oy[2] - oy[0]);
-            G.nx[c] = split_d(A.slot_n[(int64_t)tgt * 3 + c]);
-            G.ny[c] = split_d(A.slot_n[(int64_t)src * 3 + c]);
+    for (int i = tid; i < 128; i += NEAR_THREADS) tab[i] = A.sctab[i];
+    for (int i = tid; i < 64; i += NEAR_THREADS) etab[i] = A.extab[i];
+    for (int i = tid; i < 4 * A.ng; i += NEAR_THREADS) (&inner[0][0])[i] = A.inner[i];
+    if (tid < 42) {
+        // the pair's geometry, one component per thread; FP64 differences formed before the split
+        const int v = tid / 3, c = tid - 3 * v;
+        double val;
+        if (v < 12) {
+            const bool y = (v / 3) & 1, orig = v >= 6;
+            const double* P = A.slot_P + (int64_t)(y ? src : tgt) * 9 + c;
+            const int m = v % 3;
+            // reordered: (P0, P1 - P0, P2 - P1) of the rule's vertex order; original: (P0, P1 - P0, P2 - P0)
+            const int sh = y ? 10 : 4, at = orig ? m : (code >> (sh + 2 * m)) & 3;
+            const int from = orig ? 0 : (code >> (sh + 2 * (m - 1))) & 3;
+            val = P[3 * at];
+            if (m > 0) val -= P[3 * from];
+        } else {
+            val = A.slot_n[(int64_t)(v == 12 ? tgt : src) * 3 + c];
         }
-        const double ax = A.slot_area[tgt], ay = A.slot_area[src];
-        G.scale = split_d(4.0 * ax * ay);
-        G.axay = split_d(ax * ay);
+        G.v[v][c] = split_d(val);
+    } else if (tid == 42) {
+        G.scale = split_d(4.0 * A.slot_area[tgt] * A.slot_area[src] * 0.07957747154594767);
+    } else if (tid == 43) {
+        G.axay = split_d(A.slot_area[tgt] * A.slot_area[src] * 0.07957747154594767);
     }
     __syncthreads();
-    dfl acc[NACC][2];
-#pragma unroll
-    for (int i = 0; i < NACC; i++) acc[i][0] = acc[i][1] = dfl{0.0f, 0.0f};
-    if (kk.z != 0.0f || kk.w != 0.0f) near_df_body<true>(A, G, rel, pa, pb, kr, ki, live, tab, etab, acc);
-    else near_df_body<false>(A, G, rel, pa, pb, kr, ki, live, tab, etab, acc);
-    // block reduction in FP64: it runs on the FP64 pipe beside the FP32 point
-    // evaluations of the other warps (a double-float shuffle reduction was
-    // measured slower: 394 against 307 ms on the 8k-triangle rib scene, the
-    // FP32 pipe being the busier one at eight warps per SM)
-    __shared__ double red[NEAR_THREADS / 32][NACC][2];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < NACC; i++)
-#pragma unroll
-        for (int c = 0; c < 2; c++) {
-            double v = (double)acc[i][c].h + (double)acc[i][c].l;
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (lane == 0) red[warp][i][c] = v;
+    const bool atten = kk.z != 0.0f || kk.w != 0.0f;
+    const int n = A.grp_n[rel];
+    // the regular groups take the last warp of the last batch where that is free, else a batch of their own
+    const int base = (n - 1) / NEAR_THREADS * NEAR_THREADS;
+    const int reg0 = rel == 3 ? n : base + (n - base <= NEAR_THREADS - 32 ? NEAR_THREADS - 32 : NEAR_THREADS);
+    const int n_all = rel == 3 ? n : reg0 + QP;  // (not for identical pairs)
+    // lane (operator, i, j) sums its moment over its warp's groups
+    const int lane = tid & 31, warp = tid >> 5;
+    const int op = lane / 9, ij = lane - 9 * op, mi = ij / 3, mj = ij - 3 * mi;
+    dfl sr = {0.0f, 0.0f}, si = {0.0f, 0.0f};
+    for (int b = 0; b < n_all; b += NEAR_THREADS) {
+        const int idx = b + tid;
+        float2* row = rows[tid];
+        if (idx < n) {
+            if (atten) near_group<true>(A, G, rel, idx, pa, pb, kr, ki, tab, etab, inner, row);
+            else near_group<false>(A, G, rel, idx, pa, pb, kr, ki, tab, etab, inner, row);
+        } else if (idx >= reg0 && idx < n_all) {
+            if (atten) near_regular<true>(A, G, idx - reg0, kr, ki, tab, etab, row);
+            else near_regular<false>(A, G, idx - reg0, kr, ki, tab, etab, row);
         }
+        __syncwarp();
+        if (lane < NACC) {
+            for (int g = 0; g < 32; g++) {
+                const int i = b + warp * 32 + g;
+                if (!(i < n || (i >= reg0 && i < n_all))) continue;
+                const float2* r = rows[warp * 32 + g];
+                const bool xmoves = r[2 * NEAR_S + 3].x != 0.0f;
+                const float2 u = r[2 * NEAR_S + (xmoves ? mj : mi)];
+                const float2 *v = r + 2 * (3 * op + (xmoves ? mi : mj)), vr = v[0], vi = v[1];
+                dmac(sr, dfl{vr.x, vr.y}, dfl{u.x, u.y}, 1.0f);
+                dmac(si, dfl{vi.x, vi.y}, dfl{u.x, u.y}, 1.0f);
+            }
+            sr = two_sum(sr.h, sr.l);
+            si = two_sum(si.h, si.l);
+        }
+        __syncwarp();
+    }
+    if (lane < NACC) {
+        red[warp][lane][0] = (double)sr.h + (double)sr.l;
+        red[warp][lane][1] = (double)si.h + (double)si.l;
+    }
     __syncthreads();
-    if (threadIdx.x < NACC * 2) {
-        const int i = threadIdx.x >> 1, c = threadIdx.x & 1;
+    if (tid < NACC * 2) {
+        const int i = tid >> 1, c = tid & 1;
         double v = 0;
         for (int w = 0; w < NEAR_THREADS / 32; w++) v += red[w][i][c];
-        double* out = reinterpret_cast<double*>(A.raw + ((int64_t)pi * A.n_slot_k + sl) * NACC);
         out[2 * i + c] = v;
     }
 }

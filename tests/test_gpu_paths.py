@@ -58,3 +58,19 @@ def test_gemm_split_over_ctas(m, k, n):
     err = (y.cpu().to(torch.complex128) - ref).norm() / ref.norm()
     c.close()
     assert err < 2e-6
+
+
+@pytest.mark.parametrize("n_gauss", [2, 5, 6, 9])
+@pytest.mark.parametrize("name", ["shell", "two"])
+def test_near_groups_match_native_fp64(api, name, n_gauss):
+    """The double-float near build (rules as groups of points along a line)
+    against the native FP64 one over points, for Gauss orders with other group
+    counts than the default; double-float evaluations carry ~1e-13."""
+    s = scenes.shell_scene(1) if name == "shell" else scenes.two_sphere_scene(1)
+    x = scenes.smooth_trace_vector(s, 5)
+    y = []
+    for native in (0, 1):
+        c = api.Context.from_scene(s, n_gauss_singular=n_gauss, fp64_far=native)
+        y.append(c.apply(x, precision=api.FP64))
+        c.close()
+    assert rel(y[0], y[1]) < 1e-12
