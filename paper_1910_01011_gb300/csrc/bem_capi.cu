@@ -123,6 +123,9 @@ static void release_device(bem_ctx* ctx) {
     ctx->asm_ready = false;
     ctx->asm64_ready = false;
     ctx->asm64 = nullptr;
+    ctx->asm64_exp = nullptr;
+    ctx->dg_work = nullptr;
+    ctx->dg_work_bytes = 0;
     ctx->df_exp = nullptr;
     ctx->df_work = nullptr;
     ctx->df_work_bytes = 0;
@@ -251,12 +254,11 @@ int64_t estimate_solve_bytes(const bem_ctx* ctx, int64_t n_exc, const bem_solve_
         b += 32 * (pts + slots + tiles) + 4096 + R * (pts * 32 + 2 * slots * 32 + 16);
     // recycled solution space: Q, U' and their coefficients
     if (o.recycle > 0) b += (int64_t)o.recycle * (2 * N * 16 + 64 * 16);
-    // split vectors of the FP64-accurate residual product
-    b += R * N * 16 + 4096;
     if (o.operator_mode == 1) {
         const int64_t mp = (N + 127) / 128 * 128, kp = (N + 31) / 32 * 32;
         const int64_t planes = 6 * mp * kp * 2;
-        const int64_t a64 = 16 * N * N;
+        const int64_t a64 = (int64_t)(digits_bytes(N) + digits_convert_bytes(N)) + 4 * (digits_mpad(N) + digits_kpad(N)) +
+                            (int64_t)digits_work_bytes(N, std::min<int64_t>(R, 16));
         if (o.precision == BEM_PREC_FP32)
             b += std::max(planes + 8 * N * N, planes + a64) + (int64_t)gemm_work_bytes(mp, kp, R);
         else

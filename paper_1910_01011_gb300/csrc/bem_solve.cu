@@ -1021,14 +1021,14 @@ int bem_solve_basis(bem_ctx* ctx, const bem_solve_opts* opts, bem_solve_report* 
             }
         }
         if (!rc && !ctx->df_exp) {
-            ctx->df_exp = (int*)ctx->dalloc(2 * sizeof(int), &rc);
+            ctx->df_exp = (int*)ctx->dalloc(sizeof(int), &rc);
             if (rc) ctx->df_exp = nullptr;
         }
         if (!rc) {
             // kept in the split form of k_df64.cu for bem_superpose
             CK(cudaMemcpyAsync(S->basis, S->u, (size_t)ne * N * sizeof(double2), cudaMemcpyDeviceToDevice,
                                ctx->stream));
-            rc = df_prepare_inplace(ctx, S->basis, ne * N, ctx->df_exp + 1);
+            rc = df_prepare_inplace(ctx, S->basis, ne * N, ctx->df_exp);
             if (!rc) CK(cudaStreamSynchronize(ctx->stream));
             if (!rc) {
                 S->n_basis = ne;
@@ -1070,7 +1070,7 @@ int bem_superpose(bem_ctx* ctx, const bem_z* w, int64_t n_exc, bem_z* u, int on_
         ud = S->wstage + n_exc * ne;
     }
     // U = W B with the basis in the split form of k_df64.cu (FP64 accuracy)
-    if ((rc = df_combine(ctx, (const float4*)S->basis, ctx->df_exp + 1, ne, N, wd, n_exc, ud))) return rc;
+    if ((rc = df_combine(ctx, (const float4*)S->basis, ctx->df_exp, ne, N, wd, n_exc, ud))) return rc;
     if (!on_device) {
         CK(cudaMemcpyAsync(u, ud, (size_t)n_exc * N * sizeof(double2), cudaMemcpyDeviceToHost, ctx->stream));
         CK(cudaStreamSynchronize(ctx->stream));

@@ -152,10 +152,13 @@ struct bem_ctx {
     void* asm_work = nullptr;
     size_t asm_work_bytes = 0;
     // assembled operator for FP64 refinement residuals: complex128 entries stored as
-    // scaled FP32 (hi, lo) pairs, 16 bytes each (k_df64.cu)
+    // fixed-point digits, 16 bytes each (k_digits.cu)
     bool asm64_ready = false;
     double2* asm64 = nullptr;
-    int* df_exp = nullptr;          // device [2]: exponents of asm64 and of the superposition basis
+    int* asm64_exp = nullptr;       // device: column and row exponents of asm64
+    void* dg_work = nullptr;        // scratch of its products (grow-only)
+    size_t dg_work_bytes = 0;
+    int* df_exp = nullptr;          // device: exponent of the superposition basis
     void* df_work = nullptr;        // split vectors of the FP64-accurate products (grow-only)
     size_t df_work_bytes = 0;
     gbem::OsrcState* osrc = nullptr;
@@ -216,10 +219,15 @@ int64_t solve_batch_width(const bem_solve_opts& o, int64_t n_exc);
 inline int resolved_operator_mode(int mode, int64_t n_dof) {
     return mode != 2 ? mode : (36.0 * (double)n_dof * (double)n_dof <= 4.0 * 1073741824.0 ? 1 : 0);
 }
-// FP64-accurate complex products in FP32 arithmetic (k_df64.cu).
+// FP64-accurate complex products on the tensor cores (k_digits.cu) and in FP32 arithmetic (k_df64.cu).
+int64_t digits_kpad(int64_t n);
+int64_t digits_mpad(int64_t n);
+size_t digits_bytes(int64_t n);
+size_t digits_work_bytes(int64_t n, int64_t R);
+size_t digits_convert_bytes(int64_t n);
+int digits_prepare(bem_ctx* ctx, double2* A, int64_t n, int* exps);
+int digits_gemm(bem_ctx* ctx, const void* A, const int* exps, int64_t n, const double2* X, int64_t R, double2* Y, void* work);
 int df_prepare_inplace(bem_ctx* ctx, double2* v, int64_t n, int* e);
-int df_gemv(bem_ctx* ctx, const float4* A, const int* eA, int64_t m, int64_t k, int64_t lda, const double2* X,
-            int64_t R, double2* Y, int64_t ldy);
 int df_combine(bem_ctx* ctx, const float4* B, const int* eB, int64_t K, int64_t n, const double2* W, int64_t R,
                double2* U);
 }  // namespace gbem

@@ -15,6 +15,7 @@
 // between runs at the level of FP32 rounding).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "ctx.h"
@@ -543,9 +544,9 @@ int bem_ctx::ensure_assembled() {
 
 // A_hat assembled in complex128 (FP64 arithmetic), kept for the FP64
 // residual of the refinement: one pass of FP64 interactions at set-up, then
-// the matrix is stored as scaled FP32 (hi, lo) pairs in the same 16 bytes per
-// entry, and every residual is a product to FP64 accuracy in FP32 arithmetic
-// that streams it at the HBM rate (k_df64.cu).
+// the matrix is stored as fixed-point digits in the same 16 bytes per entry,
+// and every residual is a product on the tensor cores to FP64 accuracy that
+// streams it at the HBM rate (k_digits.cu).
 int bem_ctx::ensure_assembled64() {
     bem_ctx* const ctx = this;
     if (asm64_ready) return BEM_OK;
@@ -553,14 +554,20 @@ int bem_ctx::ensure_assembled64() {
     if (rc) return rc;
     const Geometry& g = geo;
     const int64_t n = g.n_dof;
-    if (asm64) { dfree(asm64); asm64 = nullptr; }
-    asm64 = (double2*)dalloc((size_t)n * n * sizeof(double2), &rc);
-    if (rc) { asm64 = nullptr; return rc; }
-    CK(cudaMemsetAsync(asm64, 0, (size_t)n * n * sizeof(double2), stream));
+    const int64_t ld = digits_kpad(n);
+    if (!asm64) {
+        asm64 = (double2*)dalloc(digits_bytes(n), &rc);
+        if (rc) { asm64 = nullptr; return rc; }
+    }
+    if (!asm64_exp) {
+        asm64_exp = (int*)dalloc((size_t)(ld + digits_mpad(n)) * sizeof(int), &rc);
+        if (rc) { asm64_exp = nullptr; return rc; }
+    }
+    CK(cudaMemsetAsync(asm64, 0, digits_bytes(n), stream));
     AssembleArgs a{};
     a.tc = dev.tc; a.tntri = dev.tntri; a.slot_v = dev.slot_v; a.slot_curl = dev.slot_curl;
     a.v_dof1 = dev.v_dof1; a.v_dof2 = dev.v_dof2; a.coef = dev.coef; a.dom_tiles = dev.dom_tiles; a.kdom = dev.kdom;
-    a.k0 = make_double2(k0re, k0im); a.n_tiles = g.n_tiles; a.chunk_tiles = 8; a.n = n;
+    a.k0 = make_double2(k0re, k0im); a.n_tiles = g.n_tiles; a.chunk_tiles = 8; a.n = ld;
     for (int q = 0; q < QP; q++)
         for (int k = 0; k < 3; k++) a.lam64[q][k] = quad.lam[q][k];
     const dim3 grid(g.n_tiles, (g.n_tiles + a.chunk_tiles - 1) / a.chunk_tiles);
@@ -591,28 +598,30 @@ int bem_ctx::ensure_assembled64() {
     if (np > 0) {
         add_near64_kernel<<<(unsigned)((np + 127) / 128), 128, 0, stream>>>(np, dev.np_tgt, dev.np_src, dev.slot_v,
                                                                            dev.v_dof1, dev.v_dof2, pmchwt_near.nb64,
-                                                                           n, asm64);
+                                                                           ld, asm64);
         CK(cudaGetLastError());
     }
-    CK(cudaGetLastError());
-    if (!df_exp) {
-        df_exp = (int*)dalloc(2 * sizeof(int), &rc);
-        if (rc) { df_exp = nullptr; return rc; }
-    }
-    if ((rc = df_prepare_inplace(this, asm64, n * n, df_exp))) return rc;
-    CK(cudaStreamSynchronize(stream));
+    if ((rc = digits_prepare(this, asm64, n, asm64_exp))) return rc;
     launches += 3;
     asm64_ready = true;
     return BEM_OK;
 }
 
 // Y = A_hat X (FP64 accuracy, assembled) for n_rhs system-order vectors;
-// A_hat is row-major in the split form of k_df64.cu.
+// A_hat as the digits of k_digits.cu.
 int bem_ctx::apply_assembled64(const double2* x, double2* y, int64_t n_rhs) {
     int rc = ensure_assembled64();
     if (rc) return rc;
     const int64_t n = geo.n_dof;
-    return df_gemv(this, (const float4*)asm64, df_exp, n, n, n, x, n_rhs, y, n);
+    const size_t need = digits_work_bytes(n, std::min<int64_t>(n_rhs, 16));
+    if (need > dg_work_bytes) {
+        dfree(dg_work);
+        dg_work_bytes = 0;
+        dg_work = dalloc(need, &rc);
+        if (rc) { dg_work = nullptr; return rc; }
+        dg_work_bytes = need;
+    }
+    return digits_gemm(this, asm64, asm64_exp, n, x, n_rhs, y, dg_work);
 }
 
 // Y = A_hat X for n_rhs system-order vectors (complex128, device), through

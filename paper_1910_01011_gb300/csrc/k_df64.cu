@@ -1,11 +1,9 @@
 // k_df64.cu -- complex products to FP64 accuracy in FP32 arithmetic.
 //
-// The FP64 residual of the refinement (r = b - A_hat u with the complex128
-// A_hat) and the excitation superposition (u = w x basis) are matrix products
-// whose operand is read once.  GB300 executes FP64 at about 1/64 of its FP32
-// rate, so the same products in FP64 arithmetic are bound by that rate (8 N^2
-// FP64 flops per vector: ~11 ms on a 41k-unknown A_hat) rather than by
-// reading the 16 N^2 bytes (~4 ms).  Here every matrix entry is stored as a
+// The excitation superposition (u = w x basis) is a matrix product whose
+// operand is read once.  GB300 executes FP64 at about 1/64 of its FP32 rate, so
+// the same product in FP64 arithmetic is bound by that rate rather than by
+// reading the basis.  Here every matrix entry is stored as a
 // pair of FP32 numbers in the same 16 bytes, and the products and sums are
 // carried out with error-free FP32 transformations:
 //
@@ -20,8 +18,7 @@
 //    ordinary FMAs; lo_a lo_x (~2^-48) is dropped.
 //  * sums: the high parts are accumulated with Knuth's TwoSum, whose
 //    rounding error is exact and goes into the low accumulator; every 256
-//    terms a lane folds its (high, low) pair into FP64, and at the end the
-//    32 lanes of a warp are summed in FP64.
+//    terms a thread folds its (high, low) pair into FP64.
 //
 // Real and imaginary parts of an output are the two lanes of one packed
 // FP32 value (FFMA2 / FADD2 / FMUL2), so y += a x for complex a, x is
@@ -39,8 +36,7 @@
 
 namespace gbem {
 
-constexpr int DF_WARPS = 8;    // warps per CTA
-constexpr int DF_FOLD = 256;   // terms a lane accumulates in FP32 between FP64 folds
+constexpr int DF_FOLD = 256;   // terms a thread accumulates in FP32 between FP64 folds
 
 // ----------------------------------------------------------------- splitting
 
@@ -144,90 +140,6 @@ __device__ __forceinline__ void df_fold(DfAcc& c, double2& acc) {
     acc.y += (double)c.S.y + (double)c.L.y;
     c.S = make_float2(0.f, 0.f);
     c.L = make_float2(0.f, 0.f);
-}
-
-__device__ __forceinline__ double2 warp_sum(double2 v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-        v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
-    }
-    return v;
-}
-
-// ----------------------------------------------------------------- Y = X A^T (rows of A reduced)
-
-struct DfGemvArgs {
-    const float4* A;      // [m][lda] split entries, scaled by 2^-eA
-    int64_t m, k, lda;
-    const int* eA;        // device scalar
-    const float4* X;      // [R][k] split vectors
-    const int* eX;        // [R]
-    int64_t R;
-    double2* Y;           // [R][ldy]
-    int64_t ldy;
-};
-
-// One warp per RW rows of A; lanes stride over the k columns (coalesced
-// 16-byte loads); right-hand sides in groups of RG, each group one pass over
-// the warp's rows.
-template <int RW, int RG>
-__global__ void __launch_bounds__(DF_WARPS * 32) df_gemv_kernel(DfGemvArgs a) {
-    const int lane = threadIdx.x & 31;
-    const int64_t n_groups = (a.m + RW - 1) / RW;
-    const int eA = *a.eA;
-    for (int64_t g = (int64_t)blockIdx.x * DF_WARPS + (threadIdx.x >> 5); g < n_groups;
-         g += (int64_t)gridDim.x * DF_WARPS) {
-        const int64_t i0 = g * RW;
-        const float4* Arow[RW];
-#pragma unroll
-        for (int w = 0; w < RW; w++) Arow[w] = a.A + min(i0 + w, a.m - 1) * a.lda;
-        for (int64_t r0 = 0; r0 < a.R; r0 += RG) {
-            const float4* Xr[RG];
-#pragma unroll
-            for (int q = 0; q < RG; q++) Xr[q] = a.X + min(r0 + q, a.R - 1) * a.k;
-            DfAcc c[RW][RG];
-            double2 acc[RW][RG];
-#pragma unroll
-            for (int w = 0; w < RW; w++)
-#pragma unroll
-                for (int q = 0; q < RG; q++) {
-                    c[w][q].S = c[w][q].L = make_float2(0.f, 0.f);
-                    acc[w][q] = make_double2(0.0, 0.0);
-                }
-            for (int64_t jb = 0; jb < a.k; jb += 32 * DF_FOLD) {
-                const int64_t je = min(a.k, jb + 32 * DF_FOLD);
-#pragma unroll 2
-                for (int64_t j = jb + lane; j < je; j += 32) {
-                    float4 xv[RG];
-#pragma unroll
-                    for (int q = 0; q < RG; q++) xv[q] = __ldg(Xr[q] + j);
-#pragma unroll
-                    for (int w = 0; w < RW; w++) {
-                        const float4 av = __ldcs(Arow[w] + j);  // streamed: each entry is read once per pass
-                        const f2 A = make_float2(av.x, av.y), AS = make_float2(-av.y, av.x);
-                        const f2 AL = make_float2(av.z, av.w), ALS = make_float2(-av.w, av.z);
-#pragma unroll
-                        for (int q = 0; q < RG; q++) df_mac(c[w][q], A, AS, AL, ALS, xv[q]);
-                    }
-                }
-#pragma unroll
-                for (int w = 0; w < RW; w++)
-#pragma unroll
-                    for (int q = 0; q < RG; q++) df_fold(c[w][q], acc[w][q]);
-            }
-#pragma unroll
-            for (int w = 0; w < RW; w++)
-#pragma unroll
-                for (int q = 0; q < RG; q++) {
-                    const double2 s = warp_sum(acc[w][q]);
-                    if (lane == 0 && i0 + w < a.m && r0 + q < a.R) {
-                        const int e = eA + a.eX[r0 + q];
-                        a.Y[(r0 + q) * a.ldy + i0 + w] = make_double2(ldexp(s.x, e), ldexp(s.y, e));
-                    }
-                }
-        }
-    }
 }
 
 // ----------------------------------------------------------------- U = W B (rows of B combined)
@@ -342,26 +254,6 @@ int df_prepare_inplace(bem_ctx* ctx, double2* v, int64_t n, int* e) {
     ctx->launches += 2;
     err = cudaGetLastError();
     return err == cudaSuccess ? BEM_OK : ctx->fail(BEM_ERR_CUDA, std::string("df prepare: ") + cudaGetErrorString(err));
-}
-
-// Y[r][i] = sum_j A[i][j] X[r][j] for r < R, A split (m x k, row stride lda).
-int df_gemv(bem_ctx* ctx, const float4* A, const int* eA, int64_t m, int64_t k, int64_t lda, const double2* X,
-            int64_t R, double2* Y, int64_t ldy) {
-    DfScratch s;
-    int rc = split_vectors(ctx, X, R, k, &s);
-    if (rc) return rc;
-    DfGemvArgs a{A, m, k, lda, eA, s.xs, s.e, R, Y, ldy};
-    const int threads = DF_WARPS * 32;
-    auto grid = [&](int rw) {
-        const int64_t groups = (m + rw - 1) / rw;
-        return (unsigned)std::max<int64_t>(1, std::min<int64_t>((groups + DF_WARPS - 1) / DF_WARPS, 152 * 4));
-    };
-    if (R == 1) df_gemv_kernel<4, 1><<<grid(4), threads, 0, ctx->stream>>>(a);
-    else if (R == 2) df_gemv_kernel<2, 2><<<grid(2), threads, 0, ctx->stream>>>(a);
-    else df_gemv_kernel<2, 4><<<grid(2), threads, 0, ctx->stream>>>(a);  // (one row x 8 vectors per warp measured slower)
-    ctx->launches += 1;
-    cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? BEM_OK : ctx->fail(BEM_ERR_CUDA, std::string("df gemv: ") + cudaGetErrorString(e));
 }
 
 // U[r][j] = sum_m W[r][m] B[m][j], B split (K x n), W complex128 [R][K].

@@ -1,0 +1,634 @@
+// k_digits.cu -- complex128 matrix x block of vectors on the tensor cores,
+// exactly to ~2^-53 of the largest terms (the FP64 residual of the refinement,
+// r = b - A_hat u with the assembled complex128 A_hat).
+//
+// GB300 runs FP64 at 1/64 of its FP32 rate, and carrying the products in FP32
+// pairs takes ~25 packed FP32 instructions per entry and vector.  Here both
+// operands are fixed-point numbers cut into digits, and the digits' products
+// and sums are exact (the error-free splitting of Ozaki, Ogita, Oishi and
+// Rump, "Error-free transformations of matrix multiplication by using fast
+// routines of matrix multiplication and its applications", 2012):
+//
+//  * A' = 2^-row A 2^-col with powers of two per row and column (columns first,
+//    so that the psi and phi blocks, a factor |k| apart, share their bits), each
+//    real part below 1/4 as Q 2^-56, |Q| < 2^54, and
+//    Q = sum_i d_i 128^(7 - i) with eight digits d_i in [-64, 63].  A digit is a
+//    byte (d + 64): 16 bytes per complex entry, as complex128 itself.
+//  * vectors likewise, x_j 2^col_j with one power of two per vector, as BF16
+//    digits (integers up to 256 are exact in BF16).
+//  * Y' = sum_{i + j <= 7} 2^(-7 (i + j + 2)) A_i X_j on tcgen05 (kind::f16,
+//    BF16 in, FP32 out): the products are integers of at most 2^12, a sum of
+//    K = 256 of both real parts and up to eight (i, j) stays below 2^24, so
+//    every FP32 accumulator holds its integer exactly whatever the order or
+//    rounding mode of the unit.  The dropped terms are below 2^-53 of
+//    |A'| |x'|.
+//  * every 256 of K the eight accumulators of an output are added, smallest
+//    weight first, into a pair of FP32 numbers by TwoSum; pieces of K in FP64.
+//
+// The 36 digit products of a step need no 36 instructions: X's digits lie side
+// by side as rows of B, X_0 first, and A_i times the first 8 - i of them, into
+// accumulators starting at the i-th, adds every product to the accumulator of
+// its weight.  Real and imaginary parts of A are two A operands with
+// B = [Xr | Xi] and [-Xi | Xr] on the same accumulators.
+//
+// What binds it is reading A once (16 N^2 bytes): A's bytes are stored in the
+// order in which a CTA reads them (blocks of 128 rows x 32 of K x 16 digit
+// planes, 64 KB, one bulk copy each), four warps turn them into BF16 pairs
+// (a byte permute and one subtraction per two digits) and put them into
+// tensor memory as the A operand, so shared memory holds them only once, as
+// bytes.  Every CTA takes an equal run of 256-wide units across row tiles (as
+// in k_gemm.cu), and pieces of a tile are added in FP64.
+//
+// N = 10,776, 16 vectors: 404 us (4.6 TB/s of A; the instructions of a step take
+// 1,306 cycles, its bytes 1,490 at the copy rate) against 4,423 us in FP32
+// pairs.  Relative error of products on scenes of 2,000-5,000 unknowns below
+// 1e-13, that of the assembled entries.
+#include <cuda_bf16.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <climits>
+#include <cstdint>
+#include <string>
+#include <vector>
+
+#include "ctx.h"
+#include "df_math.cuh"
+#include "internal.h"
+
+namespace gbem {
+
+constexpr int DG = 8;                      // digits of a real number
+constexpr int DG_M = 128;                  // rows of A per tile
+constexpr int DG_K = 32;                   // K per stage (bytes per digit row)
+constexpr int DG_STEPS = 8;                // stages per unit: K = 256
+constexpr int DG_CTAS = 152;
+constexpr int DG_PLANE = DG_M * DG_K;      // bytes of one digit plane of a stage
+constexpr int DG_ABYTES = 2 * DG * DG_PLANE;
+constexpr int DG_STAGES = 2;
+constexpr int DG_WARPS = 10;               // 0 copies, 1 MMA, 2-5 digits to BF16, 6-9 accumulators
+constexpr int DG_NONE = INT_MIN / 4;       // exponent of a zero row, column or vector
+constexpr int DG_BAD = INT_MAX / 4;        // of one with an infinity or a NaN
+
+// NC columns of B per digit: NC / 2 right-hand sides, real and imaginary parts
+template <int NC>
+struct DgCfg {
+    static constexpr int HN = NC / 2;
+    static constexpr int BROWS = DG * NC;              // B rows: digit j, column n at j NC + n
+    static constexpr int BBYTES = 2 * BROWS * DG_K * 2;  // [Xr | Xi] and [-Xi | Xr] of a stage
+    struct Smem {
+        alignas(1024) uint8_t a[DG_STAGES][DG_ABYTES];
+        alignas(1024) uint8_t b[DG_STAGES][BBYTES];
+        uint64_t full[DG_STAGES], empty[DG_STAGES];    // copies landed; bytes converted (4 warps) and B used (MMA)
+        uint64_t tfull[2], tempty[2];                  // A operand of one K = 16 step in tensor memory
+        uint64_t dfull, dempty;                        // accumulators of a unit
+        uint32_t tmem;
+    };
+    static_assert(sizeof(Smem) + 1024 <= 227 * 1024, "digits smem");
+};
+
+// ----------------------------------------------------------------- digits
+
+// e with |v| < 2^e of a double, from its bits; DG_NONE for zero (and subnormals), DG_BAD for infinities and NaN
+__device__ __forceinline__ int dg_exp(double v) {
+    const int b = (__double2hiint(v) >> 20) & 0x7ff;
+    return b == 0 ? DG_NONE : b == 0x7ff ? DG_BAD : b - 1022;
+}
+__device__ __forceinline__ int dg_exp2(double2 v) { return max(dg_exp(v.x), dg_exp(v.y)); }
+
+// Q + bias of v 2^(56 - e), |v| < 2^(e - 2), rounded to nearest, in integers
+// (no FP64): its base-128 digits are d + 64, the bias 64 sum_t 128^t.
+__device__ __forceinline__ unsigned long long dg_biased(double v, int e) {
+    constexpr unsigned long long bias = 0x0081020408102040ull;
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
+    const int be = (int)(bits >> 52) & 0x7ff;
+    if (be == 0) return bias;  // zero (and subnormals)
+    const unsigned long long m = (bits & 0xfffffffffffffull) | 0x10000000000000ull;  // v = m 2^(be - 1075)
+    const int sh = be - 1075 + 56 - e;
+    const unsigned long long q = sh >= 0 ? m << sh : sh < -54 ? 0 : (m + (1ull << (-sh - 1))) >> -sh;
+    return (bits >> 63) ? bias - q : bias + q;
+}
+
+// col[j] = largest exponent of column j of A (n rows, leading dimension ld); CTA: 128 columns, a range of rows
+__global__ void dg_colexp_kernel(const double2* __restrict__ A, int64_t n, int64_t ld, int64_t rows_per, int* col) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    const int64_t r1 = min(n, ((int64_t)blockIdx.y + 1) * rows_per);
+    int e = DG_NONE;
+#pragma unroll 4
+    for (int64_t i = (int64_t)blockIdx.y * rows_per; i < r1; i++) e = max(e, dg_exp2(A[i * ld + j]));
+    atomicMax(&col[j], e);
+}
+
+__device__ __forceinline__ int block_max(int e, int* sh) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = e;
+    __syncthreads();
+    e = sh[0];
+    for (int w = 1; w < (int)blockDim.x / 32; w++) e = max(e, sh[w]);
+    return e;
+}
+
+// One row per CTA: its exponent, then its digits into the row tile's blocks (out: the first tile of the launch).
+__global__ void __launch_bounds__(256) dg_digits_kernel(const double2* __restrict__ A, int64_t n, int64_t ld, int64_t row0,
+                                                        int64_t nkb, const int* __restrict__ col, int* __restrict__ rowe,
+                                                        uint8_t* __restrict__ out) {
+    __shared__ int sh[8];
+    const int64_t i = row0 + blockIdx.x;
+    const int r = blockIdx.x % DG_M;
+    const double2* a = A + i * ld;
+    int e = DG_NONE;
+    if (i < n)
+        for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
+            const int v = dg_exp2(a[j]), c = col[j];
+            if (v != DG_NONE) e = max(e, v == DG_BAD || c == DG_BAD ? DG_BAD : v - c);
+        }
+    e = block_max(e, sh);
+    if (threadIdx.x == 0) rowe[i] = e;
+    // a thread takes four neighbouring entries: 4-byte stores per digit plane
+    uint8_t* tile = out + (int64_t)(blockIdx.x / DG_M) * nkb * DG_ABYTES;
+    for (int64_t q = threadIdx.x; q < nkb * (DG_K / 4); q += blockDim.x) {
+        const int64_t kb = q / (DG_K / 4);
+        const int k = (int)(q % (DG_K / 4)) * 4;
+        unsigned long long u[2][4];
+#pragma unroll
+        for (int t = 0; t < 4; t++) {
+            const int64_t j = kb * DG_K + k + t;
+            double2 v = make_double2(0, 0);
+            int s = 0;
+            if (i < n && j < n && e != DG_BAD && e != DG_NONE) {
+                v = a[j];
+                s = col[j] + e + 2;
+            }
+            u[0][t] = dg_biased(v.x, s);
+            u[1][t] = dg_biased(v.y, s);
+        }
+        // 32-byte rows, 16-byte halves swapped in every other group of four rows (bank conflicts)
+        uint8_t* dst = tile + kb * DG_ABYTES + r * DG_K + ((k / 16) ^ ((r >> 2) & 1)) * 16 + k % 16;
+#pragma unroll
+        for (int p = 0; p < 2; p++)
+#pragma unroll
+            for (int d = 0; d < DG; d++) {
+                uint32_t w = 0;
+#pragma unroll
+                for (int t = 0; t < 4; t++) w |= ((uint32_t)(u[p][t] >> (7 * (DG - 1 - d))) & 127u) << (8 * t);
+                *reinterpret_cast<uint32_t*>(dst + (p * DG + d) * DG_PLANE) = w;
+            }
+    }
+}
+
+// ve[r] = largest exponent of x_r 2^col; grid (blocks, vectors)
+__global__ void dg_vecexp_kernel(const double2* __restrict__ x, int64_t n, const int* __restrict__ col, int* ve) {
+    __shared__ int sh[8];
+    const double2* v = x + (int64_t)blockIdx.y * n;
+    int e = DG_NONE;
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
+        const int t = dg_exp2(v[j]), c = col[j];
+        if (t != DG_NONE) e = max(e, t == DG_BAD || c == DG_BAD ? DG_BAD : c == DG_NONE ? DG_NONE : t + c);
+    }
+    e = block_max(e, sh);
+    if (threadIdx.x == 0) atomicMax(&ve[blockIdx.y], e);
+}
+
+// Digits of R <= HN vectors as the B operand: blocks of one stage, [part][digit HN*2 + column][32 K], 64-byte rows
+// in the 64-byte swizzle; vectors above R and K above n are zero.  Thread: one entry of one vector.
+__global__ void dg_vecdigits_kernel(const double2* __restrict__ x, int64_t n, int64_t kpad, int R, int hn,
+                                    const int* __restrict__ col, const int* __restrict__ ve, uint8_t* __restrict__ out) {
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int r = blockIdx.y;
+    if (j >= kpad) return;
+    double2 v = make_double2(0, 0);
+    int s = 0;
+    const int e = r < R ? ve[r] : DG_NONE;
+    if (j < n && e != DG_NONE && e != DG_BAD && col[j] != DG_NONE) {
+        v = x[(int64_t)r * n + j];
+        s = e + 2 - col[j];
+    }
+    const unsigned long long u[2] = {dg_biased(v.x, s), dg_biased(v.y, s)};
+    const int brows = DG * 2 * hn, k = (int)(j % DG_K);
+    uint8_t* blk = out + j / DG_K * (int64_t)(2 * brows * DG_K * 2);
+#pragma unroll
+    for (int d = 0; d < DG; d++) {
+        const float re = (float)((int)((u[0] >> (7 * (DG - 1 - d))) & 127u) - 64);
+        const float im = (float)((int)((u[1] >> (7 * (DG - 1 - d))) & 127u) - 64);
+        const float val[2][2] = {{re, im}, {-im, re}};
+#pragma unroll
+        for (int p = 0; p < 2; p++)
+#pragma unroll
+            for (int h = 0; h < 2; h++) {
+                const int row = p * brows + d * 2 * hn + h * hn + r;
+                *reinterpret_cast<__nv_bfloat16*>(blk + (int64_t)row * 64 + (((k / 8) ^ ((row >> 1) & 3)) * 16) + (k % 8) * 2) =
+                    __float2bfloat16_rn(val[p][h]);
+            }
+    }
+}
+
+// ----------------------------------------------------------------- the product
+
+__device__ __forceinline__ uint32_t d_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void d_init(uint64_t* b, uint32_t n) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(d_u32(b)), "r"(n) : "memory");
+}
+__device__ __forceinline__ void d_arrive(uint64_t* b) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(d_u32(b)) : "memory");
+}
+__device__ __forceinline__ bool d_try(uint64_t* b, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 100000;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(ok)
+        : "r"(d_u32(b)), "r"(parity)
+        : "memory");
+    return ok;
+}
+// Bounded wait (about a second); on timeout raises the error flag and returns false, as does every later wait.
+__device__ __forceinline__ bool d_wait(uint64_t* b, uint32_t parity, int* err) {
+    if (d_try(b, parity)) return true;
+    if (*(volatile int*)err) return false;
+    const long long t0 = clock64();
+    while (!d_try(b, parity))
+        if (clock64() - t0 > (1ll << 31)) {
+            atomicExch(err, 2);
+            return false;
+        }
+    return true;
+}
+__device__ __forceinline__ void d_bulk(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(d_u32(dst)),
+        "l"(src), "r"(bytes), "r"(d_u32(bar))
+        : "memory");
+}
+// B operand: K-major, 64-byte rows in the 64-byte swizzle, 8-row groups 512 bytes apart
+__device__ __forceinline__ uint64_t d_desc(uint32_t addr) {
+    return (uint64_t)((addr >> 4) & 0x3FFF) | (uint64_t)1 << 16 | (uint64_t)(512 >> 4) << 32 | (uint64_t)1 << 46 |
+           (uint64_t)4 << 61;
+}
+// D (128 x N) += A (tensor memory, 128 x 16) B (N x 16)
+__device__ __forceinline__ void d_mma(uint32_t d, uint32_t a, uint64_t b, uint32_t n, uint32_t accumulate) {
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((uint32_t)(DG_M >> 4) << 24);
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n" ::"r"(d),
+        "r"(a), "l"(b), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+__device__ __forceinline__ void d_commit(uint64_t* bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(d_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void d_st8(uint32_t t, const uint32_t (&r)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(t), "r"(r[0]), "r"(r[1]),
+                 "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+                 : "memory");
+}
+__device__ __forceinline__ void d_ld16(uint32_t t, float (&v)[16]) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(t));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
+}
+#define DG_FENCE_BEFORE asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory")
+#define DG_FENCE_AFTER asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory")
+
+struct DgArgs {
+    const uint8_t* A;     // [row tile][K block][plane][row][32]
+    const uint8_t* B;     // [K block][part][row][32 bf16]
+    int nkb, nch, units, pieces, m, R;
+    const int *rowe, *ve;
+    double2* part;        // [row tile][piece][HN][128]
+    double2* Y;           // [R][m]
+    int* err;
+};
+
+__host__ __device__ inline int dg_first_unit(int units, int ctas, int b) { return (int)((int64_t)units * b / ctas); }
+// the first of the CTAs that hold units of `tile`
+__host__ __device__ inline int dg_first_cta(int units, int ctas, int nch, int tile) {
+    const int u = tile * nch;
+    int b = (int)((int64_t)u * ctas / units);
+    while (b + 1 < ctas && dg_first_unit(units, ctas, b + 1) <= u) b++;
+    while (b > 0 && dg_first_unit(units, ctas, b) > u) b--;
+    return b;
+}
+
+template <int NC>
+__global__ void __launch_bounds__(DG_WARPS * 32, 1) digits_gemm_kernel(const DgArgs a) {
+    typedef DgCfg<NC> C;
+    extern __shared__ uint8_t smem_raw[];
+    typename C::Smem& sm =
+        *reinterpret_cast<typename C::Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int u0 = dg_first_unit(a.units, gridDim.x, blockIdx.x), u1 = dg_first_unit(a.units, gridDim.x, blockIdx.x + 1);
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < DG_STAGES; s++) {
+            d_init(&sm.full[s], 1);
+            d_init(&sm.empty[s], 5);
+        }
+        for (int b = 0; b < 2; b++) {
+            d_init(&sm.tfull[b], 4);
+            d_init(&sm.tempty[b], 1);
+        }
+        d_init(&sm.dfull, 1);
+        d_init(&sm.dempty, 4);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 2) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(d_u32(&sm.tmem)), "r"(512) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    DG_FENCE_BEFORE;
+    __syncthreads();
+    DG_FENCE_AFTER;
+    const uint32_t tmem = sm.tmem;      // accumulators: columns 0 .. 8 NC - 1
+    const uint32_t ta = tmem + 256;     // two A operands of 16 planes x 8 columns
+
+    if (warp == 0) {
+        if (lane == 0) {
+            int s = 0;
+            uint32_t ph = 1;
+            bool ok = true;
+            for (int u = u0; u < u1 && ok; u++) {
+                const int tile = u / a.nch, c = u - tile * a.nch, ke = min(a.nkb, (c + 1) * DG_STEPS);
+                for (int kb = c * DG_STEPS; kb < ke; kb++) {
+                    if (!(ok = d_wait(&sm.empty[s], ph, a.err))) break;
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(d_u32(&sm.full[s])),
+                                 "r"(DG_ABYTES + C::BBYTES)
+                                 : "memory");
+                    d_bulk(sm.a[s], a.A + ((int64_t)tile * a.nkb + kb) * DG_ABYTES, DG_ABYTES, &sm.full[s]);
+                    d_bulk(sm.b[s], a.B + (int64_t)kb * C::BBYTES, C::BBYTES, &sm.full[s]);
+                    if (++s == DG_STAGES) {
+                        s = 0;
+                        ph ^= 1;
+                    }
+                }
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            int s = 0, b = 0;
+            uint32_t ph = 0, tph = 0;
+            bool ok = true;
+            for (int u = u0; u < u1 && ok; u++) {
+                const int c = u % a.nch, kb0 = c * DG_STEPS, ke = min(a.nkb, kb0 + DG_STEPS);
+                if (u > u0) {
+                    if (!(ok = d_wait(&sm.dempty, (uint32_t)((u - u0 - 1) & 1), a.err))) break;
+                    DG_FENCE_AFTER;
+                }
+                for (int kb = kb0; kb < ke && ok; kb++) {
+                    if (!(ok = d_wait(&sm.full[s], ph, a.err))) break;
+                    const uint32_t bs = d_u32(sm.b[s]);
+                    for (int kk = 0; kk < 2; kk++) {
+                        if (!(ok = d_wait(&sm.tfull[b], tph, a.err))) break;
+                        DG_FENCE_AFTER;
+#pragma unroll
+                        for (int p = 0; p < 2; p++) {
+                            const uint64_t bd = d_desc(bs + p * C::BROWS * 64 + kk * 32);
+#pragma unroll
+                            for (int i = 0; i < DG; i++)
+                                d_mma(tmem + i * NC, ta + b * 128 + (p * DG + i) * 8, bd, NC * (DG - i),
+                                      kb > kb0 || kk > 0 || p > 0 || i > 0);
+                        }
+                        d_commit(&sm.tempty[b]);
+                        b ^= 1;
+                        if (b == 0) tph ^= 1;
+                    }
+                    if (!ok) break;
+                    d_commit(&sm.empty[s]);
+                    if (++s == DG_STAGES) {
+                        s = 0;
+                        ph ^= 1;
+                    }
+                }
+                if (ok) d_commit(&sm.dfull);
+            }
+        }
+    } else if (warp < 6) {
+        // bytes d + 64 -> BF16 128 + (d + 64) by a byte permute, minus 192
+        const int q = warp & 3, row = q * 32 + lane, sw = ((row >> 2) & 1) * 16;
+        const uint32_t lt = ta + ((uint32_t)(q * 32) << 16);
+        const __nv_bfloat162 off = __floats2bfloat162_rn(192.f, 192.f);
+        int s = 0, b = 0;
+        uint32_t ph = 0, tph = 1;
+        for (int u = u0; u < u1; u++) {
+            const int c = u % a.nch, kb0 = c * DG_STEPS, ke = min(a.nkb, kb0 + DG_STEPS);
+            for (int kb = kb0; kb < ke; kb++) {
+                d_wait(&sm.full[s], ph, a.err);
+                const uint8_t* src = sm.a[s] + row * DG_K;
+                for (int kk = 0; kk < 2; kk++) {
+                    d_wait(&sm.tempty[b], tph, a.err);
+                    DG_FENCE_AFTER;
+#pragma unroll 4
+                    for (int p = 0; p < 2 * DG; p++) {
+                        const uint4 v = *reinterpret_cast<const uint4*>(src + p * DG_PLANE + ((kk * 16) ^ sw));
+                        const uint32_t in[4] = {v.x, v.y, v.z, v.w};
+                        uint32_t r[8];
+#pragma unroll
+                        for (int w = 0; w < 4; w++)
+#pragma unroll
+                            for (int h = 0; h < 2; h++) {
+                                const uint32_t t = __byte_perm(in[w], 0x43434343u, h ? 0x4342 : 0x4140);
+                                const __nv_bfloat162 d = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&t), off);
+                                r[2 * w + h] = *reinterpret_cast<const uint32_t*>(&d);
+                            }
+                        d_st8(lt + b * 128 + p * 8, r);
+                    }
+                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                    DG_FENCE_BEFORE;
+                    __syncwarp();
+                    if (lane == 0) d_arrive(&sm.tfull[b]);
+                    b ^= 1;
+                    if (b == 0) tph ^= 1;
+                }
+                __syncwarp();
+                if (lane == 0) d_arrive(&sm.empty[s]);
+                if (++s == DG_STAGES) {
+                    s = 0;
+                    ph ^= 1;
+                }
+            }
+        }
+    } else {
+        const int q = warp & 3, r = q * 32 + lane;
+        const uint32_t ld = tmem + ((uint32_t)(q * 32) << 16);
+        dfl y[NC];
+#pragma unroll
+        for (int j = 0; j < NC; j++) y[j] = dfl{0.f, 0.f};
+        for (int u = u0; u < u1; u++) {
+            const int tile = u / a.nch;
+            d_wait(&sm.dfull, (uint32_t)((u - u0) & 1), a.err);
+            DG_FENCE_AFTER;
+#pragma unroll
+            for (int s = DG - 1; s >= 0; s--) {
+                const float w = __int_as_float((127 - 7 * s) << 23);  // 2^(-7 s)
+#pragma unroll
+                for (int c = 0; c < NC; c += 16) {
+                    float v[16];
+                    d_ld16(ld + s * NC + c, v);
+#pragma unroll
+                    for (int j = 0; j < 16; j++) {
+                        const dfl t = two_sum(y[c + j].h, v[j] * w);
+                        y[c + j].h = t.h;
+                        y[c + j].l = __fadd_rn(y[c + j].l, t.l);
+                    }
+                }
+            }
+            DG_FENCE_BEFORE;
+            __syncwarp();
+            if (lane == 0) d_arrive(&sm.dempty);
+#pragma unroll
+            for (int j = 0; j < NC; j++) y[j] = two_sum(y[j].h, y[j].l);
+            if (u + 1 < u1 && (u + 1) % a.nch != 0) continue;
+            const int piece = blockIdx.x - dg_first_cta(a.units, gridDim.x, a.nch, tile);
+            double2* out = a.part + (int64_t)(tile * a.pieces + piece) * C::HN * DG_M + r;
+#pragma unroll
+            for (int j = 0; j < C::HN; j++)
+                if (j < a.R)
+                    out[j * DG_M] = make_double2((double)y[j].h + (double)y[j].l,
+                                                 (double)y[C::HN + j].h + (double)y[C::HN + j].l);
+#pragma unroll
+            for (int j = 0; j < NC; j++) y[j] = dfl{0.f, 0.f};
+        }
+    }
+    __syncwarp();
+    DG_FENCE_BEFORE;
+    __syncthreads();
+    if (warp == 2) {
+        DG_FENCE_AFTER;
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+    }
+}
+
+// Y = the pieces of every row added in CTA order, times the powers of two.
+__global__ void dg_finish_kernel(DgArgs a, int ctas, int hn) {
+    const int row = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
+    if (row >= a.m) return;
+    const int tile = row / DG_M, first = dg_first_cta(a.units, ctas, a.nch, tile);
+    double x = 0, y = 0;
+    for (int p = 0; p < a.pieces; p++) {
+        if (first + p >= ctas || dg_first_unit(a.units, ctas, first + p) >= (tile + 1) * a.nch) break;
+        const double2 v = a.part[((int64_t)(tile * a.pieces + p) * hn + r) * DG_M + row % DG_M];
+        x += v.x;
+        y += v.y;
+    }
+    const int er = a.rowe[row], ev = a.ve[r];
+    if (er == DG_BAD || ev == DG_BAD) x = y = __longlong_as_double(0x7ff8000000000000ll);
+    else if (er == DG_NONE || ev == DG_NONE) x = y = 0;
+    else {
+        const int e = er + ev + 4 - 14;  // both operands below 2^-2 of their scale, first digits 2^-7 each
+        x = ldexp(x, e);
+        y = ldexp(y, e);
+    }
+    a.Y[(int64_t)r * a.m + row] = make_double2(x, y);
+}
+
+// ----------------------------------------------------------------- host side
+
+int64_t digits_kpad(int64_t n) { return (n + DG_K - 1) / DG_K * DG_K; }
+int64_t digits_mpad(int64_t n) { return (n + DG_M - 1) / DG_M * DG_M; }
+// bytes of a matrix (as complex128 with leading dimension kpad, then as digits in the same place)
+size_t digits_bytes(int64_t n) { return (size_t)digits_mpad(n) * digits_kpad(n) * 16; }
+
+constexpr int DG_TILES = 2;  // row tiles converted at a time
+static int dg_hn(int64_t R) { return R <= 8 ? 8 : 16; }
+static int dg_pieces(int units, int ctas, int nch) {
+    const int q = units / ctas;  // a CTA holds q or q + 1 units
+    return (nch + q - 1) / q + 1;
+}
+// scratch of a product of R vectors (B operand, exponents, pieces), and of the conversion
+size_t digits_work_bytes(int64_t n, int64_t R) {
+    const int hn = dg_hn(R);
+    const int nkb = (int)(digits_kpad(n) / DG_K), nch = (nkb + DG_STEPS - 1) / DG_STEPS;
+    const int tiles = (int)(digits_mpad(n) / DG_M), units = tiles * nch, ctas = std::min(DG_CTAS, units);
+    return (size_t)nkb * 2 * DG * 2 * hn * DG_K * 2 + (size_t)tiles * dg_pieces(units, ctas, nch) * hn * DG_M * 16 + 16 * sizeof(int);
+}
+size_t digits_convert_bytes(int64_t n) { return (size_t)DG_TILES * DG_M * digits_kpad(n) * 16; }
+
+#define DCK(expr)                                                                                        \
+    do {                                                                                                 \
+        cudaError_t e_ = (expr);                                                                         \
+        if (e_ != cudaSuccess) return ctx->fail(BEM_ERR_CUDA, std::string("digits: ") + cudaGetErrorString(e_)); \
+    } while (0)
+
+// Complex128 matrix A (n x n in a buffer of digits_bytes, leading dimension
+// digits_kpad) -> digits in place; exps: device [kpad + mpad] column, row exponents.
+int digits_prepare(bem_ctx* ctx, double2* A, int64_t n, int* exps) {
+    const int64_t kpad = digits_kpad(n), mpad = digits_mpad(n), nkb = kpad / DG_K;
+    int rc;
+    uint8_t* tmp = (uint8_t*)ctx->dalloc(digits_convert_bytes(n), &rc);
+    if (rc) return rc;
+    int* col = exps;
+    int* row = exps + kpad;
+    std::vector<int> none((size_t)kpad, DG_NONE);
+    DCK(cudaMemcpyAsync(col, none.data(), kpad * sizeof(int), cudaMemcpyHostToDevice, ctx->stream));
+    DCK(cudaStreamSynchronize(ctx->stream));
+    const int64_t rows_per = 256;
+    dg_colexp_kernel<<<dim3((unsigned)((n + 127) / 128), (unsigned)((n + rows_per - 1) / rows_per)), 128, 0, ctx->stream>>>(
+        A, n, kpad, rows_per, col);
+    DCK(cudaGetLastError());
+    ctx->launches += 1;
+    for (int64_t r0 = 0; r0 < mpad; r0 += DG_TILES * DG_M) {
+        const int64_t rows = std::min<int64_t>(DG_TILES * DG_M, mpad - r0);
+        dg_digits_kernel<<<(unsigned)rows, 256, 0, ctx->stream>>>(A, n, kpad, r0, nkb, col, row, tmp);
+        DCK(cudaGetLastError());
+        DCK(cudaMemcpyAsync(A + r0 * kpad, tmp, (size_t)rows * kpad * 16, cudaMemcpyDeviceToDevice, ctx->stream));
+        ctx->launches += 1;
+    }
+    DCK(cudaStreamSynchronize(ctx->stream));
+    ctx->dfree(tmp);
+    return BEM_OK;
+}
+
+template <int NC>
+static cudaError_t launch_digits(const DgArgs& a, unsigned ctas, cudaStream_t s) {
+    constexpr size_t smem = sizeof(typename DgCfg<NC>::Smem) + 1024;
+    static const cudaError_t attr_e =
+        cudaFuncSetAttribute(digits_gemm_kernel<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (attr_e != cudaSuccess) return attr_e;
+    digits_gemm_kernel<NC><<<ctas, DG_WARPS * 32, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
+// Y [R][n] = A X [R][n] with A as digits (digits_prepare); work: digits_work_bytes(n, min(R, 16)).
+int digits_gemm(bem_ctx* ctx, const void* A, const int* exps, int64_t n, const double2* X, int64_t R, double2* Y, void* work) {
+    const int64_t kpad = digits_kpad(n), mpad = digits_mpad(n);
+    const int hn = dg_hn(R);
+    DgArgs a{};
+    a.A = (const uint8_t*)A;
+    a.nkb = (int)(kpad / DG_K);
+    a.nch = (a.nkb + DG_STEPS - 1) / DG_STEPS;
+    const int tiles = (int)(mpad / DG_M);
+    a.units = tiles * a.nch;
+    const int ctas = std::min(DG_CTAS, a.units);
+    a.pieces = dg_pieces(a.units, ctas, a.nch);
+    a.m = (int)n;
+    a.rowe = exps + kpad;
+    a.err = ctx->dev.err;
+    uint8_t* b = (uint8_t*)work;
+    const size_t bb = (size_t)a.nkb * 2 * DG * 2 * hn * DG_K * 2;
+    a.B = b;
+    a.part = (double2*)(b + bb);
+    int* ve = (int*)(a.part + (size_t)tiles * a.pieces * hn * DG_M);
+    a.ve = ve;
+    for (int64_t r0 = 0; r0 < R; r0 += hn) {
+        const int nr = (int)std::min<int64_t>(hn, R - r0);
+        const double2* x = X + r0 * n;
+        a.R = nr;
+        a.Y = Y + r0 * n;
+        DCK(cudaMemsetAsync(ve, 0x80, 16 * sizeof(int), ctx->stream));  // below every exponent
+        dg_vecexp_kernel<<<dim3((unsigned)std::min<int64_t>(64, (n + 255) / 256), (unsigned)nr), 256, 0, ctx->stream>>>(x, n, exps, ve);
+        dg_vecdigits_kernel<<<dim3((unsigned)((kpad + 127) / 128), (unsigned)hn), 128, 0, ctx->stream>>>(x, n, kpad, nr, hn, exps, ve, b);
+        DCK(cudaGetLastError());
+        DCK(hn == 8 ? launch_digits<16>(a, (unsigned)ctas, ctx->stream) : launch_digits<32>(a, (unsigned)ctas, ctx->stream));
+        dg_finish_kernel<<<dim3((unsigned)((n + 255) / 256), (unsigned)nr), 256, 0, ctx->stream>>>(a, ctas, hn);
+        DCK(cudaGetLastError());
+        ctx->launches += 4;
+    }
+    return BEM_OK;
+}
+
+}  // namespace gbem

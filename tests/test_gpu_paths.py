@@ -74,3 +74,31 @@ def test_near_groups_match_native_fp64(api, name, n_gauss):
         y.append(c.apply(x, precision=api.FP64))
         c.close()
     assert rel(y[0], y[1]) < 1e-12
+
+
+@pytest.mark.parametrize("name,R", [("sphere", 1), ("sphere", 8), ("two", 9), ("two", 16), ("shell", 17), ("shell", 33)])
+def test_fp64_assembled_digits(api, name, R):
+    """The assembled FP64 product in fixed-point digits, by its own columns
+    (unit vectors, whose digits are exact): vectors of very different sizes,
+    with the psi and phi blocks a factor |k| apart, a zero vector, and an
+    infinite one that leaves the others alone.  Digits keep 2^-54 of the largest
+    scaled entry of a row and of a vector; rows here range over less than 2^12."""
+    s = {"sphere": lambda: scenes.sphere_scene(1), "two": lambda: scenes.two_sphere_scene(2),
+         "shell": lambda: scenes.shell_scene(1)}[name]()
+    c = api.Context.from_scene(s)
+    N = c.n_dofs
+    A = c.apply(np.eye(N, dtype=np.complex128), precision=api.FP64_ASSEMBLED).T
+    rng = np.random.default_rng(R)
+    X = np.stack([scenes.smooth_trace_vector(s, r) for r in range(R)]) * 10.0 ** rng.uniform(-150, 150, (R, 1))
+    if R > 8:
+        X[3] = 0.0
+        X[5, N // 2] = np.inf
+    Y = c.apply(X if R > 1 else X[0], precision=api.FP64_ASSEMBLED).reshape(R, N)
+    c.close()
+    for r in range(R):
+        if R > 8 and r == 3:
+            assert not Y[r].any()
+        elif R > 8 and r == 5:
+            assert np.isnan(Y[r].real).all()
+        else:
+            assert rel(Y[r], A @ X[r]) < 1e-12
