@@ -44,7 +44,18 @@ static uint64_t next_gen() {
 
 void* bem_ctx::dalloc(size_t bytes, int* rc) {
     if (bytes == 0) bytes = 16;
+    // the tensor-core far field's operands are a convenience: they go before an allocation is refused
+    auto give_back = [&] {
+        if (!mm_buf) return false;
+        cudaStreamSynchronize(stream);
+        dfree(mm_buf);
+        mm_buf = nullptr;
+        mm_bytes = 0;
+        mm_off = true;
+        return true;
+    };
     if (opts.hbm_budget_bytes > 0 && (int64_t)(used_bytes + bytes) > opts.hbm_budget_bytes) {
+        if (give_back()) return dalloc(bytes, rc);
         *rc = fail(BEM_ERR_OUT_OF_BUDGET, "device memory budget exceeded (" + std::to_string(used_bytes + bytes) +
                                               " > " + std::to_string(opts.hbm_budget_bytes) + " bytes)");
         return nullptr;
@@ -53,6 +64,7 @@ void* bem_ctx::dalloc(size_t bytes, int* rc) {
         const int64_t after = pool->fetch_add((int64_t)bytes) + (int64_t)bytes;
         if (pool_limit > 0 && after > pool_limit) {
             pool->fetch_sub((int64_t)bytes);
+            if (give_back()) return dalloc(bytes, rc);
             *rc = fail(BEM_ERR_OUT_OF_BUDGET, "shared device memory budget exceeded (" + std::to_string(after) +
                                                   " > " + std::to_string(pool_limit) + " bytes)");
             return nullptr;
@@ -62,6 +74,10 @@ void* bem_ctx::dalloc(size_t bytes, int* rc) {
     cudaError_t e = cudaMalloc(&p, bytes);
     if (e != cudaSuccess) {
         if (pool) pool->fetch_sub((int64_t)bytes);
+        if (e == cudaErrorMemoryAllocation && give_back()) {
+            cudaGetLastError();
+            return dalloc(bytes, rc);
+        }
         *rc = fail(BEM_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
         return nullptr;
     }
@@ -148,6 +164,10 @@ static void release_device(bem_ctx* ctx) {
     ctx->multi_work = nullptr;
     ctx->multi_n_work = 0;
     for (int& k : ctx->multi_key) k = -1;
+    ctx->mmg = bem_ctx::MmGeom();
+    ctx->mm_buf = nullptr;
+    ctx->mm_bytes = 0;
+    ctx->mm_off = false;
     ctx->pmchwt_near = NearSet();
     destroy_solver_state(ctx);
 }
@@ -641,12 +661,120 @@ int bem_ctx::run_apply(const double2* x, double2* y, int precision, const ApplyM
     return BEM_OK;
 }
 
+// Geometry of the tensor-core far field: source points with |g|^2, a frame
+// with the mean normal of every tile, and the close pairs of tiles.
+int bem_ctx::ensure_farmm() {
+    bem_ctx* const ctx = this;
+    if (mmg.ready) return BEM_OK;
+    const Geometry& g = geo;
+    const int nt = g.n_tiles;
+    std::vector<float4> gq(g.n_pts);
+    for (int64_t s = 0; s < g.n_slots; s++) {
+        float4 tri[QP];
+        for (int q = 0; q < QP; q++) {
+            const int64_t p = s * QP + q;
+            const float x = (float)g.pt_delta[3 * p], y = (float)g.pt_delta[3 * p + 1], z = (float)g.pt_delta[3 * p + 2];
+            tri[q] = make_float4(x, y, z, (float)((double)x * x + (double)y * y + (double)z * z));
+        }
+        pair_interleave(tri, gq.data() + s * QP);
+    }
+    std::vector<float> fr((size_t)nt * 9);
+    double rmax = 0;
+    for (int t = 0; t < nt; t++) {
+        rmax = std::max(rmax, g.tile_c[4 * t + 3]);
+        double m[3] = {0, 0, 0};
+        for (int64_t s = (int64_t)t * TT; s < (int64_t)t * TT + g.tile_ntri[t]; s++)
+            for (int c = 0; c < 3; c++) m[c] += g.slot_n[3 * s + c] * g.slot_area[s];
+        double l = std::sqrt(m[0] * m[0] + m[1] * m[1] + m[2] * m[2]);
+        if (!(l > 0)) { m[0] = m[1] = 0; m[2] = l = 1; }
+        for (double& c : m) c /= l;
+        const int ax = std::fabs(m[0]) < std::fabs(m[1]) ? (std::fabs(m[0]) < std::fabs(m[2]) ? 0 : 2)
+                                                         : (std::fabs(m[1]) < std::fabs(m[2]) ? 1 : 2);
+        double u[3] = {0, 0, 0}, d = m[ax];
+        for (int c = 0; c < 3; c++) u[c] = (c == ax) - d * m[c];
+        l = std::sqrt(u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
+        for (double& c : u) c /= l;
+        const double v[3] = {m[1] * u[2] - m[2] * u[1], m[2] * u[0] - m[0] * u[2], m[0] * u[1] - m[1] * u[0]};
+        for (int c = 0; c < 3; c++) {
+            fr[9 * t + c] = (float)u[c];
+            fr[9 * t + 3 + c] = (float)v[c];
+            fr[9 * t + 6 + c] = (float)m[c];
+        }
+    }
+    int e = 0;
+    std::frexp(rmax, &e);
+    mmg.rho = std::ldexp(1.0f, std::max(-100, std::min(100, e)));
+    mmg.near_words = (nt + 31) / 32;
+    std::vector<uint32_t> mask((size_t)nt * mmg.near_words, 0);
+    mmg.h_ptr.assign(nt + 1, 0);
+    mmg.h_idx.clear();
+    mmg.fits = true;
+    for (int t = 0; t < nt; t++) {
+        const double* a = &g.tile_c[4 * t];
+        for (int s = 0; s < nt; s++) {
+            const double* b = &g.tile_c[4 * s];
+            const double x = a[0] - b[0], y = a[1] - b[1], z = a[2] - b[2], r = FARMM_SEP * (a[3] + b[3]);
+            if (x * x + y * y + z * z < r * r || s == t) {
+                mask[(size_t)t * mmg.near_words + s / 32] |= 1u << (s % 32);
+                mmg.h_idx.push_back(s);
+            }
+        }
+        mmg.h_ptr[t + 1] = (int)mmg.h_idx.size();
+        mmg.fits &= mmg.h_ptr[t + 1] - mmg.h_ptr[t] <= CHUNK_MAX;
+    }
+    const size_t b_geo = gq.size() * sizeof(float4), b_mask = mask.size() * 4, b_fr = fr.size() * 4,
+                 b_ptr = mmg.h_ptr.size() * 4, b_idx = mmg.h_idx.size() * 4;
+    int rc;
+    mmg.buf = dalloc(b_geo + b_mask + b_fr + b_ptr + b_idx, &rc);
+    if (rc) { mmg.buf = nullptr; return rc; }
+    char* q = (char*)mmg.buf;
+    mmg.geo = (float4*)q; q += b_geo;
+    mmg.near = (uint32_t*)q; q += b_mask;
+    mmg.frame = (float*)q; q += b_fr;
+    mmg.near_ptr = (int*)q; q += b_ptr;
+    mmg.near_idx = (int*)q;
+    CK(cudaMemcpyAsync(mmg.geo, gq.data(), b_geo, cudaMemcpyHostToDevice, stream));
+    CK(cudaMemcpyAsync(mmg.near, mask.data(), b_mask, cudaMemcpyHostToDevice, stream));
+    CK(cudaMemcpyAsync(mmg.frame, fr.data(), b_fr, cudaMemcpyHostToDevice, stream));
+    CK(cudaMemcpyAsync(mmg.near_ptr, mmg.h_ptr.data(), b_ptr, cudaMemcpyHostToDevice, stream));
+    CK(cudaMemcpyAsync(mmg.near_idx, mmg.h_idx.data(), b_idx, cudaMemcpyHostToDevice, stream));
+    CK(cudaStreamSynchronize(stream));
+    mmg.ready = true;
+    return BEM_OK;
+}
+
+// Whether n_rhs vectors go to the tensor cores, with their operands' memory in
+// place: enough tiles for most pairs not to be close, and room in the budgets
+// (of a shared one at most half may be in use: other scenes' reservations do not
+// count these operands).
+bool bem_ctx::reserve_farmm(int64_t n_rhs) {
+    if (mm_off || geo.n_tiles < FARMM_MIN_TILES) return false;
+    if (ensure_farmm() || !mmg.fits) return false;
+    const size_t need = farmm_bytes(geo.n_tiles, n_rhs);
+    if (need <= mm_bytes) return true;
+    dfree(mm_buf);
+    mm_buf = nullptr;
+    mm_bytes = 0;
+    if (pool && pool_limit > 0 && 2 * (pool->load() + (int64_t)need) > pool_limit) return false;
+    int rc;
+    mm_buf = dalloc(need, &rc);
+    if (rc) {
+        mm_buf = nullptr;
+        cudaGetLastError();
+        return false;
+    }
+    mm_bytes = need;
+    return true;
+}
+
 // A_hat applied to n_rhs vectors x [n_rhs][N] -> y [n_rhs][N] at FP32 with
-// one far-field launch for all of them (far32m_kernel: the Green's function
-// and gradient factor of a pair are evaluated once per group of MRG vectors),
-// then the projection (with the near-field correction) and the reduction of
-// each vector.  Same arithmetic per vector as apply_ahat at FP32 except the
-// chunk boundaries of the source sums.
+// the far field of all of them at once, then the projection (with the
+// near-field correction) and the reduction of each vector.  Meshes of at least
+// FARMM_MIN_TILES tiles take the tensor cores for the pairs of tiles that are
+// not close (k_farmm.cu) and far32m_kernel for the close ones, whose partials
+// are one chunk more; smaller ones, and budgets that do not hold the operands,
+// far32m_kernel for all (the Green's function and gradient factor of a pair
+// are evaluated once per group of MRG vectors).
 int bem_ctx::apply_ahat_multi(const double2* x, double2* y, int64_t n_rhs) {
     bem_ctx* const ctx = this;
     int rc = ensure_near();
@@ -654,34 +782,63 @@ int bem_ctx::apply_ahat_multi(const double2* x, double2* y, int64_t n_rhs) {
     const Geometry& g = geo;
     const int n_tiles = g.n_tiles;
     const int groups = (int)((n_rhs + MRG - 1) / MRG);
-    int n_chunks, chunk_tiles;
-    multi_chunking(n_tiles, g.n_pts, n_rhs, &n_chunks, &chunk_tiles);
-    const int64_t rstride = (int64_t)n_chunks * 2 * NCOMP * g.n_pts;
-    const size_t b_pd = (size_t)n_rhs * g.n_pts * sizeof(float4);
-    const size_t b_tc = (size_t)n_rhs * 2 * g.n_slots * sizeof(float4);
-    const size_t b_part = (size_t)n_rhs * rstride * sizeof(float);
-    const size_t need = b_pd + b_tc + b_part;
-    if (need > multi_buf_bytes) {
+    int n_chunks, chunk_tiles;      // partial rows; source tiles per item
+    bool mm = reserve_farmm(n_rhs);
+    size_t b_pd, b_tc, b_part;
+    int64_t rstride;
+    while (true) {
+        if (mm) {
+            farmm_chunking(n_tiles, g.n_pts, n_rhs, &n_chunks, &chunk_tiles);
+            n_chunks += 1;          // the close tiles
+        } else {
+            multi_chunking(n_tiles, g.n_pts, n_rhs, &n_chunks, &chunk_tiles);
+        }
+        rstride = (int64_t)n_chunks * 2 * NCOMP * g.n_pts;
+        b_pd = (size_t)n_rhs * g.n_pts * sizeof(float4);
+        b_tc = (size_t)n_rhs * 2 * g.n_slots * sizeof(float4);
+        b_part = (size_t)n_rhs * rstride * sizeof(float);
+        const size_t need = b_pd + b_tc + b_part;
+        if (need <= multi_buf_bytes) break;
         dfree(multi_buf);
+        multi_buf_bytes = 0;
         multi_buf = dalloc(need, &rc);
-        if (rc) { multi_buf = nullptr; multi_buf_bytes = 0; return rc; }
-        multi_buf_bytes = need;
+        if (rc) multi_buf = nullptr;
+        else multi_buf_bytes = need;
+        if (mm && !mm_buf) {        // the operands made room for it: start over without them
+            mm = false;
+            continue;
+        }
+        if (rc && mm) {
+            mm = false;
+            continue;
+        }
+        if (rc) return rc;
+        break;
     }
     float4* pdm = (float4*)multi_buf;
     float4* tcm = (float4*)((char*)multi_buf + b_pd);
     float* part = (float*)((char*)multi_buf + b_pd + b_tc);
-    // work list: (target tile, chunk, slot, group), heaviest first
-    const int key[3] = {n_chunks, chunk_tiles, groups};
-    if (!multi_work || !std::equal(key, key + 3, multi_key)) {
+    // work list: tensor-core items (block, chunk, slot, group), groups and chunks outermost so that the CTAs of a
+    // wave share a chunk's operands through L2, then items of the FP32 kernel (target tile, chunk, slot, group),
+    // heaviest first
+    const int key[4] = {n_chunks, chunk_tiles, groups, (int)mm};
+    if (!multi_work || !std::equal(key, key + 4, multi_key)) {
+        std::vector<int4> work;
+        if (mm)
+            for (int gr = 0; gr < farmm_groups(n_rhs); gr++)
+                for (int c = 0; c + 1 < n_chunks; c++)
+                    for (int sl = 0; sl < 2; sl++)
+                        for (int b = 0; b < farmm_blocks(g.n_pts); b++) work.push_back(make_int4(b, c, sl, gr));
+        const int64_t n_far = (int64_t)work.size();
         std::vector<std::pair<int64_t, int4>> items;
-        items.reserve((size_t)n_tiles * n_chunks * 2 * groups);
         for (int t = 0; t < n_tiles; t++) {
             const int d = g.tile_dom[t];
             const int own_b = g.dom_tile_begin[d], own_e = g.dom_tile_end[d];
-            for (int c = 0; c < n_chunks; c++) {
-                const int sb = c * chunk_tiles, se = std::min(sb + chunk_tiles, n_tiles);
+            for (int c = mm ? n_chunks - 1 : 0; c < n_chunks; c++) {
+                const int sb = mm ? mmg.h_ptr[t] : c * chunk_tiles, se = mm ? mmg.h_ptr[t + 1] : std::min(sb + chunk_tiles, n_tiles);
                 int64_t w0 = 0, w1 = 0;
-                for (int s = sb; s < se; s++) {
+                for (int i = sb; i < se; i++) {
+                    const int s = mm ? mmg.h_idx[i] : i;
                     w0 += g.tile_ntri[s];
                     if (s >= own_b && s < own_e) w1 += g.tile_ntri[s];
                 }
@@ -693,16 +850,18 @@ int bem_ctx::apply_ahat_multi(const double2* x, double2* y, int64_t n_rhs) {
         }
         std::stable_sort(items.begin(), items.end(),
                          [](const std::pair<int64_t, int4>& a, const std::pair<int64_t, int4>& b) { return a.first < b.first; });
-        std::vector<int4> work(items.size());
-        for (size_t i = 0; i < items.size(); i++) work[i] = items[i].second;
+        for (const auto& it : items) work.push_back(it.second);
         dfree(multi_work);
         multi_work = nullptr;
+        for (int& k : multi_key) k = -1;
         multi_work = (int4*)dalloc(work.size() * sizeof(int4), &rc);
         if (rc) { multi_work = nullptr; return rc; }
+        if (mm && !mm_buf) return apply_ahat_multi(x, y, n_rhs);  // the operands made room for the list
         CK(cudaMemcpyAsync(multi_work, work.data(), work.size() * sizeof(int4), cudaMemcpyHostToDevice, stream));
         CK(cudaStreamSynchronize(stream));
         multi_n_work = (int64_t)work.size();
-        std::copy(key, key + 3, multi_key);
+        multi_n_far = n_far;
+        std::copy(key, key + 4, multi_key);
     }
     const int64_t N = g.n_dof;
     // 1. trial densities of every vector
@@ -716,21 +875,36 @@ int bem_ctx::apply_ahat_multi(const double2* x, double2* y, int64_t n_rhs) {
         ga.tcurl32 = tcm + r * 2 * g.n_slots;
         CK(launch_gather(ga, stream));
     }
-    // 2. far field of all vectors in one launch
-    FarArgs32M fa{};
-    fa.pg = dev.pg32; fa.pgp = dev.pgp32; fa.tg = dev.tg32; fa.tc = dev.tc; fa.tdom = dev.tdom; fa.tntri = dev.tntri;
-    fa.pd = pdm; fa.tcurl = tcm; fa.dom_tiles = dev.dom_tiles; fa.kdom = dev.kdom;
-    fa.k0 = make_double2(k0re, k0im);
-    fa.src_begin = 0; fa.src_end = n_tiles; fa.tgt_begin = 0; fa.chunk_tiles = chunk_tiles;
-    fa.R = (int)n_rhs; fa.n_pts = g.n_pts; fa.n_slots = g.n_slots; fa.rstride = rstride; fa.partial = part;
-    fa.err = dev.err; fa.work = multi_work;
+    // 2. far field of all vectors
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     if (profiling) {
         CK(cudaEventCreate(&ev0));
         CK(cudaEventCreate(&ev1));
         CK(cudaEventRecord(ev0, stream));
     }
-    CK(launch_far32_multi(fa, multi_n_work, stream));
+    if (mm) {
+        FarMmPlan p{};
+        p.pg = dev.pg32; p.tg = dev.tg32; p.tc = dev.tc; p.tdom = dev.tdom; p.dom_tiles = dev.dom_tiles; p.kdom = dev.kdom;
+        p.k0 = make_double2(k0re, k0im);
+        p.pd = pdm; p.tcurl = tcm; p.frame = mmg.frame; p.near = mmg.near; p.near_words = mmg.near_words; p.geo = mmg.geo;
+        p.rho = mmg.rho; p.n_tiles = n_tiles; p.chunk_tiles = chunk_tiles; p.R = (int)n_rhs; p.n_pts = g.n_pts;
+        p.n_slots = g.n_slots; p.rstride = rstride; p.n_work = multi_n_far; p.partial = part; p.err = dev.err;
+        p.work = multi_work; p.buf = mm_buf;
+        CK(launch_farmm(p, stream));
+        launches += 3;
+    }
+    FarArgs32M fa{};
+    fa.pg = dev.pg32; fa.pgp = dev.pgp32; fa.tg = dev.tg32; fa.tc = dev.tc; fa.tdom = dev.tdom; fa.tntri = dev.tntri;
+    fa.pd = pdm; fa.tcurl = tcm; fa.dom_tiles = dev.dom_tiles; fa.kdom = dev.kdom;
+    fa.k0 = make_double2(k0re, k0im);
+    fa.src_begin = 0; fa.src_end = n_tiles; fa.tgt_begin = 0; fa.chunk_tiles = chunk_tiles;
+    fa.R = (int)n_rhs; fa.n_pts = g.n_pts; fa.n_slots = g.n_slots; fa.rstride = rstride; fa.partial = part;
+    fa.err = dev.err; fa.work = multi_work + (mm ? multi_n_far : 0);
+    if (mm) {
+        fa.near_ptr = mmg.near_ptr;
+        fa.near_idx = mmg.near_idx;
+    }
+    CK(launch_far32_multi(fa, multi_n_work - (mm ? multi_n_far : 0), stream));
     if (profiling) {
         CK(cudaEventRecord(ev1, stream));
         far_events.push_back({ev0, ev1});

@@ -131,7 +131,23 @@ struct bem_ctx {
     std::function<int64_t(int64_t room, std::vector<double>& w)> join_hook;
     int4* multi_work = nullptr;
     int64_t multi_n_work = 0;
-    int multi_key[3] = {-1, -1, -1};  // (n_chunks, chunk_tiles, groups) the list was built for
+    int multi_key[4] = {-1, -1, -1, -1};  // (n_chunks, chunk_tiles, groups, tensor cores) the list was built for
+    struct MmGeom {                // tensor-core far field of several right-hand sides (k_farmm.cu)
+        bool ready = false;
+        bool fits = false;         // every tile's close tiles fit one item of the FP32 kernel
+        void* buf = nullptr;
+        float4* geo = nullptr;
+        float* frame = nullptr;
+        uint32_t* near = nullptr;
+        int *near_ptr = nullptr, *near_idx = nullptr;
+        std::vector<int> h_ptr, h_idx;
+        int near_words = 0;
+        float rho = 1.f;
+    } mmg;
+    void* mm_buf = nullptr;        // its B operands (grow-only; given back when the budget is needed elsewhere)
+    size_t mm_bytes = 0;
+    bool mm_off = false;           // given back once: stay with the FP32 kernel
+    int64_t multi_n_far = 0;       // work items of the tensor-core kernel at the head of multi_work
     std::vector<std::pair<void*, size_t>> allocs;
     size_t used_bytes = 0;
     size_t peak_bytes = 0;                     // largest used_bytes seen
@@ -189,6 +205,8 @@ struct bem_ctx {
     int run_apply(const double2* x, double2* y, int precision, const gbem::ApplyMode& m);
     int apply_ahat(const double2* x, double2* y, int precision);
     int apply_ahat_multi(const double2* x, double2* y, int64_t n_rhs);
+    int ensure_farmm();
+    bool reserve_farmm(int64_t n_rhs);
     int apply_ahat64_multi(const double2* x, double2* y, int64_t n_rhs);
     int ensure_fardf();
     double df_extent(bool with_transducer) const;

@@ -223,13 +223,31 @@ bool build_quadrature(Quadrature& q, int n_gauss) {
 
 // ---------------------------------------------------------------- geometry
 
-static inline uint32_t spread10(uint32_t v) {
-    v &= 1023u;
-    v = (v | (v << 16)) & 0x030000FFu;
-    v = (v | (v << 8)) & 0x0300F00Fu;
-    v = (v | (v << 4)) & 0x030C30C3u;
-    v = (v | (v << 2)) & 0x09249249u;
-    return v;
+// Triangles order[b, e) cut into tiles of TT that are as compact as their
+// count allows: halved (by whole tiles) across the longest extent of their
+// centroids until one tile is left.  (Consecutive runs of a Morton curve can
+// jump across a surface: on a 12,184-triangle kidney scene the largest of 382
+// tiles was as big as the kidney, and 19 % of the pairs of tiles came closer
+// than 1.05 times the sum of their radii; now 6.6 %.)
+static void bisect(const std::vector<double>& cen, std::vector<int>& order, int64_t b, int64_t e) {
+    const int64_t tiles = (e - b + TT - 1) / TT;
+    if (tiles <= 1) return;
+    double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
+    for (int64_t i = b; i < e; i++)
+        for (int k = 0; k < 3; k++) {
+            lo[k] = std::min(lo[k], cen[3 * (int64_t)order[i] + k]);
+            hi[k] = std::max(hi[k], cen[3 * (int64_t)order[i] + k]);
+        }
+    int ax = 0;
+    for (int k = 1; k < 3; k++)
+        if (hi[k] - lo[k] > hi[ax] - lo[ax]) ax = k;
+    const int64_t m = b + tiles / 2 * TT;
+    std::nth_element(order.begin() + b, order.begin() + m, order.begin() + e, [&](int p, int q) {
+        const double x = cen[3 * (int64_t)p + ax], y = cen[3 * (int64_t)q + ax];
+        return x < y || (x == y && p < q);
+    });
+    bisect(cen, order, b, m);
+    bisect(cen, order, m, e);
 }
 
 std::string build_geometry(const std::vector<HostDomain>& doms, const Quadrature& q, Geometry& g) {
@@ -299,19 +317,9 @@ std::string build_geometry(const std::vector<HostDomain>& doms, const Quadrature
         double diag = std::sqrt((hi[0] - lo[0]) * (hi[0] - lo[0]) + (hi[1] - lo[1]) * (hi[1] - lo[1]) +
                                 (hi[2] - lo[2]) * (hi[2] - lo[2]));
         g.max_diameter = std::max(g.max_diameter, diag);
-        double ext = std::max({hi[0] - lo[0], hi[1] - lo[1], hi[2] - lo[2], 1e-300});
-        std::vector<uint32_t> code(D.nt);
-        for (int64_t t = 0; t < D.nt; t++) {
-            uint32_t c[3];
-            for (int k = 0; k < 3; k++) {
-                double u = (cen[3 * t + k] - lo[k]) / ext;
-                c[k] = (uint32_t)std::min(1023.0, std::max(0.0, u * 1023.0));
-            }
-            code[t] = spread10(c[0]) | (spread10(c[1]) << 1) | (spread10(c[2]) << 2);
-        }
         order[d].resize(D.nt);
         std::iota(order[d].begin(), order[d].end(), 0);
-        std::stable_sort(order[d].begin(), order[d].end(), [&](int a, int b) { return code[a] < code[b]; });
+        bisect(cen, order[d], 0, D.nt);
         g.dom_tile_begin.push_back(tiles);
         tiles += (int)((D.nt + TT - 1) / TT);
         g.dom_tile_end.push_back(tiles);

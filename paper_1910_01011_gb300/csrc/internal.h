@@ -1,7 +1,7 @@
 // internal.h -- data layout shared by the library's translation units.
 //
-// Triangles are stored tile-ordered: each domain's triangles are sorted
-// along a Morton curve of their centroids and cut into tiles of TT
+// Triangles are stored tile-ordered: each domain's triangles are halved
+// recursively across the longest extent of their centroids into tiles of TT
 // triangles (the last tile of a domain is padded).  A tile carries its
 // centre in FP64; every point and plane offset of the tile is stored
 // relative to that centre, so FP32 differences between points of two tiles
@@ -157,7 +157,42 @@ struct FarArgs32M {
     float* partial;         // [R][n_chunks][2][NCOMP][n_pts]
     int* err;
     const int4* work;       // [n_work] (target tile offset, chunk, slot, group), heaviest first
+    const int* near_ptr;    // null: source tiles [chunk * chunk_tiles, ...); else the target tile's list
+    const int* near_idx;    // near_idx[near_ptr[t] .. near_ptr[t + 1]) (at most CHUNK_MAX), `chunk` being the output row only
 };
+
+// Several right-hand sides on the tensor cores (k_farmm.cu): the pairs of
+// tiles that are not close (centres at least FARMM_SEP times the sum of their
+// radii apart); the close ones go to far32m_kernel (FarArgs32M::near_ptr).
+constexpr double FARMM_SEP = 1.05;
+constexpr int FARMM_CHUNK = 48;  // source tiles per work item
+constexpr int FARMM_MIN_TILES = 96;  // below, close pairs are most of the work; measured, 4 vectors: 122 tiles 4.24 -> 2.80 ms,
+                                     // 320 tiles 21.2 -> 10.8 ms
+struct FarMmPlan {
+    const float4 *pg, *tg;
+    const double4* tc;
+    const int* tdom;
+    const int2* dom_tiles;
+    const double2* kdom;
+    double2 k0;
+    const float4 *pd, *tcurl;  // [R][n_pts], [R][2 n_slots] (gather)
+    const float* frame;        // [n_tiles][9]
+    const uint32_t* near;      // [n_tiles][near_words]
+    int near_words;
+    const float4* geo;         // [n_pts] source geometry with |g|^2
+    float rho;
+    int n_tiles, chunk_tiles, R;
+    int64_t n_pts, n_slots, rstride, n_work;
+    float* partial;
+    int* err;
+    const int4* work;          // [n_work] (block of 128 points, chunk, slot, group)
+    void* buf;                 // farmm_bytes
+};
+cudaError_t launch_farmm(const FarMmPlan& P, cudaStream_t s);
+size_t farmm_bytes(int n_tiles, int64_t R);
+void farmm_chunking(int n_tiles, int64_t n_pts, int64_t R, int* n_chunks, int* chunk_tiles);
+int farmm_blocks(int64_t n_pts);
+int farmm_groups(int64_t R);
 
 struct FarArgs64 {
     const double4* pg;      // (dx, dy, dz, w)

@@ -502,6 +502,8 @@ static_assert(STAGE_M_BYTES == 3584 + MRG * 4096, "multi stage layout");
 struct FarSmemM {
     StageM st[NSTAGE_M];
     float4 tab[2 * CHUNK_MAX];
+    int src[CHUNK_MAX];  // source tiles of the item
+    int nsrc;
     uint64_t full[NSTAGE_M];
     int cnt[NSTAGE_M];
 };
@@ -614,13 +616,22 @@ __device__ __forceinline__ void far32m_item(const FarArgs32M& A, int tx, int cy,
     const int tt = A.tgt_begin + tx;
     const int mydom = A.tdom[tt];
     const int2 dr = A.dom_tiles[mydom];
-    int sb = A.src_begin + cy * A.chunk_tiles;
-    int se = min(sb + A.chunk_tiles, A.src_end);
-    if (slot) {
-        sb = max(sb, dr.x);
-        se = min(se, dr.y);
+    // the item's source tiles (slot 1: those of the target's domain)
+    if (tid < 32) {
+        const int sb = A.near_ptr ? A.near_ptr[tt] : A.src_begin + cy * A.chunk_tiles;
+        const int se = A.near_ptr ? min(A.near_ptr[tt + 1], sb + CHUNK_MAX) : min(sb + A.chunk_tiles, A.src_end);
+        int n = 0;
+        for (int b = sb; b < se; b += 32) {
+            const int s = b + lane < se ? (A.near_ptr ? A.near_idx[b + lane] : b + lane) : -1;
+            const bool in = s >= 0 && (!slot || (s >= dr.x && s < dr.y));
+            const uint32_t m = __ballot_sync(0xffffffffu, in);
+            if (in) sm.src[n + __popc(m & ((1u << lane) - 1))] = s;
+            n += __popc(m);
+        }
+        if (lane == 0) sm.nsrc = n;
     }
-    const int nsrc = max(0, se - sb);
+    __syncthreads();
+    const int nsrc = sm.nsrc;
     const int r0 = grp * MRG;
     const int nq = min(MRG, A.R - r0);
 
@@ -637,7 +648,7 @@ __device__ __forceinline__ void far32m_item(const FarArgs32M& A, int tx, int cy,
 
     // tile-pair table: 2D, R_c^2, R_c and the FP64-reduced phase
     for (int i = tid; i < nsrc; i += TP) {
-        const double4 cs = A.tc[sb + i];
+        const double4 cs = A.tc[sm.src[i]];
         const double Dx = ct.x - cs.x, Dy = ct.y - cs.y, Dz = ct.z - cs.z;
         const double R = sqrt(Dx * Dx + Dy * Dy + Dz * Dz);
         sm.tab[2 * i] = make_float4((float)(2 * Dx), (float)(2 * Dy), (float)(2 * Dz), (float)(R * R));
@@ -653,7 +664,7 @@ __device__ __forceinline__ void far32m_item(const FarArgs32M& A, int tx, int cy,
     __syncthreads();
 
     auto issue = [&](int i, int st) {
-        const int s = sb + i;
+        const int s = sm.src[i];
         StageM& S = sm.st[st];
         mbar_arrive_expect_tx(&sm.full[st], STAGE_M_BYTES);
         bulk_g2s(S.pg, A.pgp + (int64_t)s * TP, TP * 16, &sm.full[st]);
@@ -680,7 +691,7 @@ __device__ __forceinline__ void far32m_item(const FarArgs32M& A, int tx, int cy,
     for (int i = 0; i < nsrc; i++) {
         const int st = i % NSTAGE_M;
         mbar_wait_bounded(&sm.full[st], (uint32_t)((i / NSTAGE_M) & 1), A.err);
-        const int s = sb + i;
+        const int s = sm.src[i];
         const int ntri = A.tntri[s];
         const int skip = (s == tt) ? mt : -1;
         const float4 c0 = sm.tab[2 * i], c1 = sm.tab[2 * i + 1];

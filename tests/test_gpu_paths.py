@@ -102,3 +102,51 @@ def test_fp64_assembled_digits(api, name, R):
             assert np.isnan(Y[r].real).all()
         else:
             assert rel(Y[r], A @ X[r]) < 1e-12
+
+
+@pytest.mark.parametrize("name,R", [("ribs", 2), ("kidney", 5), ("lossy", 3), ("phase", 8)])
+def test_tensor_core_far_field(api, name, R):
+    """Several right-hand sides on meshes large enough for the tensor-core far
+    field (at least 96 tiles; target blocks of 128 points straddle tiles and
+    domains, a short last group and block, attenuating interior and exterior,
+    phases over hundreds of radians), against the FP64 path at the FP32 bar;
+    vectors of very different sizes and a zero one."""
+    s = {"ribs": lambda: scenes.rib_scene(h=9e-3, freq=0.03e6), "kidney": lambda: scenes.kidney_scene(h=7.5e-3, freq=0.04e6),
+         "lossy": lambda: scenes.sphere_scene(4, k0=6.0 + 0.4j, k1=6.5 + 1.5j),
+         "phase": lambda: scenes.sphere_scene(4, k0=150.0, k1=160.0 + 0.5j)}[name]()
+    c = api.Context.from_scene(s)
+    X = np.stack([scenes.smooth_trace_vector(s, r) * 10.0 ** (6 * r - 9) for r in range(R)])
+    if R == 5:
+        X[3] = 0.0
+    Y = c.apply(X, precision=api.FP32)
+    Z = c.apply(X, precision=api.FP64)
+    for r in range(R):
+        if R == 5 and r == 3:
+            assert not Y[r].any()
+        else:
+            assert rel(Y[r], Z[r]) < 2e-5, r
+    c.close()
+
+
+def test_tensor_core_far_field_gives_its_memory_back(api):
+    """Under a budget that does not hold the operands next to the rest, the
+    product takes the FP32 kernel for all pairs, with the same result to FP32
+    accuracy; operands already held go when another allocation needs the room."""
+    s = scenes.sphere_scene(4)
+    X = np.stack([scenes.smooth_trace_vector(s, r) for r in range(16)])
+    c = api.Context.from_scene(s)
+    ref = c.apply(X, precision=api.FP32)
+    used = c.memory()[0]
+    c.close()
+    c = api.Context.from_scene(s, hbm_budget_bytes=used - (1 << 22))
+    y = c.apply(X, precision=api.FP32)
+    assert c.memory()[0] <= used - (1 << 22)
+    assert rel(y, ref) < 1e-5
+    c.close()
+    c = api.Context.from_scene(s, hbm_budget_bytes=used + (16 << 20))  # (host vectors are staged)
+    y = c.apply(X, precision=api.FP32)
+    assert np.array_equal(y, ref)
+    c.apply(X[:8], precision=api.FP64)  # its vectors and partials do not fit beside the operands
+    y = c.apply(X[:3], precision=api.FP32)
+    assert rel(y, ref[:3]) < 1e-5
+    c.close()
