@@ -4,7 +4,7 @@
 // sides in bem_solve.cu).  Sums and products are error-free transformations
 // (Knuth's TwoSum; Dekker's product through a fused multiply-add) written with
 // explicit round-to-nearest intrinsics, so the compiler fuses nothing.
-//  * dsqrt_rinv: FP32 square root and reciprocal, one Newton step each.
+//  * dsqrt_rinv: FP32 seeds, one Newton step each.
 //  * dsincos: Cody and Waite's additive reduction of the phase by multiples of
 //    pi/64 held in four FP32 parts (the first with 3 significant bits, so its
 //    product with the multiple n is exact for n < 2^21, phases below ~100,000
@@ -70,10 +70,17 @@ __device__ __forceinline__ dfl ld_h(const float4& h, const float4& l, int c) {
     return c == 0 ? dfl{h.x, l.x} : c == 1 ? dfl{h.y, l.y} : c == 2 ? dfl{h.z, l.z} : dfl{h.w, l.w};
 }
 
-// r = sqrt(R) and 1/r for R > 0 (double-float): FP32 seeds, one Newton step each
+// r = sqrt(R) and 1/r for R > 0 (double-float): FP32 seeds, one Newton step
+// each.  The seeds come from one reciprocal square root approximation, a
+// Newton step on it and one on the square root (good to an ulp), eight
+// instructions without a branch; correctly rounded square root and reciprocal
+// are about twenty with a slow path, and the double-float steps do not need them.
 __device__ __forceinline__ void dsqrt_rinv(dfl R, dfl& r, dfl& ri) {
-    const float s = __fsqrt_rn(R.h);
-    const float y = __frcp_rn(s);
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(R.h));
+    y = __fmaf_rn(y, __fmaf_rn(-__fmul_rn(0.5f, __fmul_rn(R.h, y)), y, 0.5f), y);
+    const float s0 = __fmul_rn(R.h, y);
+    const float s = __fmaf_rn(__fmul_rn(0.5f, y), __fmaf_rn(-s0, s0, R.h), s0);
     const dfl s2 = two_prod(s, s);
     const float d = __fadd_rn(__fsub_rn(R.h, s2.h), __fsub_rn(R.l, s2.l));  // R - s^2 (first difference exact)
     r = fast_two_sum(s, __fmul_rn(__fmul_rn(d, y), 0.5f));
@@ -85,7 +92,7 @@ __device__ __forceinline__ void dsqrt_rinv(dfl R, dfl& r, dfl& ri) {
 // sin and cos of th >= 0 (double-float) by reduction to |d| <= pi/128
 __device__ __forceinline__ void dsincos(dfl th, const DfConsts& A, const float4* __restrict__ tab, dfl& sn, dfl& cs) {
     const float nf = rintf(__fmul_rn(th.h, A.inv_pi64));
-    const float r1 = __fsub_rn(th.h, __fmul_rn(nf, A.pi64[0]));  // exact (n (pi/64)_1 is exact and near th)
+    const float r1 = __fmaf_rn(-nf, A.pi64[0], th.h);  // exact (n (pi/64)_1 is exact and near th)
     const dfl p2 = two_prod(nf, A.pi64[1]);                       // n (pi/64)_2 and n (pi/64)_3 exactly
     const dfl p3 = two_prod(nf, A.pi64[2]);
     const dfl s = two_sum(r1, -p2.h);

@@ -176,19 +176,21 @@ __device__ __forceinline__ dfl ddot3(const dfl (&a)[3], const dfl (&b)[3]) {
 }
 
 // G r^0 = e^{ikr} / r and F = G (ik - 1/r) / r at the difference e (without the 1 / (4 pi))
-template <bool ATTEN>
-__device__ __forceinline__ void near_gf(const dfl (&e)[3], dfl kr, dfl ki, const NearArgs& A,
+// (atten: uniform over the CTA; one body for both, which the instruction cache holds)
+__device__ __forceinline__ void near_gf(const dfl (&e)[3], dfl kr, dfl ki, bool atten, const NearArgs& A,
                                         const float4* __restrict__ tab, const float2* __restrict__ etab, dfl& Gr, dfl& Gi,
                                         dfl& Fr, dfl& Fi) {
     dfl r, ri;
     dsqrt_rinv(dadd(dadd(dsqr(e[0]), dsqr(e[1])), dsqr(e[2])), r, ri);
     dfl sn, cs;
     dsincos(dmul(kr, r), A.c, tab, sn, cs);
-    dfl a = ri;
-    if (ATTEN) a = dmul(a, dexp_neg(dmul(ki, r), A.c, etab));
+    dfl a = ri, u = dneg(ri);  // Re(ik - 1/r)
+    if (atten) {
+        a = dmul(a, dexp_neg(dmul(ki, r), A.c, etab));
+        u = dsub(u, ki);
+    }
     Gr = dmul(a, cs);
     Gi = dmul(a, sn);
-    const dfl u = ATTEN ? dsub(dneg(ki), ri) : dneg(ri);  // Re(ik - 1/r)
     Fr = dmul(dsub(dmul(Gr, u), dmul(Gi, kr)), ri);
     Fi = dmul(dadd(dmul(Gr, kr), dmul(Gi, u)), ri);
 }
@@ -204,9 +206,8 @@ __device__ __forceinline__ void bary(dfl s1, dfl s2, float c, const int (&pa)[3]
     permute3(v, pa, out);
 }
 
-template <bool ATTEN>
 __device__ __forceinline__ void near_group(const NearArgs& A, const NearGeomDF& G, int rel, int idx, const int (&pa)[3],
-                                           const int (&pb)[3], dfl kr, dfl ki, const float4* __restrict__ tab,
+                                           const int (&pb)[3], dfl kr, dfl ki, bool atten, const float4* __restrict__ tab,
                                            const float2* __restrict__ etab, const float2 (*__restrict__ inner)[4],
                                            float2* __restrict__ row) {
     const float4* T = A.grp[rel] + 4 * (int64_t)idx;
@@ -236,7 +237,7 @@ __device__ __forceinline__ void near_group(const NearArgs& A, const NearGeomDF& 
 #pragma unroll
         for (int c = 0; c < 3; c++) e[c] = dadd(e0[c], dmul(g, dv[c]));
         dfl Gr, Gi, Fr, Fi;
-        near_gf<ATTEN>(e, kr, ki, A, tab, etab, Gr, Gi, Fr, Fi);
+        near_gf(e, kr, ki, atten, A, tab, etab, Gr, Gi, Fr, Fi);
         dmac(g0[0], Gr, c0, 1.0f);
         dmac(g0[1], Gi, c0, 1.0f);
         dmac(g1[0], Gr, c1, 1.0f);
@@ -289,8 +290,7 @@ __device__ __forceinline__ void near_group(const NearArgs& A, const NearGeomDF& 
 }
 
 // Minus the regular rule the far-field kernel applied: point qa of the target against the source's points.
-template <bool ATTEN>
-__device__ __forceinline__ void near_regular(const NearArgs& A, const NearGeomDF& G, int qa, dfl kr, dfl ki,
+__device__ __forceinline__ void near_regular(const NearArgs& A, const NearGeomDF& G, int qa, dfl kr, dfl ki, bool atten,
                                              const float4* __restrict__ tab, const float2* __restrict__ etab,
                                              float2* __restrict__ row) {
     const dfl l1 = {A.rule_h[3 * qa], A.rule_l[3 * qa]}, l2 = {A.rule_h[3 * qa + 1], A.rule_l[3 * qa + 1]};
@@ -310,7 +310,7 @@ __device__ __forceinline__ void near_regular(const NearArgs& A, const NearGeomDF
         for (int c = 0; c < 3; c++)
             e[c] = dsub(x[c], dadd(dadd(G.v[9][c], dmul(m1, G.v[10][c])), dmul(m2, G.v[11][c])));
         dfl Gr, Gi, Fr, Fi;
-        near_gf<ATTEN>(e, kr, ki, A, tab, etab, Gr, Gi, Fr, Fi);
+        near_gf(e, kr, ki, atten, A, tab, etab, Gr, Gi, Fr, Fi);
         const dfl wt = dmul(w, wb), dy = dneg(ddot3(e, G.v[13])), dx = ddot3(e, G.v[12]);
         const dfl ly[3] = {dsub(dsub(dfl{1.0f, 0.0f}, m1), m2), m1, m2};
         const dfl f[3][2] = {{dmul(Gr, wt), dmul(Gi, wt)},
@@ -404,11 +404,9 @@ __global__ void __launch_bounds__(NEAR_THREADS, 4) near_build_df_kernel(NearArgs
         const int idx = b + tid;
         float2* row = rows[tid];
         if (idx < n) {
-            if (atten) near_group<true>(A, G, rel, idx, pa, pb, kr, ki, tab, etab, inner, row);
-            else near_group<false>(A, G, rel, idx, pa, pb, kr, ki, tab, etab, inner, row);
+            near_group(A, G, rel, idx, pa, pb, kr, ki, atten, tab, etab, inner, row);
         } else if (idx >= reg0 && idx < n_all) {
-            if (atten) near_regular<true>(A, G, idx - reg0, kr, ki, tab, etab, row);
-            else near_regular<false>(A, G, idx - reg0, kr, ki, tab, etab, row);
+            near_regular(A, G, idx - reg0, kr, ki, atten, tab, etab, row);
         }
         __syncwarp();
         if (lane < NACC) {
