@@ -854,6 +854,249 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(NT, 1024 / NT) cocg
     red.sync();  // no CTA may leave while another still reads its shared memory
 }
 
+// ---- loose solves of domains that fit a CTA's shared memory
+//
+// The kernels above keep the five vectors of a system in memory: an iteration
+// moves ~300 bytes per vertex through L2 (each product gathers p eight times),
+// and 384 systems of 1,370 vertices need ~19 us for it.  Here a CTA of LS_NT
+// threads owns NS systems of one domain (consecutive systems: the shifts of a
+// right-hand side) with up to NR rows per thread: r and q in registers, p, x
+// and the inverse diagonal in shared memory, so that an iteration loads only
+// the matrix (12 bytes per entry, coalesced, once for the NS systems).
+constexpr int LS_NT = 512, LS_MAX_ROWS = 8 * LS_NT;
+
+template <int NS>
+struct LocalSum32 {  // sums over the CTA, two barriers each; the two kinds alternate, so no third is needed
+    float (*sh)[3 * NS];  // [LS_NT / 32]
+    float* tot;
+    template <int NV>
+    __device__ __forceinline__ void sum(float (&v)[NV]) {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+        for (int k = 0; k < NV; k++) {
+            float t = v[k];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (lane == 0) sh[warp][k] = t;
+        }
+        __syncthreads();
+        if (warp < NV) {
+            float t = lane < LS_NT / 32 ? sh[lane][warp] : 0.f;
+#pragma unroll
+            for (int o = LS_NT / 64; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (lane == 0) tot[warp] = t;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < NV; k++) v[k] = tot[k];
+    }
+};
+
+template <int NR, int NS>
+__global__ void __launch_bounds__(LS_NT, NR <= 4 ? 2 : 1) cocg_local32_kernel(CocgArgs32 a, int n_sys, int W) {
+    extern __shared__ float4 ls_raw[];
+    __shared__ float sh2[LS_NT / 32][3 * NS], sh3[LS_NT / 32][3 * NS], tot2[2 * NS], tot3[3 * NS];
+    LocalSum32<NS> red2{sh2, tot2}, red3{sh3, tot3};
+    const int j = blockIdx.x % a.n_dom, s0 = blockIdx.x / a.n_dom * NS, t = threadIdx.x;
+    const int64_t n = a.n, v0 = a.dom_v0[j];
+    const int m = (int)(a.dom_v0[j + 1] - v0);
+    float2* ps = (float2*)ls_raw;  // [m][NS]
+    float2* xs = ps + (int64_t)m * NS;
+    float2* di = xs + (int64_t)m * NS;
+    const int32_t* eci = a.eci + v0;
+    const float *em = a.em + v0, *es = a.es + v0;
+    float2 be[NS], rho[NS];
+    float lim[NS];
+    bool done[NS], ok[NS];
+    int its[NS];
+    float2 r[NR][NS], q[NR][NS];
+    float w3[3 * NS];
+#pragma unroll
+    for (int k = 0; k < 3 * NS; k++) w3[k] = 0.f;
+#pragma unroll
+    for (int c = 0; c < NS; c++) {
+        const int s = min(s0 + c, n_sys - 1);
+        const double2 be64 = a.beta[(int64_t)s * a.n_dom + j];
+        be[c] = make_float2((float)be64.x, (float)be64.y);
+        const double2* b = a.b + (int64_t)s * n + v0;
+#pragma unroll
+        for (int u = 0; u < NR; u++) {
+            const int i = t + u * LS_NT;
+            r[u][c] = make_float2(0.f, 0.f);
+            if (i < m) {
+                const double2 b64 = b[i];
+                const float2 bi = make_float2((float)b64.x, (float)b64.y);
+                const float dm = a.dm[v0 + i], ds = a.ds[v0 + i];
+                const float2 dv = fcdiv(make_float2(1.f, 0.f), make_float2(dm - be[c].x * ds, -be[c].y * ds));
+                const float2 zi = fcmul(dv, bi);
+                di[i * NS + c] = dv;
+                xs[i * NS + c] = make_float2(0.f, 0.f);
+                ps[i * NS + c] = zi;
+                r[u][c] = bi;
+                const float2 rz = fcmul(bi, zi);
+                w3[3 * c] += rz.x;
+                w3[3 * c + 1] += rz.y;
+                w3[3 * c + 2] += bi.x * bi.x + bi.y * bi.y;
+            }
+        }
+    }
+    red3.sum(w3);  // its barriers also publish the initial p
+    bool all = true;
+#pragma unroll
+    for (int c = 0; c < NS; c++) {
+        rho[c] = make_float2(w3[3 * c], w3[3 * c + 1]);
+        lim[c] = a.tol2 * w3[3 * c + 2];
+        ok[c] = !(w3[3 * c + 2] > 0);  // zero right-hand side: x = 0 is exact
+        done[c] = ok[c] || s0 + c >= n_sys;
+        its[c] = 0;
+        all = all && done[c];
+    }
+    for (int it = 0; it < a.max_iter && !all; it++) {
+        float v2[2 * NS];
+#pragma unroll
+        for (int k = 0; k < 2 * NS; k++) v2[k] = 0.f;
+#pragma unroll
+        for (int u = 0; u < NR; u++)
+#pragma unroll
+            for (int c = 0; c < NS; c++) q[u][c] = make_float2(0.f, 0.f);
+#pragma unroll 1
+        for (int k0 = 0; k0 < W; k0 += 4) {
+#pragma unroll
+            for (int u = 0; u < NR; u++) {
+                const int i = t + u * LS_NT;
+                if (i < m) {
+#pragma unroll
+                    for (int k = 0; k < 4; k++) {
+                        const int e = (k0 + k) * (int)n + i;
+                        const int jj = eci[e] - (int)v0;
+                        const float fm = em[e], fs = es[e];
+                        float2 pj[NS];
+                        if constexpr (NS == 2) {
+                            const float4 p4 = *(const float4*)(ps + 2 * jj);
+                            pj[0] = make_float2(p4.x, p4.y);
+                            pj[1] = make_float2(p4.z, p4.w);
+                        } else {
+                            pj[0] = ps[jj];
+                        }
+#pragma unroll
+                        for (int c = 0; c < NS; c++) {
+                            const float mr = fm - be[c].x * fs, mi = -be[c].y * fs;
+                            q[u][c].x += mr * pj[c].x - mi * pj[c].y;
+                            q[u][c].y += mr * pj[c].y + mi * pj[c].x;
+                        }
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < NR; u++) {
+            const int i = t + u * LS_NT;
+            if (i < m) {
+#pragma unroll
+                for (int c = 0; c < NS; c++) {
+                    const float2 pi = ps[i * NS + c];
+                    v2[2 * c] += pi.x * q[u][c].x - pi.y * q[u][c].y;
+                    v2[2 * c + 1] += pi.x * q[u][c].y + pi.y * q[u][c].x;
+                }
+            }
+        }
+        red2.sum(v2);
+        float2 alpha[NS];
+#pragma unroll
+        for (int c = 0; c < NS; c++) {
+            if (!done[c]) its[c]++;
+            alpha[c] = fcdiv(rho[c], make_float2(v2[2 * c], v2[2 * c + 1]));
+            if (!isfinite(alpha[c].x) || !isfinite(alpha[c].y)) done[c] = true;  // breakdown: keep x
+        }
+#pragma unroll
+        for (int k = 0; k < 3 * NS; k++) w3[k] = 0.f;
+#pragma unroll
+        for (int u = 0; u < NR; u++) {
+            const int i = t + u * LS_NT;
+            if (i < m) {
+#pragma unroll
+                for (int c = 0; c < NS; c++) {
+                    if (done[c]) continue;
+                    const float2 ap = fcmul(alpha[c], ps[i * NS + c]), aq = fcmul(alpha[c], q[u][c]);
+                    float2 xi = xs[i * NS + c];
+                    xi.x += ap.x;
+                    xi.y += ap.y;
+                    xs[i * NS + c] = xi;
+                    r[u][c].x -= aq.x;
+                    r[u][c].y -= aq.y;
+                    q[u][c] = fcmul(di[i * NS + c], r[u][c]);  // z
+                    const float2 rz = fcmul(r[u][c], q[u][c]);
+                    w3[3 * c] += rz.x;
+                    w3[3 * c + 1] += rz.y;
+                    w3[3 * c + 2] += r[u][c].x * r[u][c].x + r[u][c].y * r[u][c].y;
+                }
+            }
+        }
+        red3.sum(w3);
+        all = true;
+        float2 bt[NS];
+#pragma unroll
+        for (int c = 0; c < NS; c++) {
+            if (!done[c]) {
+                if (w3[3 * c + 2] <= lim[c]) ok[c] = done[c] = true;
+                const float2 rn = make_float2(w3[3 * c], w3[3 * c + 1]);
+                bt[c] = fcdiv(rn, rho[c]);
+                if (!isfinite(bt[c].x) || !isfinite(bt[c].y)) done[c] = true;
+                rho[c] = rn;
+            }
+            all = all && done[c];
+        }
+        if (all) break;
+#pragma unroll
+        for (int u = 0; u < NR; u++) {
+            const int i = t + u * LS_NT;
+            if (i < m) {
+#pragma unroll
+                for (int c = 0; c < NS; c++) {
+                    if (done[c]) continue;
+                    const float2 bp = fcmul(bt[c], ps[i * NS + c]);
+                    ps[i * NS + c] = make_float2(q[u][c].x + bp.x, q[u][c].y + bp.y);
+                }
+            }
+        }
+        __syncthreads();  // the new p, read across rows by the next product
+    }
+#pragma unroll
+    for (int c = 0; c < NS; c++) {
+        if (s0 + c >= n_sys) continue;
+        double2* xo = a.xout + (int64_t)(s0 + c) * n + v0;
+        for (int i = t; i < m; i += LS_NT) {  // (this thread's own rows)
+            const float2 xi = xs[i * NS + c];
+            xo[i] = make_double2((double)xi.x, (double)xi.y);
+        }
+        if (t == 0) {
+            atomicAdd(&a.stat[0], (unsigned long long)its[c]);
+            if (!ok[c]) atomicAdd(&a.stat[1], 1ull);
+        }
+    }
+}
+
+template <int NR, int NS>
+static cudaError_t launch_local32(const CocgArgs32& b, int n_sys, int W, int64_t rows, cudaStream_t st) {
+    const int smem = (int)(rows * NS * 3 * sizeof(float2));
+    if (smem > 40 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(cocg_local32_kernel<NR, NS>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+    }
+    const unsigned grid = (unsigned)((n_sys + NS - 1) / NS * b.n_dom);
+    cocg_local32_kernel<NR, NS><<<grid, LS_NT, smem, st>>>(b, n_sys, W);
+    return cudaGetLastError();
+}
+
+template <int NS>
+static cudaError_t launch_local32(const CocgArgs32& b, int n_sys, int W, int64_t rows, cudaStream_t st) {
+    if (rows <= 2 * LS_NT) return launch_local32<2, NS>(b, n_sys, W, rows, st);
+    if (rows <= 3 * LS_NT) return launch_local32<3, NS>(b, n_sys, W, rows, st);
+    if (rows <= 4 * LS_NT) return launch_local32<4, NS>(b, n_sys, W, rows, st);
+    return launch_local32<8, NS>(b, n_sys, W, rows, st);
+}
+
 // ---- the Pade shifts of one right-hand side together: one cluster per (group, domain)
 //
 // The 2 N_pade Pade systems of a right-hand side come in groups of N_pade
@@ -1430,6 +1673,7 @@ static int cocg_solve(bem_ctx* ctx, int n_sys, int shifts = 1) {
     // CTA took 0.95 ms where the clusters took 1.56 ms; with fewer systems than
     // SMs the clusters spread the work wider (the 1,280-triangle sphere's solve
     // took 0.13 s with clusters, 0.16 s with one CTA per system).
+    // (FP32 solves of domains of up to LS_MAX_ROWS vertices have their own rule below.)
     const bool clustered = mode == 3 || mode == 4 ||
                            (mode == 0 && (o->max_dom_nv >= 4096 || (int64_t)n_sys * o->n_dom < 152));
     // the shifts of a group in one cluster (mode 4, or automatic once measured to pay)
@@ -1454,7 +1698,16 @@ static int cocg_solve(bem_ctx* ctx, int n_sys, int shifts = 1) {
         b.x = o->x32; b.r = o->r32; b.z = o->z32; b.p = o->p32; b.q = o->q32;
         b.dom_v0 = o->dom_v0; b.n_dom = o->n_dom; b.tol2 = (float)(o->tol * o->tol); b.max_iter = a.max_iter;
         b.stat = o->stat;
-        if (clustered) {
+        // One CTA per one or two systems wherever a domain fits its shared
+        // memory, two systems once single ones would exceed a CTA per SM.
+        // Three domains of at most 2,048 vertices, 128 / 32 systems: 141 / 59 us
+        // per application (one CTA per system on vectors in memory 189, clusters
+        // 85 us); one domain of 642 vertices, 8 and 2 systems: 24 us on average
+        // (clusters 48 us).
+        if (mode <= 1 && o->max_dom_nv <= LS_MAX_ROWS && o->n * o->ell_w < (1ll << 31)) {
+            if (ctas > 152) CK(launch_local32<2>(b, n_sys, o->ell_w, o->max_dom_nv, ctx->stream));
+            else CK(launch_local32<1>(b, n_sys, o->ell_w, o->max_dom_nv, ctx->stream));
+        } else if (clustered) {
             const unsigned grid = ctas * CL;
             if (o->ell_w == 8) cocg_cluster32_kernel<256, 8><<<grid, 256, 0, ctx->stream>>>(b);
             else if (o->ell_w == 12) cocg_cluster32_kernel<256, 12><<<grid, 256, 0, ctx->stream>>>(b);

@@ -150,3 +150,30 @@ def test_tensor_core_far_field_gives_its_memory_back(api):
     y = c.apply(X[:3], precision=api.FP32)
     assert rel(y, ref[:3]) < 1e-5
     c.close()
+
+
+@pytest.mark.parametrize("level,R,solver", [(3, 1, 0), (3, 12, 0), (4, 1, 0), (4, 5, 0), (4, 12, 0), (4, 12, 1)])
+def test_loose_solves_in_shared_memory(api, level, R, solver):
+    """The preconditioner's FP32 solves with a system's vectors in one CTA's
+    shared memory (642 and 2,562 vertices: two and eight rows per thread, one
+    and two systems per CTA) inside block GMRES (whose FP32 dots see one row
+    tile and several, full and ragged column groups): as many iterations as
+    with the vectors in memory (clusters) up to FP32 rounding, and the same
+    solution to the solve's tolerance."""
+    s = scenes.sphere_scene(level)
+    rng = np.random.default_rng(31)
+    d = rng.standard_normal((12, 3))
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    W = np.exp(2j * np.pi * rng.random((R, 12)))
+    out = []
+    for mode in (solver, 3):
+        c = api.Context.from_scene(s, n_pade=8, osrc_solver=mode, r_eps=0.1)
+        c.set_transducer(3.0 * d, -d, np.full(12, 0.1), 2.6)
+        c.set_excitations(W)
+        rep = c.solve(precision=api.FP32, tol=1e-8, restart=100, operator_mode=1, batch_rhs=R, block_gmres=1)
+        assert rep["converged"], rep
+        out.append((rep["iterations"], np.stack([c.solution(r) for r in range(R)])))
+        c.close()
+    assert abs(out[0][0] - out[1][0]) <= max(3, 0.05 * out[1][0])
+    for r in range(R):
+        assert rel(out[0][1][r], out[1][1][r]) < 1e-6, r
