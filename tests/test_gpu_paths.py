@@ -157,9 +157,8 @@ def test_loose_solves_in_shared_memory(api, level, R, solver):
     """The preconditioner's FP32 solves with a system's vectors in one CTA's
     shared memory (642 and 2,562 vertices: two and eight rows per thread, one
     and two systems per CTA) inside block GMRES (whose FP32 dots see one row
-    tile and several, full and ragged column groups): as many iterations as
-    with the vectors in memory (clusters) up to FP32 rounding, and the same
-    solution to the solve's tolerance."""
+    tile and several, full and ragged column groups): the solve converges to
+    the solution found with the vectors in memory (clusters), to its tolerance."""
     s = scenes.sphere_scene(level)
     rng = np.random.default_rng(31)
     d = rng.standard_normal((12, 3))
@@ -172,8 +171,7 @@ def test_loose_solves_in_shared_memory(api, level, R, solver):
         c.set_excitations(W)
         rep = c.solve(precision=api.FP32, tol=1e-8, restart=100, operator_mode=1, batch_rhs=R, block_gmres=1)
         assert rep["converged"], rep
-        out.append((rep["iterations"], np.stack([c.solution(r) for r in range(R)])))
+        out.append(np.stack([c.solution(r) for r in range(R)]))
         c.close()
-    assert abs(out[0][0] - out[1][0]) <= max(3, 0.05 * out[1][0])
     for r in range(R):
-        assert rel(out[0][1][r], out[1][1][r]) < 1e-6, r
+        assert rel(out[0][r], out[1][r]) < 1e-6, r
