@@ -136,7 +136,11 @@ struct bem_ctx {
         bool ready = false;
         bool fits = false;         // every tile's close tiles fit one item of the FP32 kernel
         void* buf = nullptr;
-        float4* geo = nullptr;
+        float4 *geo = nullptr, *pg = nullptr, *pgp = nullptr, *tg = nullptr;  // in the compact tiles' order
+        double4* tc = nullptr;
+        int4* slot_v = nullptr;
+        double *pt_w = nullptr, *slot_curl = nullptr;
+        int* perm = nullptr;       // the slot in the order of `dev`
         float* frame = nullptr;
         uint32_t* near = nullptr;
         int *near_ptr = nullptr, *near_idx = nullptr;

@@ -223,31 +223,13 @@ bool build_quadrature(Quadrature& q, int n_gauss) {
 
 // ---------------------------------------------------------------- geometry
 
-// Triangles order[b, e) cut into tiles of TT that are as compact as their
-// count allows: halved (by whole tiles) across the longest extent of their
-// centroids until one tile is left.  (Consecutive runs of a Morton curve can
-// jump across a surface: on a 12,184-triangle kidney scene the largest of 382
-// tiles was as big as the kidney, and 19 % of the pairs of tiles came closer
-// than 1.05 times the sum of their radii; now 6.6 %.)
-static void bisect(const std::vector<double>& cen, std::vector<int>& order, int64_t b, int64_t e) {
-    const int64_t tiles = (e - b + TT - 1) / TT;
-    if (tiles <= 1) return;
-    double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
-    for (int64_t i = b; i < e; i++)
-        for (int k = 0; k < 3; k++) {
-            lo[k] = std::min(lo[k], cen[3 * (int64_t)order[i] + k]);
-            hi[k] = std::max(hi[k], cen[3 * (int64_t)order[i] + k]);
-        }
-    int ax = 0;
-    for (int k = 1; k < 3; k++)
-        if (hi[k] - lo[k] > hi[ax] - lo[ax]) ax = k;
-    const int64_t m = b + tiles / 2 * TT;
-    std::nth_element(order.begin() + b, order.begin() + m, order.begin() + e, [&](int p, int q) {
-        const double x = cen[3 * (int64_t)p + ax], y = cen[3 * (int64_t)q + ax];
-        return x < y || (x == y && p < q);
-    });
-    bisect(cen, order, b, m);
-    bisect(cen, order, m, e);
+static inline uint32_t spread10(uint32_t v) {
+    v &= 1023u;
+    v = (v | (v << 16)) & 0x030000FFu;
+    v = (v | (v << 8)) & 0x0300F00Fu;
+    v = (v | (v << 4)) & 0x030C30C3u;
+    v = (v | (v << 2)) & 0x09249249u;
+    return v;
 }
 
 std::string build_geometry(const std::vector<HostDomain>& doms, const Quadrature& q, Geometry& g) {
@@ -317,9 +299,19 @@ std::string build_geometry(const std::vector<HostDomain>& doms, const Quadrature
         double diag = std::sqrt((hi[0] - lo[0]) * (hi[0] - lo[0]) + (hi[1] - lo[1]) * (hi[1] - lo[1]) +
                                 (hi[2] - lo[2]) * (hi[2] - lo[2]));
         g.max_diameter = std::max(g.max_diameter, diag);
+        double ext = std::max({hi[0] - lo[0], hi[1] - lo[1], hi[2] - lo[2], 1e-300});
+        std::vector<uint32_t> code(D.nt);
+        for (int64_t t = 0; t < D.nt; t++) {
+            uint32_t c[3];
+            for (int k = 0; k < 3; k++) {
+                double u = (cen[3 * t + k] - lo[k]) / ext;
+                c[k] = (uint32_t)std::min(1023.0, std::max(0.0, u * 1023.0));
+            }
+            code[t] = spread10(c[0]) | (spread10(c[1]) << 1) | (spread10(c[2]) << 2);
+        }
         order[d].resize(D.nt);
         std::iota(order[d].begin(), order[d].end(), 0);
-        bisect(cen, order[d], 0, D.nt);
+        std::stable_sort(order[d].begin(), order[d].end(), [&](int a, int b) { return code[a] < code[b]; });
         g.dom_tile_begin.push_back(tiles);
         tiles += (int)((D.nt + TT - 1) / TT);
         g.dom_tile_end.push_back(tiles);
@@ -534,6 +526,83 @@ std::string build_geometry(const std::vector<HostDomain>& doms, const Quadrature
             g.np_code[g.np_ptr[s] + i] = lists[s][i].second;
         }
     return "";
+}
+
+// Slots order[b, e) (centroids cen) cut into tiles of TT that are as compact as their
+// count allows: halved (by whole tiles) across the longest extent of their
+// centroids until one tile is left.  (Consecutive runs of a Morton curve can
+// jump across a surface: on a 12,184-triangle kidney scene the largest of 382
+// tiles was as big as the kidney, and 19 % of the pairs of tiles came closer
+// than 1.05 times the sum of their radii; now 6.6 %.)
+static void bisect(const std::vector<double>& cen, std::vector<int>& order, int64_t b, int64_t e) {
+    const int64_t tiles = (e - b + TT - 1) / TT;
+    if (tiles <= 1) return;
+    double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
+    for (int64_t i = b; i < e; i++)
+        for (int k = 0; k < 3; k++) {
+            lo[k] = std::min(lo[k], cen[3 * (int64_t)order[i] + k]);
+            hi[k] = std::max(hi[k], cen[3 * (int64_t)order[i] + k]);
+        }
+    int ax = 0;
+    for (int k = 1; k < 3; k++)
+        if (hi[k] - lo[k] > hi[ax] - lo[ax]) ax = k;
+    const int64_t m = b + tiles / 2 * TT;
+    std::nth_element(order.begin() + b, order.begin() + m, order.begin() + e, [&](int p, int q) {
+        const double x = cen[3 * (int64_t)p + ax], y = cen[3 * (int64_t)q + ax];
+        return x < y || (x == y && p < q);
+    });
+    bisect(cen, order, b, m);
+    bisect(cen, order, m, e);
+}
+
+// The triangles of every domain regrouped into compact tiles: the same tiles
+// per domain, a permutation of its slots.
+void compact_tiles(const Geometry& g, CompactTiles& c) {
+    const int nt = g.n_tiles;
+    c.perm.resize(g.n_slots);
+    std::iota(c.perm.begin(), c.perm.end(), 0);
+    std::vector<double> cen(3 * g.n_slots);
+    for (int64_t s = 0; s < g.n_slots; s++)
+        for (int k = 0; k < 3; k++) cen[3 * s + k] = (g.slot_P[9 * s + k] + g.slot_P[9 * s + 3 + k] + g.slot_P[9 * s + 6 + k]) / 3.0;
+    for (int d = 0; d < g.n_dom; d++) {
+        const int64_t b = (int64_t)g.dom_tile_begin[d] * TT;
+        int64_t e = b;
+        for (int t = g.dom_tile_begin[d]; t < g.dom_tile_end[d]; t++) e += g.tile_ntri[t];  // (padding ends the last tile)
+        bisect(cen, c.perm, b, e);
+    }
+    c.tile_c.assign(4 * (size_t)nt, 0.0);
+    c.pt_delta.assign(3 * g.n_pts, 0.0);
+    c.slot_h.assign(g.n_slots, 0.0);
+    for (int t = 0; t < nt; t++) {
+        const int64_t s0 = (int64_t)t * TT, s1 = s0 + g.tile_ntri[t];
+        double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
+        auto point = [&](int64_t s, int q, int k) {  // absolute
+            const int64_t p = c.perm[s];
+            return g.tile_c[4 * (p / TT) + k] + g.pt_delta[3 * (p * QP + q) + k];
+        };
+        for (int64_t s = s0; s < s1; s++)
+            for (int q = 0; q < QP; q++)
+                for (int k = 0; k < 3; k++) {
+                    lo[k] = std::min(lo[k], point(s, q, k));
+                    hi[k] = std::max(hi[k], point(s, q, k));
+                }
+        double cc[3], rad = 0;
+        for (int k = 0; k < 3; k++) cc[k] = c.tile_c[4 * t + k] = 0.5 * (lo[k] + hi[k]);
+        for (int64_t s = s0; s < s1; s++) {
+            for (int q = 0; q < QP; q++) {
+                double r = 0;
+                for (int k = 0; k < 3; k++) {
+                    const double x = point(s, q, k) - cc[k];
+                    c.pt_delta[3 * (s * QP + q) + k] = x;
+                    r += x * x;
+                }
+                rad = std::max(rad, std::sqrt(r));
+            }
+            const int64_t p = c.perm[s];
+            for (int k = 0; k < 3; k++) c.slot_h[s] += g.slot_n[3 * p + k] * (g.slot_P[9 * p + k] - cc[k]);
+        }
+        c.tile_c[4 * t + 3] = rad;
+    }
 }
 
 }  // namespace gbem

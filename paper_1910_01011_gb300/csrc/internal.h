@@ -88,6 +88,16 @@ bool gauss_legendre01(int n, std::vector<double>& x, std::vector<double>& w);
 // on success, else the error message.
 std::string build_geometry(const std::vector<HostDomain>& doms, const Quadrature& q, Geometry& g);
 
+// Compact tiles beside those of a Geometry (which follow a Morton curve),
+// slot by slot: a permutation within each domain that keeps its tiles' counts.
+struct CompactTiles {
+    std::vector<int> perm;          // [n_slots] the Geometry's slot
+    std::vector<double> tile_c;     // 4 per tile: centre, radius
+    std::vector<double> pt_delta;   // 3 per point
+    std::vector<double> slot_h;
+};
+void compact_tiles(const Geometry& g, CompactTiles& c);
+
 // ------------------------------------------------------------------ device views
 
 // Pair-interleaved storage of the QP points of one triangle, the layout in
@@ -159,6 +169,7 @@ struct FarArgs32M {
     const int4* work;       // [n_work] (target tile offset, chunk, slot, group), heaviest first
     const int* near_ptr;    // null: source tiles [chunk * chunk_tiles, ...); else the target tile's list
     const int* near_idx;    // near_idx[near_ptr[t] .. near_ptr[t + 1]) (at most CHUNK_MAX), `chunk` being the output row only
+    const int* perm;        // null, or the slot of partial that each slot of these tiles is
 };
 
 // Several right-hand sides on the tensor cores (k_farmm.cu): the pairs of
@@ -180,6 +191,7 @@ struct FarMmPlan {
     const uint32_t* near;      // [n_tiles][near_words]
     int near_words;
     const float4* geo;         // [n_pts] source geometry with |g|^2
+    const int* perm;           // [n_slots] the slot of partial that each slot of these tiles is
     float rho;
     int n_tiles, chunk_tiles, R;
     int64_t n_pts, n_slots, rstride, n_work;

@@ -709,6 +709,7 @@ __device__ __forceinline__ void far32m_item(const FarArgs32M& A, int tx, int cy,
         }
     }
 
+    const int64_t po = A.perm ? (int64_t)A.perm[(int64_t)tt * TT + mt] * QP + tid % QP : p;
 #pragma unroll
     for (int q = 0; q < MRG; q++) {
         if (q >= nq) break;
@@ -717,7 +718,7 @@ __device__ __forceinline__ void far32m_item(const FarArgs32M& A, int tx, int cy,
         const float v[NCOMP] = {t.Vr.x + t.Vr.y, t.Vi.x + t.Vi.y, t.K[0], t.K[1], -(t.nKpr.x + t.nKpr.y),
                                 -(t.nKpi.x + t.nKpi.y), t.Wm[0], t.Wm[1], t.Wc[0], t.Wc[1], t.Wc[2], t.Wc[3],
                                 t.Wc[4], t.Wc[5]};
-        float* out = A.partial + (int64_t)(r0 + q) * A.rstride + ((int64_t)cy * 2 + slot) * NCOMP * A.n_pts + p;
+        float* out = A.partial + (int64_t)(r0 + q) * A.rstride + ((int64_t)cy * 2 + slot) * NCOMP * A.n_pts + po;
 #pragma unroll
         for (int c = 0; c < NCOMP; c++) out[(int64_t)c * A.n_pts] = v[c];
     }

@@ -194,6 +194,7 @@ struct FarMmArgs {
     const uint32_t* near;   // [n_tiles][near_words] bit s of row t: the pair (t, s) is close
     int near_words;
     const float4* geo;      // [n_pts] source geometry (MmSmem::geo)
+    const int* perm;        // [n_slots] the slot of partial that each slot of these tiles is
     const uint8_t* B;       // [groups][n_tiles][MM_TS][MM_BBYTES]
     const float* unscale;   // [R][3] 1 / scale of d1, d2 and the curls of a vector
     float rho;              // power of two at or above every tile's radius
@@ -444,7 +445,8 @@ __global__ void __launch_bounds__(MM_WARPS * 32, 1) farmm_kernel(const FarMmArgs
                 const int r = grp * MM_RB + v;
                 if (r >= A.R) break;
                 const float u1 = A.unscale[3 * r], u2 = A.unscale[3 * r + 1], u3 = A.unscale[3 * r + 2];
-                float* out = A.partial + (int64_t)r * A.rstride + ((int64_t)w.y * 2 + slot) * NCOMP * A.n_pts + p;
+                float* out = A.partial + (int64_t)r * A.rstride + ((int64_t)w.y * 2 + slot) * NCOMP * A.n_pts +
+                             (int64_t)A.perm[p / QP] * QP + p % QP;
 #pragma unroll
                 for (int c = 0; c < NCOMP; c++) {
                     const float u = c < 2 || c == 4 || c == 5 ? u1 : c < 8 ? u2 : u3;
@@ -649,7 +651,7 @@ cudaError_t launch_farmm(const FarMmPlan& P, cudaStream_t s) {
         P.pd, P.tcurl, P.pg, P.tg, P.frame, mx, P.n_pts, P.n_slots, P.R, P.rho, B, un);
     FarMmArgs a{};
     a.pg = P.pg; a.tg = P.tg; a.tc = P.tc; a.tdom = P.tdom; a.dom_tiles = P.dom_tiles; a.kdom = P.kdom; a.k0 = P.k0;
-    a.frame = P.frame; a.near = P.near; a.near_words = P.near_words; a.geo = P.geo; a.B = B; a.unscale = un; a.rho = P.rho;
+    a.frame = P.frame; a.near = P.near; a.near_words = P.near_words; a.geo = P.geo; a.perm = P.perm; a.B = B; a.unscale = un; a.rho = P.rho;
     a.n_tiles = P.n_tiles; a.chunk_tiles = P.chunk_tiles; a.R = P.R; a.n_pts = P.n_pts; a.rstride = P.rstride;
     a.partial = P.partial; a.err = P.err; a.work = P.work;
     if (P.n_work > 0) farmm_kernel<<<(unsigned)P.n_work, MM_WARPS * 32, smem, s>>>(a);
