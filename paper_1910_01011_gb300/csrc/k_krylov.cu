@@ -326,9 +326,10 @@ __global__ void kbd_reduce(int KP, int nsplit, const double2* __restrict__ part,
 // the CTA's eight warps take every eighth basis vector, their sums added in
 // warp order at the end: a block of a few thousand unknowns fills the GPU (one
 // thread per entry and all of K left 33 CTAs on 8,200 unknowns).  There, 16
-// columns and K up to 816: FP32 67 us on average before, 20 us now; FP64, bound
+// columns and K up to 816: FP32 67 us on average before, 18 us now (20 without
+// the next coefficients in flight); FP64, bound
 // by the FP64 rate, 5.4 ms before, 1.36 ms now.
-constexpr int KC_WARPS = KV_THREADS / 32, KC_K = 64, KC_RED = 4;  // coefficient rows per stage, columns per reduction
+constexpr int KC_WARPS = KV_THREADS / 32, KC_K = 32, KC_RED = 4;  // coefficient rows per stage, columns per reduction
 
 __global__ void __launch_bounds__(KV_THREADS) kbd_combine(int64_t n, int K, int P, const double2* __restrict__ V,
                                                           const double2* __restrict__ C, double alpha,
@@ -513,7 +514,7 @@ __global__ void __launch_bounds__(KV_THREADS) kbd_dots32(int64_t n, int K, int P
 
 // C32 (may be null): the coefficients in FP32.  Two packed FMAs per column and entry,
 // (re, im) += v_re (c_re, c_im) + v_im (-c_im, c_re).
-__global__ void __launch_bounds__(KV_THREADS) kbd_combine32(int64_t n, int K, int P, const float2* __restrict__ V,
+__global__ void __launch_bounds__(KV_THREADS, 2) kbd_combine32(int64_t n, int K, int P, const float2* __restrict__ V,
                                                             const double2* __restrict__ C,
                                                             const float2* __restrict__ C32, float alpha,
                                                             const float2* base, float beta, float2* out, int c0) {
@@ -525,17 +526,28 @@ __global__ void __launch_bounds__(KV_THREADS) kbd_combine32(int64_t n, int K, in
     f2 s0[KB_COLS], s1[KB_COLS];
 #pragma unroll
     for (int c = 0; c < KB_COLS; c++) s0[c] = s1[c] = make_float2(0.f, 0.f);
+    // the coefficients of the next KC_K vectors are in flight while these are used
+    float2 nx[KC_K * KB_COLS / KV_THREADS];
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int l = 0; l < KC_K * KB_COLS / KV_THREADS; l++) {
+            const int e = l * KV_THREADS + threadIdx.x, k = k0 + e / KB_COLS, c = e % KB_COLS;
+            const int64_t at = (int64_t)k * P + c0 + c;
+            nx[l] = make_float2(0.f, 0.f);
+            if (k < K && c < nc) nx[l] = C32 ? C32[at] : make_float2((float)C[at].x, (float)C[at].y);
+        }
+    };
+    fetch(0);
     for (int k0 = 0; k0 < K; k0 += KC_K) {
         const int kn = min(KC_K, K - k0);
         __syncthreads();
-        for (int e = threadIdx.x; e < kn * KB_COLS; e += KV_THREADS) {
-            const int kk = e / KB_COLS, c = e % KB_COLS;
-            const int64_t at = (int64_t)(k0 + kk) * P + c0 + c;
-            float2 v = make_float2(0.f, 0.f);
-            if (c < nc) v = C32 ? C32[at] : make_float2((float)C[at].x, (float)C[at].y);
-            cs[kk][c] = make_float4(v.x, v.y, -v.y, v.x);
+#pragma unroll
+        for (int l = 0; l < KC_K * KB_COLS / KV_THREADS; l++) {
+            const int e = l * KV_THREADS + threadIdx.x;
+            cs[e / KB_COLS][e % KB_COLS] = make_float4(nx[l].x, nx[l].y, -nx[l].y, nx[l].x);
         }
         __syncthreads();
+        if (k0 + KC_K < K) fetch(k0 + KC_K);
 #pragma unroll 4
         for (int kk = warp; kk < kn; kk += KC_WARPS) {
             const float2* vk = V + (int64_t)(k0 + kk) * n;
