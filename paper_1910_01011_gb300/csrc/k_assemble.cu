@@ -274,10 +274,21 @@ __global__ void __launch_bounds__(TT) assemble64_kernel(AssembleArgs a, const do
     }
 }
 
-// The same assembly with the kernel values and their P1 moments in
-// double-float FP32 arithmetic (df_math.cuh), about 1e-13 relative, and the
-// coefficient epilogue in FP64 from the converted moments: GB300 runs FP64 at
-// ~1/64 of the FP32 rate, and the 36 point pairs of a triangle pair dominate.
+// The same assembly in double-float FP32 arithmetic (df_math.cuh), about
+// 1e-13 relative: GB300 runs FP64 at ~1/64 of the FP32 rate.  CTA = target
+// tile x source chunk, thread = target point; for each source triangle
+//  1. a thread forms the P1 moments of V, K and K' over the source's six points,
+//  2. the six threads of a triangle exchange them through shared memory and
+//     contract them with the test functions,
+//  3. and add the W terms,
+//  4. the sums over the triangles that meet at a vertex of the target tile
+//     (about 22 vertices for 96 corners) go to the matrix with their block
+//     coefficients: ~530 FP64 atomics per source triangle instead of 2,304,
+//     and the only FP64 arithmetic.
+// (One thread per target triangle held 54 accumulators, 255 registers and
+// eight warps on an SM with long dependent chains.)
+// 4,620-triangle rib scene, both wavenumbers: 64.6 ms before, 39.1 ms
+// now (two CTAs with 165 registers; three with 112 spilled: 41.4 ms).
 struct AssembleDf {
     const float4 *pgh, *pgl, *tgh, *tgl, *tch, *tcl;  // split geometry (bem_ctx::ensure_fardf)
     const float4* kdf;        // [n_dom] (Re k hi, lo, Im k hi, lo)
@@ -289,15 +300,76 @@ struct AssembleDf {
     float i4h, i4l;                  // 1 / (4 pi)
 };
 
+struct AsmDfSmem {
+    float4 tab[128];
+    float2 etab[64];
+    float4 sph[TP], spl[TP];  // source points of a tile
+    float4 sgh[TT], sgl[TT];  // its triangles (n, h)
+    dfl wl[TT][QP][3];        // weight x P1 values
+    dfl cs[TT][9];            // curls [3 b + c]
+    int4 sv[TT];
+    dfl ct[9][TT];            // curls of the target triangles [3 i + c]
+    dfl val[18][TP];          // V, K, K' [source vertex][re, im] of each target point
+    dfl mom[3][8][3 * TT];    // [source vertex][V, K, K', W (re, im)][corner 32 i + triangle]
+    int vert[3 * TT];         // the target tile's vertices
+    unsigned char ptr[3 * TT + 1], cor[3 * TT];  // corners of each
+    int id[3 * TT];           // vertex of each corner (-1: padding)
+    int nv;
+};
+
+__device__ __forceinline__ dfl dsplit(double v) {
+    const float h = (float)v;
+    return dfl{h, (float)(v - (double)h)};
+}
+
+// The vertices of the target tile and, for each, its corners in ascending order (one warp).
+__device__ __forceinline__ void tile_vertices(AsmDfSmem& sm, int4 tv) {
+    const int lane = threadIdx.x;
+    sm.id[lane] = tv.x;
+    sm.id[TT + lane] = tv.x < 0 ? -1 : tv.y;
+    sm.id[2 * TT + lane] = tv.x < 0 ? -1 : tv.z;
+    __syncwarp();
+    int nv = 0, nc = 0;
+    for (int i = 0; i < 3; i++) {
+        const int e = i * TT + lane, id = sm.id[e];
+        bool first = id >= 0;
+        for (int k = 0; k < e && first; k++) first = sm.id[k] != id;
+        const unsigned m = __ballot_sync(0xffffffffu, first);
+        if (first) sm.vert[nv + __popc(m & ((1u << lane) - 1))] = id;
+        nv += __popc(m);
+    }
+    __syncwarp();
+    for (int v0 = 0; v0 < nv; v0 += 32) {
+        const int v = v0 + lane, id = v < nv ? sm.vert[v] : -2;
+        int n = 0;
+        for (int k = 0; k < 3 * TT; k++) n += sm.id[k] == id;
+        int at = n;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, at, o);
+            if (lane >= o) at += t;
+        }
+        const int total = __shfl_sync(0xffffffffu, at, 31);
+        at += nc - n;
+        if (v < nv) {
+            sm.ptr[v] = (unsigned char)at;
+            for (int k = 0; k < 3 * TT; k++)
+                if (sm.id[k] == id) sm.cor[at++] = (unsigned char)k;
+        }
+        nc += total;
+    }
+    if (lane == 0) {
+        sm.ptr[nv] = (unsigned char)nc;
+        sm.nv = nv;
+    }
+}
+static_assert(TT == 32, "one warp lists a tile's vertices");
+
 template <bool ATTEN>
-__device__ __forceinline__ void assembledf_body(const AssembleArgs& a, const AssembleDf& d, double2* A64,
-                                                const float4* __restrict__ tab, const float2* __restrict__ etab) {
-    const int tt = blockIdx.x;
-    const int tl = threadIdx.x;
+__device__ __forceinline__ void assembledf_body(const AssembleArgs& a, const AssembleDf& d, double2* A64, AsmDfSmem& sm) {
+    const int tt = blockIdx.x, tid = threadIdx.x, tl = tid / QP, qx = tid % QP;
     const int64_t ts = (int64_t)tt * TT + tl;
-    const int4 tv = a.slot_v[ts];
-    if (tv.x < 0) return;
-    const int dom = tv.w;
+    const bool live = a.slot_v[ts].x >= 0;
+    const int dom = a.slot_v[(int64_t)tt * TT].w;  // (a tile's triangles are of one domain; its first slot is never padding)
     const int2 dr = a.dom_tiles[dom];
     int sb = blockIdx.y * a.chunk_tiles, se = min(sb + a.chunk_tiles, a.n_tiles);
     if (a.slot == 1) {
@@ -311,134 +383,142 @@ __device__ __forceinline__ void assembledf_body(const AssembleArgs& a, const Ass
     const float4 nh = d.tgh[ts], nl = d.tgl[ts];
     const dfl ngx = {nh.x, nl.x}, ngy = {nh.y, nl.y}, ngz = {nh.z, nl.z};
     const float4 cth = d.tch[tt], ctl = d.tcl[tt];
-    const int64_t ra[3] = {a.v_dof1[tv.x], a.v_dof1[tv.y], a.v_dof1[tv.z]};
-    const int64_t rb[3] = {a.v_dof2[tv.x], a.v_dof2[tv.y], a.v_dof2[tv.z]};
-    const dfl i4 = {d.i4h, d.i4l};
+    const float4 xh = d.pgh[ts * QP + qx], xl = d.pgl[ts * QP + qx];
+    const dfl xw = dmul(dfl{xh.w, xl.w}, dfl{d.i4h, d.i4l});
+    if (tid < TT) tile_vertices(sm, a.slot_v[(int64_t)tt * TT + tid]);
+    for (int e = tid; e < 9 * TT; e += TP) sm.ct[e % 9][e / 9] = dsplit(a.slot_curl[(int64_t)tt * TT * 9 + e]);
+    // test function and part (of 18 moments, or re / im of W) of this thread in steps 2 and 3
+    const int i = qx % 3, half = qx / 3, corner = i * TT + tl;
     for (int s = sb; s < se; s++) {
-        const float4 csh = d.tch[s], csl = d.tcl[s];
-        const dfl Dx = dsub(dfl{cth.x, ctl.x}, dfl{csh.x, csl.x});
-        const dfl Dy = dsub(dfl{cth.y, ctl.y}, dfl{csh.y, csl.y});
-        const dfl Dz = dsub(dfl{cth.z, ctl.z}, dfl{csh.z, csl.z});
         const int ntri = a.tntri[s];
+        __syncthreads();  // the last triangle of the tile before is done
+        {
+            const int64_t p = (int64_t)s * TP + tid;
+            const float4 h = d.pgh[p], l = d.pgl[p];
+            sm.sph[tid] = h;
+            sm.spl[tid] = l;
+#pragma unroll
+            for (int b = 0; b < 3; b++) sm.wl[tl][qx][b] = dmul(dfl{h.w, l.w}, dfl{d.lamh[qx][b], d.laml[qx][b]});
+            if (tid < TT) {
+                sm.sgh[tid] = d.tgh[(int64_t)s * TT + tid];
+                sm.sgl[tid] = d.tgl[(int64_t)s * TT + tid];
+                sm.sv[tid] = a.slot_v[(int64_t)s * TT + tid];
+            }
+            for (int e = tid; e < 9 * TT; e += TP) sm.cs[e / 9][e % 9] = dsplit(a.slot_curl[(int64_t)s * TT * 9 + e]);
+        }
+        const float4 csh = d.tch[s], csl = d.tcl[s];
+        const dfl Xx = dadd(dfl{xh.x, xl.x}, dsub(dfl{cth.x, ctl.x}, dfl{csh.x, csl.x}));
+        const dfl Xy = dadd(dfl{xh.y, xl.y}, dsub(dfl{cth.y, ctl.y}, dfl{csh.y, csl.y}));
+        const dfl Xz = dadd(dfl{xh.z, xl.z}, dsub(dfl{cth.z, ctl.z}, dfl{csh.z, csl.z}));
+        __syncthreads();
         for (int sl = 0; sl < ntri; sl++) {
-            const int64_t ss = (int64_t)s * TT + sl;
-            if (ss == ts) continue;
-            const float4 sgh = d.tgh[ss], sgl = d.tgl[ss];
-            const dfl snx = {sgh.x, sgl.x}, sny = {sgh.y, sgl.y}, snz = {sgh.z, sgl.z}, sh = {sgh.w, sgl.w};
-            dfl V[3][3][2], K[3][3][2], Kp[3][3][2];
+            const float4 sgh = sm.sgh[sl], sgl = sm.sgl[sl];
+            const dfl snx = {sgh.x, sgl.x}, sny = {sgh.y, sgl.y}, snz = {sgh.z, sgl.z};
+            // 1. moments over the source points
+            dfl h[18];
 #pragma unroll
-            for (int i = 0; i < 3; i++)
-#pragma unroll
-                for (int b = 0; b < 3; b++)
-#pragma unroll
-                    for (int c = 0; c < 2; c++) V[i][b][c] = K[i][b][c] = Kp[i][b][c] = dfl{0.0f, 0.0f};
-            for (int qx = 0; qx < QP; qx++) {
-                const float4 xh = d.pgh[ts * QP + qx], xl = d.pgl[ts * QP + qx];
-                const dfl Xx = dadd(dfl{xh.x, xl.x}, Dx), Xy = dadd(dfl{xh.y, xl.y}, Dy), Xz = dadd(dfl{xh.z, xl.z}, Dz);
-                const dfl fK = dsub(sh, dadd(dadd(dmul(snx, Xx), dmul(sny, Xy)), dmul(snz, Xz)));
-                dfl hV[3][2], hK[3][2], hKp[3][2];
-#pragma unroll
-                for (int b = 0; b < 3; b++)
-#pragma unroll
-                    for (int c = 0; c < 2; c++) hV[b][c] = hK[b][c] = hKp[b][c] = dfl{0.0f, 0.0f};
+            for (int k = 0; k < 18; k++) h[k] = dfl{0.0f, 0.0f};
+            if (live && (int64_t)s * TT + sl != ts) {  // (identical triangles: the near-field correction alone)
+#pragma unroll 1
                 for (int qy = 0; qy < QP; qy++) {
-                    const float4 yh = d.pgh[ss * QP + qy], yl = d.pgl[ss * QP + qy];
+                    const float4 yh = sm.sph[sl * QP + qy], yl = sm.spl[sl * QP + qy];
                     const dfl ex = dsub(Xx, dfl{yh.x, yl.x}), ey = dsub(Xy, dfl{yh.y, yl.y}), ez = dsub(Xz, dfl{yh.z, yl.z});
                     dfl r, ri;
                     dsqrt_rinv(dadd(dadd(dsqr(ex), dsqr(ey)), dsqr(ez)), r, ri);
                     dfl sn, cs;
-                    dsincos(dmul(kr, r), d.c, tab, sn, cs);
-                    const dfl am = ATTEN ? dmul(dexp_neg(dmul(ki, r), d.c, etab), ri) : ri;
+                    dsincos(dmul(kr, r), d.c, sm.tab, sn, cs);
+                    const dfl am = ATTEN ? dmul(dexp_neg(dmul(ki, r), d.c, sm.etab), ri) : ri;
                     const dfl Gr = dmul(am, cs), Gi = dmul(am, sn);
-                    const dfl u = dsub(dneg(ki), ri);
+                    const dfl u = ATTEN ? dsub(dneg(ki), ri) : dneg(ri);
                     const dfl Fr = dmul(dsub(dmul(Gr, u), dmul(Gi, kr)), ri);
                     const dfl Fi = dmul(dadd(dmul(Gr, kr), dmul(Gi, u)), ri);
                     const dfl ndot = dadd(dadd(dmul(ngx, ex), dmul(ngy, ey)), dmul(ngz, ez));
                     const dfl nFr = dmul(ndot, Fr), nFi = dmul(ndot, Fi);
-                    const dfl yw = {yh.w, yl.w};
 #pragma unroll
                     for (int b = 0; b < 3; b++) {
-                        const dfl wl = dmul(yw, dfl{d.lamh[qy][b], d.laml[qy][b]});
-                        dmac(hV[b][0], wl, Gr, 1.0f);
-                        dmac(hV[b][1], wl, Gi, 1.0f);
-                        dmac(hK[b][0], wl, Fr, 1.0f);
-                        dmac(hK[b][1], wl, Fi, 1.0f);
-                        dmac(hKp[b][0], wl, nFr, 1.0f);
-                        dmac(hKp[b][1], wl, nFi, 1.0f);
+                        const dfl wl = sm.wl[sl][qy][b];
+                        dmac(h[2 * b], wl, Gr, 1.0f);
+                        dmac(h[2 * b + 1], wl, Gi, 1.0f);
+                        dmac(h[6 + 2 * b], wl, Fr, 1.0f);
+                        dmac(h[6 + 2 * b + 1], wl, Fi, 1.0f);
+                        dmac(h[12 + 2 * b], wl, nFr, 1.0f);
+                        dmac(h[12 + 2 * b + 1], wl, nFi, 1.0f);
                     }
                 }
-                const dfl xw = dmul(dfl{xh.w, xl.w}, i4);
+                const dfl fK = dmul(xw, dsub(dfl{sgh.w, sgl.w}, dadd(dadd(dmul(snx, Xx), dmul(sny, Xy)), dmul(snz, Xz))));
 #pragma unroll
-                for (int i = 0; i < 3; i++) {
-                    const dfl wx = dmul(xw, dfl{d.lamh[qx][i], d.laml[qx][i]});
-                    const dfl wk = dmul(wx, fK);
+                for (int k = 0; k < 18; k++) h[k] = dmul(k >= 6 && k < 12 ? fK : xw, h[k]);
+            }
 #pragma unroll
-                    for (int b = 0; b < 3; b++)
+            for (int k = 0; k < 18; k++) sm.val[k][tid] = h[k];
+            __syncthreads();
+            // 2. against the test functions: moments 9 half ... 9 half + 8 of corner (triangle tl, function i)
+            {
+                dfl m[9];
 #pragma unroll
-                        for (int c = 0; c < 2; c++) {
-                            dmac(V[i][b][c], wx, hV[b][c], 1.0f);
-                            dmac(K[i][b][c], wk, hK[b][c], 1.0f);
-                            dmac(Kp[i][b][c], wx, hKp[b][c], 1.0f);
-                        }
+                for (int k = 0; k < 9; k++) m[k] = dfl{0.0f, 0.0f};
+#pragma unroll
+                for (int q = 0; q < QP; q++) {
+                    const dfl lam = {d.lamh[q][i], d.laml[q][i]};
+#pragma unroll
+                    for (int k = 0; k < 9; k++) dmac(m[k], sm.val[9 * half + k][tl * QP + q], lam, 1.0f);
+                }
+#pragma unroll
+                for (int k = 0; k < 9; k++) {
+                    const int c = 9 * half + k, kind = c / 6, b = c % 6 / 2;
+                    sm.mom[b][2 * kind + (c & 1)][corner] = m[k];
                 }
             }
-            // epilogue in FP64 (as assemble64_kernel) from the converted moments
-            double Vd[3][3][2];
-            double sr = 0, si = 0;
+            __syncthreads();
+            // 3. W: curl_i . curl_b sum V - k^2 n.n' V, real or imaginary part
+            {
+                dfl sv = {0.0f, 0.0f};
 #pragma unroll
-            for (int i = 0; i < 3; i++)
+                for (int b = 0; b < 3; b++)
+#pragma unroll
+                    for (int k = 0; k < 3; k++) sv = dadd(sv, sm.mom[b][half][k * TT + tl]);
+                const dfl nn = dneg(dadd(dadd(dmul(ngx, snx), dmul(ngy, sny)), dmul(ngz, snz)));
+                const dfl pr = dmul(nn, dsplit(cf.k2re)), pi = dmul(nn, dsplit(cf.k2im));
 #pragma unroll
                 for (int b = 0; b < 3; b++) {
-                    Vd[i][b][0] = (double)V[i][b][0].h + (double)V[i][b][0].l;
-                    Vd[i][b][1] = (double)V[i][b][1].h + (double)V[i][b][1].l;
-                    sr += Vd[i][b][0];
-                    si += Vd[i][b][1];
+                    const dfl cc = dadd(dadd(dmul(sm.ct[3 * i][tl], sm.cs[sl][3 * b]), dmul(sm.ct[3 * i + 1][tl], sm.cs[sl][3 * b + 1])),
+                                        dmul(sm.ct[3 * i + 2][tl], sm.cs[sl][3 * b + 2]));
+                    const dfl own = sm.mom[b][half][corner], other = sm.mom[b][half ^ 1][corner];
+                    dfl w = dmul(cc, sv);
+                    dmac(w, pr, own, 1.0f);
+                    dmac(w, pi, other, half ? 1.0f : -1.0f);
+                    sm.mom[b][6 + half][corner] = w;
                 }
-            const double nn = ((double)ngx.h + ngx.l) * ((double)snx.h + snx.l) +
-                              ((double)ngy.h + ngy.l) * ((double)sny.h + sny.l) +
-                              ((double)ngz.h + ngz.l) * ((double)snz.h + snz.l);
-            const int4 sv = a.slot_v[ss];
-            const int vb[3] = {sv.x, sv.y, sv.z};
-            for (int b = 0; b < 3; b++) {
-                const int64_t ca = a.v_dof1[vb[b]], cb = a.v_dof2[vb[b]];
-                for (int i = 0; i < 3; i++) {
-                    double cc = 0;
-                    for (int c = 0; c < 3; c++) cc += a.slot_curl[ts * 9 + 3 * i + c] * a.slot_curl[ss * 9 + 3 * b + c];
-                    const double kvr = cf.k2re * Vd[i][b][0] - cf.k2im * Vd[i][b][1];
-                    const double kvi = cf.k2re * Vd[i][b][1] + cf.k2im * Vd[i][b][0];
-                    const double Kr = (double)K[i][b][0].h + (double)K[i][b][0].l;
-                    const double Ki = (double)K[i][b][1].h + (double)K[i][b][1].l;
-                    const double Pr = (double)Kp[i][b][0].h + (double)Kp[i][b][0].l;
-                    const double Pi = (double)Kp[i][b][1].h + (double)Kp[i][b][1].l;
-                    double* e;
-                    e = reinterpret_cast<double*>(&A64[ra[i] * a.n + ca]);
-                    atomicAdd(e, cf.cV * Vd[i][b][0]);
-                    atomicAdd(e + 1, cf.cV * Vd[i][b][1]);
-                    e = reinterpret_cast<double*>(&A64[ra[i] * a.n + cb]);
-                    atomicAdd(e, -cf.cK * Kr);
-                    atomicAdd(e + 1, -cf.cK * Ki);
-                    e = reinterpret_cast<double*>(&A64[rb[i] * a.n + ca]);
-                    atomicAdd(e, cf.cKp * Pr);
-                    atomicAdd(e + 1, cf.cKp * Pi);
-                    e = reinterpret_cast<double*>(&A64[rb[i] * a.n + cb]);
-                    atomicAdd(e, cf.cW * (cc * sr - nn * kvr));
-                    atomicAdd(e + 1, cf.cW * (cc * si - nn * kvi));
+            }
+            __syncthreads();
+            // 4. vertex sums of one block (V, K, K' or W) into the matrix
+            const int4 sv = sm.sv[sl];
+            for (int e = tid; e < 12 * sm.nv; e += TP) {
+                const int v = e / 12, b = e % 3, blk = e % 12 / 3, vs = b == 0 ? sv.x : b == 1 ? sv.y : sv.z;
+                dfl mr = {0.0f, 0.0f}, mi = {0.0f, 0.0f};
+                for (int k = sm.ptr[v]; k < sm.ptr[v + 1]; k++) {
+                    mr = dadd(mr, sm.mom[b][2 * blk][sm.cor[k]]);
+                    mi = dadd(mi, sm.mom[b][2 * blk + 1][sm.cor[k]]);
                 }
+                const int id = sm.vert[v];
+                const int64_t row = blk < 2 ? a.v_dof1[id] : a.v_dof2[id], col = blk & 1 ? a.v_dof2[vs] : a.v_dof1[vs];
+                const double co = blk == 0 ? cf.cV : blk == 1 ? -cf.cK : blk == 2 ? cf.cKp : cf.cW;
+                double* out = reinterpret_cast<double*>(&A64[row * a.n + col]);
+                atomicAdd(out, co * ((double)mr.h + (double)mr.l));
+                atomicAdd(out + 1, co * ((double)mi.h + (double)mi.l));
             }
         }
     }
 }
 
-__global__ void __launch_bounds__(TT) assembledf_kernel(AssembleArgs a, AssembleDf d, double2* A64) {
-    __shared__ float4 tab[128];
-    __shared__ float2 etab[64];
-    for (int i = threadIdx.x; i < 128; i += blockDim.x) tab[i] = d.sctab[i];
-    for (int i = threadIdx.x; i < 64; i += blockDim.x) etab[i] = d.extab[i];
-    __syncthreads();
-    const int4 tv = a.slot_v[(int64_t)blockIdx.x * TT + threadIdx.x];
-    const float4 kk = a.slot == 0 ? d.k0df : d.kdf[tv.x >= 0 ? tv.w : 0];
-    if (kk.z != 0.0f || kk.w != 0.0f) assembledf_body<true>(a, d, A64, tab, etab);
-    else assembledf_body<false>(a, d, A64, tab, etab);
+__global__ void __launch_bounds__(TP, 2) assembledf_kernel(AssembleArgs a, AssembleDf d, double2* A64) {
+    extern __shared__ __align__(16) unsigned char asm_raw[];
+    AsmDfSmem& sm = *reinterpret_cast<AsmDfSmem*>(asm_raw);
+    for (int i = threadIdx.x; i < 128; i += blockDim.x) sm.tab[i] = d.sctab[i];
+    for (int i = threadIdx.x; i < 64; i += blockDim.x) sm.etab[i] = d.extab[i];
+    const float4 kk = a.slot == 0 ? d.k0df : d.kdf[a.slot_v[(int64_t)blockIdx.x * TT].w];
+    if (kk.z != 0.0f || kk.w != 0.0f) assembledf_body<true>(a, d, A64, sm);
+    else assembledf_body<false>(a, d, A64, sm);
 }
 
 __global__ void add_near64_kernel(int64_t n_pairs, const int32_t* pair_tgt, const int32_t* pair_src,
@@ -588,9 +668,11 @@ int bem_ctx::ensure_assembled64() {
             for (int k = 0; k < 3; k++) split((long double)quad.lam[q][k], d.lamh[q][k], d.laml[q][k]);
         split(1.0L / (4.0L * 3.141592653589793238462643383279502884L), d.i4h, d.i4l);
     }
+    if (opts.fp64_far == 0)
+        CK(cudaFuncSetAttribute(assembledf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(AsmDfSmem)));
     for (int sl = 0; sl < 2; sl++) {
         a.slot = sl;
-        if (opts.fp64_far == 0) assembledf_kernel<<<grid, TT, 0, stream>>>(a, d, asm64);
+        if (opts.fp64_far == 0) assembledf_kernel<<<grid, TP, sizeof(AsmDfSmem), stream>>>(a, d, asm64);
         else assemble64_kernel<<<grid, TT, 0, stream>>>(a, dev.pg64, dev.tg64, asm64);
         CK(cudaGetLastError());
     }
