@@ -40,7 +40,7 @@ FL_SLOT_LOSSLESS = 52.0 + 32.0 / 6.0
 FL_SLOT_LOSSY = 54.0 + 32.0 / 6.0
 # Of a slot's flops, the part that does not depend on the densities: the phase,
 # G, the gradient factor F and the sum of G w (14 + 4 flops; +2 for Im k != 0).
-# With R right-hand sides sharing a pair's G and F (far32m_kernel) the work of
+# With R right-hand sides sharing a pair's G and F the work of
 # R interactions is R x the one-vector count minus (R - 1) x this part and the
 # shared geometry.
 FL_SLOT_SHARED_LOSSLESS = 18.0
@@ -227,8 +227,9 @@ def kidney_apply_metrics(local, steps=3, n_rhs=16, peak=FP32_PEAK_TFLOPS):
     """The same operator application on the kidney + perinephric fat scene
     (61,996 triangles, 1 MHz), autotuned launch shape, L2 flushed between
     steps; then the kidney workload of 16 right-hand sides in ONE matrix-free
-    FP32 far-field launch (far32m_kernel, the pair's G and F shared by groups
-    of four vectors), as interaction-RHS per second."""
+    FP32 far field (farmm_kernel, the pair's G and F shared by groups of four
+    vectors and summed on the tensor cores; far32m_kernel for the close pairs
+    of tiles), as interaction-RHS per second."""
     import torch
 
     from paper_1910_01011_gb300.api import Context
@@ -285,11 +286,11 @@ def kidney_apply_metrics(local, steps=3, n_rhs=16, peak=FP32_PEAK_TFLOPS):
     ach_m = algorithmic_flops_multi(s, n_rhs) / (far_m / 1e3) / 1e12
     ms_med = sorted(ms_m)[len(ms_m) // 2]
     single["multi_rhs"] = {
-        "workload": f"kidney scene, {n_rhs} right-hand sides in one FP32 far-field launch (far32m_kernel)",
+        "workload": f"kidney scene, {n_rhs} right-hand sides in one FP32 far field (farmm_kernel, far32m_kernel)",
         "value": n_int * n_rhs / (ms_med / 1e3) / 1e9, "unit": "Ginteraction-RHS/s", "ms_per_apply": ms_med,
         "speedup_vs_single_rhs_applies": (ms * n_rhs / steps) / ms_med,
         "roofline": {"bound": "alu", "achieved": ach_m, "peak": peak, "unit": "TFLOP/s", "frac": ach_m / peak,
-                     "kernel": "far32m_kernel", "kernel_ms": far_m,
+                     "kernel": "farmm_kernel, far32m_kernel", "kernel_ms": far_m,
                      "work": "R x the one-vector flops minus (R-1) x the density-independent geometry, G and F"}}
     return single
 
@@ -700,7 +701,7 @@ def main():
     ap.add_argument("--block", action="store_true", help="--step solve: block GMRES instead of lockstep GMRES")
     ap.add_argument("--rhs", type=int, default=1,
                     help="right-hand sides per apply step; > 1 applies them in one matrix-free far-field launch "
-                         "(far32m_kernel) and reports interaction-RHS per second (profiling of the multi-RHS path)")
+                         "(farmm_kernel, far32m_kernel) and reports interaction-RHS per second (profiling of the multi-RHS path)")
     ap.add_argument("--serving-max-exc", type=int, default=64,
                     help="serving trace: excitations per request drawn from 1..this (default: the stated 1..64)")
     ap.add_argument("--clocks-log", default=None, help="keep the raw nvidia-smi clock samples in this CSV file")
@@ -806,7 +807,7 @@ def main():
                        "far_field_chunk_tiles": (tuned or {}).get("chunk_tiles", "built-in")},
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak_meas, "unit": "TFLOP/s",
                          "frac": achieved / peak_meas, "traffic": traffic if R == 1 else None,
-                         "kernel": "far32_kernel" if R == 1 else "far32m_kernel", "kernel_ms": far_ms,
+                         "kernel": "far32_kernel" if R == 1 else "farmm_kernel, far32m_kernel", "kernel_ms": far_ms,
                          "peak_basis": "measured: packed FFMA2 chains on every SM (bem_peak_probe), in this run",
                          "peak_derived": FP32_PEAK_TFLOPS, "frac_of_derived": achieved / FP32_PEAK_TFLOPS,
                          "peak_derived_basis": "152 SMs x 128 FP32 lanes x 2 (FFMA) x 2070 MHz max clock"},
