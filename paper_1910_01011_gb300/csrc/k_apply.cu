@@ -198,7 +198,7 @@ struct Acc {
 
 // One wavenumber slot, both lanes.
 struct PairK {
-    f2 kr, nkr, th, ki, nkil2;  // Re k, -Re k, reduced FP64 phase of the tile pair, Im k, -Im k log2(e)
+    f2 kr, th, ki, nkil2;  // Re k, reduced FP64 phase of the tile pair, Im k, -Im k log2(e)
 };
 
 // Sums over the points of one tile (V, K') and of one triangle (the rest),
@@ -230,10 +230,10 @@ __device__ __forceinline__ void pair_slot(const PairK& k, f2 rho, f2 r, f2 rinv,
         a = mul2(make_float2(ex2_approx(e.x), ex2_approx(e.y)), rinv);
     }
     const f2 Gr = mul2(a, cs), Gi = mul2(a, sn);
-    const f2 B = mul2(k.kr, rinv), nB = mul2(k.nkr, rinv);
+    const f2 B = mul2(k.kr, rinv);
     const f2 P = LOSSY ? fma2(k.ki, rinv, rinv2) : rinv2;
     const f2 nFr = fma2(P, Gr, mul2(B, Gi));
-    const f2 nFi = fma2(P, Gi, mul2(nB, Gr));
+    const f2 nFi = fma2(P, Gi, neg2(mul2(B, Gr)));
     T.Vr = fma2(Gr, d1r, fma2(Gi, nd1i, T.Vr));
     T.Vi = fma2(Gr, d1i, fma2(Gi, d1r, T.Vi));
     const f2 nFnr = mul2(ndot, nFr), nFni = mul2(ndot, nFi);
@@ -351,9 +351,9 @@ __device__ __forceinline__ void far32_item(const FarArgs32& A, int tx, int cy) {
     const int mydom = A.tdom[tt];
     const int2 dr = A.dom_tiles[mydom];
     const double2 kj = A.kdom[mydom];
-    const PairK k0{bc2((float)A.k0.x), bc2((float)-A.k0.x), bc2(0.f), bc2((float)A.k0.y),
+    const PairK k0{bc2((float)A.k0.x), bc2(0.f), bc2((float)A.k0.y),
                    bc2((float)(-A.k0.y * 1.4426950408889634))};
-    const PairK k1{bc2((float)kj.x), bc2((float)-kj.x), bc2(0.f), bc2((float)kj.y),
+    const PairK k1{bc2((float)kj.x), bc2(0.f), bc2((float)kj.y),
                    bc2((float)(-kj.y * 1.4426950408889634))};
     const bool lossy0 = A.k0.y != 0.0, lossy1 = kj.y != 0.0;
     const PairTgt X{g.x, g.y, g.z, ng.x, ng.y, ng.z, g.x * g.x + g.y * g.y + g.z * g.z,
@@ -557,10 +557,10 @@ __device__ __forceinline__ void tile_body_m(const StageM& st, int ntri, int skip
                 a = mul2(make_float2(ex2_approx(e.x), ex2_approx(e.y)), rinv);
             }
             const f2 Gr = mul2(a, cs), Gi = mul2(a, sn);
-            const f2 B = mul2(k.kr, rinv), nB = mul2(k.nkr, rinv);
+            const f2 B = mul2(k.kr, rinv);
             const f2 P = LOSSY ? fma2(k.ki, rinv, rinv2) : rinv2;
             const f2 nFr = fma2(P, Gr, mul2(B, Gi));
-            const f2 nFi = fma2(P, Gi, mul2(nB, Gr));
+            const f2 nFi = fma2(P, Gi, neg2(mul2(B, Gr)));
             const f2 nFnr = mul2(ndot, nFr), nFni = mul2(ndot, nFi);
             S2r = fma2(Gr, w, S2r);
             S2i = fma2(Gi, w, S2i);
@@ -641,7 +641,7 @@ __device__ __forceinline__ void far32m_item(const FarArgs32M& A, int tx, int cy,
     const float4 ng = A.tg[(int64_t)tt * TT + mt];
     const double4 ct = A.tc[tt];
     const double2 kk = slot ? A.kdom[mydom] : A.k0;
-    const PairK k{bc2((float)kk.x), bc2((float)-kk.x), bc2(0.f), bc2((float)kk.y),
+    const PairK k{bc2((float)kk.x), bc2(0.f), bc2((float)kk.y),
                   bc2((float)(-kk.y * 1.4426950408889634))};
     const PairTgt X{g.x, g.y, g.z, ng.x, ng.y, ng.z, g.x * g.x + g.y * g.y + g.z * g.z,
                     ng.x * g.x + ng.y * g.y + ng.z * g.z, bc2(-ng.x), bc2(-ng.y), bc2(-ng.z)};
