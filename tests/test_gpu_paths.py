@@ -175,3 +175,30 @@ def test_loose_solves_in_shared_memory(api, level, R, solver):
         c.close()
     for r in range(R):
         assert rel(out[0][r], out[1][r]) < 1e-6, r
+
+
+@pytest.mark.parametrize("precision,R", [("FP32", 1), ("FP64", 1), ("FP32", 3)])
+@pytest.mark.parametrize("name", ["sphere", "two", "ribs"])
+def test_products_back_to_back(api, name, precision, R):
+    """A chain of products, each on the one before, without the host waiting
+    in between: the same bits as with a wait after each (the kernels of a
+    product start before the ones they follow have ended)."""
+    import torch
+    s = {"sphere": lambda: scenes.sphere_scene(3), "two": lambda: scenes.two_sphere_scene(1),
+         "ribs": lambda: scenes.rib_scene(h=9e-3, freq=0.03e6)}[name]()
+    x0 = torch.from_numpy(np.stack([scenes.smooth_trace_vector(s, r) for r in range(R)])).cuda()
+    x0 = x0[0] if R == 1 else x0
+    c = api.Context.from_scene(s)
+    runs = []
+    for wait in (True, False):
+        x = x0
+        for _ in range(8):
+            y = c.apply(x, precision=getattr(api, precision))
+            if wait:
+                torch.cuda.synchronize()
+            x = y / 2.0 ** 10
+        torch.cuda.synchronize()
+        runs.append(x.cpu().numpy())
+    assert np.isfinite(runs[0]).all()
+    assert np.array_equal(runs[0], runs[1])
+    c.close()
