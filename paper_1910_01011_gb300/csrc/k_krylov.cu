@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(KV_THREADS) kbd_combine(int64_t n, int K, int 
 // part.  Every second step the sums of those 32 entries are folded into a
 // compensated (Kahan) FP32 total; the halves' totals are added and written as
 // FP64 partials part[(k P + c) nsplit + y].  8,200 unknowns, 16 columns, K up to
-// 816: 26 us on average before, 19 us now.
+// 816: 26 us on average before, 19 us at the former slices of n, 14.5 us now.
 constexpr int KD_ROWS = 64, KD_CHUNK = 32, KD_LD = KD_CHUNK + 2;  // (rows 16-byte aligned, eight in eight bank groups)
 __global__ void __launch_bounds__(KV_THREADS) kbd_dots32(int64_t n, int K, int P, const float2* __restrict__ V,
                                                          const float2* __restrict__ W, int c0, int nsplit,
@@ -957,10 +957,13 @@ namespace {
 
 using zd = std::complex<double>;
 
-// slices of n for the tiled FP32 dots: about 4 x 152 CTAs in all, slices of
-// at least 8 chunks; nsplit x gx <= max(gx, 608)
+// slices of n for the tiled FP32 dots: one wave of two CTAs per SM, slices of
+// at least two chunks (eight chunks and up to 608 CTAs left a small basis to 33
+// CTAs and put a large one in two waves: 19.1 us on average for the dots and
+// 4.4 for their reduction on 8,200 unknowns, now 14.5 and 6.3);
+// nsplit x gx <= max(gx, 304)
 int nsplit_tiled(int64_t n, int gx) {
-    return (int)std::max<int64_t>(1, std::min<int64_t>((n + 8 * KD_CHUNK - 1) / (8 * KD_CHUNK), 4 * 152 / gx));
+    return (int)std::max<int64_t>(1, std::min<int64_t>((n + 2 * KD_CHUNK - 1) / (2 * KD_CHUNK), 2 * 152 / gx));
 }
 
 int nsplit_for(int64_t n, int K) {
@@ -973,7 +976,7 @@ template <class T>
 int block_dots(bem_ctx* ctx, Krylov& k, const T* V, int K, const T* W, int P, double2* C, float2* C32 = nullptr) {
     const int64_t n = k.n;
     constexpr bool F32 = std::is_same<T, float2>::value;
-    // FP32: row tiles of KD_ROWS, slices of whole chunks, about 4 CTAs per SM
+    // FP32: row tiles of KD_ROWS, slices of whole chunks
     const int gx = F32 ? (K + KD_ROWS - 1) / KD_ROWS : K;
     const int nsplit = F32 ? nsplit_tiled(n, gx) : nsplit_for(n, K);
     const int64_t slice = F32 ? ((n + nsplit - 1) / nsplit + KD_CHUNK - 1) / KD_CHUNK * KD_CHUNK : 0;
