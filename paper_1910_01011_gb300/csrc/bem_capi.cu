@@ -392,7 +392,7 @@ int bem_ctx::upload_materials() {
     CK(cudaMemcpyAsync(dev.kdom, kd.data(), kd.size() * sizeof(double2), cudaMemcpyHostToDevice, stream));
     CK(cudaMemcpyAsync(dev.coef, cf.data(), cf.size() * sizeof(SlotCoef), cudaMemcpyHostToDevice, stream));
     CK(cudaStreamSynchronize(stream));
-    return BEM_OK;
+    return dfg.ready ? upload_df_wavenumbers() : BEM_OK;
 }
 
 // Near-field corrections: n_slot_k = 2 for the PMCHWT system (exterior and

@@ -213,6 +213,7 @@ struct bem_ctx {
     bool reserve_farmm(int64_t n_rhs);
     int apply_ahat64_multi(const double2* x, double2* y, int64_t n_rhs);
     int ensure_fardf();
+    int upload_df_wavenumbers();
     double df_extent(bool with_transducer) const;
     int check_df_phase(double kre, bool with_transducer);
     int far_df(const double4* pd, const double4* cu, int64_t R, int tgt_b, int tgt_e, int src_b, int src_e,

@@ -326,14 +326,8 @@ int bem_ctx::ensure_fardf() {
     }
     std::vector<float2> ex(64);
     for (int j = 0; j < 64; j++) split_ld(std::exp2(-(long double)j / 64.0L), ex[j].x, ex[j].y);
-    std::vector<float4> kd(g.n_dom);
-    for (int d = 0; d < g.n_dom; d++) {
-        split_ld((long double)doms[d].kre, kd[d].x, kd[d].y);
-        split_ld((long double)doms[d].kim, kd[d].z, kd[d].w);
-    }
     CK(cudaMemcpyAsync(dfg.sctab, sc.data(), sc.size() * sizeof(float4), cudaMemcpyHostToDevice, stream));
     CK(cudaMemcpyAsync(dfg.extab, ex.data(), ex.size() * sizeof(float2), cudaMemcpyHostToDevice, stream));
-    CK(cudaMemcpyAsync(dfg.kdf, kd.data(), kd.size() * sizeof(float4), cudaMemcpyHostToDevice, stream));
     // pi/64 in four parts (the first with 3 significant bits), ln2/64 in three (the first with 10)
     DfConsts& c = dfg.c;
     long double rest = PI / 64.0L;
@@ -354,7 +348,21 @@ int bem_ctx::ensure_fardf() {
     c.inv_ln64 = (float)(64.0L / LN2);
     split_ld(-1.0L / 6.0L, c.sixth[0], c.sixth[1]);
     CK(cudaStreamSynchronize(stream));  // the host tables above are freed on return
+    if ((rc = upload_df_wavenumbers())) return rc;
     dfg.ready = true;
+    return BEM_OK;
+}
+
+// The domains' wavenumbers as double-floats: with the tables above, and again whenever a material changes.
+int bem_ctx::upload_df_wavenumbers() {
+    bem_ctx* const ctx = this;
+    std::vector<float4> kd(geo.n_dom);
+    for (int d = 0; d < geo.n_dom; d++) {
+        split_ld((long double)doms[d].kre, kd[d].x, kd[d].y);
+        split_ld((long double)doms[d].kim, kd[d].z, kd[d].w);
+    }
+    CK(cudaMemcpyAsync(dfg.kdf, kd.data(), kd.size() * sizeof(float4), cudaMemcpyHostToDevice, stream));
+    CK(cudaStreamSynchronize(stream));
     return BEM_OK;
 }
 

@@ -202,3 +202,23 @@ def test_products_back_to_back(api, name, precision, R):
     assert np.isfinite(runs[0]).all()
     assert np.array_equal(runs[0], runs[1])
     c.close()
+
+
+@pytest.mark.parametrize("precision", ["FP32", "FP64", "BF16X3", "FP64_ASSEMBLED"])
+def test_new_material_after_use(api, precision):
+    """A domain's material changed after products of every kind: the next
+    product is that of a context made with it (near field, far field and both
+    assembled operators).  The assembled operators are summed by atomics."""
+    p = getattr(api, precision)
+    old, new = scenes.two_sphere_scene(1), scenes.two_sphere_scene(1, k2=4.4 + 0.3j, rho2=1.2)
+    x = scenes.smooth_trace_vector(old, 3)
+    c = api.Context.from_scene(new)
+    ref = c.apply(x, precision=p)
+    c.close()
+    c = api.Context.from_scene(old)
+    for q in (api.FP32, api.FP64, api.BF16X3, api.FP64_ASSEMBLED):
+        before = c.apply(x, precision=q)
+    assert rel(before, ref) > 1e-2
+    c.set_material(1, new.domains[1].k, new.domains[1].rho)
+    assert rel(c.apply(x, precision=p), ref) < (1e-12 if "64" in precision else 1e-6)
+    c.close()
