@@ -1076,16 +1076,16 @@ __global__ void __launch_bounds__(LS_NT, NR <= 4 ? 2 : 1) cocg_local32_kernel(Co
     }
 }
 
+// (The shared-memory limit belongs to the function, for all contexts and threads of the process: set once, to what
+// the largest domain of the instance takes.)
 template <int NR, int NS>
 static cudaError_t launch_local32(const CocgArgs32& b, int n_sys, int W, int64_t rows, cudaStream_t st) {
-    const int smem = (int)(rows * NS * 3 * sizeof(float2));
-    if (smem > 40 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(cocg_local32_kernel<NR, NS>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-    }
+    constexpr int row_bytes = NS * 3 * (int)sizeof(float2);
+    static const cudaError_t attr_e = cudaFuncSetAttribute(
+        cocg_local32_kernel<NR, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, NR * LS_NT * row_bytes);
+    if (attr_e != cudaSuccess) return attr_e;
     const unsigned grid = (unsigned)((n_sys + NS - 1) / NS * b.n_dom);
-    cocg_local32_kernel<NR, NS><<<grid, LS_NT, smem, st>>>(b, n_sys, W);
+    cocg_local32_kernel<NR, NS><<<grid, LS_NT, rows * row_bytes, st>>>(b, n_sys, W);
     return cudaGetLastError();
 }
 

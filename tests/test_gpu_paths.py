@@ -222,3 +222,34 @@ def test_new_material_after_use(api, precision):
     c.set_material(1, new.domains[1].k, new.domains[1].rho)
     assert rel(c.apply(x, precision=p), ref) < (1e-12 if "64" in precision else 1e-6)
     c.close()
+
+
+def test_loose_solves_of_two_sizes_at_once(api):
+    """Contexts solving in four threads, whose largest domains (2,562 and 2,068
+    vertices) take the same instance of the shared-memory preconditioner solver
+    with different amounts of shared memory: no launch of either is refused,
+    however the threads interleave."""
+    import threading
+    import torch
+    sc = [scenes.sphere_scene(4)] + [scenes.kidney_scene(h=6e-3, freq=0.05e6)] * 3
+    ctx = [api.Context.from_scene(s, stream=torch.cuda.Stream().cuda_stream) for s in sc]
+    errors = []
+
+    def work(c):
+        try:
+            for _ in range(20):
+                c.solve(precision=api.FP32, tol=1e-14, operator_mode=1, max_iter=100)
+        except Exception as e:  # a refused launch
+            errors.append(e)
+
+    for c in ctx:
+        c.set_plane_wave((0, 0, 1))
+        c.solve(precision=api.FP32, tol=1e-2, operator_mode=1, max_iter=20)  # set-up
+    threads = [threading.Thread(target=work, args=(c,)) for c in ctx]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for c in ctx:
+        c.close()
+    assert not errors, errors
