@@ -277,7 +277,7 @@ int64_t estimate_solve_bytes(const bem_ctx* ctx, int64_t n_exc, const bem_solve_
     if (o.operator_mode == 1) {
         const int64_t mp = (N + 127) / 128 * 128, kp = (N + 31) / 32 * 32;
         const int64_t planes = 6 * mp * kp * 2;
-        const int64_t a64 = (int64_t)(digits_bytes(N) + digits_convert_bytes(N)) + 4 * (digits_mpad(N) + digits_kpad(N)) +
+        const int64_t a64 = (int64_t)(digits_bytes(N) + digits_convert_bytes(N) + digits_exp_bytes(N)) +
                             (int64_t)digits_work_bytes(N, std::min<int64_t>(R, 16));
         if (o.precision == BEM_PREC_FP32)
             b += std::max(planes + 8 * N * N, planes + a64) + (int64_t)gemm_work_bytes(mp, kp, R);

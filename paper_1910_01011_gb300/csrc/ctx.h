@@ -175,7 +175,7 @@ struct bem_ctx {
     // fixed-point digits, 16 bytes each (k_digits.cu)
     bool asm64_ready = false;
     double2* asm64 = nullptr;
-    int* asm64_exp = nullptr;       // device: column and row exponents of asm64
+    int* asm64_exp = nullptr;       // device: exponents of asm64
     void* dg_work = nullptr;        // scratch of its products (grow-only)
     size_t dg_work_bytes = 0;
     int* df_exp = nullptr;          // device: exponent of the superposition basis
@@ -246,6 +246,7 @@ inline int resolved_operator_mode(int mode, int64_t n_dof) {
 int64_t digits_kpad(int64_t n);
 int64_t digits_mpad(int64_t n);
 size_t digits_bytes(int64_t n);
+size_t digits_exp_bytes(int64_t n);
 size_t digits_work_bytes(int64_t n, int64_t R);
 size_t digits_convert_bytes(int64_t n);
 int digits_prepare(bem_ctx* ctx, double2* A, int64_t n, int* exps);

@@ -640,7 +640,7 @@ int bem_ctx::ensure_assembled64() {
         if (rc) { asm64 = nullptr; return rc; }
     }
     if (!asm64_exp) {
-        asm64_exp = (int*)dalloc((size_t)(ld + digits_mpad(n)) * sizeof(int), &rc);
+        asm64_exp = (int*)dalloc(digits_exp_bytes(n), &rc);
         if (rc) { asm64_exp = nullptr; return rc; }
     }
     CK(cudaMemsetAsync(asm64, 0, digits_bytes(n), stream));

@@ -1,6 +1,7 @@
 // k_digits.cu -- complex128 matrix x block of vectors on the tensor cores,
-// exactly to ~2^-53 of the largest terms (the FP64 residual of the refinement,
-// r = b - A_hat u with the assembled complex128 A_hat).
+// each run of 256 columns to ~2^-51 of the largest term it can have, sums
+// exact or in FP64 (the FP64 residual of the refinement, r = b - A_hat u with
+// the assembled complex128 A_hat).
 //
 // GB300 runs FP64 at 1/64 of its FP32 rate, and carrying the products in FP32
 // pairs takes ~25 packed FP32 instructions per entry and vector.  Here both
@@ -9,21 +10,28 @@
 // Rump, "Error-free transformations of matrix multiplication by using fast
 // routines of matrix multiplication and its applications", 2012):
 //
-//  * A' = 2^-row A 2^-col with powers of two per row and column (columns first,
-//    so that the psi and phi blocks, a factor |k| apart, share their bits), each
-//    real part below 1/4 as Q 2^-56, |Q| < 2^54, and
+//  * K is cut into units of 256 columns.  In each, A' = 2^-row A 2^-col with
+//    powers of two per column and per row and unit (columns first, so that psi
+//    and phi columns, a factor |k| apart, share their bits where a unit holds
+//    both), each real part below 1/4 as Q 2^-56, |Q| < 2^54, and
 //    Q = sum_i d_i 128^(7 - i) with eight digits d_i in [-64, 63].  A digit is a
 //    byte (d + 64): 16 bytes per complex entry, as complex128 itself.
-//  * vectors likewise, x_j 2^col_j with one power of two per vector, as BF16
-//    digits (integers up to 256 are exact in BF16).
+//  * vectors likewise, x_j 2^col_j with a power of two per vector and unit (one
+//    for the whole vector and one per row lost 2^-40 of sum |a| |x| on 20,484
+//    unknowns: the phi columns hold W, whose diagonal is 2^10 and more above
+//    everything in the psi columns), as BF16 digits (integers up to 256 are
+//    exact in BF16).
 //  * Y' = sum_{i + j <= 7} 2^(-7 (i + j + 2)) A_i X_j on tcgen05 (kind::f16,
 //    BF16 in, FP32 out): the products are integers of at most 2^12, a sum of
 //    K = 256 of both real parts and up to eight (i, j) stays below 2^24, so
 //    every FP32 accumulator holds its integer exactly whatever the order or
-//    rounding mode of the unit.  The dropped terms are below 2^-53 of
-//    |A'| |x'|.
-//  * every 256 of K the eight accumulators of an output are added, smallest
-//    weight first, into a pair of FP32 numbers by TwoSum; pieces of K in FP64.
+//    rounding mode of the unit.  Dropped are the seven products with i + j = 8,
+//    at most 2^12 2^-70 each, and smaller ones: 2^-55, or 2^-51 of the largest a
+//    term can be (1/4 x 1/4).
+//  * at the end of a unit the eight accumulators of an output are added in a
+//    64-bit integer (exact; only sums of nearly the largest size lose the lowest
+//    8 of 70 bits), which goes into the FP64 sum of the CTA's run with the unit's
+//    power of two; pieces of K are added in FP64.
 //
 // The 36 digit products of a step need no 36 instructions: X's digits lie side
 // by side as rows of B, X_0 first, and A_i times the first 8 - i of them, into
@@ -39,10 +47,13 @@
 // bytes.  Every CTA takes an equal run of 256-wide units across row tiles (as
 // in k_gemm.cu), and pieces of a tile are added in FP64.
 //
-// N = 10,776, 16 vectors: 404 us (4.6 TB/s of A; the instructions of a step take
-// 1,306 cycles, its bytes 1,490 at the copy rate) against 4,423 us in FP32
-// pairs.  Relative error of products on scenes of 2,000-5,000 unknowns below
-// 1e-13, that of the assembled entries.
+// N = 10,776, 16 vectors: a call takes 422 us (4.4 TB/s of A; the instructions of
+// a step take 1,306 cycles, its bytes 1,490 at the copy rate) against 4,550 us in
+// FP32 pairs, and 430 us with one power of two per vector and row and sums in FP32
+// pairs.  Error of the product with a smooth vector on 20,484 unknowns, against
+// 128-bit sums of the entries: 3e-14, and 2^-47.7 of a row's sum |a| |x| at most
+// (FP32 pairs 2.4e-13 and 2^-43.7; one power of two per vector and row 6.7e-13 and
+// 2^-40.1).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -53,7 +64,6 @@
 #include <vector>
 
 #include "ctx.h"
-#include "df_math.cuh"
 #include "internal.h"
 
 namespace gbem {
@@ -61,7 +71,8 @@ namespace gbem {
 constexpr int DG = 8;                      // digits of a real number
 constexpr int DG_M = 128;                  // rows of A per tile
 constexpr int DG_K = 32;                   // K per stage (bytes per digit row)
-constexpr int DG_STEPS = 8;                // stages per unit: K = 256
+constexpr int DG_STEPS = 8;                // stages per unit
+constexpr int DG_UNIT = DG_K * DG_STEPS;   // K of a unit: 256
 constexpr int DG_CTAS = 152;
 constexpr int DG_PLANE = DG_M * DG_K;      // bytes of one digit plane of a stage
 constexpr int DG_ABYTES = 2 * DG * DG_PLANE;
@@ -79,6 +90,7 @@ struct DgCfg {
     struct Smem {
         alignas(1024) uint8_t a[DG_STAGES][DG_ABYTES];
         alignas(1024) uint8_t b[DG_STAGES][BBYTES];
+        double sum[NC][DG_M];                          // of the CTA's units of a tile
         uint64_t full[DG_STAGES], empty[DG_STAGES];    // copies landed; bytes converted (4 warps) and B used (MMA)
         uint64_t tfull[2], tempty[2];                  // A operand of one K = 16 step in tensor memory
         uint64_t dfull, dempty;                        // accumulators of a unit
@@ -120,37 +132,45 @@ __global__ void dg_colexp_kernel(const double2* __restrict__ A, int64_t n, int64
     atomicMax(&col[j], e);
 }
 
-__device__ __forceinline__ int block_max(int e, int* sh) {
+__device__ __forceinline__ int warp_max(int e) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = e;
-    __syncthreads();
-    e = sh[0];
-    for (int w = 1; w < (int)blockDim.x / 32; w++) e = max(e, sh[w]);
     return e;
 }
 
-// One row per CTA: its exponent, then its digits into the row tile's blocks (out: the first tile of the launch).
+// One row per CTA: its exponents (rowe [unit][mpad], rowm the largest), then its digits into the row tile's blocks
+// (out: the first tile of the launch).
 __global__ void __launch_bounds__(256) dg_digits_kernel(const double2* __restrict__ A, int64_t n, int64_t ld, int64_t row0,
-                                                        int64_t nkb, const int* __restrict__ col, int* __restrict__ rowe,
-                                                        uint8_t* __restrict__ out) {
+                                                        int64_t nkb, const int* __restrict__ col, int* __restrict__ rowm,
+                                                        int* rowe, int64_t mpad, uint8_t* __restrict__ out) {
     __shared__ int sh[8];
     const int64_t i = row0 + blockIdx.x;
-    const int r = blockIdx.x % DG_M;
+    const int r = blockIdx.x % DG_M, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const double2* a = A + i * ld;
-    int e = DG_NONE;
-    if (i < n)
-        for (int64_t j = threadIdx.x; j < n; j += blockDim.x) {
-            const int v = dg_exp2(a[j]), c = col[j];
-            if (v != DG_NONE) e = max(e, v == DG_BAD || c == DG_BAD ? DG_BAD : v - c);
-        }
-    e = block_max(e, sh);
-    if (threadIdx.x == 0) rowe[i] = e;
+    int top = DG_NONE;
+    for (int64_t u = warp; u * DG_UNIT < ld; u += 8) {
+        int e = DG_NONE;
+        if (i < n)
+            for (int64_t j = u * DG_UNIT + lane; j < min(n, (u + 1) * DG_UNIT); j += 32) {
+                const int v = dg_exp2(a[j]), c = col[j];
+                if (v != DG_NONE) e = max(e, v == DG_BAD || c == DG_BAD ? DG_BAD : v - c);
+            }
+        e = warp_max(e);
+        if (lane == 0) rowe[u * mpad + i] = e;
+        top = max(top, e);
+    }
+    if (lane == 0) sh[warp] = top;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; w++) top = max(top, sh[w]);
+        rowm[i] = top;
+    }
     // a thread takes four neighbouring entries: 4-byte stores per digit plane
     uint8_t* tile = out + (int64_t)(blockIdx.x / DG_M) * nkb * DG_ABYTES;
     for (int64_t q = threadIdx.x; q < nkb * (DG_K / 4); q += blockDim.x) {
         const int64_t kb = q / (DG_K / 4);
         const int k = (int)(q % (DG_K / 4)) * 4;
+        const int e = rowe[kb / DG_STEPS * mpad + i];
         unsigned long long u[2][4];
 #pragma unroll
         for (int t = 0; t < 4; t++) {
@@ -178,29 +198,37 @@ __global__ void __launch_bounds__(256) dg_digits_kernel(const double2* __restric
     }
 }
 
-// ve[r] = largest exponent of x_r 2^col; grid (blocks, vectors)
-__global__ void dg_vecexp_kernel(const double2* __restrict__ x, int64_t n, const int* __restrict__ col, int* ve) {
-    __shared__ int sh[8];
-    const double2* v = x + (int64_t)blockIdx.y * n;
+// ve[r][u] = largest exponent of x_r 2^col in unit u, vm[r] (set to less than any before) of all; grid (units, vectors)
+__global__ void __launch_bounds__(DG_UNIT) dg_vecexp_kernel(const double2* __restrict__ x, int64_t n, const int* __restrict__ col,
+                                                            int* __restrict__ ve, int* vm) {
+    __shared__ int sh[DG_UNIT / 32];
+    const int64_t j = (int64_t)blockIdx.x * DG_UNIT + threadIdx.x;
     int e = DG_NONE;
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-        const int t = dg_exp2(v[j]), c = col[j];
-        if (t != DG_NONE) e = max(e, t == DG_BAD || c == DG_BAD ? DG_BAD : c == DG_NONE ? DG_NONE : t + c);
+    if (j < n) {
+        const int t = dg_exp2(x[(int64_t)blockIdx.y * n + j]), c = col[j];
+        if (t != DG_NONE) e = t == DG_BAD || c == DG_BAD ? DG_BAD : c == DG_NONE ? DG_NONE : t + c;
     }
-    e = block_max(e, sh);
-    if (threadIdx.x == 0) atomicMax(&ve[blockIdx.y], e);
+    e = warp_max(e);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = e;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < DG_UNIT / 32; w++) e = max(e, sh[w]);
+        ve[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = e;
+        atomicMax(&vm[blockIdx.y], e);
+    }
 }
 
 // Digits of R <= HN vectors as the B operand: blocks of one stage, [part][digit HN*2 + column][32 K], 64-byte rows
 // in the 64-byte swizzle; vectors above R and K above n are zero.  Thread: one entry of one vector.
 __global__ void dg_vecdigits_kernel(const double2* __restrict__ x, int64_t n, int64_t kpad, int R, int hn,
-                                    const int* __restrict__ col, const int* __restrict__ ve, uint8_t* __restrict__ out) {
+                                    const int* __restrict__ col, const int* __restrict__ ve, int nch,
+                                    uint8_t* __restrict__ out) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int r = blockIdx.y;
     if (j >= kpad) return;
     double2 v = make_double2(0, 0);
     int s = 0;
-    const int e = r < R ? ve[r] : DG_NONE;
+    const int e = r < R ? ve[(int64_t)r * nch + j / DG_UNIT] : DG_NONE;
     if (j < n && e != DG_NONE && e != DG_BAD && col[j] != DG_NONE) {
         v = x[(int64_t)r * n + j];
         s = e + 2 - col[j];
@@ -282,16 +310,14 @@ __device__ __forceinline__ void d_st8(uint32_t t, const uint32_t (&r)[8]) {
                  "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
                  : "memory");
 }
-__device__ __forceinline__ void d_ld16(uint32_t t, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(t));
+__device__ __forceinline__ void d_ld8(uint32_t t, float (&v)[8]) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(t));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-    for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
+    for (int i = 0; i < 8; i++) v[i] = __uint_as_float(r[i]);
 }
 #define DG_FENCE_BEFORE asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory")
 #define DG_FENCE_AFTER asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory")
@@ -300,7 +326,8 @@ struct DgArgs {
     const uint8_t* A;     // [row tile][K block][plane][row][32]
     const uint8_t* B;     // [K block][part][row][32 bf16]
     int nkb, nch, units, pieces, m, R;
-    const int *rowe, *ve;
+    int64_t mpad;
+    const int *rowm, *rowe, *vm, *ve;
     double2* part;        // [row tile][piece][HN][128]
     double2* Y;           // [R][m]
     int* err;
@@ -455,43 +482,58 @@ __global__ void __launch_bounds__(DG_WARPS * 32, 1) digits_gemm_kernel(const DgA
     } else {
         const int q = warp & 3, r = q * 32 + lane;
         const uint32_t ld = tmem + ((uint32_t)(q * 32) << 16);
-        dfl y[NC];
-#pragma unroll
-        for (int j = 0; j < NC; j++) y[j] = dfl{0.f, 0.f};
+        bool fresh = true;  // no unit of the tile in `sum` yet
         for (int u = u0; u < u1; u++) {
-            const int tile = u / a.nch;
+            const int tile = u / a.nch, c = u - tile * a.nch;
+            const int64_t row = (int64_t)tile * DG_M + r;
+            const int er = max(a.rowe[c * a.mpad + row] - a.rowm[row], -2000);  // -2000: nothing in this unit
             d_wait(&sm.dfull, (uint32_t)((u - u0) & 1), a.err);
             DG_FENCE_AFTER;
+            // sums in 2^-49 of the first accumulator, exact, or from 2^62 on (bit set in `large`) rounded to 2^-41
+            long long y[NC];
+            uint32_t large = 0;
 #pragma unroll
-            for (int s = DG - 1; s >= 0; s--) {
-                const float w = __int_as_float((127 - 7 * s) << 23);  // 2^(-7 s)
+            for (int j0 = 0; j0 < NC; j0 += 8) {
+                long long t[2][8];
 #pragma unroll
-                for (int c = 0; c < NC; c += 16) {
-                    float v[16];
-                    d_ld16(ld + s * NC + c, v);
+                for (int h = 0; h < 2; h++)
 #pragma unroll
-                    for (int j = 0; j < 16; j++) {
-                        const dfl t = two_sum(y[c + j].h, v[j] * w);
-                        y[c + j].h = t.h;
-                        y[c + j].l = __fadd_rn(y[c + j].l, t.l);
+                    for (int s = 0; s < 4; s++) {
+                        float v[8];
+                        d_ld8(ld + (4 * h + s) * NC + j0, v);
+#pragma unroll
+                        for (int j = 0; j < 8; j++) t[h][j] = (s ? t[h][j] * 128 : 0) + __float2int_rn(v[j]);
                     }
+#pragma unroll
+                for (int j = 0; j < 8; j++) {
+                    const bool l = t[0][j] >= (1ll << 34) || t[0][j] <= -(1ll << 34);
+                    y[j0 + j] = l ? t[0][j] * (1 << 20) + ((t[1][j] + 128) >> 8) : t[0][j] * (1 << 28) + t[1][j];
+                    large |= (uint32_t)l << (j0 + j);
                 }
             }
             DG_FENCE_BEFORE;
             __syncwarp();
             if (lane == 0) d_arrive(&sm.dempty);
-#pragma unroll
-            for (int j = 0; j < NC; j++) y[j] = two_sum(y[j].h, y[j].l);
-            if (u + 1 < u1 && (u + 1) % a.nch != 0) continue;
+            const bool end = u + 1 == u1 || (u + 1) % a.nch == 0;
             const int piece = blockIdx.x - dg_first_cta(a.units, gridDim.x, a.nch, tile);
             double2* out = a.part + (int64_t)(tile * a.pieces + piece) * C::HN * DG_M + r;
 #pragma unroll
-            for (int j = 0; j < C::HN; j++)
-                if (j < a.R)
-                    out[j * DG_M] = make_double2((double)y[j].h + (double)y[j].l,
-                                                 (double)y[C::HN + j].h + (double)y[C::HN + j].l);
-#pragma unroll
-            for (int j = 0; j < NC; j++) y[j] = dfl{0.f, 0.f};
+            for (int j = 0; j < C::HN; j++) {
+                if (j >= a.R) break;
+                const int e = er + max(a.ve[(int64_t)j * a.nch + c] - a.vm[j], -2000);
+                const double fx = e < -1000 ? 0.0 : __hiloint2double((1023 + e + (large >> j & 1) * 8) << 20, 0);
+                const double fy = e < -1000 ? 0.0 : __hiloint2double((1023 + e + (large >> (C::HN + j) & 1) * 8) << 20, 0);
+                double2 s = fresh ? make_double2(0, 0) : make_double2(sm.sum[j][r], sm.sum[C::HN + j][r]);
+                s.x = fma((double)y[j], fx, s.x);
+                s.y = fma((double)y[C::HN + j], fy, s.y);
+                if (end) {
+                    out[j * DG_M] = s;
+                } else {
+                    sm.sum[j][r] = s.x;
+                    sm.sum[C::HN + j][r] = s.y;
+                }
+            }
+            fresh = end;
         }
     }
     __syncwarp();
@@ -515,11 +557,11 @@ __global__ void dg_finish_kernel(DgArgs a, int ctas, int hn) {
         x += v.x;
         y += v.y;
     }
-    const int er = a.rowe[row], ev = a.ve[r];
+    const int er = a.rowm[row], ev = a.vm[r];
     if (er == DG_BAD || ev == DG_BAD) x = y = __longlong_as_double(0x7ff8000000000000ll);
     else if (er == DG_NONE || ev == DG_NONE) x = y = 0;
     else {
-        const int e = er + ev + 4 - 14;  // both operands below 2^-2 of their scale, first digits 2^-7 each
+        const int e = er + ev + 4 - 14 - 49;  // both operands below 2^-2 of their scale, first digits 2^-7 each
         x = ldexp(x, e);
         y = ldexp(y, e);
     }
@@ -532,6 +574,9 @@ int64_t digits_kpad(int64_t n) { return (n + DG_K - 1) / DG_K * DG_K; }
 int64_t digits_mpad(int64_t n) { return (n + DG_M - 1) / DG_M * DG_M; }
 // bytes of a matrix (as complex128 with leading dimension kpad, then as digits in the same place)
 size_t digits_bytes(int64_t n) { return (size_t)digits_mpad(n) * digits_kpad(n) * 16; }
+static int64_t dg_units(int64_t n) { return (n + DG_UNIT - 1) / DG_UNIT; }
+// ... and of its exponents: columns [kpad], rows [mpad], rows of each unit [units][mpad]
+size_t digits_exp_bytes(int64_t n) { return (size_t)(digits_kpad(n) + digits_mpad(n) * (1 + dg_units(n))) * sizeof(int); }
 
 constexpr int DG_TILES = 2;  // row tiles converted at a time
 static int dg_hn(int64_t R) { return R <= 8 ? 8 : 16; }
@@ -544,7 +589,8 @@ size_t digits_work_bytes(int64_t n, int64_t R) {
     const int hn = dg_hn(R);
     const int nkb = (int)(digits_kpad(n) / DG_K), nch = (nkb + DG_STEPS - 1) / DG_STEPS;
     const int tiles = (int)(digits_mpad(n) / DG_M), units = tiles * nch, ctas = std::min(DG_CTAS, units);
-    return (size_t)nkb * 2 * DG * 2 * hn * DG_K * 2 + (size_t)tiles * dg_pieces(units, ctas, nch) * hn * DG_M * 16 + 16 * sizeof(int);
+    return (size_t)nkb * 2 * DG * 2 * hn * DG_K * 2 + (size_t)tiles * dg_pieces(units, ctas, nch) * hn * DG_M * 16 +
+           16 * (1 + nch) * sizeof(int);
 }
 size_t digits_convert_bytes(int64_t n) { return (size_t)DG_TILES * DG_M * digits_kpad(n) * 16; }
 
@@ -555,7 +601,7 @@ size_t digits_convert_bytes(int64_t n) { return (size_t)DG_TILES * DG_M * digits
     } while (0)
 
 // Complex128 matrix A (n x n in a buffer of digits_bytes, leading dimension
-// digits_kpad) -> digits in place; exps: device [kpad + mpad] column, row exponents.
+// digits_kpad) -> digits in place; exps: device, digits_exp_bytes.
 int digits_prepare(bem_ctx* ctx, double2* A, int64_t n, int* exps) {
     const int64_t kpad = digits_kpad(n), mpad = digits_mpad(n), nkb = kpad / DG_K;
     int rc;
@@ -573,7 +619,7 @@ int digits_prepare(bem_ctx* ctx, double2* A, int64_t n, int* exps) {
     ctx->launches += 1;
     for (int64_t r0 = 0; r0 < mpad; r0 += DG_TILES * DG_M) {
         const int64_t rows = std::min<int64_t>(DG_TILES * DG_M, mpad - r0);
-        dg_digits_kernel<<<(unsigned)rows, 256, 0, ctx->stream>>>(A, n, kpad, r0, nkb, col, row, tmp);
+        dg_digits_kernel<<<(unsigned)rows, 256, 0, ctx->stream>>>(A, n, kpad, r0, nkb, col, row, row + mpad, mpad, tmp);
         DCK(cudaGetLastError());
         DCK(cudaMemcpyAsync(A + r0 * kpad, tmp, (size_t)rows * kpad * 16, cudaMemcpyDeviceToDevice, ctx->stream));
         ctx->launches += 1;
@@ -606,22 +652,26 @@ int digits_gemm(bem_ctx* ctx, const void* A, const int* exps, int64_t n, const d
     const int ctas = std::min(DG_CTAS, a.units);
     a.pieces = dg_pieces(a.units, ctas, a.nch);
     a.m = (int)n;
-    a.rowe = exps + kpad;
+    a.mpad = mpad;
+    a.rowm = exps + kpad;
+    a.rowe = a.rowm + mpad;
     a.err = ctx->dev.err;
     uint8_t* b = (uint8_t*)work;
     const size_t bb = (size_t)a.nkb * 2 * DG * 2 * hn * DG_K * 2;
     a.B = b;
     a.part = (double2*)(b + bb);
-    int* ve = (int*)(a.part + (size_t)tiles * a.pieces * hn * DG_M);
+    int* vm = (int*)(a.part + (size_t)tiles * a.pieces * hn * DG_M);
+    int* ve = vm + 16;
+    a.vm = vm;
     a.ve = ve;
     for (int64_t r0 = 0; r0 < R; r0 += hn) {
         const int nr = (int)std::min<int64_t>(hn, R - r0);
         const double2* x = X + r0 * n;
         a.R = nr;
         a.Y = Y + r0 * n;
-        DCK(cudaMemsetAsync(ve, 0x80, 16 * sizeof(int), ctx->stream));  // below every exponent
-        dg_vecexp_kernel<<<dim3((unsigned)std::min<int64_t>(64, (n + 255) / 256), (unsigned)nr), 256, 0, ctx->stream>>>(x, n, exps, ve);
-        dg_vecdigits_kernel<<<dim3((unsigned)((kpad + 127) / 128), (unsigned)hn), 128, 0, ctx->stream>>>(x, n, kpad, nr, hn, exps, ve, b);
+        DCK(cudaMemsetAsync(vm, 0x80, 16 * sizeof(int), ctx->stream));  // below every exponent
+        dg_vecexp_kernel<<<dim3((unsigned)a.nch, (unsigned)nr), DG_UNIT, 0, ctx->stream>>>(x, n, exps, ve, vm);
+        dg_vecdigits_kernel<<<dim3((unsigned)((kpad + 127) / 128), (unsigned)hn), 128, 0, ctx->stream>>>(x, n, kpad, nr, hn, exps, ve, a.nch, b);
         DCK(cudaGetLastError());
         DCK(hn == 8 ? launch_digits<16>(a, (unsigned)ctas, ctx->stream) : launch_digits<32>(a, (unsigned)ctas, ctx->stream));
         dg_finish_kernel<<<dim3((unsigned)((n + 255) / 256), (unsigned)nr), 256, 0, ctx->stream>>>(a, ctas, hn);

@@ -253,3 +253,44 @@ def test_loose_solves_of_two_sizes_at_once(api):
     for c in ctx:
         c.close()
     assert not errors, errors
+
+
+def test_fp64_assembled_digits_by_columns(api):
+    """20,484 unknowns (a CTA's run covers a whole row tile): a smooth vector,
+    and rows whose terms all add up over one half of the columns and cancel
+    over the other, against 128-bit sums of the entries (products with unit
+    vectors: one term, whose digits are exact).  A term loses 7 digit products
+    of weight 2^-70 with digits of about 37 (rms), of either sign: 2^-58,
+    against a largest term of 2^-4 within its 256 columns.  Six deviations of
+    512 of them, and those of the units in quadrature; nothing from the sums."""
+    import torch
+    s = scenes.sphere_scene(5)
+    c = api.Context.from_scene(s)
+    N = c.n_dofs
+    rows = np.array([0, 137, 2561, 5000, 10241, 10242, 15000, N - 1])
+    idx = torch.from_numpy(rows).cuda()
+    A = np.empty((len(rows), N), dtype=np.complex128)
+    col = np.empty(N)  # largest part of each column
+    for b in range(0, N, 1024):
+        e = min(N, b + 1024)
+        E = torch.zeros(e - b, N, dtype=torch.complex128, device="cuda")
+        E[torch.arange(e - b), torch.arange(b, e)] = 1
+        Y = c.apply(E, precision=api.FP64_ASSEMBLED)
+        A[:, b:e] = Y[:, idx].T.cpu().numpy()
+        col[b:e] = torch.view_as_real(Y).abs().amax(dim=(1, 2)).cpu().numpy()
+    c0 = 2.0 ** np.ceil(np.log2(col))
+    X = np.exp(-1j * np.angle(A))
+    X[:, N // 2:] *= -1
+    X = np.concatenate([X, scenes.smooth_trace_vector(s, 2)[None]])
+    Y = c.apply(X, precision=api.FP64_ASSEMBLED)
+    c.close()
+    units = np.arange(0, N, 256)
+    L = np.longdouble
+    for r, i in enumerate(rows):
+        for v in (r, len(rows)):
+            ar, ai, xr, xi = (z.astype(L) for z in (A[r].real, A[r].imag, X[v].real, X[v].imag))
+            dr = abs((ar * xr - ai * xi).sum() - L(Y[v, i].real))
+            di = abs((ar * xi + ai * xr).sum() - L(Y[v, i].imag))
+            largest = np.maximum.reduceat(np.abs(A[r]) / c0, units) * np.maximum.reduceat(np.abs(X[v]) * c0, units) * 4
+            bound = 6 * np.sqrt(512) * 2.0 ** -54 * np.linalg.norm(largest)  # (4: powers of two above both)
+            assert max(dr, di) < bound, (i, v, float(max(dr, di)), bound)
