@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(NEAR_THREADS) near_build_kernel(NearArgs A) {
 // They are expanded to three sums per moving vertex for each of V, K and K'
 // (relative accuracy ~1e-13, as the evaluations), and the CTA's groups meet
 // in shared memory, where lane (operator, i, j) of each warp multiplies them
-// with the fixed point's P1 values and adds them up; four warps' sums are
+// with the fixed point's P1 values and adds up 32 groups; these sums are
 // added in FP64.  One point per thread with all 27 complex moments in
 // registers (255 of them, eight warps per SM), each reduced over the CTA by
 // FP64 shuffles, which ran on the 1/64-rate pipe for longer than the points
@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(NEAR_THREADS, 4) near_build_df_kernel(NearArgs
     // lane (operator, i, j) sums its moment over its warp's groups
     const int lane = tid & 31, warp = tid >> 5;
     const int op = lane / 9, ij = lane - 9 * op, mi = ij / 3, mj = ij - 3 * mi;
-    dfl sr = {0.0f, 0.0f}, si = {0.0f, 0.0f};
+    double tr = 0, ti = 0;
     for (int b = 0; b < n_all; b += NEAR_THREADS) {
         const int idx = b + tid;
         float2* row = rows[tid];
@@ -410,6 +410,7 @@ __global__ void __launch_bounds__(NEAR_THREADS, 4) near_build_df_kernel(NearArgs
         }
         __syncwarp();
         if (lane < NACC) {
+            dfl sr = {0.0f, 0.0f}, si = {0.0f, 0.0f};
             for (int g = 0; g < 32; g++) {
                 const int i = b + warp * 32 + g;
                 if (!(i < n || (i >= reg0 && i < n_all))) continue;
@@ -420,14 +421,14 @@ __global__ void __launch_bounds__(NEAR_THREADS, 4) near_build_df_kernel(NearArgs
                 dmac(sr, dfl{vr.x, vr.y}, dfl{u.x, u.y}, 1.0f);
                 dmac(si, dfl{vi.x, vi.y}, dfl{u.x, u.y}, 1.0f);
             }
-            sr = two_sum(sr.h, sr.l);
-            si = two_sum(si.h, si.l);
+            tr += (double)sr.h + (double)sr.l;  // 32 groups in FP32 pairs, the rest in FP64
+            ti += (double)si.h + (double)si.l;
         }
         __syncwarp();
     }
     if (lane < NACC) {
-        red[warp][lane][0] = (double)sr.h + (double)sr.l;
-        red[warp][lane][1] = (double)si.h + (double)si.l;
+        red[warp][lane][0] = tr;
+        red[warp][lane][1] = ti;
     }
     __syncthreads();
     if (tid < NACC * 2) {
