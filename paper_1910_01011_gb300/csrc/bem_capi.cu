@@ -42,43 +42,32 @@ static uint64_t next_gen() {
     return ++g;
 }
 
-void* bem_ctx::dalloc(size_t bytes, int* rc) {
+// One allocation within the context's budget and the shared one; null, *rc and why otherwise.
+void* bem_ctx::take(size_t bytes, int* rc, std::string& why) {
     if (bytes == 0) bytes = 16;
-    // the tensor-core far field's operands are a convenience: they go before an allocation is refused
-    auto give_back = [&] {
-        if (!mm_buf) return false;
-        cudaStreamSynchronize(stream);
-        dfree(mm_buf);
-        mm_buf = nullptr;
-        mm_bytes = 0;
-        mm_off = true;
-        return true;
-    };
     if (opts.hbm_budget_bytes > 0 && (int64_t)(used_bytes + bytes) > opts.hbm_budget_bytes) {
-        if (give_back()) return dalloc(bytes, rc);
-        *rc = fail(BEM_ERR_OUT_OF_BUDGET, "device memory budget exceeded (" + std::to_string(used_bytes + bytes) +
-                                              " > " + std::to_string(opts.hbm_budget_bytes) + " bytes)");
+        *rc = BEM_ERR_OUT_OF_BUDGET;
+        why = "device memory budget exceeded (" + std::to_string(used_bytes + bytes) + " > " +
+              std::to_string(opts.hbm_budget_bytes) + " bytes)";
         return nullptr;
     }
     if (pool) {
         const int64_t after = pool->fetch_add((int64_t)bytes) + (int64_t)bytes;
         if (pool_limit > 0 && after > pool_limit) {
             pool->fetch_sub((int64_t)bytes);
-            if (give_back()) return dalloc(bytes, rc);
-            *rc = fail(BEM_ERR_OUT_OF_BUDGET, "shared device memory budget exceeded (" + std::to_string(after) +
-                                                  " > " + std::to_string(pool_limit) + " bytes)");
+            *rc = BEM_ERR_OUT_OF_BUDGET;
+            why = "shared device memory budget exceeded (" + std::to_string(after) + " > " + std::to_string(pool_limit) +
+                  " bytes)";
             return nullptr;
         }
     }
     void* p = nullptr;
     cudaError_t e = cudaMalloc(&p, bytes);
     if (e != cudaSuccess) {
+        cudaGetLastError();
         if (pool) pool->fetch_sub((int64_t)bytes);
-        if (e == cudaErrorMemoryAllocation && give_back()) {
-            cudaGetLastError();
-            return dalloc(bytes, rc);
-        }
-        *rc = fail(BEM_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+        *rc = BEM_ERR_CUDA;
+        why = std::string("cudaMalloc: ") + cudaGetErrorString(e);
         return nullptr;
     }
     allocs.push_back({p, bytes});
@@ -87,6 +76,69 @@ void* bem_ctx::dalloc(size_t bytes, int* rc) {
     peak_bytes = std::max(peak_bytes, used_bytes);
     *rc = BEM_OK;
     return p;
+}
+
+// Memory that a call cannot do without: what only speeds calls up goes before it is refused.
+void* bem_ctx::dalloc(size_t bytes, int* rc) {
+    std::string why;
+    void* p = take(bytes, rc, why);
+    if (!p && give_back()) p = take(bytes, rc, why);
+    if (!p) {
+        short_of_memory = true;
+        fail(*rc, why);
+    }
+    return p;
+}
+
+// Memory that only speeds calls up: nothing else goes for it, and a refusal is not an error.
+void* bem_ctx::try_alloc(size_t bytes) {
+    int rc;
+    std::string why;
+    void* p = take(bytes, &rc, why);
+    if (!p) optional_wait = OPTIONAL_WAIT;
+    return p;
+}
+
+// Whether `grow` bytes more may go to such memory: within the context's budget,
+// at most half of a shared one (other contexts' reservations do not count it),
+// and as much again left free on the device.  After a refusal by the device
+// the next OPTIONAL_WAIT calls do not ask it again.
+bool bem_ctx::room_for(size_t grow) {
+    if (grow == 0) return true;
+    if (frugal) return false;
+    if (opts.hbm_budget_bytes > 0 && (int64_t)(used_bytes + grow) > opts.hbm_budget_bytes) return false;
+    if (pool && pool_limit > 0 && 2 * (pool->load() + (int64_t)grow) > pool_limit) return false;
+    if (optional_wait > 0) {
+        optional_wait--;
+        return false;
+    }
+    size_t free = 0, total = 0;
+    if (cudaMemGetInfo(&free, &total) != cudaSuccess || free < 2 * grow) {
+        cudaGetLastError();
+        optional_wait = OPTIONAL_WAIT;
+        return false;
+    }
+    return true;
+}
+
+// Frees what only speeds calls up, unless a call in progress holds pointers into it.
+bool bem_ctx::give_back() {
+    if (pinned > 0) return false;
+    const bool part = partial && partial_bytes > partial_need;
+    if (!part && !mm_buf) return false;
+    cudaStreamSynchronize(stream);
+    if (part) {
+        dfree(partial);
+        partial = nullptr;
+        partial_bytes = 0;
+    }
+    if (mm_buf) {
+        dfree(mm_buf);
+        mm_buf = nullptr;
+        mm_bytes = 0;
+        mm_off = true;
+    }
+    return true;
 }
 
 void bem_ctx::dfree(void* p) {
@@ -149,7 +201,8 @@ static void release_device(bem_ctx* ctx) {
     ctx->asm_work = nullptr;
     ctx->asm_work_bytes = 0;
     ctx->partial = nullptr;
-    ctx->partial_bytes = 0;
+    ctx->partial_bytes = ctx->partial_need = 0;
+    ctx->optional_wait = 0;
     ctx->field_buf = nullptr;
     ctx->field_buf_bytes = 0;
     ctx->far_work = nullptr;
@@ -484,13 +537,15 @@ int bem_ctx::ensure_near() {
     return BEM_OK;
 }
 
-int bem_ctx::ensure_partial(int n_chunks, bool fp64) {
-    size_t need = (size_t)n_chunks * 2 * NCOMP * geo.n_pts * (fp64 ? 8 : 4);
+// Partial potentials of `need` bytes; optional: where that only allows shorter chunks.
+int bem_ctx::ensure_partial(size_t need, bool optional) {
     if (need <= partial_bytes) return BEM_OK;
-    if (partial) dfree(partial);
-    int rc;
-    partial = dalloc(need, &rc);
-    if (rc) { partial = nullptr; partial_bytes = 0; return rc; }
+    if (optional && !room_for(need - partial_bytes)) return BEM_ERR_OUT_OF_BUDGET;
+    dfree(partial);
+    partial_bytes = 0;
+    int rc = BEM_OK;
+    partial = optional ? try_alloc(need) : dalloc(need, &rc);
+    if (!partial) return optional ? BEM_ERR_OUT_OF_BUDGET : rc;
     partial_bytes = need;
     return BEM_OK;
 }
@@ -563,14 +618,19 @@ int bem_ctx::plan_apply(const double2* x, double2* y, int precision, const Apply
     P.fp64 = fp64;
     const int tgt_b = g.dom_tile_begin[m.tgt_dom_lo], tgt_e = g.dom_tile_end[m.tgt_dom_hi - 1];
     const int src_b = g.dom_tile_begin[m.src_dom_lo], src_e = g.dom_tile_end[m.src_dom_hi - 1];
-    int n_chunks, chunk_tiles;
-    chunking(fill_tiles > 0 ? fill_tiles : tgt_e - tgt_b, src_e - src_b, &n_chunks, &chunk_tiles, fp64);
-    int rc = ensure_partial(n_chunks, fp64);
-    if (rc == BEM_ERR_OUT_OF_BUDGET && !fp64) {  // longer chunks where the budget does not hold the partials of short ones
-        chunking(fill_tiles > 0 ? fill_tiles : tgt_e - tgt_b, src_e - src_b, &n_chunks, &chunk_tiles, true);
-        rc = ensure_partial(n_chunks, fp64);
+    // FP32: short source chunks where there is room for their partials, else the longer ones
+    const int fill = fill_tiles > 0 ? fill_tiles : tgt_e - tgt_b;
+    const size_t per_chunk = (size_t)2 * NCOMP * g.n_pts * (fp64 ? sizeof(double) : sizeof(float));
+    int n_chunks, chunk_tiles, nc, ct, rc;
+    chunking(fill, src_e - src_b, &n_chunks, &chunk_tiles, true);
+    partial_need = std::max(partial_need, n_chunks * per_chunk);
+    chunking(fill, src_e - src_b, &nc, &ct, fp64);
+    if (nc != n_chunks && ensure_partial(nc * per_chunk, true) == BEM_OK) {
+        n_chunks = nc;
+        chunk_tiles = ct;
+    } else if ((rc = ensure_partial(n_chunks * per_chunk, false))) {
+        return rc;
     }
-    if (rc) return rc;
     P.n_tgt = tgt_e - tgt_b;
     P.n_chunks = n_chunks;
     // 1. trial densities on the source slots
@@ -626,10 +686,15 @@ int bem_ctx::plan_apply(const double2* x, double2* y, int precision, const Apply
     return BEM_OK;
 }
 
+// A call whose buffers do not fit beside memory that only speeds calls up gives that back and starts over.
+int bem_ctx::run_apply(const double2* x, double2* y, int precision, const ApplyMode& m) {
+    return without_optional_if_short([&] { return run_apply_once(x, y, precision, m); });
+}
+
 // The pipeline.  x, y: device, system order.  Modes: PMCHWT (all targets,
 // all sources at k0 plus own-domain sources at k_j), or BLOCK (targets of
 // domain j, sources of domain i, one wavenumber).
-int bem_ctx::run_apply(const double2* x, double2* y, int precision, const ApplyMode& m) {
+int bem_ctx::run_apply_once(const double2* x, double2* y, int precision, const ApplyMode& m) {
     bem_ctx* const ctx = this;
     ApplyPlan P;
     int rc = plan_apply(x, y, precision, m, P);
@@ -1350,17 +1415,8 @@ int bem_apply_block(bem_ctx* ctx, int32_t j, int32_t i, bem_z k, const bem_z* x,
     return ctx->check_device_error();
 }
 
-// Several meshes in one far-field launch (see include/bem.h).
-int bem_apply_group(bem_ctx* const* ctxs, int32_t n, const bem_z* const* x, bem_z* const* y) {
-    if (!ctxs || !x || !y || n < 1 || n > 4096) return BEM_ERR_INVALID_ARG;
+static int apply_group_once(bem_ctx* const* ctxs, int32_t n, const bem_z* const* x, bem_z* const* y) {
     bem_ctx* const ctx = ctxs[0];
-    if (!ctx) return BEM_ERR_INVALID_ARG;
-    for (int i = 0; i < n; i++) {
-        if (!ctxs[i] || !x[i] || !y[i]) return ctx->fail(BEM_ERR_INVALID_ARG, "null context or vector in the group");
-        if (ctxs[i]->device != ctx->device) return ctx->fail(BEM_ERR_INVALID_ARG, "group contexts on different devices");
-        for (int j = 0; j < i; j++)
-            if (ctxs[j] == ctxs[i]) return ctx->fail(BEM_ERR_INVALID_ARG, "a context appears twice in the group");
-    }
     CK(cudaSetDevice(ctx->device));
     // buffers and arguments of every member (no launches yet); the source
     // chunks are sized for the whole group's target tiles, so small meshes
@@ -1455,6 +1511,39 @@ int bem_apply_group(bem_ctx* const* ctxs, int32_t n, const bem_z* const* x, bem_
     CK(cudaGraphLaunch(G->exec, ctx->stream));
     ctx->launches += 1 + 3 * n;
     return BEM_OK;
+}
+
+// Several meshes in one far-field launch (see include/bem.h).
+int bem_apply_group(bem_ctx* const* ctxs, int32_t n, const bem_z* const* x, bem_z* const* y) {
+    if (!ctxs || !x || !y || n < 1 || n > 4096) return BEM_ERR_INVALID_ARG;
+    bem_ctx* const ctx = ctxs[0];
+    if (!ctx) return BEM_ERR_INVALID_ARG;
+    for (int i = 0; i < n; i++) {
+        if (!ctxs[i] || !x[i] || !y[i]) return ctx->fail(BEM_ERR_INVALID_ARG, "null context or vector in the group");
+        if (ctxs[i]->device != ctx->device) return ctx->fail(BEM_ERR_INVALID_ARG, "group contexts on different devices");
+        for (int j = 0; j < i; j++)
+            if (ctxs[j] == ctxs[i]) return ctx->fail(BEM_ERR_INVALID_ARG, "a context appears twice in the group");
+    }
+    // (as without_optional_if_short, for every member)
+    auto run = [&](bool frugal) {
+        for (int i = 0; i < n; i++) {
+            ctxs[i]->frugal = frugal;
+            ctxs[i]->short_of_memory = false;
+            ctxs[i]->pinned++;
+        }
+        const int rc = apply_group_once(ctxs, n, x, y);
+        for (int i = 0; i < n; i++) {
+            ctxs[i]->frugal = false;
+            ctxs[i]->pinned--;
+        }
+        return rc;
+    };
+    const int rc = run(false);
+    bool refused = false, given = false;
+    for (int i = 0; i < n; i++) refused |= ctxs[i]->short_of_memory;
+    if (!rc || !refused) return rc;
+    for (int i = 0; i < n; i++) given |= ctxs[i]->give_back();
+    return given ? run(true) : rc;
 }
 
 int bem_profile_enable(bem_ctx* ctx, int enable) {
@@ -1558,7 +1647,7 @@ int bem_autotune(bem_ctx* ctx, int precision, int32_t* chunk_tiles, double* best
     if (ctx->partial) {
         ctx->dfree(ctx->partial);
         ctx->partial = nullptr;
-        ctx->partial_bytes = 0;
+        ctx->partial_bytes = ctx->partial_need = 0;
     }
     if (rc) {
         ctx->opts.chunk_tiles = saved;

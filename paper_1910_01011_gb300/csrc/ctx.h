@@ -105,6 +105,13 @@ struct bem_ctx {
     std::vector<gbem::BlockCache> block_cache;
     void* partial = nullptr;
     size_t partial_bytes = 0;
+    size_t partial_need = 0;    // of the longest source chunks asked for so far; more only speeds calls up
+    // memory that only speeds calls up (room_for, give_back)
+    static constexpr int OPTIONAL_WAIT = 64;
+    int optional_wait = 0;      // calls until the device is asked for it again
+    int pinned = 0;             // calls in progress that hold pointers into it
+    bool frugal = false;        // a call that starts over without it
+    bool short_of_memory = false;  // an allocation was refused
     void* field_buf = nullptr;  // bem_field scratch (grow-only)
     size_t field_buf_bytes = 0;
     // far-field work list (heaviest (target tile, chunk) first) and the launch it was built for
@@ -195,18 +202,38 @@ struct bem_ctx {
     int64_t n_rhs = 1;
 
     int fail(int code, const std::string& msg);
+    void* take(size_t bytes, int* rc, std::string& why);
     void* dalloc(size_t bytes, int* rc);
+    void* try_alloc(size_t bytes);
+    bool room_for(size_t grow);
+    bool give_back();
+    // f with the optional memory in place; once more without it where an allocation was refused
+    template <class F>
+    int without_optional_if_short(F f) {
+        short_of_memory = false;
+        pinned++;
+        int rc = f();
+        pinned--;
+        if (!rc || !short_of_memory || frugal || !give_back()) return rc;
+        frugal = true;
+        pinned++;
+        rc = f();
+        pinned--;
+        frugal = false;
+        return rc;
+    }
     void dfree(void* p);
     int finalize();
     int upload_materials();
     int build_near(gbem::NearSet& ns, int n_slot_k, double kre, double kim, const gbem::SlotCoef* coef_dev);
     int ensure_near();
-    int ensure_partial(int n_chunks, bool fp64);
+    int ensure_partial(size_t need, bool optional);
     int ensure_far_work(int tgt_b, int tgt_e, int src_b, int src_e, int chunk_tiles, int n_chunks, int slot1);
     void chunking(int n_tgt, int n_src, int* n_chunks, int* chunk_tiles, bool fp64) const;
     int plan_apply(const double2* x, double2* y, int precision, const gbem::ApplyMode& m, gbem::ApplyPlan& P,
                    int fill_tiles = 0);
     int run_apply(const double2* x, double2* y, int precision, const gbem::ApplyMode& m);
+    int run_apply_once(const double2* x, double2* y, int precision, const gbem::ApplyMode& m);
     int apply_ahat(const double2* x, double2* y, int precision);
     int apply_ahat_multi(const double2* x, double2* y, int64_t n_rhs);
     int ensure_farmm();

@@ -1,0 +1,72 @@
+"""Device memory that only speeds calls up (the partials of short source
+chunks, the operands of the tensor-core far field): taken where there is room,
+given up without a trace where there is none or another allocation needs it."""
+import numpy as np
+import pytest
+
+from synth import scenes
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def api():
+    from paper_1910_01011_gb300 import api as a
+    return a
+
+
+def device_vectors(s, R):
+    import torch
+    return torch.from_numpy(np.stack([scenes.smooth_trace_vector(s, r) for r in range(R)])).cuda()
+
+
+def error_text(c):
+    return c.lib.bem_last_error(c.h)
+
+
+def test_long_chunks_leave_the_rest_alone(api):
+    """640 tiles: the partials of short source chunks take 0.74 GB, those of
+    four chunks 55 MB.  Under a budget for the latter only, beside the operands
+    of a product of two vectors: one-vector products have the bits of the long
+    chunks, the second allocates nothing, the operands stay in place (same bits
+    as without a budget), and no error text is left behind."""
+    s = scenes.sphere_scene(5)
+    X = device_vectors(s, 2)
+    c = api.Context.from_scene(s)
+    ref2 = c.apply(X, precision=api.FP32)
+    used = c.memory()[0]
+    c.close()
+    c = api.Context.from_scene(s, chunk_tiles=160)
+    ref1 = c.apply(X[0].contiguous(), precision=api.FP32)
+    c.close()
+    c = api.Context.from_scene(s, hbm_budget_bytes=used + (100 << 20))
+    assert (c.apply(X, precision=api.FP32) == ref2).all()
+    assert (c.apply(X[0].contiguous(), precision=api.FP32) == ref1).all()
+    held = c.memory()
+    assert (c.apply(X[0].contiguous(), precision=api.FP32) == ref1).all()
+    assert c.memory() == held
+    assert (c.apply(X, precision=api.FP32) == ref2).all()
+    assert error_text(c) == b""
+    c.close()
+
+
+def test_short_chunks_make_room(api):
+    """Partials of short source chunks that fit at first go when a later call
+    needs the room, and the product after it takes the long chunks."""
+    s = scenes.sphere_scene(5)
+    x = device_vectors(s, 1)[0]
+    c = api.Context.from_scene(s)
+    short = c.apply(x, precision=api.FP32)
+    used = c.memory()[0]
+    c.close()
+    c = api.Context.from_scene(s, chunk_tiles=160)
+    long = c.apply(x, precision=api.FP32)
+    c.close()
+    c = api.Context.from_scene(s, hbm_budget_bytes=used + (1 << 20))
+    assert (c.apply(x, precision=api.FP32) == short).all()
+    c.apply(x, precision=api.FP64)  # split vectors beside the partials
+    c.apply(x, op=api.PREC)         # vectors of the sparse solves
+    y = c.apply(x, precision=api.FP32)
+    assert (y == short).all() or (y == long).all()
+    assert c.memory()[1] <= used + (1 << 20)
+    c.close()
