@@ -124,19 +124,25 @@ bool bem_ctx::room_for(size_t grow) {
 // Frees what only speeds calls up, unless a call in progress holds pointers into it.
 bool bem_ctx::give_back() {
     if (pinned > 0) return false;
-    const bool part = partial && partial_bytes > partial_need;
-    if (!part && !mm_buf) return false;
+    const bool part = partial && partial_bytes > partial_need, multi = multi_buf && multi_buf_bytes > multi_need;
+    if (!part && !multi && !mm_buf && !mmg.buf) return false;
     cudaStreamSynchronize(stream);
     if (part) {
         dfree(partial);
         partial = nullptr;
         partial_bytes = 0;
     }
-    if (mm_buf) {
-        dfree(mm_buf);
-        mm_buf = nullptr;
-        mm_bytes = 0;
-        mm_off = true;
+    if (multi) {
+        dfree(multi_buf);
+        multi_buf = nullptr;
+        multi_buf_bytes = 0;
+    }
+    dfree(mm_buf);
+    mm_buf = nullptr;
+    mm_bytes = 0;
+    if (mmg.buf) {
+        dfree(mmg.buf);
+        mmg = MmGeom();
     }
     return true;
 }
@@ -208,7 +214,7 @@ static void release_device(bem_ctx* ctx) {
     ctx->far_work = nullptr;
     for (int& k : ctx->far_work_key) k = -1;
     ctx->multi_buf = nullptr;
-    ctx->multi_buf_bytes = 0;
+    ctx->multi_buf_bytes = ctx->multi_need = 0;
     ctx->multi64_buf = nullptr;
     ctx->multi64_buf_bytes = 0;
     ctx->dfg = bem_ctx::DfGeom();
@@ -220,7 +226,6 @@ static void release_device(bem_ctx* ctx) {
     ctx->mmg = bem_ctx::MmGeom();
     ctx->mm_buf = nullptr;
     ctx->mm_bytes = 0;
-    ctx->mm_off = false;
     ctx->pmchwt_near = NearSet();
     destroy_solver_state(ctx);
 }
@@ -806,9 +811,12 @@ int bem_ctx::ensure_farmm() {
         mmg.h_ptr[t + 1] = (int)mmg.h_idx.size();
         mmg.fits &= mmg.h_ptr[t + 1] - mmg.h_ptr[t] <= CHUNK_MAX;
     }
+    if (!mmg.fits) {  // never used
+        mmg.ready = true;
+        return BEM_OK;
+    }
     // one buffer, pieces at 256 bytes
     size_t total = 0;
-    int rc = BEM_OK;
     for (int pass = 0; pass < 2; pass++) {
         size_t at = 0;
         cudaError_t e = cudaSuccess;
@@ -826,8 +834,8 @@ int bem_ctx::ensure_farmm() {
         CK(e);
         if (!pass) {
             total = at;
-            mmg.buf = dalloc(total, &rc);
-            if (rc) { mmg.buf = nullptr; return rc; }
+            mmg.buf = try_alloc(total);
+            if (!mmg.buf) return BEM_ERR_OUT_OF_BUDGET;
         }
     }
     CK(cudaStreamSynchronize(stream));
@@ -835,28 +843,33 @@ int bem_ctx::ensure_farmm() {
     return BEM_OK;
 }
 
-// Whether n_rhs vectors go to the tensor cores, with their operands' memory in
-// place: enough tiles for most pairs not to be close, and room in the budgets
-// (of a shared one at most half may be in use: other scenes' reservations do not
-// count these operands).
-bool bem_ctx::reserve_farmm(int64_t n_rhs) {
-    if (mm_off || geo.n_tiles < FARMM_MIN_TILES) return false;
-    if (ensure_farmm() || !mmg.fits) return false;
+// Bytes of mmg.buf, at most.
+static size_t farmm_geometry_bytes(const Geometry& g) {
+    const size_t nt = g.n_tiles;
+    return (size_t)g.n_pts * 56 + (size_t)g.n_slots * 108 +
+           nt * (32 + 36 + 4 + 4 * ((nt + 31) / 32) + 4 * std::min<size_t>(nt, CHUNK_MAX)) + 14 * 256;
+}
+
+// Whether n_rhs vectors go to the tensor cores, with the memory for it in
+// place (`multi`: that of their densities and partials): enough tiles for most
+// pairs not to be close, and room.  Nothing is built or allocated where there is none.
+bool bem_ctx::reserve_farmm(int64_t n_rhs, size_t multi) {
+    if (geo.n_tiles < FARMM_MIN_TILES || (mmg.ready && !mmg.fits)) return false;
     const size_t need = farmm_bytes(geo.n_tiles, n_rhs);
-    if (need <= mm_bytes) return true;
-    dfree(mm_buf);
-    mm_buf = nullptr;
-    mm_bytes = 0;
-    if (pool && pool_limit > 0 && 2 * (pool->load() + (int64_t)need) > pool_limit) return false;
-    int rc;
-    mm_buf = dalloc(need, &rc);
-    if (rc) {
-        mm_buf = nullptr;
-        cudaGetLastError();
-        return false;
+    const size_t grow = (mmg.ready ? 0 : farmm_geometry_bytes(geo)) + (need > mm_bytes ? need - mm_bytes : 0) +
+                        (multi > multi_buf_bytes ? multi - multi_buf_bytes : 0);
+    if (!room_for(grow) || ensure_farmm() || !mmg.fits) return false;
+    if (need > mm_bytes) {
+        dfree(mm_buf);
+        mm_buf = try_alloc(need);
+        mm_bytes = mm_buf ? need : 0;
     }
-    mm_bytes = need;
-    return true;
+    if (mm_buf && multi > multi_buf_bytes) {
+        dfree(multi_buf);
+        multi_buf = try_alloc(multi);
+        multi_buf_bytes = multi_buf ? multi : 0;
+    }
+    return mm_buf && multi <= multi_buf_bytes;
 }
 
 // A_hat applied to n_rhs vectors x [n_rhs][N] -> y [n_rhs][N] at FP32 with
@@ -868,45 +881,37 @@ bool bem_ctx::reserve_farmm(int64_t n_rhs) {
 // far32m_kernel for all (the Green's function and gradient factor of a pair
 // are evaluated once per group of MRG vectors).
 int bem_ctx::apply_ahat_multi(const double2* x, double2* y, int64_t n_rhs) {
-    bem_ctx* const ctx = this;
     int rc = ensure_near();
     if (rc) return rc;
+    return without_optional_if_short([&] { return apply_ahat_multi_once(x, y, n_rhs); });
+}
+
+int bem_ctx::apply_ahat_multi_once(const double2* x, double2* y, int64_t n_rhs) {
+    bem_ctx* const ctx = this;
+    int rc;
     const Geometry& g = geo;
     const int n_tiles = g.n_tiles;
     const int groups = (int)((n_rhs + MRG - 1) / MRG);
-    int n_chunks, chunk_tiles;      // partial rows; source tiles per item
-    bool mm = reserve_farmm(n_rhs);
-    size_t b_pd, b_tc, b_part;
-    int64_t rstride;
-    while (true) {
-        if (mm) {
-            farmm_chunking(n_tiles, g.n_pts, n_rhs, &n_chunks, &chunk_tiles);
-            n_chunks += 1;          // the close tiles
-        } else {
-            multi_chunking(n_tiles, g.n_pts, n_rhs, &n_chunks, &chunk_tiles);
-        }
-        rstride = (int64_t)n_chunks * 2 * NCOMP * g.n_pts;
-        b_pd = (size_t)n_rhs * g.n_pts * sizeof(float4);
-        b_tc = (size_t)n_rhs * 2 * g.n_slots * sizeof(float4);
-        b_part = (size_t)n_rhs * rstride * sizeof(float);
-        const size_t need = b_pd + b_tc + b_part;
-        if (need <= multi_buf_bytes) break;
+    int n_chunks, chunk_tiles, nc, ct;  // partial rows; source tiles per item
+    const size_t b_pd = (size_t)n_rhs * g.n_pts * sizeof(float4);
+    const size_t b_tc = (size_t)n_rhs * 2 * g.n_slots * sizeof(float4);
+    const size_t b_row = (size_t)n_rhs * 2 * NCOMP * g.n_pts * sizeof(float);
+    multi_chunking(n_tiles, g.n_pts, n_rhs, &n_chunks, &chunk_tiles);
+    const size_t need = b_pd + b_tc + n_chunks * b_row;
+    multi_need = std::max(multi_need, need);
+    farmm_chunking(n_tiles, g.n_pts, n_rhs, &nc, &ct);
+    const bool mm = reserve_farmm(n_rhs, b_pd + b_tc + (nc + 1) * b_row);
+    if (mm) {
+        n_chunks = nc + 1;  // one more: the close tiles
+        chunk_tiles = ct;
+    } else if (need > multi_buf_bytes) {
         dfree(multi_buf);
         multi_buf_bytes = 0;
         multi_buf = dalloc(need, &rc);
-        if (rc) multi_buf = nullptr;
-        else multi_buf_bytes = need;
-        if (mm && !mm_buf) {        // the operands made room for it: start over without them
-            mm = false;
-            continue;
-        }
-        if (rc && mm) {
-            mm = false;
-            continue;
-        }
         if (rc) return rc;
-        break;
+        multi_buf_bytes = need;
     }
+    const int64_t rstride = (int64_t)n_chunks * 2 * NCOMP * g.n_pts;
     float4* pdm = (float4*)multi_buf;
     float4* tcm = (float4*)((char*)multi_buf + b_pd);
     float* part = (float*)((char*)multi_buf + b_pd + b_tc);
@@ -947,8 +952,7 @@ int bem_ctx::apply_ahat_multi(const double2* x, double2* y, int64_t n_rhs) {
         multi_work = nullptr;
         for (int& k : multi_key) k = -1;
         multi_work = (int4*)dalloc(work.size() * sizeof(int4), &rc);
-        if (rc) { multi_work = nullptr; return rc; }
-        if (mm && !mm_buf) return apply_ahat_multi(x, y, n_rhs);  // the operands made room for the list
+        if (rc) return rc;
         CK(cudaMemcpyAsync(multi_work, work.data(), work.size() * sizeof(int4), cudaMemcpyHostToDevice, stream));
         CK(cudaStreamSynchronize(stream));
         multi_n_work = (int64_t)work.size();

@@ -120,6 +120,7 @@ struct bem_ctx {
     // several right-hand sides in one far-field launch: densities, partials and the work list
     void* multi_buf = nullptr;
     size_t multi_buf_bytes = 0;
+    size_t multi_need = 0;      // of the FP32 kernel alone; more is for the tensor cores
     void* multi64_buf = nullptr;  // FP64 multi-vector far field: densities, curls, partial potentials
     size_t multi64_buf_bytes = 0;
     struct DfGeom {                // double-float far field: split geometry, tables, constants
@@ -155,9 +156,8 @@ struct bem_ctx {
         int near_words = 0;
         float rho = 1.f;
     } mmg;
-    void* mm_buf = nullptr;        // its B operands (grow-only; given back when the budget is needed elsewhere)
+    void* mm_buf = nullptr;        // its B operands
     size_t mm_bytes = 0;
-    bool mm_off = false;           // given back once: stay with the FP32 kernel
     int64_t multi_n_far = 0;       // work items of the tensor-core kernel at the head of multi_work
     std::vector<std::pair<void*, size_t>> allocs;
     size_t used_bytes = 0;
@@ -236,8 +236,9 @@ struct bem_ctx {
     int run_apply_once(const double2* x, double2* y, int precision, const gbem::ApplyMode& m);
     int apply_ahat(const double2* x, double2* y, int precision);
     int apply_ahat_multi(const double2* x, double2* y, int64_t n_rhs);
+    int apply_ahat_multi_once(const double2* x, double2* y, int64_t n_rhs);
     int ensure_farmm();
-    bool reserve_farmm(int64_t n_rhs);
+    bool reserve_farmm(int64_t n_rhs, size_t multi);
     int apply_ahat64_multi(const double2* x, double2* y, int64_t n_rhs);
     int ensure_fardf();
     int upload_df_wavenumbers();

@@ -70,3 +70,44 @@ def test_short_chunks_make_room(api):
     assert (y == short).all() or (y == long).all()
     assert c.memory()[1] <= used + (1 << 20)
     c.close()
+
+
+def test_tensor_core_operands_come_back(api):
+    """The operands of several vectors' products go when another allocation
+    needs their room (vectors staged from the host), and are there again, with
+    the same bits, once that room is free."""
+    s = scenes.sphere_scene(4)
+    X = device_vectors(s, 16)
+    c = api.Context.from_scene(s)
+    ref = c.apply(X, precision=api.FP32)
+    used = c.memory()[0]
+    c.close()
+    c = api.Context.from_scene(s, hbm_budget_bytes=used + (1 << 20))
+    assert (c.apply(X, precision=api.FP32) == ref).all()
+    y = c.apply(X.cpu().numpy(), precision=api.FP32)  # 2.6 MB of staging
+    assert np.linalg.norm(y - ref.cpu().numpy()) < 1e-5 * np.linalg.norm(y)
+    assert c.memory()[0] < used - (1 << 22)
+    assert (c.apply(X, precision=api.FP32) == ref).all()
+    assert error_text(c) == b""
+    c.close()
+
+
+def test_no_room_for_the_operands(api):
+    """A budget that misses the operands of 16 vectors by 4 MiB: the product by
+    the FP32 kernel alone, nothing of the tensor cores' memory held, no error
+    text, and nothing allocated by the second product."""
+    s = scenes.sphere_scene(4)
+    X = device_vectors(s, 16)
+    c = api.Context.from_scene(s)
+    ref = c.apply(X, precision=api.FP32)
+    used = c.memory()[0]
+    c.close()
+    c = api.Context.from_scene(s, hbm_budget_bytes=used - (1 << 22))
+    y = c.apply(X, precision=api.FP32)
+    assert (y - ref).norm() < 1e-5 * ref.norm()
+    assert error_text(c) == b""
+    held = c.memory()
+    assert (c.apply(X, precision=api.FP32) == y).all()
+    assert c.memory() == held
+    assert error_text(c) == b""
+    c.close()
