@@ -286,7 +286,8 @@ int bem_memory_info(const bem_ctx* ctx, int64_t* used_bytes, int64_t* peak_bytes
  * options alone (no device work): geometry, near-field blocks and their
  * build scratch, far-field partials, right-hand sides, GMRES basis, the
  * preconditioner's batched vectors and, with operator_mode 1, the assembled
- * operators. */
+ * operators.  Memory that only speeds products up, taken where the budget has
+ * room beyond this and given back when it is needed, is not counted. */
 int bem_estimate_solve_bytes(const bem_ctx* ctx, int64_t n_exc, const bem_solve_opts* opts, int64_t* bytes);
 
 /* Several meshes at once (no counterpart in the paper; for many small

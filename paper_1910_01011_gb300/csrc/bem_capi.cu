@@ -83,7 +83,9 @@ void* bem_ctx::dalloc(size_t bytes, int* rc) {
     std::string why;
     void* p = take(bytes, rc, why);
     if (!p && give_back()) p = take(bytes, rc, why);
-    if (!p) {
+    if (p) {
+        note_need();
+    } else {
         short_of_memory = true;
         fail(*rc, why);
     }
@@ -100,14 +102,17 @@ void* bem_ctx::try_alloc(size_t bytes) {
 }
 
 // Whether `grow` bytes more may go to such memory: within the context's budget,
-// at most half of a shared one (other contexts' reservations do not count it),
-// and as much again left free on the device.  After a refusal by the device
+// within half of a shared one next to all that is held of and promised out of
+// it, and as much again left free on the device.  After a refusal by the device
 // the next OPTIONAL_WAIT calls do not ask it again.
 bool bem_ctx::room_for(size_t grow) {
     if (grow == 0) return true;
     if (frugal) return false;
     if (opts.hbm_budget_bytes > 0 && (int64_t)(used_bytes + grow) > opts.hbm_budget_bytes) return false;
-    if (pool && pool_limit > 0 && 2 * (pool->load() + (int64_t)grow) > pool_limit) return false;
+    if (pool_wanted && pool_wanted->load()) return false;
+    if (pool && pool_limit > 0 &&
+        2 * (pool->load() + (pool_reserved ? pool_reserved->load() : 0) + (int64_t)grow) > pool_limit)
+        return false;
     if (optional_wait > 0) {
         optional_wait--;
         return false;
@@ -144,7 +149,19 @@ bool bem_ctx::give_back() {
         dfree(mmg.buf);
         mmg = MmGeom();
     }
+    note_need();
     return true;
+}
+
+size_t bem_ctx::optional_bytes() const {
+    return (partial_bytes > partial_need ? partial_bytes - partial_need : 0) +
+           (multi_buf_bytes > multi_need ? multi_buf_bytes - multi_need : 0) + mm_bytes + mmg.bytes;
+}
+
+void bem_ctx::note_need() {
+    const size_t o = optional_bytes();
+    optional_now.store((int64_t)o);
+    peak_need = std::max(peak_need, used_bytes - std::min(o, used_bytes));
 }
 
 void bem_ctx::dfree(void* p) {
@@ -226,6 +243,7 @@ static void release_device(bem_ctx* ctx) {
     ctx->mmg = bem_ctx::MmGeom();
     ctx->mm_buf = nullptr;
     ctx->mm_bytes = 0;
+    ctx->optional_now.store(0);
     ctx->pmchwt_near = NearSet();
     destroy_solver_state(ctx);
 }
@@ -288,11 +306,11 @@ int64_t estimate_solve_bytes(const bem_ctx* ctx, int64_t n_exc, const bem_solve_
     b += pts * 152 + slots * 460 + pairs * 12 + N * 64 + tiles * 64;
     // near-field blocks (c128 + c64) and their build scratch
     b += pairs * 36 * 24 + std::min<int64_t>(pairs, 1 << 20) * 2 * 27 * 16;
-    // far-field partial potentials (one buffer for the FP32 operator and the FP64 residual)
-    int nc = 1, nc64 = 1, ct = 1;
-    ctx->chunking((int)tiles, (int)tiles, &nc, &ct, false);
-    ctx->chunking((int)tiles, (int)tiles, &nc64, &ct, true);
-    b += std::max((int64_t)nc * 4, (int64_t)nc64 * 8) * 2 * NCOMP * pts;
+    // far-field partial potentials of the longest chunks (one buffer for the FP32 operator and the FP64 residual, which
+    // is the larger); short chunks' and the tensor-core far field's memory is not needed and not counted
+    int nc = 1, ct = 1;
+    ctx->chunking((int)tiles, (int)tiles, &nc, &ct, true);
+    b += (int64_t)nc * 2 * NCOMP * pts * 8;
     // right-hand sides, solutions, piston data
     b += n_exc * (2 * N * 16 + slots * 6 * 16 + ne * 16) + ne * 32 * 32 + 3 * N * 16;
     // GMRES basis and work (per lockstep column)
@@ -836,6 +854,7 @@ int bem_ctx::ensure_farmm() {
             total = at;
             mmg.buf = try_alloc(total);
             if (!mmg.buf) return BEM_ERR_OUT_OF_BUDGET;
+            mmg.bytes = total;
         }
     }
     CK(cudaStreamSynchronize(stream));

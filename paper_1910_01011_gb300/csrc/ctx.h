@@ -112,6 +112,7 @@ struct bem_ctx {
     int pinned = 0;             // calls in progress that hold pointers into it
     bool frugal = false;        // a call that starts over without it
     bool short_of_memory = false;  // an allocation was refused
+    std::atomic<int64_t> optional_now{0};  // bytes of it held, for the request loop
     void* field_buf = nullptr;  // bem_field scratch (grow-only)
     size_t field_buf_bytes = 0;
     // far-field work list (heaviest (target tile, chunk) first) and the launch it was built for
@@ -155,6 +156,7 @@ struct bem_ctx {
         std::vector<int> h_ptr, h_idx;
         int near_words = 0;
         float rho = 1.f;
+        size_t bytes = 0;
     } mmg;
     void* mm_buf = nullptr;        // its B operands
     size_t mm_bytes = 0;
@@ -162,10 +164,13 @@ struct bem_ctx {
     std::vector<std::pair<void*, size_t>> allocs;
     size_t used_bytes = 0;
     size_t peak_bytes = 0;                     // largest used_bytes seen
+    size_t peak_need = 0;                      // the same without memory that only speeds calls up
     uint64_t gen = 0;                          // bumped by every device allocation and release
     gbem::GroupCache* group = nullptr;         // bem_apply_group state when this context leads a group
     std::atomic<int64_t>* pool = nullptr;      // shared device-memory counter (serving), or null
     int64_t pool_limit = 0;                    // limit of the shared counter (0: none)
+    const std::atomic<int64_t>* pool_reserved = nullptr;  // promised out of it to admitted solves
+    const std::atomic<bool>* pool_wanted = nullptr;       // a request waits for optional memory of running solves
     bool own_stream = false;                   // stream created by the library, destroyed with the context
     long long launches = 0;
     bool profiling = false;
@@ -207,19 +212,24 @@ struct bem_ctx {
     void* try_alloc(size_t bytes);
     bool room_for(size_t grow);
     bool give_back();
+    size_t optional_bytes() const;
+    void note_need();
     // f with the optional memory in place; once more without it where an allocation was refused
     template <class F>
     int without_optional_if_short(F f) {
+        if (pool_wanted && pool_wanted->load()) give_back();
         short_of_memory = false;
         pinned++;
         int rc = f();
         pinned--;
+        note_need();
         if (!rc || !short_of_memory || frugal || !give_back()) return rc;
         frugal = true;
         pinned++;
         rc = f();
         pinned--;
         frugal = false;
+        note_need();
         return rc;
     }
     void dfree(void* p);

@@ -48,7 +48,7 @@ struct Scene {
     int64_t n_elem = 0;
     int64_t n_dofs = 0;
     bool busy = false;
-    int64_t peak = 0;        // largest device footprint seen (bytes)
+    int64_t peak = 0;        // largest device footprint seen (bytes), without memory that only speeds calls up
     Clock::time_point last;  // last use, for eviction
 };
 
@@ -78,7 +78,8 @@ struct bem_server {
     std::map<int64_t, std::unique_ptr<Request>> reqs;
     std::deque<int64_t> queue;
     std::atomic<int64_t> pool{0};  // device bytes held by all scenes
-    int64_t reserved = 0;          // admitted growth not yet allocated
+    std::atomic<int64_t> reserved{0};  // admitted growth not yet allocated
+    std::atomic<bool> wanted{false};   // running solves give their optional memory back for a waiting request
     int64_t next_handle = 1;
     int running = 0;
     bool stop = false;
@@ -142,7 +143,10 @@ bool bem_server::pick(std::vector<Request*>& group, Scene*& sc, int64_t& extra) 
             need = std::max(need, s->peak + s->peak / 4);
             if (opts.hbm_budget_bytes > 0) need = std::min<int64_t>(need, opts.hbm_budget_bytes);
         }
-        int64_t grow = std::max<int64_t>(0, need - (int64_t)s->ctx->used_bytes);
+        auto growth = [&] {
+            return std::max<int64_t>(0, need - ((int64_t)s->ctx->used_bytes - s->ctx->optional_now.load()));
+        };
+        int64_t grow = growth();
         if (budget > 0 && need > budget) {
             // r0 alone can never fit (the group holds only r0 then)
             r0->state = BEM_REQ_FAILED;
@@ -153,6 +157,12 @@ bool bem_server::pick(std::vector<Request*>& group, Scene*& sc, int64_t& extra) 
             queue.erase(queue.begin() + qi);
             cv_done.notify_all();
             return pick(group, sc, extra);
+        }
+        // memory of idle scenes that only speeds their calls up goes first
+        if (budget > 0 && pool.load() + reserved + grow > budget) {
+            for (auto& o : scenes)
+                if (!o->busy) o->ctx->give_back();
+            grow = growth();
         }
         while (budget > 0 && pool.load() + reserved + grow > budget) {
             // evict the least recently used idle scene that holds memory
@@ -171,7 +181,12 @@ bool bem_server::pick(std::vector<Request*>& group, Scene*& sc, int64_t& extra) 
                 grow = need;
                 if (pool.load() + reserved + grow > budget) return false;
             } else {
-                return false;  // wait for a running solve to finish (keeps FIFO order)
+                // wait for a running solve to finish (keeps FIFO order), or to give back what it can do without
+                int64_t optional = 0;
+                for (auto& o : scenes)
+                    if (o->busy) optional += o->ctx->optional_now.load();
+                wanted = optional > 0 && pool.load() + reserved + grow - optional <= budget;
+                return false;
             }
         }
         // admit
@@ -182,8 +197,10 @@ bool bem_server::pick(std::vector<Request*>& group, Scene*& sc, int64_t& extra) 
         sc = s;
         extra = grow;
         reserved += grow;
+        wanted = false;
         return true;
     }
+    wanted = false;
     return false;
 }
 
@@ -194,7 +211,10 @@ void bem_server::worker() {
         std::vector<Request*> group;
         Scene* s = nullptr;
         int64_t extra = 0;
-        while (!stop && !pick(group, s, extra)) cv_work.wait(lk);
+        while (!stop && !pick(group, s, extra)) {
+            if (wanted) cv_work.wait_for(lk, std::chrono::milliseconds(5));
+            else cv_work.wait(lk);
+        }
         if (stop) return;
         running++;
         const auto t0 = Clock::now();
@@ -229,7 +249,8 @@ void bem_server::worker() {
                     const int64_t add = std::max<int64_t>(
                         0, estimate_solve_bytes(ctx, n_cur + k + r->n_exc, opts.solve) -
                                estimate_solve_bytes(ctx, n_cur + k, opts.solve));
-                    if (opts.hbm_budget_bytes > 0 && pool.load() + reserved + add > opts.hbm_budget_bytes) {
+                    auto over = [&] { return opts.hbm_budget_bytes > 0 && pool.load() + reserved + add > opts.hbm_budget_bytes; };
+                    if (over() && (!ctx->give_back() || over())) {
                         qi++;
                         continue;
                     }
@@ -267,7 +288,7 @@ void bem_server::worker() {
         reserved -= extra;
         s->busy = false;
         s->last = t1;
-        s->peak = std::max<int64_t>(s->peak, (int64_t)ctx->peak_bytes);
+        s->peak = std::max<int64_t>(s->peak, (int64_t)ctx->peak_need);
         peak_pool = std::max(peak_pool, pool.load());
         batches++;
         batch_exc_sum += n;
@@ -352,6 +373,8 @@ int bem_server_destroy(bem_server* s) {
     for (auto& t : s->workers) t.join();
     for (auto& sc : s->scenes) {
         sc->ctx->pool = nullptr;
+        sc->ctx->pool_reserved = nullptr;
+        sc->ctx->pool_wanted = nullptr;
         bem_destroy(sc->ctx);
     }
     delete s;
@@ -369,6 +392,8 @@ int bem_server_add_scene(bem_server* s, bem_ctx* ctx, int32_t* scene_id) {
     s->pool += (int64_t)ctx->used_bytes;
     ctx->pool = &s->pool;
     ctx->pool_limit = s->opts.hbm_budget_bytes;
+    ctx->pool_reserved = &s->reserved;
+    ctx->pool_wanted = &s->wanted;
     if (!ctx->stream) {
         // a stream of its own, so that this scene's kernels overlap with the
         // other scenes' (the legacy default stream would serialise them)

@@ -111,3 +111,53 @@ def test_no_room_for_the_operands(api):
     assert c.memory() == held
     assert error_text(c) == b""
     c.close()
+
+
+def test_estimate_counts_what_a_solve_needs(api):
+    """640 tiles: the solve's estimate is that of the longest source chunks,
+    and the solve runs under it."""
+    s = scenes.sphere_scene(5)
+    kw = dict(precision=api.FP32, tol=1e-3, operator_mode=0, max_iter=60)
+    est = []
+    for chunk in (160, 0):
+        c = api.Context.from_scene(s, chunk_tiles=chunk, r_eps=0.2)
+        est.append(c.estimate_solve_bytes(1, **kw))
+        c.close()
+    assert est[0] == est[1]
+    c = api.Context.from_scene(s, hbm_budget_bytes=est[0], r_eps=0.2)
+    c.set_plane_wave((0, 0, 1))
+    c.solve(**kw)
+    assert c.memory()[1] <= est[0]
+    c.close()
+
+
+@pytest.mark.parametrize("share", [1.25, 3.5])
+def test_served_scenes_share_a_budget(api, share):
+    """Two scenes whose matrix-free solves of eight excitations take the
+    tensor-core far field where the budget has room, under one that holds a
+    little more than one of them (idle scenes are evicted) and one that holds
+    both running: every request completes, within the budget, with the
+    solutions found without a limit."""
+    tr = scenes.bowl_transducer(seed=0, n_elem=6, R=4.0, aperture=3.0, piston_radius=0.3, gap=0.05)
+    kw = dict(precision=api.FP32, tol=1e-8, operator_mode=0, batch_rhs=8, block_gmres=1)
+    W = [np.exp(2j * np.pi * np.random.default_rng(i).random((8, 6))) for i in range(2)]
+
+    def serve(budget, rounds):
+        srv = api.Server(slots=2, max_batch_rhs=8, hbm_budget_bytes=budget, join=0, **kw)
+        ids = [srv.add_scene(scenes.sphere_scene(4, k0=4.0 + i), transducer=tr, omega_rho0=2.6, r_eps=0.2) for i in range(2)]
+        est = max(srv.estimate(i, 8) for i in ids)
+        hs = [(i, srv.submit(ids[i], W[i])) for _ in range(rounds) for i in range(2)]
+        out = {}
+        for i, h in hs:
+            assert srv.wait(h, 600) == 2, srv.error(h)
+            out[i] = srv.result(h, 8, ids[i])[0]
+        st = srv.stats()
+        srv.close()
+        assert st["completed"] == 2 * rounds and st["failed"] == 0
+        assert budget == 0 or st["peak_device_bytes"] <= budget
+        return out, est
+
+    ref, est = serve(0, 1)
+    out, _ = serve(int(share * est), 3)
+    for i in range(2):
+        assert np.linalg.norm(out[i] - ref[i]) < 1e-6 * np.linalg.norm(ref[i])
