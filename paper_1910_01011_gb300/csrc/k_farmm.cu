@@ -13,12 +13,13 @@
 // further right-hand side; here they are a tcgen05 contraction, and the FP32
 // and MUFU pipes only evaluate G and F.
 //
-//  * Precision: every FP32 value is split into two FP16 numbers, 11 bits in
-//    the first and the rest, rounded to 11, in the second: 2^-23 of the value,
-//    below FP32's own rounding in a sum of such terms.  Products with FP16
-//    operands are exact in FP32.  Three of the four products are kept
-//    (2^-22 of a term dropped), hi hi in one accumulator, the two cross terms
-//    in another.  Powers of two bring G and F (by the distance of the tiles)
+//  * Precision: every FP32 value is split into two FP16 numbers of 11 bits:
+//    densities rounded to the first and the rest rounded to the second (2^-23
+//    of the value at most), G and F truncated, which takes fewer instructions,
+//    and the rest rounded (2^-22).  Products with FP16 operands are exact in
+//    FP32.  Three of the four products are kept, hi hi in one accumulator, the
+//    two cross terms in another; the fourth is at most 2^-21 of a term, and of
+//    either sign because the densities' second numbers are.  Powers of two bring G and F (by the distance of the tiles)
 //    and the densities (by the vector's largest) to 2^8 at most, so that
 //    nothing leaves FP16's range and small values keep 2^-33 of the largest.
 //    The tensor cores truncate when they accumulate, so an accumulator takes
@@ -41,8 +42,9 @@
 //    eight points still takes 400 of its 550 cycles; the tensor pipe itself needs
 //    242).  Kidney scene of 12,184 triangles, 16 right-hand sides: far field
 //    139.6 ms with far32m_kernel for all pairs of tiles, now 58 + 9 ms (close
-//    pairs); relative error against 64 bits on 127-146 tiles 1.0-1.4e-6 (5.5e-6
-//    at k r of several hundred), before 1.5-2.4e-6 (1.3e-5).
+//    pairs); relative error against 64 bits on 121-178 tiles 0.9-1.3e-6 (5.4e-6
+//    at k r of several hundred; 1.0-1.4e-6 with densities truncated too), before
+//    1.5-2.4e-6 (1.3e-5).
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -594,8 +596,8 @@ __global__ void __launch_bounds__(64) farmm_pack_kernel(const float4* __restrict
     }
     // K of this point within its step of eight: (Gr, Gr, Gi, Gi) per pair of points
     const int kk = k >> 3, pt = k & 7, kre = kk * 16 + (pt >> 1) * 4 + (pt & 1), kim = kre + 2;
-    auto put = [&](int row, int kx, float x) {
-        *reinterpret_cast<__half*>(sb + row * 64 + (((kx >> 3) ^ ((row >> 1) & 3)) << 4) + (kx & 7) * 2) = __float2half_rn(x);
+    auto put = [&](int row, int kx, __half x) {
+        *reinterpret_cast<__half*>(sb + row * 64 + (((kx >> 3) ^ ((row >> 1) & 3)) << 4) + (kx & 7) * 2) = x;
     };
 #pragma unroll
     for (int f = 0; f < 2; f++)
@@ -604,12 +606,12 @@ __global__ void __launch_bounds__(64) farmm_pack_kernel(const float4* __restrict
 #pragma unroll
             for (int z = 0; z < 2; z++) {  // output part: re = Gr d.re - Gi d.im, im = Gr d.im + Gi d.re
                 const float a = col[f][c][z], b = z ? col[f][c][0] : -col[f][c][1];
-                const float ah = __uint_as_float(__float_as_uint(a) & 0xffffe000u), bh = __uint_as_float(__float_as_uint(b) & 0xffffe000u);
+                const __half ah = __float2half_rn(a), bh = __float2half_rn(b);
                 const int row = f * 2 * MM_N + v * 16 + 2 * c + z;
                 put(row, kre, ah);
                 put(row, kim, bh);
-                put(row + MM_N, kre, a - ah);
-                put(row + MM_N, kim, b - bh);
+                put(row + MM_N, kre, __float2half_rn(a - __half2float(ah)));
+                put(row + MM_N, kim, __float2half_rn(b - __half2float(bh)));
             }
     __syncthreads();
     uint4* dst = reinterpret_cast<uint4*>(out + ((int64_t)grp * gridDim.x + stage) * MM_BBYTES);

@@ -294,3 +294,19 @@ def test_fp64_assembled_digits_by_columns(api):
             largest = np.maximum.reduceat(np.abs(A[r]) / c0, units) * np.maximum.reduceat(np.abs(X[v]) * c0, units) * 4
             bound = 6 * np.sqrt(512) * 2.0 ** -54 * np.linalg.norm(largest)  # (4: powers of two above both)
             assert max(dr, di) < bound, (i, v, float(max(dr, di)), bound)
+
+
+@pytest.mark.parametrize("name,R", [("ribs", 4), ("kidney", 6)])
+def test_tensor_core_far_field_error(api, name, R):
+    """The same product to the accuracy of its numbers: FP32 evaluation of the
+    phase, 1/r and the gradient factor is good to a few 2^-23 of a term, the
+    FP16 pairs keep 2^-21 of it, and the sums are rounded to nearest per
+    source tile: together 2^-18 leaves a factor of four."""
+    s = {"ribs": lambda: scenes.rib_scene(h=9e-3, freq=0.03e6), "kidney": lambda: scenes.kidney_scene(h=7.5e-3, freq=0.04e6)}[name]()
+    c = api.Context.from_scene(s)
+    X = np.stack([scenes.smooth_trace_vector(s, r) for r in range(R)])
+    Y = c.apply(X, precision=api.FP32)
+    Z = c.apply(X, precision=api.FP64)
+    c.close()
+    for r in range(R):
+        assert rel(Y[r], Z[r]) < 2.0 ** -18, r
