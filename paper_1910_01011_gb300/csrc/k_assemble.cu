@@ -280,15 +280,20 @@ __global__ void __launch_bounds__(TT) assemble64_kernel(AssembleArgs a, const do
 //  1. a thread forms the P1 moments of V, K and K' over the source's six points,
 //  2. the six threads of a triangle exchange them through shared memory and
 //     contract them with the test functions,
-//  3. and add the W terms,
-//  4. the sums over the triangles that meet at a vertex of the target tile
+//  3. the sums over the triangles that meet at a vertex of the target tile
 //     (about 22 vertices for 96 corners) go to the matrix with their block
 //     coefficients: ~530 FP64 atomics per source triangle instead of 2,304,
-//     and the only FP64 arithmetic.
+//  4. and W from the same V: curl . curl' V, whose sums over a vertex cancel to
+//     (h k)^2 of their terms, in FP64, each target vertex's sum of curl V once
+//     for the three source vertices; -k^2 n.n' V, which does not cancel, in
+//     FP32 pairs up to the vertex and FP64 from there.
 // (One thread per target triangle held 54 accumulators, 255 registers and
 // eight warps on an SM with long dependent chains.)
-// 4,620-triangle rib scene, both wavenumbers: 64.6 ms before, 39.1 ms
-// now (two CTAs with 165 registers; three with 112 spilled: 41.4 ms).
+// New exterior medium of the 4,620-triangle rib scene 114 ms, 135 ms with that
+// kernel (two CTAs with 164 registers an SM; three with 112 spilled).  All of W
+// in FP32 pairs took 110 ms, but the entries' error against native FP64, six
+// scenes on average, grew from 1.780e-14 to 1.884e-14 (now 1.778e-14), and row
+// sums of W, which are zero without a wavenumber, fivefold.
 struct AssembleDf {
     const float4 *pgh, *pgl, *tgh, *tgl, *tch, *tcl;  // split geometry (bem_ctx::ensure_fardf)
     const float4* kdf;        // [n_dom] (Re k hi, lo, Im k hi, lo)
@@ -306,20 +311,30 @@ struct AsmDfSmem {
     float4 sph[TP], spl[TP];  // source points of a tile
     float4 sgh[TT], sgl[TT];  // its triangles (n, h)
     dfl wl[TT][QP][3];        // weight x P1 values
-    dfl cs[TT][9];            // curls [3 b + c]
+    double cs[TT][9];         // curls [3 b + c]
     int4 sv[TT];
-    dfl ct[9][TT];            // curls of the target triangles [3 i + c]
+    double ct[3][3 * TT];     // curls [component][corner] of the target triangles
     dfl val[18][TP];          // V, K, K' [source vertex][re, im] of each target point
-    dfl mom[3][8][3 * TT];    // [source vertex][V, K, K', W (re, im)][corner 32 i + triangle]
+    dfl mom[3][6][3 * TT];    // [source vertex][V, K, K' (re, im)][corner 32 i + triangle]
+    double vsum[2][3 * TT];   // [re, im][corner]: V over the source's vertices
+    dfl nn[TT];               // n.n'
     int vert[3 * TT];         // the target tile's vertices
     unsigned char ptr[3 * TT + 1], cor[3 * TT];  // corners of each
     int id[3 * TT];           // vertex of each corner (-1: padding)
     int nv;
 };
 
-__device__ __forceinline__ dfl dsplit(double v) {
-    const float h = (float)v;
-    return dfl{h, (float)(v - (double)h)};
+// A sum of FP32 pairs to FP64: the leading sum, its errors and the low parts in a second, the errors of that in a third.
+__device__ __forceinline__ double pair_sum(const dfl (&v)[3]) {
+    float s = 0.0f, e = 0.0f, f = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const dfl a = two_sum(s, v[k].h), b = two_sum(e, a.l), c = two_sum(b.h, v[k].l);
+        s = a.h;
+        e = c.h;
+        f = __fadd_rn(f, __fadd_rn(b.l, c.l));
+    }
+    return (double)s + ((double)e + (double)f);
 }
 
 // The vertices of the target tile and, for each, its corners in ascending order (one warp).
@@ -386,9 +401,9 @@ __device__ __forceinline__ void assembledf_body(const AssembleArgs& a, const Ass
     const float4 xh = d.pgh[ts * QP + qx], xl = d.pgl[ts * QP + qx];
     const dfl xw = dmul(dfl{xh.w, xl.w}, dfl{d.i4h, d.i4l});
     if (tid < TT) tile_vertices(sm, a.slot_v[(int64_t)tt * TT + tid]);
-    for (int e = tid; e < 9 * TT; e += TP) sm.ct[e % 9][e / 9] = dsplit(a.slot_curl[(int64_t)tt * TT * 9 + e]);
-    // test function and part (of 18 moments, or re / im of W) of this thread in steps 2 and 3
-    const int i = qx % 3, half = qx / 3, corner = i * TT + tl;
+    for (int e = tid; e < 9 * TT; e += TP) sm.ct[e % 3][e % 9 / 3 * TT + e / 9] = a.slot_curl[(int64_t)tt * TT * 9 + e];
+    // test function, and real or imaginary parts, of this thread in step 2
+    const int i = qx % 3, part = qx / 3, corner = i * TT + tl;
     for (int s = sb; s < se; s++) {
         const int ntri = a.tntri[s];
         __syncthreads();  // the last triangle of the tile before is done
@@ -404,7 +419,7 @@ __device__ __forceinline__ void assembledf_body(const AssembleArgs& a, const Ass
                 sm.sgl[tid] = d.tgl[(int64_t)s * TT + tid];
                 sm.sv[tid] = a.slot_v[(int64_t)s * TT + tid];
             }
-            for (int e = tid; e < 9 * TT; e += TP) sm.cs[e / 9][e % 9] = dsplit(a.slot_curl[(int64_t)s * TT * 9 + e]);
+            for (int e = tid; e < 9 * TT; e += TP) sm.cs[e / 9][e % 9] = a.slot_curl[(int64_t)s * TT * 9 + e];
         }
         const float4 csh = d.tch[s], csl = d.tcl[s];
         const dfl Xx = dadd(dfl{xh.x, xl.x}, dsub(dfl{cth.x, ctl.x}, dfl{csh.x, csl.x}));
@@ -452,60 +467,73 @@ __device__ __forceinline__ void assembledf_body(const AssembleArgs& a, const Ass
 #pragma unroll
             for (int k = 0; k < 18; k++) sm.val[k][tid] = h[k];
             __syncthreads();
-            // 2. against the test functions: moments 9 half ... 9 half + 8 of corner (triangle tl, function i)
+            // 2. against the test functions: real or imaginary parts of corner (triangle tl, function i)
             {
-                dfl m[9];
+                dfl m[3][3];
 #pragma unroll
-                for (int k = 0; k < 9; k++) m[k] = dfl{0.0f, 0.0f};
+                for (int k = 0; k < 3; k++)
+#pragma unroll
+                    for (int b = 0; b < 3; b++) m[k][b] = dfl{0.0f, 0.0f};
 #pragma unroll
                 for (int q = 0; q < QP; q++) {
                     const dfl lam = {d.lamh[q][i], d.laml[q][i]};
 #pragma unroll
-                    for (int k = 0; k < 9; k++) dmac(m[k], sm.val[9 * half + k][tl * QP + q], lam, 1.0f);
+                    for (int k = 0; k < 3; k++)
+#pragma unroll
+                        for (int b = 0; b < 3; b++) dmac(m[k][b], sm.val[6 * k + 2 * b + part][tl * QP + q], lam, 1.0f);
                 }
 #pragma unroll
-                for (int k = 0; k < 9; k++) {
-                    const int c = 9 * half + k, kind = c / 6, b = c % 6 / 2;
-                    sm.mom[b][2 * kind + (c & 1)][corner] = m[k];
-                }
+                for (int k = 0; k < 3; k++)
+#pragma unroll
+                    for (int b = 0; b < 3; b++) sm.mom[b][2 * k + part][corner] = m[k][b];
+                sm.vsum[part][corner] = pair_sum(m[0]);
+                if (qx == QP - 1) sm.nn[tl] = dadd(dadd(dmul(ngx, snx), dmul(ngy, sny)), dmul(ngz, snz));
             }
             __syncthreads();
-            // 3. W: curl_i . curl_b sum V - k^2 n.n' V, real or imaginary part
-            {
-                dfl sv = {0.0f, 0.0f};
-#pragma unroll
-                for (int b = 0; b < 3; b++)
-#pragma unroll
-                    for (int k = 0; k < 3; k++) sv = dadd(sv, sm.mom[b][half][k * TT + tl]);
-                const dfl nn = dneg(dadd(dadd(dmul(ngx, snx), dmul(ngy, sny)), dmul(ngz, snz)));
-                const dfl pr = dmul(nn, dsplit(cf.k2re)), pi = dmul(nn, dsplit(cf.k2im));
-#pragma unroll
-                for (int b = 0; b < 3; b++) {
-                    const dfl cc = dadd(dadd(dmul(sm.ct[3 * i][tl], sm.cs[sl][3 * b]), dmul(sm.ct[3 * i + 1][tl], sm.cs[sl][3 * b + 1])),
-                                        dmul(sm.ct[3 * i + 2][tl], sm.cs[sl][3 * b + 2]));
-                    const dfl own = sm.mom[b][half][corner], other = sm.mom[b][half ^ 1][corner];
-                    dfl w = dmul(cc, sv);
-                    dmac(w, pr, own, 1.0f);
-                    dmac(w, pi, other, half ? 1.0f : -1.0f);
-                    sm.mom[b][6 + half][corner] = w;
-                }
-            }
-            __syncthreads();
-            // 4. vertex sums of one block (V, K, K' or W) into the matrix
+            // 3. vertex sums of V, K and K' into the matrix
             const int4 sv = sm.sv[sl];
-            for (int e = tid; e < 12 * sm.nv; e += TP) {
-                const int v = e / 12, b = e % 3, blk = e % 12 / 3, vs = b == 0 ? sv.x : b == 1 ? sv.y : sv.z;
+            auto put = [&](int v, int b, int blk, double co, double xr, double xi) {
+                const int id = sm.vert[v], vs = b == 0 ? sv.x : b == 1 ? sv.y : sv.z;
+                const int64_t row = blk < 2 ? a.v_dof1[id] : a.v_dof2[id], col = blk & 1 ? a.v_dof2[vs] : a.v_dof1[vs];
+                double* out = reinterpret_cast<double*>(&A64[row * a.n + col]);
+                atomicAdd(out, co * xr);
+                atomicAdd(out + 1, co * xi);
+            };
+            for (int e = tid; e < 9 * sm.nv; e += TP) {
+                const int v = e / 9, b = e % 3, blk = e % 9 / 3;
                 dfl mr = {0.0f, 0.0f}, mi = {0.0f, 0.0f};
                 for (int k = sm.ptr[v]; k < sm.ptr[v + 1]; k++) {
                     mr = dadd(mr, sm.mom[b][2 * blk][sm.cor[k]]);
                     mi = dadd(mi, sm.mom[b][2 * blk + 1][sm.cor[k]]);
                 }
-                const int id = sm.vert[v];
-                const int64_t row = blk < 2 ? a.v_dof1[id] : a.v_dof2[id], col = blk & 1 ? a.v_dof2[vs] : a.v_dof1[vs];
-                const double co = blk == 0 ? cf.cV : blk == 1 ? -cf.cK : blk == 2 ? cf.cKp : cf.cW;
-                double* out = reinterpret_cast<double*>(&A64[row * a.n + col]);
-                atomicAdd(out, co * ((double)mr.h + (double)mr.l));
-                atomicAdd(out + 1, co * ((double)mi.h + (double)mi.l));
+                put(v, b, blk, blk == 0 ? cf.cV : blk == 1 ? -cf.cK : cf.cKp, (double)mr.h + (double)mr.l,
+                    (double)mi.h + (double)mi.l);
+            }
+            // 4. W in FP64: three lanes per vertex of the target, the last warps first
+            const int lane = tid & 31, b = lane % 3;
+            for (int v0 = (TP / 32 - 1 - tid / 32) * 10; v0 < sm.nv; v0 += TP / 32 * 10) {
+                const int v = v0 + lane / 3;
+                const bool on = lane < 30 && v < sm.nv;
+                double gr = 0, gi = 0;  // component b of the sum of curl x V over the vertex's triangles
+                dfl vr = {0.0f, 0.0f}, vi = {0.0f, 0.0f};
+                for (int k = on ? sm.ptr[v] : 0, e = on ? sm.ptr[v + 1] : 0; k < e; k++) {
+                    const int c = sm.cor[k], t = c % TT;
+                    gr += sm.ct[b][c] * (sm.vsum[0][t] + sm.vsum[0][TT + t] + sm.vsum[0][2 * TT + t]);
+                    gi += sm.ct[b][c] * (sm.vsum[1][t] + sm.vsum[1][TT + t] + sm.vsum[1][2 * TT + t]);
+                    vr = dadd(vr, dmul(sm.nn[t], sm.mom[b][0][c]));
+                    vi = dadd(vi, dmul(sm.nn[t], sm.mom[b][1][c]));
+                }
+                double wr = 0, wi = 0;
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    const double cc = sm.cs[sl][3 * b + c];
+                    wr += cc * __shfl_sync(0xffffffffu, gr, lane - b + c);
+                    wi += cc * __shfl_sync(0xffffffffu, gi, lane - b + c);
+                }
+                if (on) {
+                    const double xr = (double)vr.h + (double)vr.l, xi = (double)vi.h + (double)vi.l;
+                    put(v, b, 3, cf.cW, wr - (cf.k2re * xr - cf.k2im * xi), wi - (cf.k2re * xi + cf.k2im * xr));
+                }
             }
         }
     }

@@ -310,3 +310,22 @@ def test_tensor_core_far_field_error(api, name, R):
     c.close()
     for r in range(R):
         assert rel(Y[r], Z[r]) < 2.0 ** -18, r
+
+
+@pytest.mark.parametrize("level", [2, 3])
+def test_fp64_assembled_hypersingular_rows(api, level):
+    """W keeps FP64's rounding in the double-float assembly.  Without a
+    wavenumber its rows add up to zero whatever the errors of V, because a
+    source triangle's three curls do; what is left is the rounding of its terms
+    and their sums, FP64 in the native assembly as well: at most twice that
+    one's, on average over the rows (sums by atomics: the order differs)."""
+    s = scenes.sphere_scene(level, k0=1e-9, k1=1e-9)
+    left = []
+    for native in (0, 1):
+        c = api.Context.from_scene(s, fp64_far=native)
+        N = c.n_dofs
+        A = c.apply(np.eye(N, dtype=np.complex128), precision=api.FP64_ASSEMBLED).T
+        c.close()
+        W = A[N // 2:, N // 2:].real.astype(np.longdouble)
+        left.append(np.mean(np.abs(W.sum(axis=1)) / np.sqrt((W ** 2).sum(axis=1))))
+    assert left[0] < 2 * left[1], [float(v) for v in left]
