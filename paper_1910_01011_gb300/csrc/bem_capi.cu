@@ -273,8 +273,10 @@ void multi_chunking(int n_tiles, int64_t n_pts, int64_t R, int* n_chunks, int* c
 }
 
 // Chunks of the FP64 multi-vector far field: about 8 CTAs per SM over
-// (target tile, chunk, slot, group), no more (each chunk adds R x 2 x NCOMP
-// x n_pts doubles of partial potentials).
+// (target tile, chunk, slot, group of RG64), no more (each chunk adds R x 2 x
+// NCOMP x n_pts doubles of partial potentials).  The double-float kernel has
+// groups of two, so up to twice as many CTAs: 2,964-triangle rib scene, 5
+// vectors, 40.2 ms; with its own groups counted, and so longer chunks, 41.0 ms.
 void multi64_chunking(int n_tiles, int64_t R, int* n_chunks, int* chunk_tiles) {
     const int64_t groups = (R + RG64 - 1) / RG64;
     int64_t nc = (152 * 8 + 2 * groups * n_tiles - 1) / std::max<int64_t>(1, 2 * groups * n_tiles);
@@ -1048,9 +1050,10 @@ int bem_ctx::apply_ahat_multi_once(const double2* x, double2* y, int64_t n_rhs) 
 }
 
 // A_hat applied to n_rhs vectors at FP64 with one far-field launch for all of
-// them (far64m_kernel: the kernel values of a pair evaluated once per group of
-// RG64 vectors), then the projection (with the FP64 near-field correction) and
-// the reduction of each vector.
+// them (the kernel values of a pair evaluated once per group: two vectors in
+// fardf_kernel, RG64 in far64m_kernel where native FP64 is asked for), then the
+// projection (with the FP64 near-field correction) and the reduction of each
+// vector.
 int bem_ctx::apply_ahat64_multi(const double2* x, double2* y, int64_t n_rhs) {
     bem_ctx* const ctx = this;
     int rc = ensure_near();

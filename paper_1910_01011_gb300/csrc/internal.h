@@ -1,12 +1,12 @@
 // internal.h -- data layout shared by the library's translation units.
 //
-// Triangles are stored tile-ordered: each domain's triangles are halved
-// recursively across the longest extent of their centroids into tiles of TT
-// triangles (the last tile of a domain is padded).  A tile carries its
-// centre in FP64; every point and plane offset of the tile is stored
-// relative to that centre, so FP32 differences between points of two tiles
-// keep their accuracy (the far-field phase is reconstructed from an FP64
-// tile-pair distance plus an FP32 local offset).
+// Triangles are stored tile-ordered: each domain's triangles, sorted along a
+// Morton curve of their centroids, are cut into tiles of TT triangles (the last
+// tile of a domain is padded; the tensor-core far field has tiles of its own,
+// CompactTiles).  A tile carries its centre in FP64; every point and plane
+// offset of the tile is stored relative to that centre, so FP32 differences
+// between points of two tiles keep their accuracy (the far-field phase is
+// reconstructed from an FP64 tile-pair distance plus an FP32 local offset).
 #pragma once
 
 #include <cuda_runtime.h>

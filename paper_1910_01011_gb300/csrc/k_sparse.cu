@@ -1723,7 +1723,12 @@ static int cocg_solve(bem_ctx* ctx, int n_sys, int shifts = 1) {
         // Three domains of at most 2,048 vertices, 128 / 32 systems: 141 / 59 us
         // per application (one CTA per system on vectors in memory 189, clusters
         // 85 us); one domain of 642 vertices, 8 and 2 systems: 24 us on average
-        // (clusters 48 us).
+        // (clusters 48 us).  Above 2,048 vertices, whole solves of 60 iterations
+        // with one domain and 1 / 16 / 32 right-hand sides (8, 128, 256 systems
+        // and the closing ones): 2,532 vertices 38 / 53 / 75 ms (clusters, and one
+        // CTA per system on vectors in memory where they are many: 51 / 86 / 135
+        // ms), 3,520 vertices 53 / 71 / 106 ms (57 / 102 / 202 ms), 4,016 vertices
+        // 60 / 90 / 124 ms (70 / 120 / 251 ms).
         if (mode <= 1 && o->max_dom_nv <= LS_MAX_ROWS && o->n * o->ell_w < (1ll << 31)) {
             if (ctas > 152) CK(launch_local32<2>(b, n_sys, o->ell_w, o->max_dom_nv, ctx->stream));
             else CK(launch_local32<1>(b, n_sys, o->ell_w, o->max_dom_nv, ctx->stream));
