@@ -23,6 +23,7 @@
 #include <type_traits>
 
 #include "internal.h"
+#include "launch.cuh"
 #include "pair_math.h"
 
 namespace gbem {
@@ -76,31 +77,6 @@ __device__ __forceinline__ void mbar_wait_bounded(uint64_t* b, uint32_t parity, 
             return;
         }
     }
-}
-
-// The kernels of one product overlap at their ends: each is launched as soon as
-// every CTA of the one before has called dependents_may_start, does what needs
-// none of that one's results (tile-pair tables, near pairs), and waits in
-// inputs_ready for it to have completed.  A kernel calls dependents_may_start
-// only after its own wait, so whatever runs early follows every kernel but the
-// last.  (Launched without the attribute of launch_after, the wait returns at once.)
-// A product of 300 triangles, all latency: 59.4 -> 48.1 us; 8,172 triangles 4.93 -> 4.91 ms.
-__device__ __forceinline__ void inputs_ready() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
-template <class Args>
-static cudaError_t launch_after(void (*kernel)(Args), dim3 grid, int threads, size_t smem, cudaStream_t s, const Args& a) {
-    cudaLaunchConfig_t c{};
-    c.gridDim = grid;
-    c.blockDim = dim3((unsigned)threads);
-    c.dynamicSmemBytes = smem;
-    c.stream = s;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    c.attrs = &at;
-    c.numAttrs = 1;
-    return cudaLaunchKernelEx(&c, kernel, a);
 }
 
 // x - 2 pi round(x / 2 pi) in FP64 (2 pi split in two doubles), as float.

@@ -40,17 +40,22 @@
 // B = [Xr | Xi] and [-Xi | Xr] on the same accumulators.
 //
 // What binds it is reading A once (16 N^2 bytes): A's bytes are stored in the
-// order in which a CTA reads them (blocks of 128 rows x 32 of K x 16 digit
-// planes, 64 KB, one bulk copy each), four warps turn them into BF16 pairs
-// (a byte permute and one subtraction per two digits) and put them into
-// tensor memory as the A operand, so shared memory holds them only once, as
-// bytes.  Every CTA takes an equal run of 256-wide units across row tiles (as
-// in k_gemm.cu), and pieces of a tile are added in FP64.
+// order in which a CTA reads them (stages of 128 rows x 32 of K x 16 digit
+// planes, 64 KB, in two bulk copies, real and imaginary digits), four warps turn
+// them into BF16 pairs (a byte permute and one subtraction per two digits) and
+// put them into tensor memory as the A operand, so shared memory holds them only
+// once, as bytes.  Every CTA takes an equal run of stages across row tiles, and
+// pieces of a tile are added in FP64.  The copies of A and the set-up of a CTA do
+// not wait for the vectors' digits, and where the accumulators take half of their
+// columns (up to eight vectors) a second set takes the next unit while the first
+// is read.  With whole units per CTA (15 for some, 14 for others), one set of
+// accumulators, 64 KB copies and two more launches, one vector took 223 us on
+// N = 8,200 and 36 us on N = 324 (FP32 pairs 193 and 28 us), now 193 and 20 us.
 //
-// N = 10,776, 16 vectors: a call takes 422 us (4.4 TB/s of A; the instructions of
-// a step take 1,306 cycles, its bytes 1,490 at the copy rate) against 4,550 us in
-// FP32 pairs, and 430 us with one power of two per vector and row and sums in FP32
-// pairs.  Error of the product with a smooth vector on 20,484 unknowns, against
+// N = 10,776, 16 vectors: a call takes 410 us (4.5 TB/s of A; the instructions of
+// half a stage take 1,306 cycles, its bytes 1,490 at the copy rate) against 4,550
+// us in FP32 pairs; N = 10,608, one vector 306 us (5.9 TB/s) against 403 us.
+// Error of the product with a smooth vector on 20,484 unknowns, against
 // 128-bit sums of the entries: 3e-14, and 2^-47.7 of a row's sum |a| |x| at most
 // (FP32 pairs 2.4e-13 and 2^-43.7; one power of two per vector and row 6.7e-13 and
 // 2^-40.1).
@@ -65,6 +70,7 @@
 
 #include "ctx.h"
 #include "internal.h"
+#include "launch.cuh"
 
 namespace gbem {
 
@@ -76,7 +82,6 @@ constexpr int DG_UNIT = DG_K * DG_STEPS;   // K of a unit: 256
 constexpr int DG_CTAS = 152;
 constexpr int DG_PLANE = DG_M * DG_K;      // bytes of one digit plane of a stage
 constexpr int DG_ABYTES = 2 * DG * DG_PLANE;
-constexpr int DG_STAGES = 2;
 constexpr int DG_WARPS = 10;               // 0 copies, 1 MMA, 2-5 digits to BF16, 6-9 accumulators
 constexpr int DG_NONE = INT_MIN / 4;       // exponent of a zero row, column or vector
 constexpr int DG_BAD = INT_MAX / 4;        // of one with an infinity or a NaN
@@ -87,14 +92,17 @@ struct DgCfg {
     static constexpr int HN = NC / 2;
     static constexpr int BROWS = DG * NC;              // B rows: digit j, column n at j NC + n
     static constexpr int BBYTES = 2 * BROWS * DG_K * 2;  // [Xr | Xi] and [-Xi | Xr] of a stage
+    static constexpr int ACC = 256 / (DG * NC);        // sets of accumulators in 256 columns of tensor memory
+    static constexpr int RING = NC == 16 ? 5 : 4;      // half stages (the real or the imaginary digits of A) in flight
     struct Smem {
-        alignas(1024) uint8_t a[DG_STAGES][DG_ABYTES];
-        alignas(1024) uint8_t b[DG_STAGES][BBYTES];
+        alignas(1024) uint8_t a[RING][DG_ABYTES / 2];
+        alignas(1024) uint8_t b[RING][BBYTES / 2];
         double sum[NC][DG_M];                          // of the CTA's units of a tile
-        uint64_t full[DG_STAGES], empty[DG_STAGES];    // copies landed; bytes converted (4 warps) and B used (MMA)
-        uint64_t tfull[2], tempty[2];                  // A operand of one K = 16 step in tensor memory
-        uint64_t dfull, dempty;                        // accumulators of a unit
+        uint64_t full[RING], empty[RING];              // copies landed; bytes converted (4 warps) and B used (MMA)
+        uint64_t tfull[2], tempty[2];                  // A operand of a half stage in tensor memory
+        uint64_t dfull[ACC], dempty[ACC];              // accumulators of a unit
         uint32_t tmem;
+        int vmax[HN];
     };
     static_assert(sizeof(Smem) + 1024 <= 227 * 1024, "digits smem");
 };
@@ -198,41 +206,34 @@ __global__ void __launch_bounds__(256) dg_digits_kernel(const double2* __restric
     }
 }
 
-// ve[r][u] = largest exponent of x_r 2^col in unit u, vm[r] (set to less than any before) of all; grid (units, vectors)
-__global__ void __launch_bounds__(DG_UNIT) dg_vecexp_kernel(const double2* __restrict__ x, int64_t n, const int* __restrict__ col,
-                                                            int* __restrict__ ve, int* vm) {
+// Digits of R <= hn vectors as the B operand: blocks of one stage, [part][digit HN*2 + column][32 K], 64-byte rows
+// in the 64-byte swizzle; vectors above R and K above n are zero.  ve[r][u] = largest exponent of x_r 2^col in unit u.
+// Grid (units, hn), a thread an entry.
+__global__ void __launch_bounds__(DG_UNIT) dg_vector_kernel(const double2* __restrict__ x, int64_t n, int64_t kpad, int R, int hn,
+                                                            const int* __restrict__ col, int* __restrict__ ve,
+                                                            uint8_t* __restrict__ out) {
     __shared__ int sh[DG_UNIT / 32];
+    dependents_may_start();
     const int64_t j = (int64_t)blockIdx.x * DG_UNIT + threadIdx.x;
-    int e = DG_NONE;
-    if (j < n) {
-        const int t = dg_exp2(x[(int64_t)blockIdx.y * n + j]), c = col[j];
+    const int r = blockIdx.y;
+    double2 v = make_double2(0, 0);
+    int c = DG_NONE, e = DG_NONE;
+    if (r < R && j < n) {
+        v = x[(int64_t)r * n + j];
+        c = col[j];
+        const int t = dg_exp2(v);
         if (t != DG_NONE) e = t == DG_BAD || c == DG_BAD ? DG_BAD : c == DG_NONE ? DG_NONE : t + c;
     }
     e = warp_max(e);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = e;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < DG_UNIT / 32; w++) e = max(e, sh[w]);
-        ve[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = e;
-        atomicMax(&vm[blockIdx.y], e);
-    }
-}
-
-// Digits of R <= HN vectors as the B operand: blocks of one stage, [part][digit HN*2 + column][32 K], 64-byte rows
-// in the 64-byte swizzle; vectors above R and K above n are zero.  Thread: one entry of one vector.
-__global__ void dg_vecdigits_kernel(const double2* __restrict__ x, int64_t n, int64_t kpad, int R, int hn,
-                                    const int* __restrict__ col, const int* __restrict__ ve, int nch,
-                                    uint8_t* __restrict__ out) {
-    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int r = blockIdx.y;
+#pragma unroll
+    for (int w = 0; w < DG_UNIT / 32; w++) e = max(e, sh[w]);
+    if (r < R && threadIdx.x == 0) ve[(int64_t)r * gridDim.x + blockIdx.x] = e;
     if (j >= kpad) return;
-    double2 v = make_double2(0, 0);
     int s = 0;
-    const int e = r < R ? ve[(int64_t)r * nch + j / DG_UNIT] : DG_NONE;
-    if (j < n && e != DG_NONE && e != DG_BAD && col[j] != DG_NONE) {
-        v = x[(int64_t)r * n + j];
-        s = e + 2 - col[j];
-    }
+    if (e == DG_NONE || e == DG_BAD || c == DG_NONE) v = make_double2(0, 0);
+    else s = e + 2 - c;
     const unsigned long long u[2] = {dg_biased(v.x, s), dg_biased(v.y, s)};
     const int brows = DG * 2 * hn, k = (int)(j % DG_K);
     uint8_t* blk = out + j / DG_K * (int64_t)(2 * brows * DG_K * 2);
@@ -325,23 +326,33 @@ __device__ __forceinline__ void d_ld8(uint32_t t, float (&v)[8]) {
 struct DgArgs {
     const uint8_t* A;     // [row tile][K block][plane][row][32]
     const uint8_t* B;     // [K block][part][row][32 bf16]
-    int nkb, nch, units, pieces, m, R;
+    int nkb, stages, pieces, m, R;  // K blocks; stages (row tiles x K blocks)
     int64_t mpad;
-    const int *rowm, *rowe, *vm, *ve;
+    const int *rowm, *rowe, *ve;
     double2* part;        // [row tile][piece][HN][128]
     double2* Y;           // [R][m]
     int* err;
 };
 
-__host__ __device__ inline int dg_first_unit(int units, int ctas, int b) { return (int)((int64_t)units * b / ctas); }
-// the first of the CTAs that hold units of `tile`
-__host__ __device__ inline int dg_first_cta(int units, int ctas, int nch, int tile) {
-    const int u = tile * nch;
-    int b = (int)((int64_t)u * ctas / units);
-    while (b + 1 < ctas && dg_first_unit(units, ctas, b + 1) <= u) b++;
-    while (b > 0 && dg_first_unit(units, ctas, b) > u) b--;
+__host__ __device__ inline int dg_first_stage(int stages, int ctas, int b) { return (int)((int64_t)stages * b / ctas); }
+// the first of the CTAs that hold stages of `tile`
+__host__ __device__ inline int dg_first_cta(int stages, int ctas, int nkb, int tile) {
+    const int g = tile * nkb;
+    int b = (int)((int64_t)g * ctas / stages);
+    while (b + 1 < ctas && dg_first_stage(stages, ctas, b + 1) <= g) b++;
+    while (b > 0 && dg_first_stage(stages, ctas, b) > g) b--;
     return b;
 }
+// The part of a unit that starts at stage g of a run up to g1: its row tile, unit and K blocks.
+struct DgSpan {
+    int tile, unit, kb0, kb1;
+    __device__ __forceinline__ DgSpan(int g, int g1, int nkb) {
+        tile = g / nkb;
+        kb0 = g - tile * nkb;
+        unit = kb0 / DG_STEPS;
+        kb1 = min(min(nkb, (unit + 1) * DG_STEPS), kb0 + g1 - g);
+    }
+};
 
 template <int NC>
 __global__ void __launch_bounds__(DG_WARPS * 32, 1) digits_gemm_kernel(const DgArgs a) {
@@ -350,9 +361,9 @@ __global__ void __launch_bounds__(DG_WARPS * 32, 1) digits_gemm_kernel(const DgA
     typename C::Smem& sm =
         *reinterpret_cast<typename C::Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int u0 = dg_first_unit(a.units, gridDim.x, blockIdx.x), u1 = dg_first_unit(a.units, gridDim.x, blockIdx.x + 1);
+    const int g0 = dg_first_stage(a.stages, gridDim.x, blockIdx.x), g1 = dg_first_stage(a.stages, gridDim.x, blockIdx.x + 1);
     if (threadIdx.x == 0) {
-        for (int s = 0; s < DG_STAGES; s++) {
+        for (int s = 0; s < C::RING; s++) {
             d_init(&sm.full[s], 1);
             d_init(&sm.empty[s], 5);
         }
@@ -360,8 +371,10 @@ __global__ void __launch_bounds__(DG_WARPS * 32, 1) digits_gemm_kernel(const DgA
             d_init(&sm.tfull[b], 4);
             d_init(&sm.tempty[b], 1);
         }
-        d_init(&sm.dfull, 1);
-        d_init(&sm.dempty, 4);
+        for (int d = 0; d < C::ACC; d++) {
+            d_init(&sm.dfull[d], 1);
+            d_init(&sm.dempty[d], 4);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 2) {
@@ -371,28 +384,30 @@ __global__ void __launch_bounds__(DG_WARPS * 32, 1) digits_gemm_kernel(const DgA
     DG_FENCE_BEFORE;
     __syncthreads();
     DG_FENCE_AFTER;
-    const uint32_t tmem = sm.tmem;      // accumulators: columns 0 .. 8 NC - 1
-    const uint32_t ta = tmem + 256;     // two A operands of 16 planes x 8 columns
+    const uint32_t tmem = sm.tmem;      // accumulators: sets of 8 NC columns
+    const uint32_t ta = tmem + 256;     // two A operands: [K = 16 step][plane] x 8 columns
 
     if (warp == 0) {
         if (lane == 0) {
             int s = 0;
             uint32_t ph = 1;
             bool ok = true;
-            for (int u = u0; u < u1 && ok; u++) {
-                const int tile = u / a.nch, c = u - tile * a.nch, ke = min(a.nkb, (c + 1) * DG_STEPS);
-                for (int kb = c * DG_STEPS; kb < ke; kb++) {
+            for (int g = g0; g < g1 && ok;) {
+                const DgSpan w(g, g1, a.nkb);
+                for (int h = 2 * w.kb0; h < 2 * w.kb1; h++) {
                     if (!(ok = d_wait(&sm.empty[s], ph, a.err))) break;
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(d_u32(&sm.full[s])),
-                                 "r"(DG_ABYTES + C::BBYTES)
+                                 "r"((DG_ABYTES + C::BBYTES) / 2)
                                  : "memory");
-                    d_bulk(sm.a[s], a.A + ((int64_t)tile * a.nkb + kb) * DG_ABYTES, DG_ABYTES, &sm.full[s]);
-                    d_bulk(sm.b[s], a.B + (int64_t)kb * C::BBYTES, C::BBYTES, &sm.full[s]);
-                    if (++s == DG_STAGES) {
+                    d_bulk(sm.a[s], a.A + ((int64_t)w.tile * a.nkb * 2 + h) * (DG_ABYTES / 2), DG_ABYTES / 2, &sm.full[s]);
+                    if (g == g0 && h == 2 * w.kb0) inputs_ready();  // (A was there before the vectors)
+                    d_bulk(sm.b[s], a.B + (int64_t)h * (C::BBYTES / 2), C::BBYTES / 2, &sm.full[s]);
+                    if (++s == C::RING) {
                         s = 0;
                         ph ^= 1;
                     }
                 }
+                g += w.kb1 - w.kb0;
             }
         }
     } else if (warp == 1) {
@@ -400,38 +415,38 @@ __global__ void __launch_bounds__(DG_WARPS * 32, 1) digits_gemm_kernel(const DgA
             int s = 0, b = 0;
             uint32_t ph = 0, tph = 0;
             bool ok = true;
-            for (int u = u0; u < u1 && ok; u++) {
-                const int c = u % a.nch, kb0 = c * DG_STEPS, ke = min(a.nkb, kb0 + DG_STEPS);
-                if (u > u0) {
-                    if (!(ok = d_wait(&sm.dempty, (uint32_t)((u - u0 - 1) & 1), a.err))) break;
+            int d = 0;
+            uint32_t dph = 1;
+            for (int g = g0; g < g1 && ok;) {
+                const DgSpan w(g, g1, a.nkb);
+                if (!(ok = d_wait(&sm.dempty[d], dph, a.err))) break;  // (at once the first time)
+                DG_FENCE_AFTER;
+                const uint32_t acc = tmem + d * DG * NC;
+                for (int h = 2 * w.kb0; h < 2 * w.kb1; h++) {
+                    if (!(ok = d_wait(&sm.full[s], ph, a.err) && d_wait(&sm.tfull[b], tph, a.err))) break;
                     DG_FENCE_AFTER;
-                }
-                for (int kb = kb0; kb < ke && ok; kb++) {
-                    if (!(ok = d_wait(&sm.full[s], ph, a.err))) break;
                     const uint32_t bs = d_u32(sm.b[s]);
-                    for (int kk = 0; kk < 2; kk++) {
-                        if (!(ok = d_wait(&sm.tfull[b], tph, a.err))) break;
-                        DG_FENCE_AFTER;
 #pragma unroll
-                        for (int p = 0; p < 2; p++) {
-                            const uint64_t bd = d_desc(bs + p * C::BROWS * 64 + kk * 32);
+                    for (int kk = 0; kk < 2; kk++)
 #pragma unroll
-                            for (int i = 0; i < DG; i++)
-                                d_mma(tmem + i * NC, ta + b * 128 + (p * DG + i) * 8, bd, NC * (DG - i),
-                                      kb > kb0 || kk > 0 || p > 0 || i > 0);
-                        }
-                        d_commit(&sm.tempty[b]);
-                        b ^= 1;
-                        if (b == 0) tph ^= 1;
-                    }
-                    if (!ok) break;
+                        for (int i = 0; i < DG; i++)
+                            d_mma(acc + i * NC, ta + b * 128 + (kk * DG + i) * 8, d_desc(bs + kk * 32), NC * (DG - i),
+                                  h > 2 * w.kb0 || kk > 0 || i > 0);
+                    d_commit(&sm.tempty[b]);
                     d_commit(&sm.empty[s]);
-                    if (++s == DG_STAGES) {
+                    b ^= 1;
+                    if (b == 0) tph ^= 1;
+                    if (++s == C::RING) {
                         s = 0;
                         ph ^= 1;
                     }
                 }
-                if (ok) d_commit(&sm.dfull);
+                if (ok) d_commit(&sm.dfull[d]);
+                if (++d == C::ACC) {
+                    d = 0;
+                    dph ^= 1;
+                }
+                g += w.kb1 - w.kb0;
             }
         }
     } else if (warp < 6) {
@@ -441,53 +456,65 @@ __global__ void __launch_bounds__(DG_WARPS * 32, 1) digits_gemm_kernel(const DgA
         const __nv_bfloat162 off = __floats2bfloat162_rn(192.f, 192.f);
         int s = 0, b = 0;
         uint32_t ph = 0, tph = 1;
-        for (int u = u0; u < u1; u++) {
-            const int c = u % a.nch, kb0 = c * DG_STEPS, ke = min(a.nkb, kb0 + DG_STEPS);
-            for (int kb = kb0; kb < ke; kb++) {
-                d_wait(&sm.full[s], ph, a.err);
-                const uint8_t* src = sm.a[s] + row * DG_K;
+        for (int h = 2 * g0; h < 2 * g1; h++) {
+            d_wait(&sm.full[s], ph, a.err);
+            const uint8_t* src = sm.a[s] + row * DG_K;
+            d_wait(&sm.tempty[b], tph, a.err);
+            DG_FENCE_AFTER;
+#pragma unroll 2
+            for (int p = 0; p < DG; p++)
+#pragma unroll
                 for (int kk = 0; kk < 2; kk++) {
-                    d_wait(&sm.tempty[b], tph, a.err);
-                    DG_FENCE_AFTER;
-#pragma unroll 4
-                    for (int p = 0; p < 2 * DG; p++) {
-                        const uint4 v = *reinterpret_cast<const uint4*>(src + p * DG_PLANE + ((kk * 16) ^ sw));
-                        const uint32_t in[4] = {v.x, v.y, v.z, v.w};
-                        uint32_t r[8];
+                    const uint4 v = *reinterpret_cast<const uint4*>(src + p * DG_PLANE + ((kk * 16) ^ sw));
+                    const uint32_t in[4] = {v.x, v.y, v.z, v.w};
+                    uint32_t r[8];
 #pragma unroll
-                        for (int w = 0; w < 4; w++)
+                    for (int w = 0; w < 4; w++)
 #pragma unroll
-                            for (int h = 0; h < 2; h++) {
-                                const uint32_t t = __byte_perm(in[w], 0x43434343u, h ? 0x4342 : 0x4140);
-                                const __nv_bfloat162 d = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&t), off);
-                                r[2 * w + h] = *reinterpret_cast<const uint32_t*>(&d);
-                            }
-                        d_st8(lt + b * 128 + p * 8, r);
-                    }
-                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                    DG_FENCE_BEFORE;
-                    __syncwarp();
-                    if (lane == 0) d_arrive(&sm.tfull[b]);
-                    b ^= 1;
-                    if (b == 0) tph ^= 1;
+                        for (int hb = 0; hb < 2; hb++) {
+                            const uint32_t t = __byte_perm(in[w], 0x43434343u, hb ? 0x4342 : 0x4140);
+                            const __nv_bfloat162 d = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&t), off);
+                            r[2 * w + hb] = *reinterpret_cast<const uint32_t*>(&d);
+                        }
+                    d_st8(lt + b * 128 + (kk * DG + p) * 8, r);
                 }
-                __syncwarp();
-                if (lane == 0) d_arrive(&sm.empty[s]);
-                if (++s == DG_STAGES) {
-                    s = 0;
-                    ph ^= 1;
-                }
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+            DG_FENCE_BEFORE;
+            __syncwarp();
+            if (lane == 0) {
+                d_arrive(&sm.tfull[b]);
+                d_arrive(&sm.empty[s]);
+            }
+            b ^= 1;
+            if (b == 0) tph ^= 1;
+            if (++s == C::RING) {
+                s = 0;
+                ph ^= 1;
             }
         }
     } else {
         const int q = warp & 3, r = q * 32 + lane;
         const uint32_t ld = tmem + ((uint32_t)(q * 32) << 16);
+        // the largest exponent of each vector: eight lanes a vector
+        inputs_ready();
+        dependents_may_start();
+        const int nch = (a.nkb + DG_STEPS - 1) / DG_STEPS;
+        for (int j = (warp - 6) * 4 + lane / 8; j < a.R; j += 16) {
+            int e = DG_NONE;
+            for (int u = lane % 8; u < nch; u += 8) e = max(e, a.ve[(int64_t)j * nch + u]);
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffu << (lane & 24), e, o));
+            if (lane % 8 == 0) sm.vmax[j] = e;
+        }
+        asm volatile("bar.sync 1, 128;" ::: "memory");  // (these four warps)
         bool fresh = true;  // no unit of the tile in `sum` yet
-        for (int u = u0; u < u1; u++) {
-            const int tile = u / a.nch, c = u - tile * a.nch;
-            const int64_t row = (int64_t)tile * DG_M + r;
-            const int er = max(a.rowe[c * a.mpad + row] - a.rowm[row], -2000);  // -2000: nothing in this unit
-            d_wait(&sm.dfull, (uint32_t)((u - u0) & 1), a.err);
+        int d = 0;
+        uint32_t dph = 0;
+        for (int g = g0; g < g1;) {
+            const DgSpan w(g, g1, a.nkb);
+            const int64_t row = (int64_t)w.tile * DG_M + r;
+            const int er = max(a.rowe[w.unit * a.mpad + row] - a.rowm[row], -2000);  // -2000: nothing in this unit
+            d_wait(&sm.dfull[d], dph, a.err);
             DG_FENCE_AFTER;
             // sums in 2^-49 of the first accumulator, exact, or from 2^62 on (bit set in `large`) rounded to 2^-41
             long long y[NC];
@@ -500,7 +527,7 @@ __global__ void __launch_bounds__(DG_WARPS * 32, 1) digits_gemm_kernel(const DgA
 #pragma unroll
                     for (int s = 0; s < 4; s++) {
                         float v[8];
-                        d_ld8(ld + (4 * h + s) * NC + j0, v);
+                        d_ld8(ld + (d * DG + 4 * h + s) * NC + j0, v);
 #pragma unroll
                         for (int j = 0; j < 8; j++) t[h][j] = (s ? t[h][j] * 128 : 0) + __float2int_rn(v[j]);
                     }
@@ -513,14 +540,19 @@ __global__ void __launch_bounds__(DG_WARPS * 32, 1) digits_gemm_kernel(const DgA
             }
             DG_FENCE_BEFORE;
             __syncwarp();
-            if (lane == 0) d_arrive(&sm.dempty);
-            const bool end = u + 1 == u1 || (u + 1) % a.nch == 0;
-            const int piece = blockIdx.x - dg_first_cta(a.units, gridDim.x, a.nch, tile);
-            double2* out = a.part + (int64_t)(tile * a.pieces + piece) * C::HN * DG_M + r;
+            if (lane == 0) d_arrive(&sm.dempty[d]);
+            if (++d == C::ACC) {
+                d = 0;
+                dph ^= 1;
+            }
+            g += w.kb1 - w.kb0;
+            const bool end = g == g1 || w.kb1 == a.nkb;
+            const int piece = blockIdx.x - dg_first_cta(a.stages, gridDim.x, a.nkb, w.tile);
+            double2* out = a.part + (int64_t)(w.tile * a.pieces + piece) * C::HN * DG_M + r;
 #pragma unroll
             for (int j = 0; j < C::HN; j++) {
                 if (j >= a.R) break;
-                const int e = er + max(a.ve[(int64_t)j * a.nch + c] - a.vm[j], -2000);
+                const int e = er + max(a.ve[(int64_t)j * nch + w.unit] - sm.vmax[j], -2000);
                 const double fx = e < -1000 ? 0.0 : __hiloint2double((1023 + e + (large >> j & 1) * 8) << 20, 0);
                 const double fy = e < -1000 ? 0.0 : __hiloint2double((1023 + e + (large >> (C::HN + j) & 1) * 8) << 20, 0);
                 double2 s = fresh ? make_double2(0, 0) : make_double2(sm.sum[j][r], sm.sum[C::HN + j][r]);
@@ -545,19 +577,30 @@ __global__ void __launch_bounds__(DG_WARPS * 32, 1) digits_gemm_kernel(const DgA
     }
 }
 
-// Y = the pieces of every row added in CTA order, times the powers of two.
-__global__ void dg_finish_kernel(DgArgs a, int ctas, int hn) {
-    const int row = blockIdx.x * blockDim.x + threadIdx.x, r = blockIdx.y;
+// Y = the pieces of every row added in CTA order, times the powers of two.  Grid (blocks of rows, vectors).
+struct DgFinish {
+    DgArgs a;
+    int ctas, hn;
+};
+constexpr int DG_FT = 128;
+__global__ void __launch_bounds__(DG_FT) dg_finish_kernel(DgFinish f) {
+    const DgArgs& a = f.a;
+    const int row = blockIdx.x * DG_FT + threadIdx.x, r = blockIdx.y, lane = threadIdx.x & 31;
+    const int nch = (a.nkb + DG_STEPS - 1) / DG_STEPS;
+    const int tile = min(row, a.m - 1) / DG_M, first = dg_first_cta(a.stages, f.ctas, a.nkb, tile);
+    inputs_ready();
+    int ev = DG_NONE;
+    for (int u = lane; u < nch; u += 32) ev = max(ev, a.ve[(int64_t)r * nch + u]);
+    ev = warp_max(ev);
     if (row >= a.m) return;
-    const int tile = row / DG_M, first = dg_first_cta(a.units, ctas, a.nch, tile);
     double x = 0, y = 0;
     for (int p = 0; p < a.pieces; p++) {
-        if (first + p >= ctas || dg_first_unit(a.units, ctas, first + p) >= (tile + 1) * a.nch) break;
-        const double2 v = a.part[((int64_t)(tile * a.pieces + p) * hn + r) * DG_M + row % DG_M];
+        if (first + p >= f.ctas || dg_first_stage(a.stages, f.ctas, first + p) >= (tile + 1) * a.nkb) break;
+        const double2 v = a.part[((int64_t)(tile * a.pieces + p) * f.hn + r) * DG_M + row % DG_M];
         x += v.x;
         y += v.y;
     }
-    const int er = a.rowm[row], ev = a.vm[r];
+    const int er = a.rowm[row];
     if (er == DG_BAD || ev == DG_BAD) x = y = __longlong_as_double(0x7ff8000000000000ll);
     else if (er == DG_NONE || ev == DG_NONE) x = y = 0;
     else {
@@ -580,17 +623,20 @@ size_t digits_exp_bytes(int64_t n) { return (size_t)(digits_kpad(n) + digits_mpa
 
 constexpr int DG_TILES = 2;  // row tiles converted at a time
 static int dg_hn(int64_t R) { return R <= 8 ? 8 : 16; }
-static int dg_pieces(int units, int ctas, int nch) {
-    const int q = units / ctas;  // a CTA holds q or q + 1 units
-    return (nch + q - 1) / q + 1;
+// CTAs of a product: every one a run of equal length, at least two stages for
+// up to eight vectors and four for more, whose pieces are dearer (N = 1,284, 16
+// vectors: 48 us with runs of three stages, 38 us with four, 39 us with eight).
+static int dg_ctas(int stages, int hn) { return std::max(1, std::min(DG_CTAS, stages / (hn == 8 ? 2 : 4))); }
+static int dg_pieces(int stages, int nkb, int hn) {
+    const int q = stages / dg_ctas(stages, hn);  // a CTA holds q or q + 1 stages
+    return (nkb + q - 1) / q + 1;
 }
 // scratch of a product of R vectors (B operand, exponents, pieces), and of the conversion
 size_t digits_work_bytes(int64_t n, int64_t R) {
     const int hn = dg_hn(R);
-    const int nkb = (int)(digits_kpad(n) / DG_K), nch = (nkb + DG_STEPS - 1) / DG_STEPS;
-    const int tiles = (int)(digits_mpad(n) / DG_M), units = tiles * nch, ctas = std::min(DG_CTAS, units);
-    return (size_t)nkb * 2 * DG * 2 * hn * DG_K * 2 + (size_t)tiles * dg_pieces(units, ctas, nch) * hn * DG_M * 16 +
-           16 * (1 + nch) * sizeof(int);
+    const int nkb = (int)(digits_kpad(n) / DG_K), tiles = (int)(digits_mpad(n) / DG_M), stages = tiles * nkb;
+    return (size_t)nkb * 2 * DG * 2 * hn * DG_K * 2 + (size_t)tiles * dg_pieces(stages, nkb, hn) * hn * DG_M * 16 +
+           16 * (size_t)dg_units(n) * sizeof(int);
 }
 size_t digits_convert_bytes(int64_t n) { return (size_t)DG_TILES * DG_M * digits_kpad(n) * 16; }
 
@@ -635,8 +681,7 @@ static cudaError_t launch_digits(const DgArgs& a, unsigned ctas, cudaStream_t s)
     static const cudaError_t attr_e =
         cudaFuncSetAttribute(digits_gemm_kernel<NC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (attr_e != cudaSuccess) return attr_e;
-    digits_gemm_kernel<NC><<<ctas, DG_WARPS * 32, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_after(digits_gemm_kernel<NC>, dim3(ctas), DG_WARPS * 32, smem, s, a);
 }
 
 // Y [R][n] = A X [R][n] with A as digits (digits_prepare); work: digits_work_bytes(n, min(R, 16)).
@@ -646,11 +691,10 @@ int digits_gemm(bem_ctx* ctx, const void* A, const int* exps, int64_t n, const d
     DgArgs a{};
     a.A = (const uint8_t*)A;
     a.nkb = (int)(kpad / DG_K);
-    a.nch = (a.nkb + DG_STEPS - 1) / DG_STEPS;
     const int tiles = (int)(mpad / DG_M);
-    a.units = tiles * a.nch;
-    const int ctas = std::min(DG_CTAS, a.units);
-    a.pieces = dg_pieces(a.units, ctas, a.nch);
+    a.stages = tiles * a.nkb;
+    const int ctas = dg_ctas(a.stages, hn);
+    a.pieces = dg_pieces(a.stages, a.nkb, hn);
     a.m = (int)n;
     a.mpad = mpad;
     a.rowm = exps + kpad;
@@ -660,23 +704,19 @@ int digits_gemm(bem_ctx* ctx, const void* A, const int* exps, int64_t n, const d
     const size_t bb = (size_t)a.nkb * 2 * DG * 2 * hn * DG_K * 2;
     a.B = b;
     a.part = (double2*)(b + bb);
-    int* vm = (int*)(a.part + (size_t)tiles * a.pieces * hn * DG_M);
-    int* ve = vm + 16;
-    a.vm = vm;
+    int* ve = (int*)(a.part + (size_t)tiles * a.pieces * hn * DG_M);
     a.ve = ve;
     for (int64_t r0 = 0; r0 < R; r0 += hn) {
         const int nr = (int)std::min<int64_t>(hn, R - r0);
-        const double2* x = X + r0 * n;
         a.R = nr;
         a.Y = Y + r0 * n;
-        DCK(cudaMemsetAsync(vm, 0x80, 16 * sizeof(int), ctx->stream));  // below every exponent
-        dg_vecexp_kernel<<<dim3((unsigned)a.nch, (unsigned)nr), DG_UNIT, 0, ctx->stream>>>(x, n, exps, ve, vm);
-        dg_vecdigits_kernel<<<dim3((unsigned)((kpad + 127) / 128), (unsigned)hn), 128, 0, ctx->stream>>>(x, n, kpad, nr, hn, exps, ve, a.nch, b);
+        dg_vector_kernel<<<dim3((unsigned)dg_units(n), (unsigned)hn), DG_UNIT, 0, ctx->stream>>>(X + r0 * n, n, kpad, nr, hn,
+                                                                                               exps, ve, b);
         DCK(cudaGetLastError());
         DCK(hn == 8 ? launch_digits<16>(a, (unsigned)ctas, ctx->stream) : launch_digits<32>(a, (unsigned)ctas, ctx->stream));
-        dg_finish_kernel<<<dim3((unsigned)((n + 255) / 256), (unsigned)nr), 256, 0, ctx->stream>>>(a, ctas, hn);
-        DCK(cudaGetLastError());
-        ctx->launches += 4;
+        const DgFinish f{a, ctas, hn};
+        DCK(launch_after(dg_finish_kernel, dim3((unsigned)((n + DG_FT - 1) / DG_FT), (unsigned)nr), DG_FT, 0, ctx->stream, f));
+        ctx->launches += 3;
     }
     return BEM_OK;
 }

@@ -329,3 +329,21 @@ def test_fp64_assembled_hypersingular_rows(api, level):
         W = A[N // 2:, N // 2:].real.astype(np.longdouble)
         left.append(np.mean(np.abs(W.sum(axis=1)) / np.sqrt((W ** 2).sum(axis=1))))
     assert left[0] < 2 * left[1], [float(v) for v in left]
+
+
+@pytest.mark.parametrize("name,R", [("sphere", 1), ("sphere", 9), ("two", 2), ("two", 16), ("two1", 3), ("two1", 12)])
+def test_fp64_assembled_digits_short_runs(api, name, R):
+    """One block of 32 columns in all (24 unknowns), two (48), and runs of two
+    and four blocks that start inside a unit of 256 columns and whose pieces
+    make up a row tile (168): by the product's own columns, whose digits are
+    exact, to 2^-54 of the largest scaled entry of a row and of a vector; rows
+    here range over less than 2^12."""
+    s = {"sphere": lambda: scenes.sphere_scene(0), "two": lambda: scenes.two_sphere_scene(0),
+         "two1": lambda: scenes.two_sphere_scene(1)}[name]()
+    c = api.Context.from_scene(s)
+    A = c.apply(np.eye(c.n_dofs, dtype=np.complex128), precision=api.FP64_ASSEMBLED).T
+    X = np.stack([scenes.smooth_trace_vector(s, r) for r in range(R)])
+    Y = c.apply(X if R > 1 else X[0], precision=api.FP64_ASSEMBLED).reshape(R, -1)
+    c.close()
+    for r in range(R):
+        assert rel(Y[r], A @ X[r]) < 1e-12
