@@ -289,8 +289,9 @@ __global__ void __launch_bounds__(TT) assemble64_kernel(AssembleArgs a, const do
 //     FP32 pairs up to the vertex and FP64 from there.
 // (One thread per target triangle held 54 accumulators, 255 registers and
 // eight warps on an SM with long dependent chains.)
-// New exterior medium of the 4,620-triangle rib scene 114 ms, 135 ms with that
-// kernel (two CTAs with 164 registers an SM; three with 112 spilled).  All of W
+// New exterior medium of the 4,620-triangle rib scene 112.8 ms (114.0 with the
+// sums over a target triangle inside the sums over its vertices), 135 ms with that
+// kernel (two CTAs with 167 registers an SM; three with 112 spilled).  All of W
 // in FP32 pairs took 110 ms, but the entries' error against native FP64, six
 // scenes on average, grew from 1.780e-14 to 1.884e-14 (now 1.778e-14), and row
 // sums of W, which are zero without a wavenumber, fivefold.
@@ -317,6 +318,7 @@ struct AsmDfSmem {
     dfl val[18][TP];          // V, K, K' [source vertex][re, im] of each target point
     dfl mom[3][6][3 * TT];    // [source vertex][V, K, K' (re, im)][corner 32 i + triangle]
     double vsum[2][3 * TT];   // [re, im][corner]: V over the source's vertices
+    double tsum[2][TT];       // ... and over the target triangle's
     dfl nn[TT];               // n.n'
     int vert[3 * TT];         // the target tile's vertices
     unsigned char ptr[3 * TT + 1], cor[3 * TT];  // corners of each
@@ -499,6 +501,10 @@ __device__ __forceinline__ void assembledf_body(const AssembleArgs& a, const Ass
                 atomicAdd(out, co * xr);
                 atomicAdd(out + 1, co * xi);
             };
+            if (tid >= TP - 2 * TT) {
+                const int t = (tid - TP + 2 * TT) % TT, p = (tid - TP + 2 * TT) / TT;
+                sm.tsum[p][t] = sm.vsum[p][t] + sm.vsum[p][TT + t] + sm.vsum[p][2 * TT + t];
+            }
             for (int e = tid; e < 9 * sm.nv; e += TP) {
                 const int v = e / 9, b = e % 3, blk = e % 9 / 3;
                 dfl mr = {0.0f, 0.0f}, mi = {0.0f, 0.0f};
@@ -509,17 +515,19 @@ __device__ __forceinline__ void assembledf_body(const AssembleArgs& a, const Ass
                 put(v, b, blk, blk == 0 ? cf.cV : blk == 1 ? -cf.cK : cf.cKp, (double)mr.h + (double)mr.l,
                     (double)mi.h + (double)mi.l);
             }
-            // 4. W in FP64: three lanes per vertex of the target, the last warps first
+            // 4. W in FP64: three lanes per vertex of the target, the last three warps
+            if (tid < TP / 2) continue;
+            asm volatile("bar.sync 1, 96;" ::: "memory");  // tsum
             const int lane = tid & 31, b = lane % 3;
-            for (int v0 = (TP / 32 - 1 - tid / 32) * 10; v0 < sm.nv; v0 += TP / 32 * 10) {
+            for (int v0 = (TP / 32 - 1 - tid / 32) * 10; v0 < sm.nv; v0 += 30) {
                 const int v = v0 + lane / 3;
                 const bool on = lane < 30 && v < sm.nv;
                 double gr = 0, gi = 0;  // component b of the sum of curl x V over the vertex's triangles
                 dfl vr = {0.0f, 0.0f}, vi = {0.0f, 0.0f};
                 for (int k = on ? sm.ptr[v] : 0, e = on ? sm.ptr[v + 1] : 0; k < e; k++) {
                     const int c = sm.cor[k], t = c % TT;
-                    gr += sm.ct[b][c] * (sm.vsum[0][t] + sm.vsum[0][TT + t] + sm.vsum[0][2 * TT + t]);
-                    gi += sm.ct[b][c] * (sm.vsum[1][t] + sm.vsum[1][TT + t] + sm.vsum[1][2 * TT + t]);
+                    gr += sm.ct[b][c] * sm.tsum[0][t];
+                    gi += sm.ct[b][c] * sm.tsum[1][t];
                     vr = dadd(vr, dmul(sm.nn[t], sm.mom[b][0][c]));
                     vi = dadd(vi, dmul(sm.nn[t], sm.mom[b][1][c]));
                 }
